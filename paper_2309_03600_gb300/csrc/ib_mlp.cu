@@ -11,6 +11,7 @@
 #include <array>
 #include <cmath>
 #include <cstring>
+#include <type_traits>
 #include <vector>
 
 #include "ib_common.cuh"
@@ -43,11 +44,9 @@ struct ib_mlp {
     // training scratch (rows <= cap)
     int64_t cap = 0;
     bf16* act = nullptr;                // hidden activations, [nl - 1][cap][n_hidden]
-    float* y = nullptr;                 // [cap][n_out]
-    float* g32 = nullptr;               // [cap][max dim]
-    bf16* g16a = nullptr;
-    bf16* g16b = nullptr;
-    float* part = nullptr;              // [1024] loss partial sums
+    bf16* g16 = nullptr;                // gradients of the layers' outputs, [nl][cap][max(n_hidden, n_out rounded up to 8)]
+    bf16* xg = nullptr;                 // gathered inputs, [cap][n_in rounded up to 8]
+    float* bpart = nullptr;             // [row tiles of cap][sum of layer widths], then the loss partials
     // inference scratch (rows per chunk)
     int64_t icap = 0;
     bf16* ia = nullptr;
@@ -122,33 +121,44 @@ __global__ void k_features(int ndim, int64_t n0, int64_t n1, int64_t n2, double 
     }
 }
 
-// C = A B with bfloat16 operands and FP32 accumulation on the tensor cores.
-//   A(m, k) = A[row_a(m) * a_sm + k * a_sk], row_a(m) = a_idx ? a_idx[m] : m
-//   B(k, n) = B[row_b(k) * b_sk + n * b_sn], row_b(k) = b_idx ? b_idx[k] : k
-enum { EPI_BIAS_F32 = 0, EPI_BIAS_RELU_BF16 = 1, EPI_RELU_GRAD = 2, EPI_F32 = 3 };
+// C = A B with bfloat16 operands and FP32 accumulation on the tensor cores
+// (mma.sync m16n8k16 over ascending k, so that a sum does not depend on the tiling).
+// A is [m][k]; B is [n][k] (forward: the weights) or [k][n] (input gradients).
+//   128 x 128 x 32 tiles of 8 warps (64 x 32 each), four cp.async stages (82 KB, two
+// blocks per SM), fragments by ldmatrix (.trans for the [k][*] layouts).  Copies are 16
+// bytes where the operand's rows allow it, 8 bytes for rows of 4 j elements (260 network
+// inputs), single elements otherwise.
+//   What bounds the training step is the number of blocks, passes and launches, not the
+// tensor pipe: the epilogues form the loss and its gradient, the ReLU mask and the column
+// sums of the bias gradients, so no FP32 gradient is stored, and the weight gradients of
+// all layers are one launch (k_weight_grad).
+enum { EPI_BIAS_F32 = 0, EPI_BIAS_RELU_BF16 = 1, EPI_RELU_GRAD = 2, EPI_MSE = 3 };
+struct Operand {
+    const bf16* p;
+    int64_t ld;              // elements between rows
+    int rows, ext;           // valid rows; valid elements of a row (copies stay inside)
+};
 struct Gemm {
     int M, N, K;
-    const bf16* A;
-    int64_t a_sm, a_sk;
-    const int64_t* a_idx;
-    const bf16* B;
-    int64_t b_sk, b_sn;
-    const int64_t* b_idx;
-    int mode;
-    const float* bias;      // [N]
-    const bf16* act;        // EPI_RELU_GRAD: forward activation [m][n] (ld act_ld); gradient kept where > 0
-    int64_t act_ld;
-    float* c32;
-    bf16* c16;
+    Operand a, b;
+    const float* bias;       // [N]
+    const bf16* act;         // EPI_RELU_GRAD: forward activation [m][n] (ld ldc); gradient kept where > 0
+    float* c32;              // EPI_BIAS_F32: [m][ldc]
+    bf16* c16;               // [m][ldc]
     int64_t ldc;
+    float* colpart;          // [gridDim.y][N] column sums of the tile's gradient
+    const float* T;          // EPI_MSE: targets [*][N], rows t_idx
+    const int64_t* t_idx;
+    float scale;             // EPI_MSE: 2 / (rows N)
+    float* losspart;         // EPI_MSE: [gridDim.y][gridDim.x] sums of (Y - T)^2
 };
 
-#define GBM 64
-#define GBN 64
+#define GBM 128
+#define GBN 128
 #define GBK 32
-#define GLD (GBK + 8)
-
-__device__ __forceinline__ uint32_t ld_pair(const bf16* p) { return *reinterpret_cast<const uint32_t*>(p); }
+#define GST 4
+#define GLDK (GBK + 8)    // [m][k] tile row (80 bytes: ldmatrix rows fall in distinct banks)
+#define GLDM (GBN + 8)    // [k][n] tile row (272 bytes)
 
 __device__ __forceinline__ void mma_16816(float* d, const uint32_t* a, const uint32_t* b) {
     asm volatile(
@@ -157,168 +167,330 @@ __device__ __forceinline__ void mma_16816(float* d, const uint32_t* a, const uin
         : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
 }
+template <bool TRANS>
+__device__ __forceinline__ void ldsm4(uint32_t* r, const bf16* p) {
+    const uint32_t a = (uint32_t)__cvta_generic_to_shared(p);
+    if (TRANS)
+        asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+                     : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a) : "memory");
+    else
+        asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+                     : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a) : "memory");
+}
 
-__global__ void __launch_bounds__(128) k_gemm(Gemm g) {
-    __shared__ __align__(16) bf16 As[GBM * GLD];
-    __shared__ __align__(16) bf16 Bs[GBN * GLD];
+// rows r0 .. r0 + R - 1, elements c0 .. c0 + C - 1 of an operand into a tile of row pitch LD,
+// zero beyond its rows and row extent; VEC elements per copy (8 or 4: cp.async, 1: plain)
+template <int VEC, int R, int C, int LD>
+__device__ __forceinline__ void load_tile(bf16* dst, const Operand& o, int r0, int c0, int tid) {
+    constexpr int CH = C / VEC;
+#pragma unroll
+    for (int i = 0; i < R * CH / 256; ++i) {
+        const int e = tid + 256 * i, r = e / CH, c = (e - r * CH) * VEC;
+        const bool ok = r0 + r < o.rows && c0 + c < o.ext;
+        const bf16* src = o.p;
+        if (ok) src += (int64_t)(r0 + r) * o.ld + c0 + c;
+        bf16* d = dst + r * LD + c;
+        if (VEC == 1) {
+            *d = ok ? *src : __float2bfloat16(0.f);
+        } else {
+            const uint32_t s = (uint32_t)__cvta_generic_to_shared(d);
+            if (VEC == 8)
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(s), "l"(src), "r"(ok ? 16 : 0) : "memory");
+            else
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;\n" ::"r"(s), "l"(src), "r"(ok ? 8 : 0) : "memory");
+        }
+    }
+}
+
+template <bool BK, int MODE, int VA, int VB>
+__global__ void __launch_bounds__(256, 2) k_gemm(Gemm g) {
+    constexpr int SA = GBM * GLDK, SB = BK ? GBN * GLDK : GBK * GLDM;
+    extern __shared__ __align__(16) unsigned char gemm_sm[];
+    bf16* As = reinterpret_cast<bf16*>(gemm_sm);
+    bf16* Bs = As + GST * SA;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int m0 = blockIdx.y * GBM, n0 = blockIdx.x * GBN;
-    const int wm = (warp >> 1) * 32, wn = (warp & 1) * 32;
-    const int gr = lane >> 2, tc = (lane & 3) * 2;
-    float acc[2][4][4];
+    const int wm = (warp >> 2) * 64, wn = (warp & 3) * 32;
+    const int nk = (g.K + GBK - 1) / GBK;
+    float acc[4][4][4];
 #pragma unroll
-    for (int i = 0; i < 2; ++i)
+    for (int i = 0; i < 4; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j)
 #pragma unroll
             for (int e = 0; e < 4; ++e) acc[i][j][e] = 0.f;
-    const bool a_kfast = g.a_sk == 1, b_kfast = g.b_sk == 1;
-    const bf16 zero = __float2bfloat16(0.f);
-    for (int k0 = 0; k0 < g.K; k0 += GBK) {
-        for (int e = tid; e < GBM * GBK; e += 128) {
-            int r, kk;
-            if (a_kfast) {
-                r = e / GBK;
-                kk = e - r * GBK;
-            } else {
-                kk = e / GBM;
-                r = e - kk * GBM;
-            }
-            const int m = m0 + r, k = k0 + kk;
-            bf16 v = zero;
-            if (m < g.M && k < g.K) {
-                const int64_t row = g.a_idx ? g.a_idx[m] : (int64_t)m;
-                v = g.A[row * g.a_sm + (int64_t)k * g.a_sk];
-            }
-            As[r * GLD + kk] = v;
+    auto fetch = [&](int t) {
+        if (t < nk) {
+            const int k0 = t * GBK;
+            bf16* a = As + (t % GST) * SA;
+            bf16* b = Bs + (t % GST) * SB;
+            load_tile<VA, GBM, GBK, GLDK>(a, g.a, m0, k0, tid);
+            if (BK) load_tile<VB, GBN, GBK, GLDK>(b, g.b, n0, k0, tid);
+            else load_tile<VB, GBK, GBN, GLDM>(b, g.b, k0, n0, tid);
         }
-        for (int e = tid; e < GBN * GBK; e += 128) {
-            int c, kk;
-            if (b_kfast) {
-                c = e / GBK;
-                kk = e - c * GBK;
-            } else {
-                kk = e / GBN;
-                c = e - kk * GBN;
-            }
-            const int n = n0 + c, k = k0 + kk;
-            bf16 v = zero;
-            if (n < g.N && k < g.K) {
-                const int64_t kr = g.b_idx ? g.b_idx[k] : (int64_t)k;
-                v = g.B[kr * g.b_sk + (int64_t)n * g.b_sn];
-            }
-            Bs[c * GLD + kk] = v;
-        }
-        __syncthreads();
+        asm volatile("cp.async.commit_group;\n" ::: "memory");
+    };
+#pragma unroll
+    for (int t = 0; t < GST - 1; ++t) fetch(t);
+    for (int t = 0; t < nk; ++t) {
+        asm volatile("cp.async.wait_group %0;\n" ::"n"(GST - 2) : "memory");
+        __syncthreads();   // tile t has landed, tile t - 1 is consumed
+        fetch(t + GST - 1);
+        const bf16* a = As + (t % GST) * SA;
+        const bf16* b = Bs + (t % GST) * SB;
 #pragma unroll
         for (int ks = 0; ks < GBK; ks += 16) {
-            uint32_t af[2][4], bfr[4][2];
+            uint32_t af[4][4], bfr[2][4];
 #pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                const bf16* p = As + (wm + i * 16 + gr) * GLD + ks + tc;
-                af[i][0] = ld_pair(p);
-                af[i][1] = ld_pair(p + 8 * GLD);
-                af[i][2] = ld_pair(p + 8);
-                af[i][3] = ld_pair(p + 8 * GLD + 8);
+            for (int i = 0; i < 4; ++i) {
+                ldsm4<false>(af[i], a + (wm + i * 16 + (lane & 15)) * GLDK + ks + 8 * (lane >> 4));
             }
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const bf16* p = Bs + (wn + j * 8 + gr) * GLD + ks + tc;
-                bfr[j][0] = ld_pair(p);
-                bfr[j][1] = ld_pair(p + 8);
+            for (int j = 0; j < 2; ++j) {   // two n8 blocks each: (n, k), (n, k + 8), (n + 8, k), (n + 8, k + 8)
+                const int n = wn + j * 16;
+                if (BK) ldsm4<false>(bfr[j], b + (n + (lane & 7) + 8 * (lane >> 4)) * GLDK + ks + 8 * ((lane >> 3) & 1));
+                else ldsm4<true>(bfr[j], b + (ks + (lane & 15)) * GLDM + n + 8 * (lane >> 4));
             }
 #pragma unroll
-            for (int i = 0; i < 2; ++i)
+            for (int i = 0; i < 4; ++i)
 #pragma unroll
-                for (int j = 0; j < 4; ++j) mma_16816(acc[i][j], af[i], bfr[j]);
+                for (int j = 0; j < 4; ++j) mma_16816(acc[i][j], af[i], bfr[j >> 1] + 2 * (j & 1));
         }
-        __syncthreads();
     }
+    // thread's elements: rows m0 + wm + 16 i + (lane >> 2) + 8 h, columns n0 + wn + 8 j + 2 (lane & 3) + {0, 1}
+    const int gr = lane >> 2, tc = (lane & 3) * 2;
+    float loss = 0.f, col[4][2];
 #pragma unroll
-    for (int i = 0; i < 2; ++i)
+    for (int j = 0; j < 4; ++j) col[j][0] = col[j][1] = 0.f;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const int n = n0 + wn + j * 8 + tc;
+        float bias[2] = {0.f, 0.f};
+        if (MODE == EPI_BIAS_F32 || MODE == EPI_BIAS_RELU_BF16 || MODE == EPI_MSE) {
+            if (n < g.N) bias[0] = g.bias[n];
+            if (n + 1 < g.N) bias[1] = g.bias[n + 1];
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int m = m0 + wm + i * 16 + gr + 8 * h;
+                if (m >= g.M) continue;
+                const float x0 = acc[i][j][2 * h], x1 = acc[i][j][2 * h + 1];
+                if (MODE == EPI_BIAS_F32) {
+                    float* c = g.c32 + (int64_t)m * g.ldc + n;
+                    if (n < g.N) c[0] = x0 + bias[0];
+                    if (n + 1 < g.N) c[1] = x1 + bias[1];
+                } else if (MODE == EPI_BIAS_RELU_BF16) {   // N is even: n < N covers the pair
+                    if (n < g.N)
+                        *reinterpret_cast<__nv_bfloat162*>(g.c16 + (int64_t)m * g.ldc + n) =
+                            __floats2bfloat162_rn(fmaxf(x0 + bias[0], 0.f), fmaxf(x1 + bias[1], 0.f));
+                } else if (MODE == EPI_RELU_GRAD) {
+                    if (n < g.N) {
+                        const __nv_bfloat162 f = *reinterpret_cast<const __nv_bfloat162*>(g.act + (int64_t)m * g.ldc + n);
+                        const float k0 = __low2float(f) > 0.f ? x0 : 0.f, k1 = __high2float(f) > 0.f ? x1 : 0.f;
+                        col[j][0] += k0;
+                        col[j][1] += k1;
+                        *reinterpret_cast<__nv_bfloat162*>(g.c16 + (int64_t)m * g.ldc + n) = __floats2bfloat162_rn(k0, k1);
+                    }
+                } else {   // EPI_MSE: d = Y - T, gradient scale * d; the row's padding up to ldc is zero
+                    const float* t = g.T + g.t_idx[m] * g.N;
+                    float g0 = 0.f, g1 = 0.f;
+                    if (n < g.N) {
+                        const float d = (x0 + bias[0]) - t[n];
+                        loss += d * d;
+                        g0 = g.scale * d;
+                    }
+                    if (n + 1 < g.N) {
+                        const float d = (x1 + bias[1]) - t[n + 1];
+                        loss += d * d;
+                        g1 = g.scale * d;
+                    }
+                    col[j][0] += g0;
+                    col[j][1] += g1;
+                    if (n < g.ldc)
+                        *reinterpret_cast<__nv_bfloat162*>(g.c16 + (int64_t)m * g.ldc + n) = __floats2bfloat162_rn(g0, g1);
+                }
+            }
+    }
+    if (MODE == EPI_RELU_GRAD || MODE == EPI_MSE) {
+        // column sums of the tile: over the 8 lanes of a column, then the two warps along m
+        asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+        __syncthreads();
+        float* red = reinterpret_cast<float*>(gemm_sm);   // [2][GBN], then 8 loss sums
 #pragma unroll
         for (int j = 0; j < 4; ++j)
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const int m = m0 + wm + i * 16 + gr + (e >> 1) * 8;
-                const int n = n0 + wn + j * 8 + tc + (e & 1);
-                if (m >= g.M || n >= g.N) continue;
-                const float x = acc[i][j][e];
-                const int64_t q = (int64_t)m * g.ldc + n;
-                if (g.mode == EPI_BIAS_F32) {
-                    g.c32[q] = x + g.bias[n];
-                } else if (g.mode == EPI_BIAS_RELU_BF16) {
-                    g.c16[q] = __float2bfloat16(fmaxf(x + g.bias[n], 0.f));
-                } else if (g.mode == EPI_RELU_GRAD) {
-                    const float keep = __bfloat162float(g.act[(int64_t)m * g.act_ld + n]) > 0.f ? x : 0.f;
-                    g.c32[q] = keep;
-                    g.c16[q] = __float2bfloat16(keep);
-                } else {
-                    g.c32[q] = x;
-                }
+            for (int e = 0; e < 2; ++e) {
+                float v = col[j][e];
+                v += __shfl_xor_sync(0xffffffffu, v, 4);
+                v += __shfl_xor_sync(0xffffffffu, v, 8);
+                v += __shfl_xor_sync(0xffffffffu, v, 16);
+                if (gr == 0) red[(warp >> 2) * GBN + wn + j * 8 + tc + e] = v;
             }
-}
-
-// dY = 2 (Y - T[idx]) / (n n_out) (FP32 and bfloat16), per-block partial sums of (Y - T)^2
-__global__ void k_mse_grad(const float* Y, const float* T, const int64_t* idx, int64_t n, int no, float scale,
-                           float* g32, bf16* g16, float* part) {
-    __shared__ float red[8];
-    float acc = 0.f;
-    const int64_t total = n * no;
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total;
-         e += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t i = e / no;
-        const int j = (int)(e - i * no);
-        const float d = Y[e] - T[idx[i] * no + j];
-        acc += d * d;
-        const float gv = scale * d;
-        g32[e] = gv;
-        g16[e] = __float2bfloat16(gv);
-    }
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        float t = 0.f;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w];
-        part[blockIdx.x] = t;
+        if (MODE == EPI_MSE) {
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, o);
+            if (lane == 0) red[2 * GBN + warp] = loss;
+        }
+        __syncthreads();
+        if (tid < GBN && n0 + tid < g.N) g.colpart[(int64_t)blockIdx.y * g.N + n0 + tid] = red[tid] + red[GBN + tid];
+        if (MODE == EPI_MSE && tid == 0) {
+            float t = 0.f;
+            for (int w = 0; w < 8; ++w) t += red[2 * GBN + w];
+            g.losspart[blockIdx.y * gridDim.x + blockIdx.x] = t;
+        }
     }
 }
 
-__global__ void k_loss_final(const float* part, int nb, float inv, float* loss) {
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
+// Weight gradients of every layer, dW_l [No][Ki] = G_l^T X_l over the minibatch rows, in one
+// launch: 64 x 32 tiles of 8 warps (16 x 16 each), the whole k = rows of a tile summed by one
+// warp in ascending order (the order of a plain loop: a split along the rows changes the
+// FP32 result by more than its own rounding, 6.6e-5 of the gradient at 16384 rows).  Both
+// operands have their row index as k, so the tiles are [64 rows][64] and [64 rows][32] and
+// the fragments come by ldmatrix.trans; DWST stages hide the L2 latency of the long k loop.
+// The layers together give 144 tiles for a 260 -> 4 x 256 -> 81 network, where one launch
+// per layer had 8-24 blocks.
+#define DWK 64
+#define DWM 64
+#define DWN 32
+#define DWST 6
+#define DWLG (DWM + 8)    // 144 and 80 bytes: ldmatrix rows fall in distinct banks
+#define DWLX (DWN + 8)
+struct DwLayer {
+    Operand g, x;         // [row][o], [row][k]
+    int No, Ki, tile0, ntx;
+    float* out;
+};
+struct DwArgs {
+    int nl, rows;
+    DwLayer l[MLP_MAX_LINEAR];
+};
+__global__ void __launch_bounds__(256) k_weight_grad(const __grid_constant__ DwArgs A) {
+    extern __shared__ __align__(16) unsigned char gemm_sm[];
+    bf16* Gs = reinterpret_cast<bf16*>(gemm_sm);      // [DWST][DWK][DWLG]
+    bf16* Xs = Gs + DWST * DWK * DWLG;                // [DWST][DWK][DWLX]
+    int li = 0;
+    while (li + 1 < A.nl && (int)blockIdx.x >= A.l[li + 1].tile0) ++li;
+    const DwLayer L = A.l[li];
+    const int tile = blockIdx.x - L.tile0, m0 = tile / L.ntx * DWM, n0 = tile % L.ntx * DWN;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int wm = (warp >> 1) * 16, wn = (warp & 1) * 16;
+    const int nk = (A.rows + DWK - 1) / DWK;
+    float acc[2][4];
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) acc[j][e] = 0.f;
+    auto fetch = [&](int t) {
+        if (t < nk) {
+            load_tile<8, DWK, DWM, DWLG>(Gs + (t % DWST) * DWK * DWLG, L.g, t * DWK, m0, tid);
+            load_tile<8, DWK, DWN, DWLX>(Xs + (t % DWST) * DWK * DWLX, L.x, t * DWK, n0, tid);
+        }
+        asm volatile("cp.async.commit_group;\n" ::: "memory");
+    };
+#pragma unroll
+    for (int t = 0; t < DWST - 1; ++t) fetch(t);
+    for (int t = 0; t < nk; ++t) {
+        asm volatile("cp.async.wait_group %0;\n" ::"n"(DWST - 2) : "memory");
+        __syncthreads();   // tile t has landed, tile t - 1 is consumed
+        fetch(t + DWST - 1);
+        const bf16* g = Gs + (t % DWST) * DWK * DWLG + ((lane & 7) + 8 * (lane >> 4)) * DWLG + wm + 8 * ((lane >> 3) & 1);
+        const bf16* x = Xs + (t % DWST) * DWK * DWLX + (lane & 15) * DWLX + wn + 8 * (lane >> 4);
+        uint32_t af[DWK / 16][4], bfr[DWK / 16][4];
+#pragma unroll
+        for (int q = 0; q < DWK / 16; ++q) {
+            ldsm4<true>(af[q], g + 16 * q * DWLG);
+            ldsm4<true>(bfr[q], x + 16 * q * DWLX);
+        }
+#pragma unroll
+        for (int q = 0; q < DWK / 16; ++q) {
+            mma_16816(acc[0], af[q], bfr[q]);
+            mma_16816(acc[1], af[q], bfr[q] + 2);
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const int m = m0 + wm + (lane >> 2) + 8 * (e >> 1), n = n0 + wn + j * 8 + (lane & 3) * 2 + (e & 1);
+            if (m < L.No && n < L.Ki) L.out[(int64_t)m * L.Ki + n] = acc[j][e];
+        }
+}
+
+// The minibatch's input rows, gathered once per step into rows of pad8(n_in) (16-byte copies
+// for both GEMMs that read them, no index in their loops); VEC elements per copy.
+template <int VEC>
+__global__ void __launch_bounds__(256) k_gather_rows(const bf16* __restrict__ X, int n_in, int ld,
+                                                     const int64_t* __restrict__ idx, int64_t n, bf16* out) {
+    typedef typename std::conditional<VEC == 4, uint2, unsigned short>::type V;
+    const int ch = ld / VEC;
+    const int64_t total = n * ch;
+    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t i = e / ch;
+        const int c = (int)(e - i * ch) * VEC;
+        V v = V();
+        if (c < n_in) v = *reinterpret_cast<const V*>(X + idx[i] * n_in + c);
+        *reinterpret_cast<V*>(out + i * ld + c) = v;
+    }
+}
+
+// Bias gradients from the tiles' column sums (in a fixed order), then Adam (Kingma & Ba,
+// Algorithm 1; bc1 = 1 - beta1^t, bc2 = 1 - beta2^t) and the bfloat16 copies of the weights.
+// Block 0 also sums the loss.
+// A training step of 16384 rows, 260 -> 4 x 256 -> 81 on GB300: 11.9 ms with one GEMM of
+// 8-24 blocks per weight gradient, FP32 gradients stored, and a column-sum pass per layer;
+// 282 us now (92 us of it k_weight_grad, whose long sums keep one warp per 16 x 16 outputs).
+struct GradLayers {
+    int nl;
+    int64_t w_off[MLP_MAX_LINEAR], b_off[MLP_MAX_LINEAR], wb_off[MLP_MAX_LINEAR];
+    int n_b[MLP_MAX_LINEAR];
+    const float* bpart[MLP_MAX_LINEAR];   // [nby][n_b]
+    int nby;
+    const float* losspart;
+    int nloss;
+    float loss_scale;
+    float* loss;
+};
+__global__ void __launch_bounds__(256) k_grad_adam(GradLayers L, int64_t n, float* p, float* g, float* m, float* v,
+                                                   bf16* wb, float lr, float b1, float b2, float eps, float bc1,
+                                                   float bc2) {
+    if (blockIdx.x == 0 && threadIdx.x < 32) {
         double t = 0.0;
-        for (int i = 0; i < nb; ++i) t += part[i];
-        *loss = (float)(t * inv);
+        for (int i = threadIdx.x; i < L.nloss; i += 32) t += (double)L.losspart[i];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+        if (threadIdx.x == 0) *L.loss = (float)(t * (double)L.loss_scale);
     }
-}
-
-// db[n] = sum_m G[m][n]; block (32, 8) per 32 columns
-__global__ void k_colsum(const float* G, int64_t M, int N, float* out) {
-    __shared__ float red[8][33];
-    const int n = blockIdx.x * 32 + threadIdx.x;
-    float a = 0.f;
-    if (n < N)
-        for (int64_t m = threadIdx.y; m < M; m += 8) a += G[m * N + n];
-    red[threadIdx.y][threadIdx.x] = a;
-    __syncthreads();
-    if (threadIdx.y == 0 && n < N) {
-        float t = 0.f;
-        for (int r = 0; r < 8; ++r) t += red[r][threadIdx.x];
-        out[n] = t;
-    }
-}
-
-// Adam (Kingma & Ba, Algorithm 1); bc1 = 1 - beta1^t, bc2 = 1 - beta2^t
-__global__ void k_adam(int64_t n, float* p, const float* g, float* m, float* v, float lr, float b1, float b2,
-                       float eps, float bc1, float bc2) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const float gi = g[i];
+    auto adam = [&](int64_t i, float gi) {
         const float mi = b1 * m[i] + (1.f - b1) * gi;
         const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
         m[i] = mi;
         v[i] = vi;
-        p[i] -= lr * (mi / bc1) / (sqrtf(vi / bc2) + eps);
+        return p[i] = p[i] - lr * (mi / bc1) / (sqrtf(vi / bc2) + eps);
+    };
+    // biases: one warp each, lanes over the row tiles
+    const int lane = threadIdx.x & 31;
+    int64_t wid = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    const int64_t nw = (int64_t)gridDim.x * blockDim.x >> 5;
+    for (int l = 0; l < L.nl; ++l) {
+        for (; wid < L.n_b[l]; wid += nw) {
+            float s = 0.f;
+            for (int c = lane; c < L.nby; c += 32) s += L.bpart[l][(int64_t)c * L.n_b[l] + wid];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            if (lane == 0) {
+                g[L.b_off[l] + wid] = s;
+                adam(L.b_off[l] + wid, s);
+            }
+        }
+        wid -= L.n_b[l];
+    }
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        int l = 0;
+        while (l + 1 < L.nl && i >= L.w_off[l + 1]) ++l;
+        if (i >= L.b_off[l]) continue;
+        wb[L.wb_off[l] + (i - L.w_off[l])] = __float2bfloat16(adam(i, g[i]));
     }
 }
 
@@ -390,6 +562,26 @@ static ib_status mlp_alloc(T** p, int64_t n) {
     return IB_OK;
 }
 
+static int pad8(int n) { return (n + 7) & ~7; }
+
+// elements per copy an operand allows: its rows start on a multiple of 16 (8) bytes and
+// hold whole copies
+static int copy_vec(const Operand& o) {
+    const uintptr_t a = reinterpret_cast<uintptr_t>(o.p);
+    if (a % 16 == 0 && o.ld % 8 == 0 && o.ext % 8 == 0) return 8;
+    if (a % 8 == 0 && o.ld % 4 == 0 && o.ext % 4 == 0) return 4;
+    return 1;
+}
+
+template <bool BK, int MODE, int VA, int VB>
+static void launch_gemm_v(const Gemm& g, dim3 grid, cudaStream_t s) {
+    constexpr size_t sm = sizeof(bf16) * GST * (GBM * GLDK + (BK ? GBN * GLDK : GBK * GLDM));
+    // per launch: right whatever device is current
+    cudaFuncSetAttribute(k_gemm<BK, MODE, VA, VB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    k_gemm<BK, MODE, VA, VB><<<grid, 256, sm, s>>>(g);
+}
+
+template <bool BK, int MODE>
 static ib_status launch_gemm(const Gemm& g, cudaStream_t s) {
     if (g.M <= 0 || g.N <= 0) return IB_OK;
     dim3 grid((g.N + GBN - 1) / GBN, (g.M + GBM - 1) / GBM);
@@ -397,25 +589,27 @@ static ib_status launch_gemm(const Gemm& g, cudaStream_t s) {
         ib_set_error("GEMM too tall");
         return IB_ERR_ARG;
     }
-    k_gemm<<<grid, 128, 0, s>>>(g);
+    const int va = copy_vec(g.a), vb = copy_vec(g.b);
+    if (va == 8 && vb == 8) launch_gemm_v<BK, MODE, 8, 8>(g, grid, s);
+    else if (va == 8 && vb == 4) launch_gemm_v<BK, MODE, 8, 4>(g, grid, s);
+    else if (va >= 4 && vb >= 4) launch_gemm_v<BK, MODE, 4, 4>(g, grid, s);
+    else if (va == 8) launch_gemm_v<BK, MODE, 8, 1>(g, grid, s);
+    else launch_gemm_v<BK, MODE, 1, 1>(g, grid, s);
     IB_CHECK_LAUNCH("k_gemm");
     ib_count_launch("mlp_gemm_bf16");
     return IB_OK;
 }
 
-static Gemm gemm_fwd(const ib_mlp* m, int l, const bf16* Xin, int64_t ldx, const int64_t* idx, int64_t n) {
+
+// layer l on n rows of Xin (ext readable elements each, zero past the layer's inputs)
+static Gemm gemm_fwd(const ib_mlp* m, int l, const bf16* Xin, int64_t ldx, int ext, int64_t n) {
     Gemm g;
     memset(&g, 0, sizeof g);
     g.M = (int)n;
     g.N = m->dims[l + 1];
     g.K = m->dims[l];
-    g.A = Xin;
-    g.a_sm = ldx;
-    g.a_sk = 1;
-    g.a_idx = idx;
-    g.B = m->wb + m->wb_off[l];   // W_l [N][K]: B(k, n) = W[n][k]
-    g.b_sk = 1;
-    g.b_sn = g.K;
+    g.a = {Xin, ldx, (int)n, ext};
+    g.b = {m->wb + m->wb_off[l], g.K, g.N, g.K};   // W_l [N][K]
     g.bias = m->params + m->b_off[l];
     return g;
 }
@@ -472,7 +666,6 @@ extern "C" ib_status ib_mlp_create(const ib_mlp_config* cfg, ib_mlp** out) {
     if ((st = mlp_alloc(&m->in_off, 3 * (int64_t)inb.size())) != IB_OK) return fail(st);
     const int W = 2 * m->out_R + 1;
     if ((st = mlp_alloc(&m->out_lut, (int64_t)W * W * W)) != IB_OK) return fail(st);
-    if ((st = mlp_alloc(&m->part, 1024)) != IB_OK) return fail(st);
     std::vector<int8_t> ho;
     for (auto& o : inb)
         for (int a = 0; a < 3; ++a) ho.push_back((int8_t)o[a]);
@@ -496,7 +689,7 @@ extern "C" ib_status ib_mlp_create(const ib_mlp_config* cfg, ib_mlp** out) {
 extern "C" void ib_mlp_free(ib_mlp* m) {
     if (!m) return;
     void* ptrs[] = {m->params, m->grads, m->adam_m, m->adam_v, m->wb, m->in_off, m->out_lut, m->act,
-                    m->y, m->g32, m->g16a, m->g16b, m->part, m->ia, m->ib, m->ix};
+                    m->g16, m->xg, m->bpart, m->ia, m->ib, m->ix};
     for (void* q : ptrs)
         if (q) cudaFree(q);
     delete m;
@@ -602,19 +795,17 @@ static ib_status forward(ib_mlp* m, const bf16* X, int64_t n, float* Y, cudaStre
         int64_t ldi = m->n_in;
         bf16* bufs[2] = {m->ia, m->ib};
         for (int l = 0; l < m->nl; ++l) {
-            Gemm g = gemm_fwd(m, l, in, ldi, nullptr, cn);
+            Gemm g = gemm_fwd(m, l, in, ldi, m->dims[l], cn);
             if (l + 1 < m->nl) {
-                g.mode = EPI_BIAS_RELU_BF16;
                 g.c16 = bufs[l & 1];
                 g.ldc = H;
-                TRY(launch_gemm(g, s));
+                TRY((launch_gemm<true, EPI_BIAS_RELU_BF16>(g, s)));
                 in = bufs[l & 1];
                 ldi = H;
             } else {
-                g.mode = EPI_BIAS_F32;
                 g.c32 = Y + c0 * m->n_out;
                 g.ldc = m->n_out;
-                TRY(launch_gemm(g, s));
+                TRY((launch_gemm<true, EPI_BIAS_F32>(g, s)));
             }
         }
     }
@@ -633,21 +824,20 @@ extern "C" ib_status ib_mlp_forward(ib_mlp* m, const void* X_dev, int64_t n, flo
 static ib_status ensure_train(ib_mlp* m, int64_t n) {
     if (n <= m->cap) return IB_OK;
     const int H = m->cfg.n_hidden;
-    int mxd = 0;
-    for (int l = 0; l <= m->nl; ++l) mxd = std::max(mxd, m->dims[l]);
-    void* ptrs[] = {m->act, m->y, m->g32, m->g16a, m->g16b};
+    const int mxd = std::max(H, pad8(m->n_out));
+    int64_t sum_b = 0;
+    for (int l = 0; l < m->nl; ++l) sum_b += m->dims[l + 1];
+    const int64_t nby = (n + GBM - 1) / GBM;
+    void* ptrs[] = {m->act, m->g16, m->xg, m->bpart};
     for (void* q : ptrs)
         if (q) cudaFree(q);
-    m->act = nullptr;
-    m->y = nullptr;
-    m->g32 = nullptr;
-    m->g16a = m->g16b = nullptr;
+    m->act = m->g16 = m->xg = nullptr;
+    m->bpart = nullptr;
     m->cap = 0;
     TRY(mlp_alloc(&m->act, (int64_t)(m->nl - 1) * n * H));
-    TRY(mlp_alloc(&m->y, n * m->n_out));
-    TRY(mlp_alloc(&m->g32, n * mxd));
-    TRY(mlp_alloc(&m->g16a, n * mxd));
-    TRY(mlp_alloc(&m->g16b, n * mxd));
+    TRY(mlp_alloc(&m->g16, (int64_t)m->nl * n * mxd));
+    TRY(mlp_alloc(&m->xg, n * pad8(m->n_in)));
+    TRY(mlp_alloc(&m->bpart, nby * (sum_b + (m->n_out + GBN - 1) / GBN)));
     m->cap = n;
     return IB_OK;
 }
@@ -669,92 +859,105 @@ extern "C" ib_status ib_mlp_train_step(ib_mlp* m, const void* X_dev, const float
     const int H = m->cfg.n_hidden, L = m->nl;
     const bf16* X = (const bf16*)X_dev;
     auto act = [&](int l) { return m->act + (int64_t)(l - 1) * m->cap * H; };   // input of layer l >= 1
-    // forward, keeping each layer's input
+    // forward, keeping each layer's input; the last layer's epilogue forms the loss and its
+    // gradient (rows of pad8(n_out), zero in the padding)
+    const int64_t nby = (n + GBM - 1) / GBM;
+    const int ldo = pad8(m->n_out);
+    auto grad = [&](int l) { return m->g16 + (int64_t)l * m->cap * std::max(H, ldo); };   // of layer l's output
+    GradLayers R;
+    memset(&R, 0, sizeof R);
+    R.nl = L;
+    R.nby = (int)nby;
+    {
+        float* bp = m->bpart;
+        for (int l = 0; l < L; ++l) {
+            R.w_off[l] = m->w_off[l];
+            R.b_off[l] = m->b_off[l];
+            R.wb_off[l] = m->wb_off[l];
+            R.n_b[l] = m->dims[l + 1];
+            R.bpart[l] = bp;
+            bp += nby * R.n_b[l];
+        }
+        R.losspart = bp;
+        R.nloss = (int)(nby * ((m->n_out + GBN - 1) / GBN));
+        R.loss_scale = (float)(1.0 / ((double)n * m->n_out));
+        R.loss = loss_dev;
+    }
+    const int ldx = pad8(m->n_in);
+    if (m->n_in % 4 == 0 && reinterpret_cast<uintptr_t>(X) % 8 == 0)
+        k_gather_rows<4><<<grid1(n * ldx / 4, 256), 256, 0, s>>>(X, m->n_in, ldx, idx_dev, n, m->xg);
+    else
+        k_gather_rows<1><<<grid1(n * ldx, 256), 256, 0, s>>>(X, m->n_in, ldx, idx_dev, n, m->xg);
+    IB_CHECK_LAUNCH("k_gather_rows");
+    ib_count_launch("mlp_setup");
     for (int l = 0; l < L; ++l) {
-        Gemm g = l == 0 ? gemm_fwd(m, 0, X, m->n_in, idx_dev, n) : gemm_fwd(m, l, act(l), H, nullptr, n);
+        Gemm g = l == 0 ? gemm_fwd(m, 0, m->xg, ldx, ldx, n) : gemm_fwd(m, l, act(l), H, H, n);
         if (l + 1 < L) {
-            g.mode = EPI_BIAS_RELU_BF16;
             g.c16 = act(l + 1);
             g.ldc = H;
+            TRY((launch_gemm<true, EPI_BIAS_RELU_BF16>(g, s)));
         } else {
-            g.mode = EPI_BIAS_F32;
-            g.c32 = m->y;
-            g.ldc = m->n_out;
+            g.c16 = grad(l);
+            g.ldc = ldo;
+            g.T = T_dev;
+            g.t_idx = idx_dev;
+            g.scale = (float)(2.0 / ((double)n * m->n_out));
+            g.colpart = const_cast<float*>(R.bpart[l]);
+            g.losspart = const_cast<float*>(R.losspart);
+            TRY((launch_gemm<true, EPI_MSE>(g, s)));
         }
-        TRY(launch_gemm(g, s));
     }
-    // loss and output gradient
-    const int nb = std::min(1024, grid1(n * m->n_out, 256));
-    k_mse_grad<<<nb, 256, 0, s>>>(m->y, T_dev, idx_dev, n, m->n_out, (float)(2.0 / ((double)n * m->n_out)), m->g32,
-                                  m->g16a, m->part);
-    IB_CHECK_LAUNCH("k_mse_grad");
-    ib_count_launch("mlp_loss");
-    k_loss_final<<<1, 32, 0, s>>>(m->part, nb, (float)(1.0 / ((double)n * m->n_out)), loss_dev);
-    IB_CHECK_LAUNCH("k_loss_final");
-    ib_count_launch("mlp_loss");
-    // backward: g16 holds d loss / d (output of layer l), g32 its FP32 value
-    bf16* gcur = m->g16a;
-    bf16* gnext = m->g16b;
-    for (int l = L - 1; l >= 0; --l) {
-        const int No = m->dims[l + 1], Ki = m->dims[l];
-        // dW_l [No][Ki] = G^T X_l
-        Gemm gw;
-        memset(&gw, 0, sizeof gw);
-        gw.M = No;
-        gw.N = Ki;
-        gw.K = (int)n;
-        gw.A = gcur;          // A(o, r) = G[r][o]
-        gw.a_sm = 1;
-        gw.a_sk = No;
-        if (l == 0) {
-            gw.B = X;         // B(r, k) = X[idx[r]][k]
-            gw.b_sk = m->n_in;
-            gw.b_idx = idx_dev;
-        } else {
-            gw.B = act(l);
-            gw.b_sk = H;
-        }
-        gw.b_sn = 1;
-        gw.mode = EPI_F32;
-        gw.c32 = m->grads + m->w_off[l];
-        gw.ldc = Ki;
-        TRY(launch_gemm(gw, s));
-        // db_l = column sums of G (FP32)
-        k_colsum<<<(No + 31) / 32, dim3(32, 8), 0, s>>>(m->g32, n, No, m->grads + m->b_off[l]);
-        IB_CHECK_LAUNCH("k_colsum");
-        ib_count_launch("mlp_colsum");
-        if (l > 0) {
-            // G_{l-1} = (G W_l) * [X_l > 0]
-            Gemm gx;
-            memset(&gx, 0, sizeof gx);
-            gx.M = (int)n;
-            gx.N = Ki;
-            gx.K = No;
-            gx.A = gcur;
-            gx.a_sm = No;
-            gx.a_sk = 1;
-            gx.B = m->wb + m->wb_off[l];   // B(o, k) = W[o][k]
-            gx.b_sk = Ki;
-            gx.b_sn = 1;
-            gx.mode = EPI_RELU_GRAD;
-            gx.act = act(l);
-            gx.act_ld = H;
-            gx.c32 = m->g32;
-            gx.c16 = gnext;
-            gx.ldc = Ki;
-            TRY(launch_gemm(gx, s));
-            std::swap(gcur, gnext);
-        }
+    // backward: G_{l-1} = (G_l W_l) * [X_l > 0], with the column sums of db_{l-1}
+    for (int l = L - 1; l > 0; --l) {
+        const int No = m->dims[l + 1], Ki = m->dims[l], ldg = l == L - 1 ? ldo : H;
+        Gemm gx;
+        memset(&gx, 0, sizeof gx);
+        gx.M = (int)n;
+        gx.N = Ki;
+        gx.K = No;
+        gx.a = {grad(l), ldg, (int)n, ldg};
+        gx.b = {m->wb + m->wb_off[l], Ki, No, Ki};
+        gx.act = act(l);
+        gx.c16 = grad(l - 1);
+        gx.ldc = Ki;
+        gx.colpart = const_cast<float*>(R.bpart[l - 1]);
+        TRY((launch_gemm<false, EPI_RELU_GRAD>(gx, s)));
+    }
+    // dW_l of all layers
+    DwArgs D;
+    memset(&D, 0, sizeof D);
+    D.nl = L;
+    D.rows = (int)n;
+    int tiles = 0;
+    for (int l = 0; l < L; ++l) {
+        const int No = m->dims[l + 1], Ki = m->dims[l], ldg = l == L - 1 ? ldo : H;
+        DwLayer& d = D.l[l];
+        d.g = {grad(l), ldg, (int)n, ldg};
+        if (l == 0) d.x = {m->xg, ldx, (int)n, ldx};
+        else d.x = {act(l), H, (int)n, H};
+        d.No = No;
+        d.Ki = Ki;
+        d.tile0 = tiles;
+        d.ntx = (Ki + DWN - 1) / DWN;
+        d.out = m->grads + m->w_off[l];
+        tiles += d.ntx * ((No + DWM - 1) / DWM);
+    }
+    {
+        constexpr size_t sm = sizeof(bf16) * DWST * DWK * (DWLG + DWLX);
+        cudaFuncSetAttribute(k_weight_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        k_weight_grad<<<tiles, 256, sm, s>>>(D);
+        IB_CHECK_LAUNCH("k_weight_grad");
+        ib_count_launch("mlp_gemm_bf16");
     }
     // Adam
     m->step += 1;
     const double bc1 = 1.0 - std::pow((double)beta1, (double)m->step);
     const double bc2 = 1.0 - std::pow((double)beta2, (double)m->step);
-    k_adam<<<grid1(m->n_params, 256), 256, 0, s>>>(m->n_params, m->params, m->grads, m->adam_m, m->adam_v, lr, beta1,
-                                                   beta2, eps, (float)bc1, (float)bc2);
-    IB_CHECK_LAUNCH("k_adam");
+    k_grad_adam<<<grid1(m->n_params, 256), 256, 0, s>>>(R, m->n_params, m->params, m->grads, m->adam_m, m->adam_v, m->wb,
+                                                        lr, beta1, beta2, eps, (float)bc1, (float)bc2);
+    IB_CHECK_LAUNCH("k_grad_adam");
     ib_count_launch("mlp_adam");
-    return sync_weights(m, s);
+    return IB_OK;
 }
 
 extern "C" ib_status ib_mlp_targets(const ib_table* t, const ib_mlp* m, int64_t* nodes_dev, float* T_dev,

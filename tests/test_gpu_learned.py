@@ -95,6 +95,35 @@ def test_gradient_and_loss_match_oracle(ib):
             o += sz
 
 
+@pytest.mark.parametrize("n_in_radius,width,layers,n", [(4.0, 8, 1, 1), (4.0, 136, 3, 129), (1.0, 64, 2, 700), (0.0, 264, 2, 65)])
+def test_gradient_tile_edges(ib, n_in_radius, width, layers, n):
+    """Widths, row counts and input counts off the GEMM tiles (128 x 128 x 32; weight gradients 64 x 32 x 64),
+    and input rows of odd length; per tensor against float64 on the same bfloat16 weights and inputs.
+    Tolerance: bfloat16 keeps 8 bits, so each rounded activation and gradient is off by at most 2^-9
+    relative; 2 (layers + 1) such roundings in a row bound the relative error by 2 (layers + 1) 2^-9 to first
+    order (a random walk of them stays below), and ReLU switches near zero add the same again."""
+    net = ib.Mlp(3, 8, n_hidden=width, n_layers=layers, in_radius=n_in_radius)
+    p = inputs.mlp_init(net.n_in, width, layers, net.n_out, seed=n)
+    net.set_params(p)
+    rng = np.random.default_rng(n)
+    Xf = omlp.bf16(rng.normal(size=(n + 7, net.n_in)))
+    Tf = rng.normal(size=(n + 7, net.n_out)).astype(np.float32)
+    idx = rng.permutation(n + 7)[:n].astype(np.int64)
+    X = torch.as_tensor(Xf, device="cuda").to(torch.bfloat16)
+    loss = ib.ib_mlp_train_step(net, X, torch.as_tensor(Tf, device="cuda"), torch.as_tensor(idx, device="cuda"), lr=1e-9)
+    torch.cuda.synchronize()
+    g = net.buffers()[1].double().cpu().numpy()
+    go, lo = omlp.backward(p.astype(np.float64), _sizes(net), Xf[idx], Tf[idx].astype(np.float64), emulate=True)
+    tol = 4 * (layers + 1) * 2.0 ** -9
+    assert abs(float(loss.item()) - lo) <= tol * lo
+    o = 0
+    for no, ni in _sizes(net):
+        for sz in (no * ni, no):
+            a, b = g[o:o + sz], go[o:o + sz]
+            assert np.linalg.norm(a - b) <= tol * np.linalg.norm(b) + 1e-12, (o, sz)
+            o += sz
+
+
 def test_adam_step_matches_oracle(ib):
     net, p, Xf, Tf, idx, X, T, I = _train_case(ib, seed=6)
     params, grads, m, v = net.buffers()
