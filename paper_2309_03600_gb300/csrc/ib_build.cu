@@ -507,6 +507,9 @@ struct FitParams {
     double accept_tol;
     double* resid;              // [nrows] exactness residual of the prediction
     uint8_t* accepted;          // [nrows]
+    int check_only;             // check the predictions and leave the other rows (k_fit_rows fits them)
+    const int32_t* sel;         // rows to fit (null: all)
+    int64_t nsel;
 };
 
 __constant__ double c_inv_int[10] = {0.0, 1.0, 0.5, 1.0 / 3.0, 0.25, 0.2, 1.0 / 6.0, 1.0 / 7.0, 0.125, 1.0 / 9.0};
@@ -1164,7 +1167,8 @@ __global__ void __launch_bounds__(FIT_THREADS) k_fit(FitParams P) {
     S.scal = S.bps + FIT_MAX_BP;          // [0..63]
     int* scan_tmp = S.scal + 16;
 
-    for (int64_t row = blockIdx.x; row < P.nrows; row += gridDim.x) {
+    for (int64_t at = blockIdx.x; at < (P.sel ? P.nsel : P.nrows); at += gridDim.x) {
+        const int64_t row = P.sel ? (int64_t)P.sel[at] : at;
         const int64_t lin = P.rows[row];
         int64_t node[3];
         node[0] = lin % P.g.n[0];
@@ -1336,6 +1340,10 @@ __global__ void __launch_bounds__(FIT_THREADS) k_fit(FitParams P) {
                         used_r2 = (int)lrint(2.0 * r);
                         used_nbp = nbp;
                         nsup_final = nsup;
+                        done = true;
+                        break;
+                    }
+                    if (P.check_only) {
                         done = true;
                         break;
                     }
@@ -1520,6 +1528,8 @@ __global__ void __launch_bounds__(FIT_THREADS) k_fit(FitParams P) {
         __syncthreads();
     }
 }
+
+#include "ib_fit.cuh"
 
 // ---------------------------------------------------------------------------
 // packing
@@ -1778,9 +1788,238 @@ static ib_status pack_pool(ib_table* t, const FitKind& fk, const int64_t* rows, 
     return IB_OK;
 }
 
+template <class T>
+static ib_status upload(DevBuf& tmp, const std::vector<T>& v, const T** out) {
+    T* d;
+    TRY(tmp.alloc(&d, (int64_t)v.size()));
+    if (!v.empty()) IB_CUDA(cudaMemcpy(d, v.data(), sizeof(T) * v.size(), cudaMemcpyHostToDevice));
+    *out = d;
+    return IB_OK;
+}
+
+// Tables of k_fit_rows for the orders of P (same indices, balls and stencil).  *ok stays
+// false where a fit does not suit it: a basis order above 4 (its moments would outgrow the
+// integers and the registers), more than 35 unknowns (3D coupled rows: their Gram matrix
+// alone takes 44 KB), or a ball beyond 768 offsets or 6 nodes.
+static ib_status row_fit_tables(ib_table* t, const Geo& g, const FitKind& fk, const FitParams& P,
+                                const std::vector<int>& orders, const std::vector<int8_t>* off,
+                                const std::vector<int32_t>* ball_q, const int64_t* bp_owner, int64_t nbp, RowFit& R,
+                                cudaStream_t s, DevBuf& tmp, bool* ok) {
+    const int d = g.ndim;
+    *ok = false;
+    memset(&R, 0, sizeof R);
+    if (P.ngrow + 1 > RF_GROW || P.rule.nE > 32) return IB_OK;
+    for (int oi = 0; oi < P.norders; ++oi)
+        if (orders[oi] > 4 || fk.nf * P.ord[oi].T > RF_MAXCOL) return IB_OK;
+    for (int f = 0; f < fk.nf; ++f) {
+        R.ncand[f] = P.nball[f];
+        if (P.nball[f] > 768) return IB_OK;
+        for (int c = 0; c < P.nball[f]; ++c)
+            for (int a = 0; a < d; ++a)
+                if (abs(2 * off[f][3 * c + a] + fk.fshift2[f][a] - fk.x0shift2[a]) > 12) return IB_OK;
+    }
+    auto fact = [](int k) {
+        double v = 1.0;
+        for (int i = 2; i <= k; ++i) v *= i;
+        return v;
+    };
+    for (int oi = 0; oi < P.norders; ++oi) {
+        RowOrder& o = R.ord[oi];
+        const int Mp = orders[oi];
+        const std::vector<MI> K = multi_indices(d, Mp), Gm = multi_indices(d, 2 * Mp);
+        const int T = (int)K.size(), n = fk.nf * T;
+        o.order = Mp;
+        o.T = T;
+        o.n = n;
+        o.np = n * (n + 1) / 2;
+        o.r0 = P.ord[oi].r0;
+        o.gpad = ((int)Gm.size() + 31) / 32 * 32;
+        if (o.gpad > 192 || fk.nf * o.gpad > RF_CAP) return IB_OK;
+        std::map<MI, int> kid, gid;
+        for (int k = 0; k < T; ++k) kid[K[k]] = k;
+        for (int k = 0; k < (int)Gm.size(); ++k) gid[Gm[k]] = k;
+        // candidates: moments (doubled coordinates), monomials
+        std::vector<int32_t> mom;
+        std::vector<long long> full((size_t)fk.nf * RF_GROW * o.gpad, 0);
+        std::vector<double> phi, phiT((size_t)0);
+        for (int f = 0; f < fk.nf; ++f) {
+            const int nc = P.nball[f];
+            std::vector<double> pT((size_t)T * nc);
+            for (int gi = 0; gi <= P.ngrow; ++gi) {
+                const double r = o.r0 + 0.5 * gi;
+                const int qlim = (int)floor(4.0 * r * r + 1e-9);
+                int nb = 0;
+                while (nb < nc && ball_q[f][nb] <= qlim) ++nb;
+                o.nb[f][gi] = nb;
+            }
+            for (int c = 0; c < nc; ++c) {
+                int x[3] = {0, 0, 0};
+                for (int a = 0; a < d; ++a) x[a] = 2 * off[f][3 * c + a] + fk.fshift2[f][a] - fk.x0shift2[a];
+                for (int k = 0; k < o.gpad; ++k) {
+                    long long v = 0;
+                    if (k < (int)Gm.size()) {
+                        v = 1;
+                        for (int a = 0; a < 3; ++a)
+                            for (int e = 0; e < Gm[k][a]; ++e) v *= x[a];
+                    }
+                    mom.push_back((int32_t)v);
+                    for (int gi = 0; gi <= P.ngrow; ++gi)
+                        if (c < o.nb[f][gi]) full[((size_t)f * RF_GROW + gi) * o.gpad + k] += v;
+                }
+                for (int k = 0; k < T; ++k) {
+                    double v = 1.0;
+                    for (int a = 0; a < 3; ++a)
+                        for (int e = 1; e <= K[k][a]; ++e) v *= 0.5 * x[a] / e;
+                    phi.push_back(v);
+                    pT[(size_t)k * nc + c] = v;
+                }
+            }
+            phiT.insert(phiT.end(), pT.begin(), pT.end());
+            if (f + 1 < fk.nf && P.nball[f + 1] != nc) return IB_OK;   // one candidate count per field
+        }
+        TRY(upload(tmp, mom, &o.mom));
+        TRY(upload(tmp, full, &o.full));
+        TRY(upload(tmp, phi, &o.phi));
+        TRY(upload(tmp, phiT, &o.phiT));
+        // boundary-condition rows
+        const HostTemplate ht = bc_template(fk.vector_bc, t->bc, d, Mp);
+        o.nbc = (int)ht.rows.size();
+        std::vector<int32_t> pptr;
+        std::vector<uint32_t> prog;
+        std::vector<double> pc, crow;
+        o.ident = -1;
+        for (const auto& row : ht.rows) {
+            std::vector<int32_t> rp(1, 0);
+            std::vector<uint32_t> rw;
+            std::vector<double> rc, cst(n, 0.0);
+            bool constant = true, ident = fk.nf == 1;
+            for (int c = 0; c < n; ++c) {
+                for (const DevTerm& tm : row) {
+                    if (tm.field != c / T) continue;
+                    MI b = K[c % T];
+                    for (int a = 0; a < 3; ++a) b[a] -= tm.alpha[a];
+                    if (b[0] < 0 || b[1] < 0 || b[2] < 0) continue;
+                    const int k = kid[b];
+                    rw.push_back((uint32_t)k | (uint32_t)(tm.axis + 1) << 8);
+                    rc.push_back(tm.coef);
+                    cst[c] += tm.coef;
+                    constant = constant && k == 0 && tm.axis < 0;
+                    ident = ident && k == c && tm.axis < 0 && tm.coef == 1.0;
+                }
+                rp.push_back((int32_t)rw.size());
+                ident = ident && rp[c + 1] == rp[c] + 1;
+            }
+            if (constant) {
+                crow.insert(crow.end(), cst.begin(), cst.end());
+                ++o.nconst;
+                continue;
+            }
+            if (ident) o.ident = o.nrow;
+            for (int32_t v : rp) pptr.push_back(v + (int32_t)prog.size());
+            prog.insert(prog.end(), rw.begin(), rw.end());
+            pc.insert(pc.end(), rc.begin(), rc.end());
+            ++o.nrow;
+        }
+        if (o.nrow > 8 || o.nconst > 2) return IB_OK;
+        TRY(upload(tmp, pptr, &o.prog_ptr));
+        TRY(upload(tmp, prog, &o.prog));
+        TRY(upload(tmp, pc, &o.prog_c));
+        TRY(upload(tmp, crow, &o.crow));
+        R.bc_doubles = std::max(R.bc_doubles, (T + (o.nrow - (o.ident >= 0 ? 1 : 0)) * n) * RF_PITCH);
+        // element list of the upper triangle
+        std::vector<uint16_t> pair;
+        std::vector<int16_t> pgam;
+        std::vector<double> pcoef, pconst;
+        for (int i = 0; i < n; ++i)
+            for (int j = i; j < n; ++j) {
+                pair.push_back((uint16_t)(i | j << 8));
+                const MI &a = K[i % T], &b = K[j % T];
+                const MI sum = {a[0] + b[0], a[1] + b[1], a[2] + b[2]};
+                pgam.push_back((int16_t)(i / T == j / T ? (i / T) * o.gpad + gid[sum] : -1));
+                double v = ldexp(1.0, -(sum[0] + sum[1] + sum[2]));
+                for (int x = 0; x < 3; ++x) v /= fact(a[x]) * fact(b[x]);
+                pcoef.push_back(v);
+                double q = 0.0;
+                for (int c = 0; c < o.nconst; ++c) q += crow[(size_t)c * n + i] * crow[(size_t)c * n + j];
+                pconst.push_back(q);
+            }
+        TRY(upload(tmp, pair, &o.pair));
+        TRY(upload(tmp, pgam, &o.pgam));
+        TRY(upload(tmp, pcoef, &o.pcoef));
+        TRY(upload(tmp, pconst, &o.pconst));
+        // exterior stencil points
+        std::vector<double> uE((size_t)P.rule.nE * n, 0.0);
+        for (int e = 0; e < P.rule.nE; ++e) {
+            int fi = 0;
+            for (int f = 0; f < fk.nf; ++f)
+                if (fk.fkind[f] == P.rule.Efield[e]) fi = f;
+            for (int k = 0; k < T; ++k) {
+                double v = P.rule.Ew[e];
+                for (int a = 0; a < d; ++a) {
+                    const double x = 0.5 * (2 * P.rule.Eoff[e][a] + fk.fshift2[fi][a] - fk.x0shift2[a]);
+                    for (int q = 1; q <= K[k][a]; ++q) v *= x / q;
+                }
+                uE[(size_t)e * n + fi * T + k] = v;
+            }
+        }
+        TRY(upload(tmp, uE, &o.uE));
+        std::vector<uint32_t> mono(T, 0);
+        for (int k = 1; k < T; ++k) {
+            int a = 2;
+            while (K[k][a] == 0) --a;
+            MI b = K[k];
+            --b[a];
+            mono[k] = (uint32_t)kid[b] | (uint32_t)a << 8 | (uint32_t)K[k][a] << 16 |
+                      (uint32_t)(K[k][0] + K[k][1] + K[k][2]) << 24;
+        }
+        TRY(upload(tmp, mono, &o.mono));
+        for (int gi = 0; gi <= P.ngrow; ++gi) {
+            const double r = o.r0 + 0.5 * gi;
+            for (int a = 0; a < d; ++a) {
+                o.lo[a][gi] = (int)ceil(0.5 * fk.x0shift2[a] - r - 0.5 - 1e-12);
+                o.hi[a][gi] = (int)floor(0.5 * fk.x0shift2[a] + r + 0.5 + 1e-12);
+            }
+        }
+    }
+    for (int f = 0; f < fk.nf; ++f) {
+        uint8_t* kept;
+        TRY(tmp.alloc(&kept, t->L.N));
+        k_kept<<<grid_for(t->L.N, 256), 256, 0, s>>>(g, fk.fkind[f], kept);
+        ib_count_launch("setup");
+        if (fk.feta[f] > 0.0 && nbp) {
+            EtaBox b;
+            b.reach = (int)ceil(fk.feta[f] + 1.0);
+            b.eta = fk.feta[f];
+            for (int a = 0; a < 3; ++a) b.shift2[a] = fk.fshift2[f][a];
+            const int W = 2 * b.reach + 1;
+            k_eta_drop<<<grid_for(nbp * (d == 3 ? W * W * W : W * W), 256), 256, 0, s>>>(g, nbp, bp_owner, P.bp_xb, b, kept);
+            ib_count_launch("setup");
+        }
+        IB_CHECK_LAUNCH("k_kept");
+        R.kept[f] = kept;
+    }
+    *ok = true;
+    return IB_OK;
+}
+
+template <int NMAX>
+static ib_status launch_fit_rows(const FitParams& P, RowFit& R, cudaStream_t s) {
+    R.bc_doubles = std::max(R.bc_doubles, NMAX * NMAX / 2);   // also the rank test's FP32 matrix
+    const size_t shm = sizeof(double) * (NMAX * (NMAX + 1) / 2 + R.bc_doubles + 7 * NMAX + RF_CAP + 8 * RF_CB) +
+                       4 * (NMAX * NMAX + 40 + 72 + RF_BP) + 2 * RF_CAP;
+    IB_CUDA(cudaFuncSetAttribute(k_fit_rows<NMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
+    int per_sm = 1;
+    IB_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_fit_rows<NMAX>, 32, shm));
+    const int64_t blocks = std::min<int64_t>(P.nrows, (int64_t)152 * std::max(per_sm, 1));
+    k_fit_rows<NMAX><<<(unsigned)blocks, 32, shm, s>>>(P, R);
+    IB_CHECK_LAUNCH("k_fit_rows");
+    ib_count_launch("setup");
+    return IB_OK;
+}
+
 static ib_status run_fit(ib_table* t, const Geo& g, const FitKind& fk, const int32_t* bp_index,
-                         const double* bp_xb, const double* bp_n, int op_first, cudaStream_t s,
-                         DevBuf& tmp) {
+                         const double* bp_xb, const double* bp_n, const int64_t* bp_owner, int64_t nbp, int op_first,
+                         cudaStream_t s, DevBuf& tmp) {
     const int d = g.ndim;
     const Layout& L = t->L;
     // rows
@@ -1857,11 +2096,13 @@ static ib_status run_fit(ib_table* t, const Geo& g, const FitKind& fk, const int
         return IB_ERR_ARG;
     }
     P.ncol_max = std::max(ncol_max, FIT_PB);
+    std::vector<int8_t> ball_off[3];
+    std::vector<int32_t> ball_q[3];
     for (int f = 0; f < fk.nf; ++f) {
         int frac2[3];
         for (int a = 0; a < 3; ++a) frac2[a] = fk.fshift2[f][a] - fk.x0shift2[a];
-        std::vector<int8_t> off;
-        std::vector<int32_t> q;
+        std::vector<int8_t>& off = ball_off[f];
+        std::vector<int32_t>& q = ball_q[f];
         make_ball(d, frac2, rmax, off, q);
         int8_t* doff;
         int32_t* dq;
@@ -1903,13 +2144,29 @@ static ib_status run_fit(ib_table* t, const Geo& g, const FitKind& fk, const int
     TRY(tmp.alloc(&cnt, std::max<int64_t>(nrows, 1)));
     TRY(tmp.alloc(&start, std::max<int64_t>(nrows, 1)));
     IB_CUDA(cudaMemsetAsync(cnt, 0, sizeof(int32_t) * std::max<int64_t>(nrows, 1), s));
-    int64_t cap = std::max<int64_t>(nrows * 48 * fk.nf, 1024);
+    // room for every row's support at the first radius (a 3D order-8 row holds 64 entries of
+    // its 81 on average; the few rows that grow take what the cut supports leave): an
+    // overflow fits every row again
+    int64_t per_row = 0;
+    for (int f = 0; f < fk.nf; ++f) {
+        const int qlim = (int)floor(4.0 * P.ord[0].r0 * P.ord[0].r0 + 1e-9);
+        for (int32_t q : ball_q[f]) per_row += q <= qlim;
+    }
+    int64_t cap = std::max<int64_t>(nrows * per_row, 1024);
     int32_t* pool_code;
     int8_t* pool_field;
     double* pool_w;
     unsigned long long* top;
     TRY(tmp.alloc(&top, 1));
-    std::vector<int64_t> redo;
+    RowFit R;
+    bool by_rows = false;
+    int32_t* redo = nullptr;
+    unsigned long long* queue = nullptr;   // next row; then the number of rows left to k_fit
+    if (nrows) TRY(row_fit_tables(t, g, fk, P, orders, ball_off, ball_q, bp_owner, nbp, R, s, tmp, &by_rows));
+    if (by_rows) {
+        TRY(tmp.alloc(&redo, nrows));
+        TRY(tmp.alloc(&queue, 2));
+    }
     for (int attempt = 0; attempt < 3; ++attempt) {
         TRY(tmp.alloc(&pool_code, cap));
         TRY(tmp.alloc(&pool_field, cap));
@@ -1931,11 +2188,34 @@ static ib_status run_fit(ib_table* t, const Geo& g, const FitKind& fk, const int
                                        ncm + 4 * ncm + 6 * FIT_MAX_BP + 48) +
                      sizeof(int32_t) * (FIT_MAX_SUP + FIT_MAX_BP + 64);
         IB_CUDA(cudaFuncSetAttribute(k_fit, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
-        if (nrows > 0) {
-            int blocks = (int)std::min<int64_t>(nrows, 152 * 16);
+        const int blocks = (int)std::min<int64_t>(nrows, 152 * 16);
+        if (nrows > 0 && (!by_rows || P.pred)) {
+            P.check_only = by_rows;
             k_fit<<<blocks, FIT_THREADS, shm, s>>>(P);
             IB_CHECK_LAUNCH("k_fit");
             ib_count_launch("setup");
+            P.check_only = 0;
+        }
+        if (by_rows) {
+            IB_CUDA(cudaMemsetAsync(queue, 0, 16, s));
+            R.next = queue;
+            R.redo = redo;
+            R.nredo = (unsigned int*)(queue + 1);
+            if (ncol_max <= 16) TRY(launch_fit_rows<16>(P, R, s));
+            else if (ncol_max <= 32) TRY(launch_fit_rows<32>(P, R, s));
+            else TRY(launch_fit_rows<36>(P, R, s));
+            unsigned int nredo = 0;
+            IB_CUDA(cudaMemcpyAsync(&nredo, R.nredo, sizeof nredo, cudaMemcpyDeviceToHost, s));
+            IB_CUDA(cudaStreamSynchronize(s));
+            if (nredo) {
+                FitParams Q = P;
+                Q.pred = nullptr;
+                Q.sel = redo;
+                Q.nsel = nredo;
+                k_fit<<<(int)std::min<int64_t>(nredo, 152 * 16), FIT_THREADS, shm, s>>>(Q);
+                IB_CHECK_LAUNCH("k_fit");
+                ib_count_launch("setup");
+            }
         }
         IB_CUDA(cudaStreamSynchronize(s));
         // pool overflow?
@@ -2356,7 +2636,7 @@ static ib_status build_impl(const ib_grid* grid, const double* sdf, ib_bc bc, ib
         if (o.extrapolation == IB_EXTRAP_1D)
             st = run_fit1d(t, g, fk, M, w2, s, tmp);
         else
-            st = run_fit(t, g, fk, bp_index, bp_xb, bp_n, 0, s, tmp);
+            st = run_fit(t, g, fk, bp_index, bp_xb, bp_n, bplist, nbp, 0, s, tmp);
         if (st != IB_OK) return fail(st);
     } else {
         std::vector<double> c1 = ib_staggered_first(M);
@@ -2380,7 +2660,7 @@ static ib_status build_impl(const ib_grid* grid, const double* sdf, ib_bc bc, ib
             fk.feta[0] = o.eta_p;
             fk.x0shift2[a] = 1;
             fk.vector_bc = false;
-            if ((st = run_fit(t, g, fk, bp_index, bp_xb, bp_n, a, s, tmp)) != IB_OK) return fail(st);
+            if ((st = run_fit(t, g, fk, bp_index, bp_xb, bp_n, bplist, nbp, a, s, tmp)) != IB_OK) return fail(st);
         }
         // divergence at p nodes: v_a at j + k e_a, k = -H..H-1, weight c1[k + H]
         FitKind fk;
@@ -2403,7 +2683,7 @@ static ib_status build_impl(const ib_grid* grid, const double* sdf, ib_bc bc, ib
             fk.feta[a] = o.eta_v;
         }
         fk.vector_bc = true;
-        if ((st = run_fit(t, g, fk, bp_index, bp_xb, bp_n, d, s, tmp)) != IB_OK) return fail(st);
+        if ((st = run_fit(t, g, fk, bp_index, bp_xb, bp_n, bplist, nbp, d, s, tmp)) != IB_OK) return fail(st);
     }
     if (cudaStreamSynchronize(s) != cudaSuccess) return fail(IB_ERR_CUDA);
     t->setup_seconds = ib_wall_seconds() - t0;
