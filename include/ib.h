@@ -240,10 +240,10 @@ ib_status ib_adjoint(const ib_table* table, const ib_shot* shot, int32_t precisi
 /*
  * ib_forward_batch -- many independent shots, each with its own table (grid
  * and topography), advanced together: every time step is one launch that
- * covers the tiles (or z-marched strips of tiles) of all shots, and all steps
- * are one captured CUDA graph.  The tile shape is timed on the first batch of
- * a size class and remembered; the environment variable IB_BATCH_SHAPE=<0..9>
- * fixes it instead (IB_ERR_ARG outside that range).  Same semantics per shot
+ * covers the blocks of all shots, and all steps are one captured CUDA graph.
+ * The blocks' shape follows from the batch's number of grid points; the
+ * environment variable IB_BATCH_SHAPE=<0..9> fixes it instead (IB_ERR_ARG
+ * outside that range).  Same semantics per shot
  * as ib_forward (precision 32, no checkpoints).  tables[i] and shots[i] are
  * host arrays of length nshot.
  */
@@ -266,7 +266,7 @@ ib_status ib_forward_batch_ckpt(const ib_table* const* tables, const ib_shot* sh
 /*
  * ib_adjoint_batch -- ib_adjoint (same transpose, same checkpoint segments)
  * for many shots at once: every recompute step and every adjoint step is one
- * launch over the tiles of all shots, and the whole backward pass is one
+ * launch over the blocks of all shots, and the whole backward pass is one
  * captured graph.  Per shot i: checkpoints ckpts[i] from ib_forward_batch_ckpt
  * or ib_forward with the same dt, nt and n_ckpt; residuals[i] [nrec][nt];
  * grads[i] [N] receives dJ/dc (overwritten).  Host arrays of nshot device

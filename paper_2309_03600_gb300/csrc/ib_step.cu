@@ -75,16 +75,14 @@ struct PointSet {          // multilinear weights: 8 corner slots per point
     const T* w;
 };
 
-// rows of a small gather table (receiver residual injection in the adjoint)
+// immersed-boundary rows of an operator: padded nodes, entry ranges, packed column offsets
 template <typename T>
-struct RowView {
-    const int64_t* row_pad;
-    const int64_t* row_ptr;
-    const int64_t* col;
+struct RowList {
+    int64_t n;
+    const int64_t* pad;
+    const int64_t* ptr;
+    const int32_t* code;
     const T* w;
-    const int32_t* tile_ptr;
-    const int32_t* perm;
-    int64_t ntx;
 };
 
 // Each warp takes chunks of 32 consecutive entries, four chunks at a time so that
@@ -191,8 +189,9 @@ struct StepArgs {
     // batched runs: the two wavefield buffers (p^n is buf[step & 1])
     T* buf0;
     T* buf1;
-    int64_t ntx;         // tiles along x
-    int64_t ntiles;      // tiles of the shot (blocks beyond only record receivers)
+    RowList<T> rows;     // 2D: the immersed-boundary rows (ib_leap2d.cuh) ...
+    int64_t nrb, ntx;    // ... their blocks, and column blocks along x
+    const T* damp;       // 2D: g of each node (dw > 0)
     int dw;              // absorbing layer width in nodes (0: none)
     T da;                // its largest a = eta_max dt / 2
 };
@@ -248,543 +247,7 @@ __device__ __forceinline__ void cp_async(void* dst, const void* src, bool valid)
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 
-template <typename T, int H, int TX, int TZ>
-__device__ __forceinline__ void leap2d_tile(const StepArgs<T>& a, int64_t bx, int64_t bz, T (*tile)[TX + 2 * H],
-                                            T* acc, T* sadd) {
-    static_assert((TZ * TX) % 256 == 0, "whole points per thread");
-    constexpr int PT = TZ * TX / 256;
-    const int tid = threadIdx.x;
-    const int64_t x0 = bx * TX, z0 = bz * TZ;
-    const Layout& L = a.L;
-    // the halo tile arrives by cp.async (zero fill past the padded array) ...
-    for (int i = tid; i < (TZ + 2 * H) * (TX + 2 * H); i += 256) {
-        const int lz = i / (TX + 2 * H), lx = i - lz * (TX + 2 * H);
-        const int64_t x = x0 + lx - H, z = z0 + lz - H;
-        const bool ok = x < L.nx + H && z < L.nz + H;
-        cp_async<(int)sizeof(T)>(&tile[lz][lx], ok ? a.p + L.base + z * L.px + x : a.p, ok);
-    }
-    cp_async_commit();
-    for (int i = tid; i < TZ * TX; i += 256) sadd[i] = (T)0;
-    // ... while this thread's p_prev and K, and the tile's correction range, load
-    const int64_t origin = L.base + z0 * L.px + x0;
-    T pmv[PT], khv[PT];
-#pragma unroll
-    for (int j = 0; j < PT; ++j) {
-        const int i = tid + 256 * j, lz = i / TX, lx = i - lz * TX;
-        const bool in = x0 + lx < L.nx && z0 + lz < L.nz;
-        const int64_t q = origin + lz * L.px + lx;
-        pmv[j] = in ? a.pm[q] : (T)0;
-        khv[j] = in ? a.Kh[q] : (T)0;
-    }
-    int32_t e0 = 0, e1 = 0;
-    if (a.op.ptr) {
-        e0 = a.op.ptr[bz * a.op.ntx + bx];
-        e1 = a.op.ptr[bz * a.op.ntx + bx + 1];
-    }
-    cp_async_wait_all();
-    __syncthreads();
-    // Laplacian in difference form, sum_k w_k sum_axes (p_{+k} - p_0 + p_{-k} - p_0): the
-    // discrete operator annihilates constants exactly in floating point (row sum zero)
-    for (int i = tid; i < TZ * TX; i += 256) {
-        int lz = i / TX, lx = i - lz * TX;
-        T c = tile[lz + H][lx + H];
-        T s = 0;
-#pragma unroll
-        for (int k = 1; k <= H; ++k)
-            s += a.w2[k] * (((tile[lz + H][lx + H + k] - c) + (tile[lz + H][lx + H - k] - c)) +
-                            ((tile[lz + H + k][lx + H] - c) + (tile[lz + H - k][lx + H] - c)));
-        acc[i] = s;
-    }
-    const T wv = a.src.n ? a.wavelet[a.step] : (T)0;
-    tile_sources<T, TX, TZ>(a.src, wv, origin, L.px, sadd, tid);
-    __syncthreads();
-    if (e1 > e0) add_entries_range(a.op, e0, e1, a.p, origin, acc, tid, 256);
-    __syncthreads();
-    const bool damped = damp_box(L, a.dw, x0, x0 + TX - 1, 0, 0, z0 + TZ - 1);
-#pragma unroll
-    for (int j = 0; j < PT; ++j) {
-        const int i = tid + 256 * j, lz = i / TX, lx = i - lz * TX;
-        if (x0 + lx >= L.nx || z0 + lz >= L.nz) continue;
-        const int64_t q = origin + lz * L.px + lx;
-        const T c = tile[lz + H][lx + H];
-        T u = c + ((c - pmv[j]) + khv[j] * acc[i]) + sadd[i];
-        if (damped) u -= damp_g<T>(L, a.dw, a.da, x0 + lx, 0, z0 + lz) * (u - pmv[j]);
-        a.out[q] = u;
-    }
-}
-
-template <typename T, int H, int TX, int TZ>
-__global__ void __launch_bounds__(256) k_leap2d(StepArgs<T> a) {
-    __shared__ T tile[TZ + 2 * H][TX + 2 * H];
-    __shared__ T acc[TZ * TX];
-    __shared__ T sadd[TZ * TX];
-    const int64_t blk = (int64_t)blockIdx.y * gridDim.x + blockIdx.x;
-    record_receivers(a.rec, a.p, a.traces, a.nt, a.rec_step, blk * 256 + threadIdx.x, launch_threads());
-    leap2d_tile<T, H, TX, TZ>(a, blockIdx.x, blockIdx.y, tile, acc, sadd);
-}
-
-// many shots in one launch: block -> (shot, tile) through the per-shot tile offsets
-template <typename T, int H, int TX, int TZ>
-__global__ void __launch_bounds__(256) k_leap2d_batch(const StepArgs<T>* __restrict__ shots,
-                                                      const int64_t* __restrict__ tile0,
-                                                      const int32_t* __restrict__ shot_of, int nshot, int step) {
-    __shared__ T tile[TZ + 2 * H][TX + 2 * H];
-    __shared__ T acc[TZ * TX];
-    __shared__ T sadd[TZ * TX];
-    const int64_t b = blockIdx.x;
-    const int lo = shot_of[b];            // the shot whose tiles include block b
-    StepArgs<T> a = shots[lo];
-    const int64_t local = b - tile0[lo];
-    T* cur = (step & 1) ? a.buf1 : a.buf0;
-    T* prev = (step & 1) ? a.buf0 : a.buf1;
-    a.p = cur;
-    a.pm = prev;
-    a.out = prev;
-    a.step = step;
-    a.rec_step = step - 1;
-    record_receivers(a.rec, a.p, a.traces, a.nt, a.rec_step, local * 256 + threadIdx.x,
-                     (tile0[lo + 1] - tile0[lo]) * 256);
-    if (local >= a.ntiles) return;   // uniform per block
-    leap2d_tile<T, H, TX, TZ>(a, local % a.ntx, local / a.ntx, tile, acc, sadd);
-}
-
-template <int N>
-__device__ __forceinline__ void cp_async_wait_group() {
-    asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
-}
-
-// A strip 64 wide and up to NSUB tiles of 64 x 8 deep, marched in z with D tiles
-// in flight.  Everything a tile reads arrives by 16-byte cp.async: the strip's
-// rows of p (columns x0-4 .. x0+67; x0-4 is a multiple of 4 because the row pitch
-// is a multiple of 32) into a buffer that holds the whole strip, p_prev and K into
-// D+1 stages.  Each thread owns two vertically adjacent points of every tile and
-// walks a pointer down its column, so the stencil's shared-memory offsets are
-// immediates.  Arithmetic per point is that of leap2d_tile.
-template <int H, int NSUB, int D>
-struct Strip2D {
-    static constexpr int TX = 64, TZ = 8, W = TX + 8, CH = W / 4, ROWS = NSUB * TZ + 2 * H;
-    static_assert(H <= 4 && TZ * CH <= 256 && 2 * H <= TZ, "one chunk per thread and tile");
-    float rows[ROWS][W];   // row j holds z = zs - H + j
-    float pm[D + 1][TZ * TX];
-    float kh[D + 1][TZ * TX];
-    float acc[TZ * TX];
-    float sadd[TZ * TX];
-};
-
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, bool valid) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(dst), "l"(src), "r"(valid ? 16 : 0)
-                 : "memory");
-}
-
-template <int H, int NSUB, int D>
-__device__ __forceinline__ void leap2d_strip(const StepArgs<float>& a, int64_t bx, int64_t bzc,
-                                             Strip2D<H, NSUB, D>& sm) {
-    using S = Strip2D<H, NSUB, D>;
-    constexpr int TX = S::TX, TZ = S::TZ, W = S::W, CH = S::CH;
-    const int tid = threadIdx.x;
-    const Layout& L = a.L;
-    const int64_t ntz = (L.nz + TZ - 1) / TZ;
-    const int64_t bz0 = bzc * NSUB;
-    const int nsub = (int)(ntz - bz0 < NSUB ? ntz - bz0 : NSUB);
-    const int64_t x0 = bx * TX, zs = bz0 * TZ;
-    const int64_t tstep = TZ * L.px;   // elements from one tile's rows to the next
-    // This thread's copies: chunk (pr, pc) of each tile's new rows of p (tid < TZ * CH)
-    // and chunk (qr, qc) of p_prev (tid < 128) or K (tid >= 128).  A chunk is zero-filled
-    // when its row is past the last row a stored point reads, or when it would end past
-    // the allocation; it feeds no stored point then.  The chunks move down tstep
-    // elements per tile: their offsets, rows and shared addresses are carried along.
-    const int pr = tid / CH, pc = tid - pr * CH;
-    const bool pcopy = tid < TZ * CH;
-    auto copy_row = [&](int j) {   // strip row j (tile 0 only)
-        const int64_t z = zs - H + j;
-        const int64_t q = (z + H + 1) * L.px + x0 - 4 + 4 * pc;
-        const bool ok = z < L.nz + H && q + 4 <= L.total;
-        cp_async16(smem_u32(&sm.rows[j][4 * pc]), ok ? a.p + q : a.p, ok);
-    };
-    int64_t pq = (zs + TZ + 2 * H + pr + 1) * L.px + x0 - 4 + 4 * pc;   // tile 1: strip row TZ + 2H + pr
-    const int nzh = (int)(L.nz + H), nzi = (int)L.nz;   // row limits (2D rows < 2^31)
-    const int64_t qlim = L.total - 4;                 // last chunk start inside the allocation
-    int pz = (int)(zs + TZ + H + pr);
-    uint32_t pdst = smem_u32(&sm.rows[0][0]) + 4u * (uint32_t)((TZ + 2 * H + pr) * W + 4 * pc);
-    const int qr = (tid & 127) >> 4, qc = tid & 15;
-    const float* qsrc = tid < 128 ? a.pm : a.Kh;
-    int64_t qq = (zs + qr + H + 1) * L.px + x0 + 4 * qc;                // tile 0
-    int qz = (int)(zs + qr);
-    const uint32_t qdst0 = smem_u32((tid < 128 ? &sm.pm[0][0] : &sm.kh[0][0]) + qr * TX + 4 * qc);
-    int qst = 0;
-    // group t (issued in order t = 0, 1, ...): tile t's new rows of p (rows 0 .. TZ + 2H - 1
-    // for t = 0), its p_prev and K
-    auto issue = [&](int t) {
-        if (t < nsub) {
-            if (pcopy) {
-                if (t == 0) {
-                    copy_row(pr);
-                    if (pr < 2 * H) copy_row(pr + TZ);
-                } else {
-                    const bool ok = pz < nzh && pq <= qlim;
-                    cp_async16(pdst, ok ? a.p + pq : a.p, ok);
-                    pq += tstep;
-                    pz += TZ;
-                    pdst += 4u * TZ * W;
-                }
-            }
-            const bool ok = qz < nzi && qq <= qlim;
-            cp_async16(qdst0 + 4u * TZ * TX * qst, ok ? qsrc + qq : qsrc, ok);
-            qq += tstep;
-            qz += TZ;
-            qst = qst == D ? 0 : qst + 1;
-        }
-        cp_async_commit();   // empty groups keep the count uniform
-    };
-    const int lx = tid & (TX - 1), lz0 = 2 * (tid >> 6);
-    const int i0 = lz0 * TX + lx;
-    sm.sadd[i0] = 0.f;
-    sm.sadd[i0 + TX] = 0.f;
-#pragma unroll
-    for (int t = 0; t < D; ++t) issue(t);
-    // this thread's source corner (tid < 8 n) as (row, column) from the strip origin
-    int srow = -1, scol = 0;
-    float sw = 0.f;
-    const float wv = a.src.n ? a.wavelet[a.step] : 0.f;
-    if (tid < 8 * a.src.n) {
-        const int64_t rel = a.src.idx[tid] - (L.base + zs * L.px + x0);
-        if (rel >= 0) {
-            const int64_t r = rel / L.px, c = rel - r * L.px;
-            if (r < NSUB * TZ && c < TX && a.src.w[tid] != 0.f) {
-                srow = (int)r;
-                scol = (int)c;
-                sw = a.src.w[tid] * wv;
-            }
-        }
-    }
-    const int32_t* pp = a.op.ptr ? a.op.ptr + bz0 * a.op.ntx + bx : nullptr;   // tile s's entry range
-    int32_t e0 = 0, e1 = 0;
-    if (pp) {
-        e0 = pp[0];
-        e1 = pp[1];
-    }
-    const float* colp = &sm.rows[lz0][lx + 4];   // this thread's column, tile s
-    const bool xin = x0 + lx < L.nx;
-    const int zleft = nzi - (int)zs - lz0;       // rows of this thread's column left to store
-    float* outp = a.out + (zs + lz0 + H + 1) * L.px + x0 + lx;
-    int64_t origin = L.base + zs * L.px + x0;    // tile s
-    int st = 0;                                   // stage of tile s
-#pragma unroll 1
-    for (int s = 0; s < nsub; ++s) {
-        cp_async_wait_group<D - 1>();
-        __syncthreads();   // tile s has landed; tile s - 1 is done with its buffers
-        issue(s + D);
-        int32_t f0 = 0, f1 = 0;
-        if (s + 1 < nsub && pp) {
-            pp += a.op.ntx;
-            f0 = pp[0];
-            f1 = pp[1];
-        }
-        // rows z0 + lz0 - H .. z0 + lz0 + 1 + H of this thread's column
-        float v[2 * H + 2];
-#pragma unroll
-        for (int m = 0; m < 2 * H + 2; ++m) v[m] = colp[m * W];
-        float cv[2];
-#pragma unroll
-        for (int j = 0; j < 2; ++j) {
-            const float* r0 = colp + (H + j) * W;
-            const float c = v[H + j];
-            float sum = 0.f;
-#pragma unroll
-            for (int k = 1; k <= H; ++k)
-                sum += a.w2[k] * (((r0[k] - c) + (r0[-k] - c)) + ((v[H + j + k] - c) + (v[H + j - k] - c)));
-            sm.acc[i0 + j * TX] = sum;
-            cv[j] = c;
-        }
-        {
-            const int ly = srow - s * TZ;
-            if (srow >= 0 && ly >= 0 && ly < TZ) atomicAdd(&sm.sadd[ly * TX + scol], sw);
-        }
-        __syncthreads();
-        if (e1 > e0) {
-            add_entries_range(a.op, e0, e1, a.p, origin, sm.acc, tid, 256);
-            __syncthreads();
-        }
-        const float* pmS = sm.pm[st];
-        const float* khS = sm.kh[st];
-        const bool damped = damp_box(L, a.dw, x0, x0 + TX - 1, 0, 0, zs + (s + 1) * TZ - 1);
-#pragma unroll
-        for (int j = 0; j < 2; ++j) {
-            const int i = i0 + j * TX;
-            if (xin && s * TZ + j < zleft) {
-                const float c = cv[j];
-                float u = c + ((c - pmS[i]) + khS[i] * sm.acc[i]) + sm.sadd[i];
-                if (damped) u -= damp_g<float>(L, a.dw, a.da, x0 + lx, 0, zs + s * TZ + lz0 + j) * (u - pmS[i]);
-                outp[j * L.px] = u;
-            }
-            sm.sadd[i] = 0.f;
-        }
-        e0 = f0;
-        e1 = f1;
-        colp += TZ * W;
-        outp += tstep;
-        origin += tstep;
-        st = st == D ? 0 : st + 1;
-    }
-    cp_async_wait_group<0>();   // the empty groups past the strip's end
-}
-
-// many shots in one launch, each block a z-marched strip (leap2d_strip)
-template <int H, int NSUB, int D, int MINB>
-__global__ void __launch_bounds__(256, MINB) k_leap2d_batch_m(const StepArgs<float>* __restrict__ shots,
-                                                              const int64_t* __restrict__ tile0,
-                                                              const int32_t* __restrict__ shot_of, int nshot,
-                                                              int step) {
-    __shared__ __align__(16) Strip2D<H, NSUB, D> sm;
-    const int64_t b = blockIdx.x;
-    const int lo = shot_of[b];
-    StepArgs<float> a = shots[lo];
-    const int64_t local = b - tile0[lo];
-    float* cur = (step & 1) ? a.buf1 : a.buf0;
-    float* prev = (step & 1) ? a.buf0 : a.buf1;
-    a.p = cur;
-    a.pm = prev;
-    a.out = prev;
-    a.step = step;
-    a.rec_step = step - 1;
-    record_receivers(a.rec, a.p, a.traces, a.nt, a.rec_step, local * 256 + threadIdx.x,
-                     (tile0[lo + 1] - tile0[lo]) * 256);
-    if (local >= a.ntiles) return;   // uniform per block
-    leap2d_strip<H, NSUB, D>(a, local % a.ntx, local / a.ntx, sm);
-}
-
-// one shot, FP32: block (x, y) is the z-marched strip of column x and chunk y
-template <int H, int NSUB, int D>
-__global__ void __launch_bounds__(256, 4) k_leap2d_m(StepArgs<float> a) {
-    __shared__ __align__(16) Strip2D<H, NSUB, D> sm;
-    const int64_t blk = (int64_t)blockIdx.y * gridDim.x + blockIdx.x;
-    record_receivers(a.rec, a.p, a.traces, a.nt, a.rec_step, blk * 256 + threadIdx.x, launch_threads());
-    leap2d_strip<H, NSUB, D>(a, blockIdx.x, blockIdx.y, sm);
-}
-
-// ---------------------------------------------------------------------------
-// Strips of 64 x 16 tiles with four points per thread (two x-adjacent columns
-// of two rows): the z-marched strip of leap2d_strip with the x-pair layout of
-// the 3D step.  Per tile a thread loads its two columns' 2H + 2 rows as 8-byte
-// pairs and each of its rows' x neighbours (-4 .. +5) in five 8-byte loads, and
-// the copy issue, waits, barriers and epilogue serve four points.  The strip is
-// NSUB tiles deep and held whole in shared memory; D tiles are in flight.  The
-// arithmetic per point is that of leap2d_tile.
-// ---------------------------------------------------------------------------
-template <int H, int NSUB, int D>
-struct Strip4 {
-    static constexpr int TX = 64, TZ = 16, W = TX + 8, CH = W / 4, ROWS = NSUB * TZ + 2 * H;
-    static constexpr int STAGE = TZ * TX;
-    // floats: rows, p_prev and K stages, acc, sadd
-    static constexpr size_t FLOATS = (size_t)ROWS * W + 2 * (D + 1) * STAGE + 2 * STAGE;
-    static_assert(H <= 4 && 2 * H <= TZ, "x halo of 4 and one tile of look-ahead rows");
-};
-
-template <int H, int NSUB, int D>
-__device__ __forceinline__ void leap2d_strip4(const StepArgs<float>& a, int64_t bx, int64_t bzc, float* smem) {
-    using S = Strip4<H, NSUB, D>;
-    constexpr int TX = S::TX, TZ = S::TZ, W = S::W, CH = S::CH, STAGE = S::STAGE;
-    float* rows = smem;                                  // [ROWS][W], row j <-> z = zs - H + j
-    float* pm = rows + S::ROWS * W;                      // [D + 1][STAGE]
-    float* kh = pm + (D + 1) * STAGE;                    // [D + 1][STAGE]
-    float* acc = kh + (D + 1) * STAGE;                   // [STAGE]
-    float* sadd = acc + STAGE;                           // [STAGE]
-    const int tid = threadIdx.x;
-    const Layout& L = a.L;
-    const int64_t ntz = (L.nz + TZ - 1) / TZ;
-    const int64_t bz0 = bzc * NSUB;
-    const int nsub = (int)(ntz - bz0 < NSUB ? ntz - bz0 : NSUB);
-    const int64_t x0 = bx * TX, zs = bz0 * TZ;
-    const int64_t qlim = L.total - 4;
-    // copies of tile t: its new rows of p (all TZ + 2H rows for t = 0), and its
-    // p_prev and K (chunk tid of each: row tid >> 4, columns 4 (tid & 15) ..)
-    auto issue = [&](int t) {
-        if (t < nsub) {
-            const int j0 = t == 0 ? 0 : t * TZ + 2 * H;           // first strip row to fetch
-            const int nr = t == 0 ? TZ + 2 * H : TZ;
-            for (int c = tid; c < nr * CH; c += 256) {
-                const int r = c / CH, pc = c - r * CH;
-                const int j = j0 + r;
-                const int64_t z = zs - H + j;
-                const int64_t q = (z + H + 1) * L.px + x0 - 4 + 4 * pc;
-                const bool ok = z < L.nz + H && q <= qlim;
-                cp_async16(smem_u32(rows + j * W + 4 * pc), ok ? a.p + q : a.p, ok);
-            }
-            const int st = t % (D + 1);
-            const int qr = tid >> 4, qc = tid & 15;
-            const int64_t z = zs + (int64_t)t * TZ + qr;
-            const int64_t q = (z + H + 1) * L.px + x0 + 4 * qc;
-            const bool ok = z < L.nz && q <= qlim;
-            cp_async16(smem_u32(pm + st * STAGE + qr * TX + 4 * qc), ok ? a.pm + q : a.pm, ok);
-            cp_async16(smem_u32(kh + st * STAGE + qr * TX + 4 * qc), ok ? a.Kh + q : a.Kh, ok);
-        }
-        cp_async_commit();   // empty groups keep the count uniform
-    };
-    const int cx = tid & 31, rz = tid >> 5;
-    const int lx = 2 * cx, lz0 = 2 * rz;                // points (lz0 + j, lx + k), j, k in {0, 1}
-    const int i0 = lz0 * TX + lx;
-    *reinterpret_cast<float2*>(sadd + i0) = make_float2(0.f, 0.f);
-    *reinterpret_cast<float2*>(sadd + i0 + TX) = make_float2(0.f, 0.f);
-#pragma unroll
-    for (int t = 0; t < D; ++t) issue(t);
-    int srow = -1, scol = 0;
-    float sw = 0.f;
-    const float wv = a.src.n ? a.wavelet[a.step] : 0.f;
-    if (tid < 8 * a.src.n) {
-        const int64_t rel = a.src.idx[tid] - (L.base + zs * L.px + x0);
-        if (rel >= 0) {
-            const int64_t r = rel / L.px, c = rel - r * L.px;
-            if (r < NSUB * TZ && c < TX && a.src.w[tid] != 0.f) {
-                srow = (int)r;
-                scol = (int)c;
-                sw = a.src.w[tid] * wv;
-            }
-        }
-    }
-    const int32_t* pp = a.op.ptr ? a.op.ptr + bz0 * a.op.ntx + bx : nullptr;
-    int32_t e0 = 0, e1 = 0;
-    if (pp) {
-        e0 = pp[0];
-        e1 = pp[1];
-    }
-    const float* colp = rows + lz0 * W + lx + 4;        // this thread's column pair, tile s
-    const bool xa = x0 + lx < L.nx, xb = x0 + lx + 1 < L.nx;
-    const int zleft = (int)(L.nz - zs) - lz0;           // rows of this thread left to store
-    float* outp = a.out + (zs + lz0 + H + 1) * L.px + x0 + lx;
-    int64_t origin = L.base + zs * L.px + x0;
-#pragma unroll 1
-    for (int s = 0; s < nsub; ++s) {
-        cp_async_wait_group<D - 1>();
-        __syncthreads();   // tile s has landed; tile s - 1 is done with its buffers
-        issue(s + D);
-        int32_t f0 = 0, f1 = 0;
-        if (s + 1 < nsub && pp) {
-            pp += a.op.ntx;
-            f0 = pp[0];
-            f1 = pp[1];
-        }
-        float2 v[2 * H + 2];   // rows lz0 - H .. lz0 + 1 + H of the two columns
-#pragma unroll
-        for (int m = 0; m < 2 * H + 2; ++m) v[m] = *reinterpret_cast<const float2*>(colp + m * W);
-        float2 cv[2];
-#pragma unroll
-        for (int j = 0; j < 2; ++j) {
-            const float* r0 = colp + (H + j) * W;
-            float2 xr[5];   // r0[-4 .. 5]
-#pragma unroll
-            for (int i = 0; i < 5; ++i) xr[i] = *reinterpret_cast<const float2*>(r0 + 2 * i - 4);
-            auto X = [&](int o) -> float {
-                const int i = o + 4;
-                return (i & 1) ? xr[i >> 1].y : xr[i >> 1].x;
-            };
-            const float ca = v[H + j].x, cb = v[H + j].y;
-            float sa = 0.f, sb = 0.f;
-#pragma unroll
-            for (int k = 1; k <= H; ++k) {
-                sa += a.w2[k] * (((X(k) - ca) + (X(-k) - ca)) + ((v[H + j + k].x - ca) + (v[H + j - k].x - ca)));
-                sb += a.w2[k] * (((X(1 + k) - cb) + (X(1 - k) - cb)) + ((v[H + j + k].y - cb) + (v[H + j - k].y - cb)));
-            }
-            *reinterpret_cast<float2*>(acc + i0 + j * TX) = make_float2(sa, sb);
-            cv[j] = make_float2(ca, cb);
-        }
-        {
-            const int ly = srow - s * TZ;
-            if (srow >= 0 && ly >= 0 && ly < TZ) atomicAdd(&sadd[ly * TX + scol], sw);
-        }
-        __syncthreads();
-        if (e1 > e0) {
-            add_entries_range(a.op, e0, e1, a.p, origin, acc, tid, 256);
-            __syncthreads();
-        }
-        const int st = s % (D + 1);
-        const float* pmS = pm + st * STAGE;
-        const float* khS = kh + st * STAGE;
-        const bool damped = damp_box(L, a.dw, x0, x0 + TX - 1, 0, 0, zs + (s + 1) * TZ - 1);
-#pragma unroll
-        for (int j = 0; j < 2; ++j) {
-            const int i = i0 + j * TX;
-            const float2 pmv = *reinterpret_cast<const float2*>(pmS + i);
-            const float2 khv = *reinterpret_cast<const float2*>(khS + i);
-            const float2 ac = *reinterpret_cast<const float2*>(acc + i);
-            const float2 sd = *reinterpret_cast<const float2*>(sadd + i);
-            const float c0 = cv[j].x, c1 = cv[j].y;
-            float u0 = c0 + ((c0 - pmv.x) + khv.x * ac.x) + sd.x;
-            float u1 = c1 + ((c1 - pmv.y) + khv.y * ac.y) + sd.y;
-            if (damped) {
-                const int64_t z = zs + s * TZ + lz0 + j;
-                u0 -= damp_g<float>(L, a.dw, a.da, x0 + lx, 0, z) * (u0 - pmv.x);
-                u1 -= damp_g<float>(L, a.dw, a.da, x0 + lx + 1, 0, z) * (u1 - pmv.y);
-            }
-            if (s * TZ + j < zleft) {
-                if (xb) *reinterpret_cast<float2*>(outp + j * L.px) = make_float2(u0, u1);
-                else if (xa) outp[j * L.px] = u0;
-            }
-            *reinterpret_cast<float2*>(sadd + i) = make_float2(0.f, 0.f);
-        }
-        e0 = f0;
-        e1 = f1;
-        colp += TZ * W;
-        outp += TZ * L.px;
-        origin += TZ * L.px;
-    }
-    cp_async_wait_group<0>();   // the empty groups past the strip's end
-}
-
-// many shots in one launch, each block a z-marched strip of 64 x 16 tiles
-template <int H, int NSUB, int D, int MINB>
-__global__ void __launch_bounds__(256, MINB) k_leap2d_batch_m4(const StepArgs<float>* __restrict__ shots,
-                                                               const int64_t* __restrict__ tile0,
-                                                               const int32_t* __restrict__ shot_of, int nshot,
-                                                               int step) {
-    extern __shared__ __align__(16) float strip4_sm[];
-    const int64_t b = blockIdx.x;
-    const int lo = shot_of[b];
-    StepArgs<float> a = shots[lo];
-    const int64_t local = b - tile0[lo];
-    float* cur = (step & 1) ? a.buf1 : a.buf0;
-    float* prev = (step & 1) ? a.buf0 : a.buf1;
-    a.p = cur;
-    a.pm = prev;
-    a.out = prev;
-    a.step = step;
-    a.rec_step = step - 1;
-    record_receivers(a.rec, a.p, a.traces, a.nt, a.rec_step, local * 256 + threadIdx.x,
-                     (tile0[lo + 1] - tile0[lo]) * 256);
-    if (local >= a.ntiles) return;   // uniform per block
-    leap2d_strip4<H, NSUB, D>(a, local % a.ntx, local / a.ntx, strip4_sm);
-}
-
-// one shot, FP32: block (x, y) is the z-marched strip of column x and chunk y
-template <int H, int NSUB, int D>
-__global__ void __launch_bounds__(256, 3) k_leap2d_m4(StepArgs<float> a) {
-    extern __shared__ __align__(16) float strip4_sm[];
-    const int64_t blk = (int64_t)blockIdx.y * gridDim.x + blockIdx.x;
-    record_receivers(a.rec, a.p, a.traces, a.nt, a.rec_step, blk * 256 + threadIdx.x, launch_threads());
-    leap2d_strip4<H, NSUB, D>(a, blockIdx.x, blockIdx.y, strip4_sm);
-}
-
-// Batched recompute step n of a checkpoint segment, on z-marched strips: the
-// shot's segment buffer (buf0) holds p^{c-1+j} in slot j, and step n = c + j
-// writes slot j + 2.  The block map counts strips, ntx * ceil(ceil(nz / 8) / NSUB)
-// per shot.
-template <int H, int NSUB, int D>
-__global__ void __launch_bounds__(256, 4) k_leap2d_batch_seg_m(const StepArgs<float>* __restrict__ shots,
-                                                               const int64_t* __restrict__ tile0,
-                                                               const int32_t* __restrict__ shot_of, int n, int j) {
-    __shared__ __align__(16) Strip2D<H, NSUB, D> sm;
-    const int64_t b = blockIdx.x;
-    const int sh = shot_of[b];
-    StepArgs<float> a = shots[sh];
-    const int64_t local = b - tile0[sh];
-    const int64_t nstrip = a.ntx * (((a.L.nz + 7) / 8 + NSUB - 1) / NSUB);
-    if (local >= nstrip) return;   // uniform per block
-    const int64_t tot = a.L.total;
-    a.p = a.buf0 + (int64_t)(j + 1) * tot;
-    a.pm = a.buf0 + (int64_t)j * tot;
-    a.out = a.buf0 + (int64_t)(j + 2) * tot;
-    a.step = n;
-    leap2d_strip<H, NSUB, D>(a, local % a.ntx, local / a.ntx, sm);
-}
+#include "ib_leap2d.cuh"
 
 // Per-shot field copies between wavefield buffers, checkpoints and segment buffers
 template <typename T>
@@ -1828,210 +1291,6 @@ __global__ void __launch_bounds__(256, 4) k_stag_p2d(StagArgs<T> a) {
 }
 
 // ---------------------------------------------------------------------------
-// 2D adjoint of the leapfrog map and the velocity gradient
-//   mu^m = 2 mu^{m+1} - mu^{m+2} + mask (L^T (K mu^{m+1})) + R^T res^{m-1}
-//   g   += mu^m (2 / c) (p^m - 2 p^{m-1} + p^{m-2} - s^{m-1})
-//   gw[m-1] = S . mu^m
-// ---------------------------------------------------------------------------
-template <typename T>
-struct AdjArgs {
-    Layout L;
-    T w2[5];
-    const T* mu;         // mu^{m+1}
-    const T* mum;        // mu^{m+2}
-    T* out;              // mu^m (may alias mum)
-    const T* Kh;         // dt^2 c^2 / h^2
-    const uint8_t* mask;
-    T two_dt_over_h;     // 2 dt / h  (2 / c = two_dt_over_h / sqrt(Kh))
-    TileView<T> opT;     // transposed corrections, keyed by column node
-    RowView<T> inj;      // receiver injection: col = receiver id
-    const T* res;        // [nrec][nt]
-    int nt;
-    int m;
-    const T* pm0;        // p^m
-    const T* pm1;        // p^{m-1}
-    const T* pm2;        // p^{m-2}
-    T* grad;             // padded accumulator
-    PointSet<T> src;
-    const T* wavelet;
-    T* gw;               // [nt] or null
-    int dw;              // absorbing layer (as StepArgs); the stored multiplier is
-    T da;                // nu^m = mu^m / (1 + a)
-};
-
-// one adjoint tile (bx, bz); shared arrays from the calling kernel
-template <typename T, int H, int TX, int TZ>
-__device__ __forceinline__ void adj2d_tile(const AdjArgs<T>& a, int64_t bx, int64_t bz, T (*tile)[TX + 8], T* tmu,
-                                           T* acc, T* sw) {
-    static_assert((TZ * TX) % 256 == 0, "whole points per thread");
-    constexpr int W = TX + 8, V = 16 / (int)sizeof(T), CHR = W / V;
-    constexpr int PT = TZ * TX / 256, NT = (TZ + 2 * H) * W;
-    static_assert(H <= 4 && TX % 64 == 0, "columns x0-4 .. x0+TX+3 in 16-byte chunks");
-    const int tid = threadIdx.x;
-    const int64_t x0 = bx * TX, z0 = bz * TZ;
-    const Layout& L = a.L;
-    const int64_t origin = L.base + z0 * L.px + x0;
-    const int64_t tile_id = bz * a.opT.ntx + bx;
-    // K and mu halo tiles arrive by 16-byte cp.async: rows z0-H .. z0+TZ+H-1, columns
-    // x0-4 .. x0+TX+3 (x0-4 is 16-byte aligned: the row pitch is a multiple of 32
-    // elements).  Rows past nz+H-1 and chunks that would end past the allocation are
-    // zero-filled; columns past nx+H-1 feed no stored point ...
-    for (int i = tid; i < (TZ + 2 * H) * CHR; i += 256) {
-        const int r = i / CHR, c = i - r * CHR;
-        const int64_t z = z0 - H + r;
-        const int64_t q = (z + H + 1) * L.px + x0 - 4 + V * c;
-        const bool ok = z < L.nz + H && q + V <= L.total;
-        cp_async<16>(&tile[r][V * c], ok ? a.Kh + q : a.Kh, ok);
-        cp_async<16>(&tmu[r * W + V * c], ok ? a.mu + q : a.mu, ok);
-    }
-    cp_async_commit();
-    for (int i = tid; i < TZ * TX; i += 256) sw[i] = (T)0;
-    // ... while this thread's operands and the tile's entry ranges load
-    T mu_v[PT], mum_v[PT], kh_v[PT], p0_v[PT], p1_v[PT], p2_v[PT], g_v[PT];
-    bool msk[PT];
-#pragma unroll
-    for (int j = 0; j < PT; ++j) {
-        const int i = tid + 256 * j, lz = i / TX, lx = i - lz * TX;
-        const bool in = x0 + lx < L.nx && z0 + lz < L.nz;
-        const int64_t q = origin + lz * L.px + lx;
-        mu_v[j] = in ? a.mu[q] : (T)0;
-        mum_v[j] = in ? a.mum[q] : (T)0;
-        kh_v[j] = in ? a.Kh[q] : (T)0;
-        msk[j] = in ? a.mask[q] != 0 : false;
-        p0_v[j] = in ? a.pm0[q] : (T)0;
-        p1_v[j] = in ? a.pm1[q] : (T)0;
-        p2_v[j] = in ? a.pm2[q] : (T)0;
-        g_v[j] = in ? a.grad[q] : (T)0;
-    }
-    int32_t e0 = 0, e1 = 0, j0 = 0, j1 = 0;
-    if (a.opT.ptr) {
-        e0 = a.opT.ptr[tile_id];
-        e1 = a.opT.ptr[tile_id + 1];
-    }
-    if (a.inj.tile_ptr) {
-        j0 = a.inj.tile_ptr[tile_id];
-        j1 = a.inj.tile_ptr[tile_id + 1];
-    }
-    cp_async_wait_all();
-    __syncthreads();
-    for (int i = tid; i < NT; i += 256) (&tile[0][0])[i] *= tmu[i];
-    __syncthreads();
-    for (int i = tid; i < TZ * TX; i += 256) {
-        int lz = i / TX, lx = i - lz * TX;
-        T c = tile[lz + H][lx + 4];
-        T s = 0;
-#pragma unroll
-        for (int k = 1; k <= H; ++k)
-            s += a.w2[k] * (((tile[lz + H][lx + 4 + k] - c) + (tile[lz + H][lx + 4 - k] - c)) +
-                            ((tile[lz + H + k][lx + 4] - c) + (tile[lz + H - k][lx + 4] - c)));
-        acc[i] = s;
-    }
-    tile_sources<T, TX, TZ>(a.src, (T)1, origin, L.px, sw, tid);
-    __syncthreads();
-    for (int32_t e = e0 + tid; e < e1; e += 256) {
-        int64_t s = origin + a.opT.src[e];
-        atomicAdd(&acc[a.opT.loc[e]], a.opT.w[e] * (a.Kh[s] * a.mu[s]));
-    }
-    __syncthreads();
-#pragma unroll
-    for (int j = 0; j < PT; ++j) {
-        const int i = tid + 256 * j;
-        if (!msk[j]) acc[i] = (T)0;
-    }
-    __syncthreads();
-    if (j1 > j0) {
-        const int warp = tid >> 5, lane = tid & 31;
-        for (int k = j0 + warp; k < j1; k += 8) {
-            const int32_t r = a.inj.perm[k];
-            const int64_t q = a.inj.row_pad[r];
-            T s = 0;
-            for (int64_t j = a.inj.row_ptr[r] + lane; j < a.inj.row_ptr[r + 1]; j += 32)
-                s += a.inj.w[j] * a.res[a.inj.col[j] * (int64_t)a.nt + (a.m - 1)];
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-            if (lane == 0) {
-                int64_t loc = q - origin;
-                int64_t dz = loc / L.px;
-                acc[dz * TX + (loc - dz * L.px)] += s;
-            }
-        }
-    }
-    __syncthreads();
-    const T wv = a.src.n ? a.wavelet[a.m - 1] : (T)0;
-    const bool damped = damp_box(L, a.dw, x0, x0 + TX - 1, 0, 0, z0 + TZ - 1);
-#pragma unroll
-    for (int j = 0; j < PT; ++j) {
-        const int i = tid + 256 * j, lz = i / TX, lx = i - lz * TX;
-        if (x0 + lx >= L.nx || z0 + lz >= L.nz) continue;
-        const int64_t q = origin + lz * L.px + lx;
-        // With an absorbing layer the buffers hold nu = mu / (1 + a): the transpose of
-        // p^{n+1} = ((2 + K L) p^n - (1 - a) p^{n-1} + s) / (1 + a) is
-        // mu^m = 2 nu^{m+1} - (1 - a) nu^{m+2} + L^T (K nu^{m+1}) + R^T res^{m-1}.
-        const T av = damped ? damp_a<T>(L, a.dw, a.da, x0 + lx, 0, z0 + lz) : (T)0;
-        T mu_new = (T)2 * mu_v[j] - ((T)1 - av) * mum_v[j] + acc[i];
-        if (damped) mu_new = mu_new / ((T)1 + av);
-        a.out[q] = mu_new;
-        const T Kq = kh_v[j];
-        if (Kq > (T)0) {
-            // dt^2 c^2 (L p^{m-1}) = (1 + a) p^m - 2 p^{m-1} + (1 - a) p^{m-2} - s^{m-1}
-            T d2 = (p0_v[j] - p1_v[j]) - (p1_v[j] - p2_v[j]);
-            if (damped) d2 += av * (p0_v[j] - p2_v[j]);
-            const T srcw = sw[i];
-            d2 -= srcw * wv;
-            a.grad[q] = g_v[j] + mu_new * (a.two_dt_over_h / sqrt(Kq)) * d2;
-            if (a.gw && srcw != (T)0) atomicAdd(&a.gw[a.m - 1], srcw * mu_new);
-        }
-    }
-}
-
-template <typename T, int H, int TX, int TZ>
-__global__ void __launch_bounds__(256) k_adj2d(AdjArgs<T> a) {
-    __shared__ __align__(16) T tile[TZ + 2 * H][TX + 8];     // K mu on the halo tile
-    __shared__ __align__(16) T tmu[(TZ + 2 * H) * (TX + 8)];
-    __shared__ T acc[TZ * TX];
-    __shared__ T sw[TZ * TX];                      // source weights landing in the tile
-    adj2d_tile<T, H, TX, TZ>(a, blockIdx.x, blockIdx.y, tile, tmu, acc, sw);
-}
-
-// Batched adjoint step m of segment [c, e) over many shots: block -> (shot, tile)
-// by table.  mu^{m+1} / mu^{m+2} alternate between the shot's two buffers with
-// the number of steps taken (nt - m); the segment buffer holds p^{c-1+j} in slot j.
-template <typename T>
-struct AdjBatch {
-    AdjArgs<T> a;
-    T* mu1;
-    T* mu2;
-    T* seg;               // segment buffer: (seg_len + 2) padded fields
-};
-
-template <typename T, int H, int TX, int TZ>
-__global__ void __launch_bounds__(256, 3) k_adj2d_batch(const AdjBatch<T>* __restrict__ shots,
-                                                     const int64_t* __restrict__ tile0,
-                                                     const int32_t* __restrict__ shot_of, int m, int j, int nt) {
-    __shared__ __align__(16) T tile[TZ + 2 * H][TX + 8];
-    __shared__ __align__(16) T tmu[(TZ + 2 * H) * (TX + 8)];
-    __shared__ T acc[TZ * TX];
-    __shared__ T sw[TZ * TX];
-    const int64_t b = blockIdx.x;
-    const int sh = shot_of[b];
-    const AdjBatch<T>& B = shots[sh];
-    AdjArgs<T> a = B.a;
-    const bool even = ((nt - m) & 1) == 0;
-    a.mu = even ? B.mu1 : B.mu2;
-    a.mum = even ? B.mu2 : B.mu1;
-    a.out = const_cast<T*>(a.mum);
-    a.m = m;
-    const int64_t tot = a.L.total;
-    a.pm0 = B.seg + (int64_t)(j + 1) * tot;
-    a.pm1 = B.seg + (int64_t)j * tot;
-    a.pm2 = B.seg + (int64_t)(j - 1) * tot;
-    const int64_t local = b - tile0[sh];
-    const int64_t ntiles = a.opT.ntx * ((a.L.nz + TZ - 1) / TZ);
-    if (local >= ntiles) return;   // uniform per block
-    adj2d_tile<T, H, TX, TZ>(a, local % a.opT.ntx, local / a.opT.ntx, tile, tmu, acc, sw);
-}
-
-// ---------------------------------------------------------------------------
 // setup kernels (coefficients formed in FP64, rounded once)
 // ---------------------------------------------------------------------------
 template <typename T>
@@ -2099,14 +1358,6 @@ __global__ void k_interp_setup(int n, const double* xyz, int ndim, double inv_h,
     }
 }
 
-template <typename T>
-__global__ void k_unpad(Layout L, const T* pad, T* out) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < L.N; i += (int64_t)gridDim.x * blockDim.x) {
-        int64_t x = i % L.nx, r = i / L.nx, y = r % L.ny, z = r / L.ny;
-        out[i] = pad[L.idx(x, y, z)];
-    }
-}
-
 // ---------------------------------------------------------------------------
 // stability checks
 //   - every forward / adjoint run ends with a pass over its final fields; a
@@ -2117,8 +1368,6 @@ __global__ void k_unpad(Layout L, const T* pad, T* out) {
 //     renormalises every STAB_BLOCK steps: a power iteration on the one-step
 //     map whose per-step growth estimates its spectral radius.
 // ---------------------------------------------------------------------------
-static __device__ int g_dev_status;
-
 template <typename T>
 __global__ void k_check_finite(int64_t n, const T* __restrict__ a, const T* __restrict__ b,
                                const T* __restrict__ c) {
@@ -2128,7 +1377,7 @@ __global__ void k_check_finite(int64_t n, const T* __restrict__ a, const T* __re
         if (b) bad |= !isfinite(b[i]);
         if (c) bad |= !isfinite(c[i]);
     }
-    if (__any_sync(0xffffffffu, bad) && (threadIdx.x & 31) == 0) atomicOr(&g_dev_status, 1);
+    if (__any_sync(0xffffffffu, bad) && (threadIdx.x & 31) == 0) atomicOr(&g_dev_status, STATUS_UNSTABLE);
 }
 
 // SplitMix64 output function (Steele, Lea & Flood, "Fast splittable
@@ -2279,8 +1528,6 @@ static TileView<T> tview(const TileBins* b) {
     return v;
 }
 
-static const int TX2 = 64, TZ2 = 8;
-
 // cuTensorMapEncodeTiled through the runtime's driver entry point (no libcuda link)
 static PFN_cuTensorMapEncodeTiled_v12000 tma_encode_fn() {
     static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
@@ -2405,35 +1652,192 @@ extern "C" int64_t ib_checkpoint_bytes(const ib_table* t, int32_t precision, int
     return (int64_t)n_ckpt * 2 * t->L.total * es;
 }
 
-static const int STRIP_NSUB = 8, STRIP_D = 3;   // z-marched strips: 8 tiles of 64 x 8, 3 in flight
+// Shapes of the 2D steps: vx columns a thread; rz rows (burst) or a march of zc rows.
+struct LeapShape {
+    int vx, rz, zc;
+};
+static const int kNumShapes = 10;
+static const LeapShape kShapes[kNumShapes] = {{1, 1, 0},  {2, 2, 0},  {2, 4, 0},  {4, 2, 0},  {4, 0, 16},
+                                              {4, 0, 24}, {4, 0, 32}, {4, 0, 48}, {4, 0, 64}, {4, 0, 128}};
+static int64_t shape_ntx(const LeapShape& p, const Layout& L) { return (L.nx + 32 * p.vx - 1) / (32 * p.vx); }
+static int64_t shape_blocks(const LeapShape& p, const Layout& L) {
+    const int64_t rows = (int64_t)LEAP_WARPS * (p.rz ? p.rz : p.zc);
+    return shape_ntx(p, L) * ((L.nz + rows - 1) / rows);
+}
 
-// One FP32 shot runs on strips when there are enough of them to fill the GPU
-// (a strip is 8 tiles of work: on small grids the tile kernel keeps more blocks
-// in flight).  IB_STRIP=0 / IB_STRIP=1 turn strips off / on whatever the size.
-static bool use_strips(const Layout& L) {
-    const int64_t nblk = ((L.nx + TX2 - 1) / TX2) * (((L.nz + TZ2 - 1) / TZ2 + STRIP_NSUB - 1) / STRIP_NSUB);
+static int64_t row_blocks(int64_t rows, int rz) {
+    const int64_t per = rz ? RowsPer<1>::N : RowsPer<0>::N;
+    return (rows + per - 1) / per;
+}
+
+// IB_STRIP=0 / 1 forces bursts / marches (one FP32 shot and both adjoints); -1: not set
+static int strip_switch() {
     const char* e = getenv("IB_STRIP");
-    if (e && *e) return e[0] != '0';
-    return nblk >= 1024;
+    return e && *e ? e[0] != '0' : -1;
+}
+// Shape of a step over `points` grid points in one launch.  A small grid needs many threads
+// with little to do, a large one few instructions a point; the march has a floor of about 25 us
+// (its 8 dependent steps).  us per step, order 8, damped, set-up included (a launch takes the
+// host about 7):
+//   10^6 points        0.16   0.42   0.79   2.1    4.2    7.5   16.8   33.6
+//   burst 1 x 1         7.2    9.3   12.3   23.9   43.6   79.3   178    358
+//   burst 2 x 2         7.1    7.2    9.2   15.7   25.2   48.5   109    219
+//   burst 4 x 2         7.2    9.0    9.2   13.6   21.0   40.3    91    182
+//   march, 16 rows     25.5   25.6   25.4   27.0   27.8   38.1    77    147
+// Longer marches were slower at every size.  Batches cross at the same sizes: 12 shots with
+// 6.5 x 10^6 points 82 (burst 4 x 2) and 70, 48 shots with 28.9 x 10^6 points 353 and 226.
+static int leap_shape(int64_t points) {
+    if (points >= 6000000) return 4;
+    if (points >= 1200000) return 3;
+    return points >= 150000 ? 1 : 0;
+}
+static int leap_shape_shot(const Layout& L) {
+    const int f = strip_switch();
+    return f < 0 ? leap_shape(L.nx * L.nz) : f ? 4 : 1;
 }
 
 template <typename T>
-static void launch_leap2d(const StepArgs<T>& a, int H, dim3 grid, cudaStream_t s) {
-    PROF_LAUNCH(kname<T>("leap2d_f32", "leap2d_f64"), s, {
-        if (H == 1) k_leap2d<T, 1, TX2, TZ2><<<grid, 256, 0, s>>>(a);
-        else if (H == 2) k_leap2d<T, 2, TX2, TZ2><<<grid, 256, 0, s>>>(a);
-        else if (H == 3) k_leap2d<T, 3, TX2, TZ2><<<grid, 256, 0, s>>>(a);
-        else k_leap2d<T, 4, TX2, TZ2><<<grid, 256, 0, s>>>(a);
-    });
+static RowList<T> row_list(const IbOp& op) {
+    return {op.nrows, op.row_pad, op.row_ptr, op.col_code,
+            (const T*)(sizeof(T) == 8 ? (const void*)op.w64 : (const void*)op.w32)};
 }
 
-static void launch_leap2d_strip(const StepArgs<float>& a, int H, dim3 grid, cudaStream_t s) {
-    PROF_LAUNCH("leap2d_strip_f32", s, {
-        if (H == 1) k_leap2d_m<1, STRIP_NSUB, STRIP_D><<<grid, 256, 0, s>>>(a);
-        else if (H == 2) k_leap2d_m<2, STRIP_NSUB, STRIP_D><<<grid, 256, 0, s>>>(a);
-        else if (H == 3) k_leap2d_m<3, STRIP_NSUB, STRIP_D><<<grid, 256, 0, s>>>(a);
-        else k_leap2d_m<4, STRIP_NSUB, STRIP_D><<<grid, 256, 0, s>>>(a);
+// calls f(H as a constant, shape's VX and RZ as constants)
+template <int VX, int RZ, class F>
+static void with_h(int H, F f) {
+    std::integral_constant<int, VX> vx;
+    std::integral_constant<int, RZ> rz;
+    if (H == 1) f(std::integral_constant<int, 1>(), vx, rz);
+    else if (H == 2) f(std::integral_constant<int, 2>(), vx, rz);
+    else if (H == 3) f(std::integral_constant<int, 3>(), vx, rz);
+    else f(std::integral_constant<int, 4>(), vx, rz);
+}
+template <class F>
+static void with_shape(int si, int H, F f) {
+    const LeapShape& p = kShapes[si];
+    if (p.rz == 1) with_h<1, 1>(H, f);
+    else if (p.vx == 2 && p.rz == 2) with_h<2, 2>(H, f);
+    else if (p.vx == 2 && p.rz == 4) with_h<2, 4>(H, f);
+    else if (p.rz == 2) with_h<4, 2>(H, f);
+    else with_h<4, 0>(H, f);
+}
+
+// one step of one shot; a.nrb and a.ntx are set here
+static void launch_leap2d(StepArgs<float>& a, int si, int H, cudaStream_t s) {
+    const LeapShape& p = kShapes[si];
+    a.nrb = row_blocks(a.rows.n, p.rz);
+    a.ntx = shape_ntx(p, a.L);
+    const unsigned grid = (unsigned)(a.nrb + shape_blocks(p, a.L));
+    PROF_LAUNCH(p.rz ? "leap2d_f32" : "leap2d_strip_f32", s, {
+        with_shape(si, H, [&](auto h, auto vx, auto rz) {
+            constexpr size_t sm = leap_smem<h.value, rz.value>();
+            if (sm > 48 * 1024)
+                cudaFuncSetAttribute(k_leap2d<float, h.value, vx.value, rz.value>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)sm);
+            k_leap2d<float, h.value, vx.value, rz.value><<<grid, LEAP_THREADS, sm, s>>>(a, p.zc);
+        });
     });
+}
+static void launch_leap2d(StepArgs<double>& a, int, int H, cudaStream_t s) {
+    const LeapShape& p = kShapes[0];
+    a.nrb = row_blocks(a.rows.n, p.rz);
+    a.ntx = shape_ntx(p, a.L);
+    const unsigned grid = (unsigned)(a.nrb + shape_blocks(p, a.L));
+    PROF_LAUNCH("leap2d_f64", s, {
+        with_h<1, 1>(H, [&](auto h, auto, auto) { k_leap2d<double, h.value, 1, 1><<<grid, LEAP_THREADS, 0, s>>>(a, 0); });
+    });
+}
+// the absorbing layer's factor at every node (null without a layer)
+template <typename T>
+static ib_status damp_field(const Layout& L, int dw, T da, bool adjoint, Scratch& S, const T** out) {
+    *out = nullptr;
+    if (!dw) return IB_OK;
+    T* f;
+    TRY(S.alloc(&f, L.total, true));
+    k_damp_field<T><<<grid1(L.N, 256), 256, 0, S.s>>>(L, dw, da, adjoint, f);
+    IB_CHECK_LAUNCH("k_damp_field");
+    ib_count_launch("setup");
+    *out = f;
+    return IB_OK;
+}
+// Small grids: all steps between two checkpoints in one cooperative launch (k_leap2d_run), if
+// one block per SM can hold the grid with 1 or 4 points a thread (about 430 000 points;
+// with 16, for twice that, a step took 13.9 us at 1013 x 777 against 9.2 us launch by launch).
+// us per step in one launch and launch by launch, FP32 order 8: 201 x 201 3.5 and 7.2, 400 x 400
+// 4.4 and 7.1, 700 x 600 5.4 and 7.2; FP64 order 4, 201 x 201: 3.9, and 12.4 on the tiles before.
+struct RunPlan {
+    int vx, rz, cw;
+    int64_t blocks;          // 0: the grid does not fit
+};
+template <typename T>
+static RunPlan run_plan(const Layout& L, int H) {
+    int dev = 0, sms = 0, coop = 0;
+    RunPlan none = {0, 0, 0, 0};
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess || !coop)
+        return none;
+    const int shapes[2][2] = {{1, 1}, {2, 2}};
+    const int threads[2] = {sizeof(T) == 8 ? (H <= 2 ? 1024 : 512) : 1024, 768};
+    for (int i = 0; i < (sizeof(T) == 8 ? 1 : 2); ++i) {
+        const int vx = shapes[i][0], rz = shapes[i][1], most = threads[i] / 32 - RUN_RW;
+        const int64_t ntx = (L.nx + 32 * vx - 1) / (32 * vx);
+        if (ntx > sms) continue;
+        const int64_t cw = (L.nz + (sms / ntx) * rz - 1) / ((sms / ntx) * rz);
+        if (cw <= most) return {vx, rz, (int)cw, ntx * ((L.nz + cw * rz - 1) / (cw * rz))};
+    }
+    return none;
+}
+template <typename T, int H, int VX, int RZ>
+static cudaError_t launch_run_shape(RunArgs<T>& r, const RunPlan& p, cudaStream_t s) {
+    const int threads = 32 * (p.cw + RUN_RW);
+    const size_t sm = sizeof(RunRow<T>) * RUN_ROWS + (sizeof(T) + sizeof(int)) * RUN_ENT + sizeof(T) * 2 * VX * RZ * threads;
+    cudaError_t e = cudaFuncSetAttribute(k_leap2d_run<T, H, VX, RZ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (e != cudaSuccess) return e;
+    r.cw = p.cw;
+    r.a.ntx = (r.a.L.nx + 32 * VX - 1) / (32 * VX);
+    void* args[] = {&r};
+    return cudaLaunchCooperativeKernel((const void*)k_leap2d_run<T, H, VX, RZ>, dim3((unsigned)p.blocks), dim3(threads), args,
+                                       sm, s);
+}
+template <typename T, int H>
+static cudaError_t launch_run_h(RunArgs<T>& r, const RunPlan& p, cudaStream_t s) {
+    if (p.vx == 1) return launch_run_shape<T, H, 1, 1>(r, p, s);
+    if constexpr (sizeof(T) == 4) {
+        if (p.vx == 2) return launch_run_shape<T, H, 2, 2>(r, p, s);
+    }
+    return cudaErrorInvalidValue;
+}
+// steps n0 .. n1 - 1; bar: a zeroed word of this launch
+template <typename T>
+static ib_status launch_run(const StepArgs<T>& a, const RunPlan& p, int H, T* buf0, T* buf1, int64_t stride, int n0, int n1,
+                            unsigned* bar, cudaStream_t s) {
+    RunArgs<T> r;
+    memset(&r, 0, sizeof r);
+    r.a = a;
+    r.buf0 = buf0;
+    r.buf1 = buf1;
+    r.stride = stride;
+    r.n0 = n0;
+    r.n1 = n1;
+    r.bar = bar;
+    cudaError_t e = cudaSuccess;
+    PROF_LAUNCH(kname<T>("leap2d_run_f32", "leap2d_run_f64"), s, {
+        if (H == 1) e = launch_run_h<T, 1>(r, p, s);
+        else if (H == 2) e = launch_run_h<T, 2>(r, p, s);
+        else if (H == 3) e = launch_run_h<T, 3>(r, p, s);
+        else e = launch_run_h<T, 4>(r, p, s);
+    });
+    if (e != cudaSuccess) return ib_cuda_fail(e, "k_leap2d_run", __FILE__, __LINE__);
+    return IB_OK;
+}
+
+template <typename T>
+static ib_status mark_rows(const RowList<T>& r, T* Kh, cudaStream_t s) {
+    if (r.n == 0) return IB_OK;
+    k_mark_rows<T><<<grid1(r.n, 256), 256, 0, s>>>(r.n, r.pad, Kh);
+    IB_CHECK_LAUNCH("k_mark_rows");
+    ib_count_launch("setup");
+    return IB_OK;
 }
 
 // ---------------------------------------------------------------------------
@@ -2817,32 +2221,6 @@ static void launch_tb2(const TbArgs& a, int H, int R, dim3 grid, cudaStream_t s)
     });
 }
 
-// Single FP32 shots on strips use 64 x 16 tiles with two columns per thread
-// (IB_STRIP4=0 selects the 64 x 8 strips): 134 against 176 us per step at
-// 8192 x 4096, order 8.
-static bool strip4_enabled() {
-    const char* e = getenv("IB_STRIP4");
-    return !(e && e[0] == '0');
-}
-
-template <int H>
-static void launch_strip4_h(const StepArgs<float>& a, dim3 grid, cudaStream_t s) {
-    constexpr size_t sm = Strip4<H, 4, 2>::FLOATS * sizeof(float);
-    static const bool attr = (cudaFuncSetAttribute(k_leap2d_m4<H, 4, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   (int)sm),
-                              true);
-    (void)attr;
-    k_leap2d_m4<H, 4, 2><<<grid, 256, sm, s>>>(a);
-}
-static void launch_leap2d_strip4(const StepArgs<float>& a, int H, dim3 grid, cudaStream_t s) {
-    PROF_LAUNCH("leap2d_strip_f32", s, {
-        if (H == 1) launch_strip4_h<1>(a, grid, s);
-        else if (H == 2) launch_strip4_h<2>(a, grid, s);
-        else if (H == 3) launch_strip4_h<3>(a, grid, s);
-        else launch_strip4_h<4>(a, grid, s);
-    });
-}
-
 template <typename T>
 static ib_status forward_2nd(ib_table* t, const ib_shot* sh, double dt, int nt, void* ckpt, int n_ckpt,
                              cudaStream_t s, const Probe* probe = nullptr) {
@@ -2866,8 +2244,7 @@ static ib_status forward_2nd(ib_table* t, const ib_shot* sh, double dt, int nt, 
     Geom<T> g;
     TRY(setup_points<T>(t, sh, dt * dt / pow(t->grid.h, d), S, g));
     const TileBins* bins = nullptr;
-    if (d == 2) TRY(ib_table_bins(t, 0, false, TX2, 1, TZ2, &bins, s));
-    else TRY(ib_table_bins(t, 0, false, 32, 8, 1, &bins, s));
+    if (d == 3) TRY(ib_table_bins(t, 0, false, 32, 8, 1, &bins, s));
     StepArgs<T> a;
     memset(&a, 0, sizeof a);
     a.L = L;
@@ -2877,6 +2254,7 @@ static ib_status forward_2nd(ib_table* t, const ib_shot* sh, double dt, int nt, 
     }
     a.Kh = Kh;
     a.op = tview<T>(bins);
+    a.rows = row_list<T>(t->ops[0]);
     a.src = g.src;
     a.wavelet = (const T*)sh->wavelet_dev;
     a.rec = g.rec;
@@ -2886,17 +2264,8 @@ static ib_status forward_2nd(ib_table* t, const ib_shot* sh, double dt, int nt, 
     const int64_t seg = ckpt ? ckpt_seg(nt, n_ckpt) : 0;
     T* cur = p0;   // p^n
     T* prev = p1;  // p^{n-1}
-    dim3 grid2((unsigned)((L.nx + TX2 - 1) / TX2), (unsigned)((L.nz + TZ2 - 1) / TZ2));
-    const bool strips = d == 2 && sizeof(T) == 4 && use_strips(L);
-    // strips of 64 x 16 tiles, two columns per thread (default; IB_STRIP4=0: 64 x 8)
-    const bool strip4 = strips && strip4_enabled();
-    StepArgs<T> a4 = a;
-    dim3 grid4((unsigned)((L.nx + 63) / 64), (unsigned)(((L.nz + 15) / 16 + 3) / 4));
-    if (strip4) {
-        const TileBins* b4 = nullptr;
-        TRY(ib_table_bins(t, 0, false, 64, 1, 16, &b4, s));
-        a4.op = tview<T>(b4);
-    }
+    const int shape = d == 2 ? leap_shape_shot(L) : 0;
+    if (d == 2) TRY(damp_field<T>(L, a.dw, a.da, false, S, &a.damp));
     // two steps per launch (FP32 2D; not with checkpoints or the stability probe)
     int tbR = 0;
     TileBins tbb;
@@ -2916,8 +2285,6 @@ static ib_status forward_2nd(ib_table* t, const ib_shot* sh, double dt, int nt, 
             TRY(S.alloc(&tb_o2, L.total, true));
         }
     }
-    dim3 grids((unsigned)((L.nx + TX2 - 1) / TX2),
-               (unsigned)(((L.nz + TZ2 - 1) / TZ2 + STRIP_NSUB - 1) / STRIP_NSUB));
     // planes per 3D block (IB_ZCHUNK overrides it for tuning)
     int zchunk = 32;
     if (const char* e = getenv("IB_ZCHUNK")) zchunk = std::max(1, atoi(e));
@@ -3001,6 +2368,28 @@ static ib_status forward_2nd(ib_table* t, const ib_shot* sh, double dt, int nt, 
             ib_count_launch("setup");
         }
     }
+    // (the two-step kernel reads the coefficients unmarked)
+    if (d == 2) TRY(mark_rows<T>(a.rows, Kh, s));
+    const char* forced = getenv("IB_STRIP");
+    const RunPlan plan = d == 2 && !(forced && *forced) && !tb_enabled() ? run_plan<T>(L, H) : RunPlan{0, 0, 0, 0};
+    if (plan.blocks) {
+        // up to the next checkpoint (or renormalisation of the probe) in one launch
+        const int64_t part = ckpt ? seg : probe ? STAB_BLOCK : nt;
+        unsigned* bars;
+        TRY(S.alloc(&bars, (nt + part - 1) / part, true));
+        for (; n0 < nt; n0 = (int)std::min<int64_t>(n0 + part, nt)) {
+            if (ckpt) {
+                T* slot = (T*)ckpt + (n0 / seg) * 2 * L.total;
+                IB_CUDA(cudaMemcpyAsync(slot, cur, sizeof(T) * L.total, cudaMemcpyDeviceToDevice, s));
+                IB_CUDA(cudaMemcpyAsync(slot + L.total, prev, sizeof(T) * L.total, cudaMemcpyDeviceToDevice, s));
+            }
+            const int n1 = (int)std::min<int64_t>(n0 + part, nt);
+            TRY(launch_run<T>(a, plan, H, cur, prev, 0, n0, n1, bars + n0 / part, s));
+            if ((n1 - n0) & 1) std::swap(cur, prev);
+            if (probe && n1 % STAB_BLOCK == 0)
+                TRY(probe_rescale<T>(probe, n1 / STAB_BLOCK, L.total, cur, prev, (T*)nullptr, s));
+        }
+    }
     for (int n = n0; n < nt; ++n) {
         if (ckpt && n % seg == 0) {
             T* slot = (T*)ckpt + (int64_t)(n / seg) * 2 * L.total;
@@ -3012,17 +2401,8 @@ static ib_status forward_2nd(ib_table* t, const ib_shot* sh, double dt, int nt, 
         a.out = prev;
         a.step = n;
         a.rec_step = n - 1;
-        if (strip4) {
-            a4.p = a.p;
-            a4.pm = a.pm;
-            a4.out = a.out;
-            a4.step = a.step;
-            a4.rec_step = a.rec_step;
-            launch_leap2d_strip4(*reinterpret_cast<const StepArgs<float>*>(&a4), H, grid4, s);
-        } else if (strips) {
-            launch_leap2d_strip(*reinterpret_cast<const StepArgs<float>*>(&a), H, grids, s);
-        } else if (d == 2) {
-            launch_leap2d<T>(a, H, grid2, s);
+        if (d == 2) {
+            launch_leap2d(a, shape, H, s);
         } else if (use_tma) {
             dim3 blk(32, 8);
             const CUtensorMap& tmc = (cur == p0) ? tmap[0] : tmap[1];
@@ -3685,9 +3065,8 @@ extern "C" ib_status ib_forward(const ib_table* tc, const ib_shot* sh, int32_t p
 
 // receiver injection rows: node -> (receiver, weight), regrouped on the host
 template <typename T>
-static ib_status build_injection(const Layout& L, const PointSet<T>& rec, Scratch& S, RowView<T>& view,
-                                 std::vector<TileBins>& keep) {
-    memset(&view, 0, sizeof view);
+static ib_status build_injection(const PointSet<T>& rec, Scratch& S, AdjArgs<T>& a) {
+    a.n_inj = 0;
     if (rec.n == 0) return IB_OK;
     std::vector<int64_t> idx(8 * (size_t)rec.n);
     std::vector<T> w(8 * (size_t)rec.n);
@@ -3726,18 +3105,85 @@ static ib_status build_injection(const Layout& L, const PointSet<T>& rec, Scratc
     IB_CUDA(cudaMemcpyAsync(dptr, ptr.data(), 8 * ptr.size(), cudaMemcpyHostToDevice, S.s));
     IB_CUDA(cudaMemcpyAsync(dcol, col.data(), 8 * col.size(), cudaMemcpyHostToDevice, S.s));
     IB_CUDA(cudaMemcpyAsync(dw, ww.data(), sizeof(T) * ww.size(), cudaMemcpyHostToDevice, S.s));
-    TileBins b;
-    TRY(ib_make_bins_ext(L, (int64_t)rows.size(), drows, TX2, 1, TZ2, b, S.s));
-    keep.push_back(b);
-    view.row_pad = drows;
-    view.row_ptr = dptr;
-    view.col = dcol;
-    view.w = dw;
-    view.tile_ptr = b.tile_ptr;
-    view.perm = b.perm;
-    view.ntx = b.ntx;
+    a.n_inj = (int64_t)rows.size();
+    a.i_pad = drows;
+    a.i_ptr = dptr;
+    a.i_rec = dcol;
+    a.i_w = dw;
     IB_CUDA(cudaStreamSynchronize(S.s));
     return IB_OK;
+}
+
+// Adjoint step arguments of one shot: coefficients marked at the nodes of the transposed rows
+// and of the receiver injection, their lists and the map between them.
+template <typename T>
+static ib_status adj_setup(ib_table* t, const ib_shot* sh, double dt, int nt, const PointSet<T>& rec,
+                           const PointSet<T>& src, const T* res, Scratch& S, AdjArgs<T>& a) {
+    const Layout& L = t->L;
+    IbOp& op = t->ops[0];
+    TRY(ib_table_transpose(t, 0, S.s));
+    memset(&a, 0, sizeof a);
+    a.L = L;
+    T c1u[4];
+    stencil_weights<T>(t->opts.space_order, a.w2, c1u);
+    T* Kh;
+    int32_t* map;
+    TRY(S.alloc(&Kh, L.total, true));
+    TRY(S.alloc(&map, L.total, true));
+    TRY(S.alloc(&a.grad, L.total, true));
+    k_leap_coef<T><<<grid1(L.N, 256), 256, 0, S.s>>>(L, (const T*)sh->vel_dev, t->mask_pad[0], dt / t->grid.h, Kh);
+    IB_CHECK_LAUNCH("k_leap_coef");
+    ib_count_launch("setup");
+    a.nt_rows = op.t_nrows;
+    a.t_pad = op.t_row_pad;
+    a.t_ptr = op.t_ptr;
+    a.t_off = op.t_src_off;
+    a.t_w = (const T*)(sizeof(T) == 8 ? (const void*)op.t_w64 : (const void*)op.t_w32);
+    TRY(build_injection<T>(rec, S, a));
+    if (a.nt_rows) k_map_nodes<T><<<grid1(a.nt_rows, 256), 256, 0, S.s>>>(a.nt_rows, a.t_pad, false, map, Kh);
+    if (a.n_inj) k_map_nodes<T><<<grid1(a.n_inj, 256), 256, 0, S.s>>>(a.n_inj, a.i_pad, true, map, Kh);
+    IB_CHECK_LAUNCH("k_map_nodes");
+    ib_count_launch("setup");
+    a.Kh = Kh;
+    a.nodemap = map;
+    a.res = res;
+    a.nt = nt;
+    a.src = src;
+    a.wavelet = (const T*)sh->wavelet_dev;
+    set_damping<T>(sh, dt, a.dw, a.da);
+    return damp_field<T>(L, a.dw, a.da, true, S, &a.damp);
+}
+
+static const int kAdjRows = 32;   // rows a warp of the adjoint marches
+// Shape of an adjoint step over `points` grid points: 0 one point a thread, 1 a march of 128
+// columns.  Whole gradients, us per step: 2 shots (10^6 points) 86 and 144, 6 shots (3.5 x 10^6)
+// 223 and 265, 12 shots (6.5 x 10^6) 449 and 403, 24 shots (13 x 10^6) 854 and 686.
+static int adj_shape(int64_t points) {
+    const int f = strip_switch();
+    return f < 0 ? points >= 5000000 : f;
+}
+static int64_t adj_ntx(int si, const Layout& L) { return (L.nx + (si ? 128 : 32) - 1) / (si ? 128 : 32); }
+static int64_t adj_blocks(int si, const Layout& L) {
+    const int64_t rows = (int64_t)LEAP_WARPS * (si ? kAdjRows : 1);
+    return adj_ntx(si, L) * ((L.nz + rows - 1) / rows);
+}
+template <class F>
+static void with_adj_shape(int si, int H, F f) {
+    if (si == 0) with_h<1, 1>(H, f);
+    else with_h<4, 0>(H, f);
+}
+
+static void launch_adj2d(const AdjArgs<float>& a, int si, int H, unsigned grid, cudaStream_t s) {
+    with_adj_shape(si, H, [&](auto h, auto vx, auto rz) {
+        constexpr size_t sm = adj_smem<h.value, rz.value>();
+        if (sm)
+            cudaFuncSetAttribute(k_adj2d<float, h.value, vx.value, rz.value>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)sm);
+        k_adj2d<float, h.value, vx.value, rz.value><<<grid, LEAP_THREADS, sm, s>>>(a, kAdjRows);
+    });
+}
+static void launch_adj2d(const AdjArgs<double>& a, int, int H, unsigned grid, cudaStream_t s) {
+    with_h<1, 1>(H, [&](auto h, auto, auto) { k_adj2d<double, h.value, 1, 1><<<grid, LEAP_THREADS, 0, s>>>(a, 0); });
 }
 
 template <typename T>
@@ -3752,23 +3198,17 @@ static ib_status adjoint_2nd(ib_table* t, const ib_shot* sh, double dt, int nt, 
     const int M = t->opts.space_order;
     const int H = M / 2;
     Scratch S(s);
-    T *Kh, *mu1, *mu2, *grad;
+    T *Kh, *mu1, *mu2;
     TRY(S.alloc(&Kh, L.total, true));
     TRY(S.alloc(&mu1, L.total, true));
     TRY(S.alloc(&mu2, L.total, true));
-    TRY(S.alloc(&grad, L.total, true));
     k_leap_coef<T><<<grid1(L.N, 256), 256, 0, s>>>(L, (const T*)sh->vel_dev, t->mask_pad[0], dt / t->grid.h, Kh);
     IB_CHECK_LAUNCH("k_leap_coef");
     ib_count_launch("setup");
     Geom<T> g;
     TRY(setup_points<T>(t, sh, dt * dt / pow(t->grid.h, d), S, g));
-    const TileBins* fb = nullptr;
-    const TileBins* tb = nullptr;
-    TRY(ib_table_bins(t, 0, false, TX2, 1, TZ2, &fb, s));
-    TRY(ib_table_bins(t, 0, true, TX2, 1, TZ2, &tb, s));
-    std::vector<TileBins> keep;
-    RowView<T> inj;
-    TRY(build_injection<T>(L, g.rec, S, inj, keep));
+    AdjArgs<T> aa;
+    TRY(adj_setup<T>(t, sh, dt, nt, g.rec, g.src, res, S, aa));
     const int64_t seg = ckpt_seg(nt, n_ckpt);
     T* segbuf;
     TRY(S.alloc(&segbuf, (seg + 2) * L.total, true));
@@ -3781,32 +3221,23 @@ static ib_status adjoint_2nd(ib_table* t, const ib_shot* sh, double dt, int nt, 
         stencil_weights<T>(M, fa.w2, c1u);
     }
     fa.Kh = Kh;
-    fa.op = tview<T>(fb);
+    fa.rows = row_list<T>(t->ops[0]);
+    TRY(mark_rows<T>(fa.rows, Kh, s));
     fa.src = g.src;
     fa.wavelet = (const T*)sh->wavelet_dev;
     fa.rec.n = 0;
     fa.rec_step = -1;
     fa.nt = nt;
     set_damping<T>(sh, dt, fa.dw, fa.da);
-    AdjArgs<T> aa;
-    memset(&aa, 0, sizeof aa);
-    aa.L = L;
-    for (int k = 0; k < 5; ++k) aa.w2[k] = fa.w2[k];
-    aa.Kh = Kh;
-    aa.mask = t->mask_pad[0];
-    aa.two_dt_over_h = (T)(2.0 * dt / t->grid.h);
-    aa.opT = tview<T>(tb);
-    aa.opT.ntx = (L.nx + TX2 - 1) / TX2;
-    aa.inj = inj;
-    aa.inj.ntx = aa.opT.ntx;
-    aa.res = res;
-    aa.nt = nt;
-    aa.grad = grad;
-    aa.src = g.src;
-    aa.wavelet = (const T*)sh->wavelet_dev;
+    TRY(damp_field<T>(L, fa.dw, fa.da, false, S, &fa.damp));
     aa.gw = gw;
-    set_damping<T>(sh, dt, aa.dw, aa.da);
-    dim3 grid2((unsigned)((L.nx + TX2 - 1) / TX2), (unsigned)((L.nz + TZ2 - 1) / TZ2));
+    const int fshape = leap_shape_shot(L), ashape = sizeof(T) == 8 ? 0 : adj_shape(L.nx * L.nz);
+    aa.ntx = adj_ntx(ashape, L);
+    aa.nrb = row_blocks(aa.nt_rows + aa.n_inj, ashape ? 0 : 1);
+    const unsigned agrid = (unsigned)(aa.nrb + adj_blocks(ashape, L));
+    const RunPlan plan = run_plan<T>(L, H);
+    unsigned* bars;
+    TRY(S.alloc(&bars, n_ckpt, true));
     T* mu_a = mu1;   // mu^{m+1}
     T* mu_b = mu2;   // mu^{m+2}
     for (int k = n_ckpt - 1; k >= 0; --k) {
@@ -3817,12 +3248,13 @@ static ib_status adjoint_2nd(ib_table* t, const ib_shot* sh, double dt, int nt, 
         // segment slots j hold p^{c - 1 + j}
         IB_CUDA(cudaMemcpyAsync(segbuf, slot + L.total, sizeof(T) * L.total, cudaMemcpyDeviceToDevice, s));
         IB_CUDA(cudaMemcpyAsync(segbuf + L.total, slot, sizeof(T) * L.total, cudaMemcpyDeviceToDevice, s));
-        for (int64_t n = c; n < e; ++n) {
+        if (plan.blocks) TRY(launch_run<T>(fa, plan, H, segbuf, segbuf, L.total, (int)c, (int)e, bars + k, s));
+        else for (int64_t n = c; n < e; ++n) {
             fa.p = segbuf + (n - c + 1) * L.total;
             fa.pm = segbuf + (n - c) * L.total;
             fa.out = segbuf + (n - c + 2) * L.total;
             fa.step = (int)n;
-            launch_leap2d<T>(fa, H, grid2, s);
+            launch_leap2d(fa, fshape, H, s);
             IB_CHECK_LAUNCH("recompute step");
         }
         for (int64_t m = e; m >= c + 1; --m) {
@@ -3833,22 +3265,16 @@ static ib_status adjoint_2nd(ib_table* t, const ib_shot* sh, double dt, int nt, 
             aa.pm0 = segbuf + (m - c + 1) * L.total;
             aa.pm1 = segbuf + (m - c) * L.total;
             aa.pm2 = segbuf + (m - c - 1) * L.total;
-            PROF_LAUNCH(kname<T>("adj2d_f32", "adj2d_f64"), s, {
-                if (H == 1) k_adj2d<T, 1, TX2, TZ2><<<grid2, 256, 0, s>>>(aa);
-                else if (H == 2) k_adj2d<T, 2, TX2, TZ2><<<grid2, 256, 0, s>>>(aa);
-                else if (H == 3) k_adj2d<T, 3, TX2, TZ2><<<grid2, 256, 0, s>>>(aa);
-                else k_adj2d<T, 4, TX2, TZ2><<<grid2, 256, 0, s>>>(aa);
-            });
+            PROF_LAUNCH(kname<T>("adj2d_f32", "adj2d_f64"), s, { launch_adj2d(aa, ashape, H, agrid, s); });
             IB_CHECK_LAUNCH("adjoint step");
             std::swap(mu_a, mu_b);
         }
     }
-    k_unpad<T><<<grid1(L.N, 256), 256, 0, s>>>(L, grad, grad_out);
+    k_unpad_grad<T><<<grid1(L.N, 256), 256, 0, s>>>(L, aa.grad, aa.Kh, (T)(2.0 * dt / t->grid.h), grad_out);
     IB_CHECK_LAUNCH("k_unpad");
     ib_count_launch("setup");
     TRY(check_finite<T>(L.N, grad_out, (const T*)nullptr, (const T*)nullptr, s));
     IB_CUDA(cudaStreamSynchronize(s));
-    for (auto& b : keep) ib_free_bins(b);
     return IB_OK;
 }
 
@@ -3875,73 +3301,20 @@ extern "C" ib_status ib_adjoint(const ib_table* tc, const ib_shot* sh, int32_t p
 }
 
 // ---------------------------------------------------------------------------
-// batched shots: one launch per time step over the tiles of every shot,
-// captured with all nt steps into one CUDA graph; the tile shape is chosen by
-// timing the candidates on the batch itself (cached per shape class)
+// batched shots: one launch per time step over the blocks of every shot, captured with all
+// nt steps into one CUDA graph
 // ---------------------------------------------------------------------------
-struct TileShape {
-    int tx, tz, nsub;   // nsub > 1: z-marched strips of nsub tiles (k_leap2d_batch_m)
-};
-static const int kNumShapes = 10;
-static const TileShape kShapes[kNumShapes] = {{64, 8, 1},  {32, 16, 1}, {128, 4, 1}, {64, 4, 1},
-                                              {64, 8, 8},  {64, 8, 8},  {64, 8, 8},  {64, 8, 8},
-                                              {64, 16, 4}, {64, 16, 4}};
-
-template <int H, int TX, int TZ>
-static void launch_batch(const StepArgs<float>* args, const int64_t* tile0, const int32_t* shot_of, int nshot,
-                         int step, int64_t nblk,
-                         cudaStream_t s) {
-    k_leap2d_batch<float, H, TX, TZ><<<(unsigned)nblk, 256, 0, s>>>(args, tile0, shot_of, nshot, step);
-}
-
-template <int H, int NSUB, int D, int MINB>
-static void launch_batch_m(const StepArgs<float>* args, const int64_t* tile0, const int32_t* shot_of, int nshot,
-                           int step, int64_t nblk, cudaStream_t s) {
-    k_leap2d_batch_m<H, NSUB, D, MINB><<<(unsigned)nblk, 256, 0, s>>>(args, tile0, shot_of, nshot, step);
-}
-
-template <int H, int NSUB, int D, int MINB>
-static void launch_batch_m4(const StepArgs<float>* args, const int64_t* tile0, const int32_t* shot_of, int nshot,
-                            int step, int64_t nblk, cudaStream_t s) {
-    constexpr size_t sm = Strip4<H, NSUB, D>::FLOATS * sizeof(float);
-    static const bool attr = (cudaFuncSetAttribute(k_leap2d_batch_m4<H, NSUB, D, MINB>,
-                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm),
-                              true);
-    (void)attr;
-    k_leap2d_batch_m4<H, NSUB, D, MINB><<<(unsigned)nblk, 256, sm, s>>>(args, tile0, shot_of, nshot, step);
-}
-
-template <int H>
-static void launch_batch_shape(int si, const StepArgs<float>* args, const int64_t* tile0, const int32_t* shot_of,
-                               int nshot, int step,
-                               int64_t nblk, cudaStream_t s) {
-    switch (si) {
-        case 0: launch_batch<H, 64, 8>(args, tile0, shot_of, nshot, step, nblk, s); break;
-        case 1: launch_batch<H, 32, 16>(args, tile0, shot_of, nshot, step, nblk, s); break;
-        case 2: launch_batch<H, 128, 4>(args, tile0, shot_of, nshot, step, nblk, s); break;
-        case 3: launch_batch<H, 64, 4>(args, tile0, shot_of, nshot, step, nblk, s); break;
-        case 4: launch_batch_m<H, 8, 2, 4>(args, tile0, shot_of, nshot, step, nblk, s); break;
-        case 5: launch_batch_m<H, 8, 3, 4>(args, tile0, shot_of, nshot, step, nblk, s); break;
-        case 6: launch_batch_m<H, 8, 2, 5>(args, tile0, shot_of, nshot, step, nblk, s); break;
-        case 7: launch_batch_m<H, 8, 3, 5>(args, tile0, shot_of, nshot, step, nblk, s); break;
-        case 8: launch_batch_m4<H, 4, 2, 3>(args, tile0, shot_of, nshot, step, nblk, s); break;
-        default: launch_batch_m4<H, 4, 3, 3>(args, tile0, shot_of, nshot, step, nblk, s); break;
-    }
-}
-
-static void launch_batch_any(int H, int si, const StepArgs<float>* args, const int64_t* tile0, const int32_t* shot_of,
-                             int nshot, int step,
-                             int64_t nblk, cudaStream_t s) {
-    PROF_LAUNCH("leap2d_batch_f32", s, {
-        if (H == 1) launch_batch_shape<1>(si, args, tile0, shot_of, nshot, step, nblk, s);
-        else if (H == 2) launch_batch_shape<2>(si, args, tile0, shot_of, nshot, step, nblk, s);
-        else if (H == 3) launch_batch_shape<3>(si, args, tile0, shot_of, nshot, step, nblk, s);
-        else launch_batch_shape<4>(si, args, tile0, shot_of, nshot, step, nblk, s);
+static void launch_batch(int si, int H, const StepArgs<float>* args, const int64_t* tile0, const int32_t* shot_of,
+                         int step, int seg, int64_t nblk, cudaStream_t s) {
+    with_shape(si, H, [&](auto h, auto vx, auto rz) {
+        constexpr size_t sm = leap_smem<h.value, rz.value>();
+        if (sm > 48 * 1024)
+            cudaFuncSetAttribute(k_leap2d_batch<h.value, vx.value, rz.value>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)sm);
+        k_leap2d_batch<h.value, vx.value, rz.value>
+            <<<(unsigned)nblk, LEAP_THREADS, sm, s>>>(args, tile0, shot_of, step, seg, kShapes[si].zc);
     });
 }
-
-static std::mutex g_tune_mu;
-static std::map<std::pair<int, int64_t>, int> g_tuned;   // (H, total points / 2^18) -> shape index
 
 struct BatchSetup {
     std::vector<StepArgs<float>> args;
@@ -3956,21 +3329,18 @@ static ib_status batch_prepare(ib_table* const* ts, const ib_shot* shots, int ns
                                const std::vector<float*>& buf0, const std::vector<float*>& buf1,
                                const std::vector<float*>& Kh, const std::vector<Geom<float>>& geo, Scratch& S,
                                BatchSetup& B) {
-    const int tx = kShapes[si].tx, tz = kShapes[si].tz;
     B.args.assign(nshot, StepArgs<float>());
     B.tile0.assign(nshot + 1, 0);
     for (int i = 0; i < nshot; ++i) {
         ib_table* t = ts[i];
         const Layout& L = t->L;
-        const TileBins* bins = nullptr;
-        TRY(ib_table_bins(t, 0, false, tx, 1, tz, &bins, S.s));
         StepArgs<float>& a = B.args[i];
         memset(&a, 0, sizeof a);
         a.L = L;
         float c1u[4];
         stencil_weights<float>(t->opts.space_order, a.w2, c1u);
         a.Kh = Kh[i];
-        a.op = tview<float>(bins);
+        a.rows = row_list<float>(t->ops[0]);
         a.src = geo[i].src;
         a.wavelet = (const float*)shots[i].wavelet_dev;
         a.rec = geo[i].rec;
@@ -3979,13 +3349,10 @@ static ib_status batch_prepare(ib_table* const* ts, const ib_shot* shots, int ns
         a.buf0 = buf0[i];
         a.buf1 = buf1[i];
         set_damping<float>(&shots[i], dt, a.dw, a.da);
-        a.ntx = (L.nx + tx - 1) / tx;
-        const int nsub = kShapes[si].nsub;
-        int64_t ntiles = a.ntx * ((((L.nz + tz - 1) / tz) + nsub - 1) / nsub);
-        a.ntiles = ntiles;
-        // receivers are recorded by the first blocks of the shot: make sure there are enough
-        int64_t need = (shots[i].nrec + 255) / 256;
-        B.tile0[i + 1] = B.tile0[i] + std::max(ntiles, need);
+        TRY(damp_field<float>(L, a.dw, a.da, false, S, &a.damp));
+        a.ntx = shape_ntx(kShapes[si], L);
+        a.nrb = row_blocks(a.rows.n, kShapes[si].rz);
+        B.tile0[i + 1] = B.tile0[i] + a.nrb + shape_blocks(kShapes[si], L);
     }
     B.nblk = B.tile0[nshot];
     TRY(S.alloc(&B.d_args, nshot));
@@ -4047,60 +3414,18 @@ static ib_status forward_batch_impl(const ib_table* const* tables, const ib_shot
                                                            dt / ts[i]->grid.h, Kh[i]);
         IB_CHECK_LAUNCH("k_leap_coef");
         ib_count_launch("setup");
+        TRY(mark_rows<float>(row_list<float>(ts[i]->ops[0]), Kh[i], s));
         TRY(setup_points<float>(ts[i], &shots[i], dt * dt / pow(ts[i]->grid.h, 2), S, geo[i]));
         total += L.N;
     }
-    // ---- tile-shape autotuning (first batch of a shape class); IB_BATCH_SHAPE=<index
-    // into kShapes> fixes the shape instead
-    int best = 0;
+    // the shape by the batch's size; IB_BATCH_SHAPE=<index into kShapes> fixes it instead
+    int best = leap_shape(total);
     const char* forced = getenv("IB_BATCH_SHAPE");
     if (forced && *forced) {
         best = atoi(forced);
         if (best < 0 || best >= kNumShapes) {
-            ib_set_error("IB_BATCH_SHAPE must name a tile shape index in [0, 10)");
+            ib_set_error("IB_BATCH_SHAPE must name a shape index in [0, 10)");
             return IB_ERR_ARG;
-        }
-    } else {
-        std::pair<int, int64_t> key(H, total >> 18);
-        bool have = false;
-        {
-            std::lock_guard<std::mutex> lk(g_tune_mu);
-            auto it = g_tuned.find(key);
-            if (it != g_tuned.end()) {
-                best = it->second;
-                have = true;
-            }
-        }
-        if (!have) {
-            float best_ms = 1e30f;
-            cudaEvent_t e0, e1;
-            IB_CUDA(cudaEventCreate(&e0));
-            IB_CUDA(cudaEventCreate(&e1));
-            for (int si = 0; si < kNumShapes; ++si) {
-                BatchSetup B;
-                TRY(batch_prepare(ts.data(), shots, nshot, si, dt, nt, b0, b1, Kh, geo, S, B));
-                const int trial = std::min(nt, 12);
-                for (int n = 0; n < 2; ++n) launch_batch_any(H, si, B.d_args, B.d_tile0, B.d_shot_of, nshot, n, B.nblk, s);
-                IB_CUDA(cudaEventRecord(e0, s));
-                for (int n = 0; n < trial; ++n) launch_batch_any(H, si, B.d_args, B.d_tile0, B.d_shot_of, nshot, n, B.nblk, s);
-                IB_CUDA(cudaEventRecord(e1, s));
-                IB_CUDA(cudaEventSynchronize(e1));
-                float ms = 0.f;
-                IB_CUDA(cudaEventElapsedTime(&ms, e0, e1));
-                if (ms < best_ms) {
-                    best_ms = ms;
-                    best = si;
-                }
-            }
-            cudaEventDestroy(e0);
-            cudaEventDestroy(e1);
-            std::lock_guard<std::mutex> lk(g_tune_mu);
-            g_tuned[key] = best;
-            // trial steps wrote the wavefields: start the real run from zero
-            for (int i = 0; i < nshot; ++i) {
-                IB_CUDA(cudaMemsetAsync(b0[i], 0, sizeof(float) * ts[i]->L.total, s));
-                IB_CUDA(cudaMemsetAsync(b1[i], 0, sizeof(float) * ts[i]->L.total, s));
-            }
         }
     }
     BatchSetup B;
@@ -4136,13 +3461,7 @@ static ib_status forward_batch_impl(const ib_table* const* tables, const ib_shot
     IB_CUDA(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
     for (int n = 0; n < nt; ++n) {
         if (d_items && n % seg == 0) k_ckpt_batch<float><<<cgrid, 256, 0, cs>>>(d_items, n, (int)(n / seg));
-        StepArgs<float>* dargs = B.d_args;
-        switch (H) {
-            case 1: launch_batch_shape<1>(best, dargs, B.d_tile0, B.d_shot_of, nshot, n, B.nblk, cs); break;
-            case 2: launch_batch_shape<2>(best, dargs, B.d_tile0, B.d_shot_of, nshot, n, B.nblk, cs); break;
-            case 3: launch_batch_shape<3>(best, dargs, B.d_tile0, B.d_shot_of, nshot, n, B.nblk, cs); break;
-            default: launch_batch_shape<4>(best, dargs, B.d_tile0, B.d_shot_of, nshot, n, B.nblk, cs); break;
-        }
+        launch_batch(best, H, B.d_args, B.d_tile0, B.d_shot_of, n, -1, B.nblk, cs);
     }
     cudaError_t ce = cudaStreamEndCapture(cs, &graph);
     if (ce != cudaSuccess) return ib_cuda_fail(ce, "graph capture", __FILE__, __LINE__);
@@ -4192,19 +3511,22 @@ extern "C" ib_status ib_forward_batch_ckpt(const ib_table* const* tables, const 
 // batched adjoint: every shot's segments in lockstep, one graph for the whole
 // backward pass (segment restore, batched recompute steps, batched adjoint steps)
 // ---------------------------------------------------------------------------
-// block maps: tile0 / shot_of over 64 x 8 tiles (adjoint steps), stile0 / sshot_of
-// over z-marched strips (recompute steps)
-template <int H>
-static void launch_adj_batch_h(const StepArgs<float>* fargs, const AdjBatch<float>* aargs, const ShotCopy<float>* rst,
-                               const int64_t* tile0, const int32_t* shot_of, int64_t nblk, const int64_t* stile0,
-                               const int32_t* sshot_of, int64_t nsblk, dim3 cgrid, int nt, int64_t c, int64_t e,
-                               int k, cudaStream_t s) {
+// block maps: tile0 / shot_of of the adjoint steps, stile0 / sshot_of of the recompute steps
+static void launch_adj_batch(int H, int fshape, int ashape, const StepArgs<float>* fargs, const AdjBatch<float>* aargs,
+                             const ShotCopy<float>* rst, const int64_t* tile0, const int32_t* shot_of, int64_t nblk,
+                             const int64_t* stile0, const int32_t* sshot_of, int64_t nsblk, dim3 cgrid, int nt, int64_t c,
+                             int64_t e, int k, cudaStream_t s) {
     k_seg_restore_batch<float><<<cgrid, 256, 0, s>>>(rst, k);
-    for (int64_t n = c; n < e; ++n)
-        k_leap2d_batch_seg_m<H, STRIP_NSUB, STRIP_D><<<(unsigned)nsblk, 256, 0, s>>>(fargs, stile0, sshot_of, (int)n,
-                                                                                      (int)(n - c));
+    for (int64_t n = c; n < e; ++n) launch_batch(fshape, H, fargs, stile0, sshot_of, (int)n, (int)(n - c), nsblk, s);
     for (int64_t m = e; m >= c + 1; --m)
-        k_adj2d_batch<float, H, 64, 8><<<(unsigned)nblk, 256, 0, s>>>(aargs, tile0, shot_of, (int)m, (int)(m - c), nt);
+        with_adj_shape(ashape, H, [&](auto h, auto vx, auto rz) {
+            constexpr size_t sm = adj_smem<h.value, rz.value>();
+            if (sm)
+                cudaFuncSetAttribute(k_adj2d_batch<h.value, vx.value, rz.value>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)sm);
+            k_adj2d_batch<h.value, vx.value, rz.value><<<(unsigned)nblk, LEAP_THREADS, sm, s>>>(
+                aargs, tile0, shot_of, (int)m, (int)(m - c), nt, kAdjRows);
+        });
 }
 
 extern "C" ib_status ib_adjoint_batch(const ib_table* const* tables, const ib_shot* shots, int32_t nshot,
@@ -4246,9 +3568,10 @@ extern "C" ib_status ib_adjoint_batch(const ib_table* const* tables, const ib_sh
     std::vector<StepArgs<float>> fargs(nshot);
     std::vector<AdjBatch<float>> aargs(nshot);
     std::vector<ShotCopy<float>> rst(nshot);
-    std::vector<float*> grad(nshot);
     std::vector<int64_t> tile0(nshot + 1, 0), stile0(nshot + 1, 0);
-    std::vector<TileBins> keep;
+    int64_t points = 0;
+    for (int i = 0; i < nshot; ++i) points += ts[i]->L.N;
+    const int fshape = leap_shape(points), ashape = adj_shape(points);
     int64_t maxtot = 0;
     for (int i = 0; i < nshot; ++i) {
         ib_table* t = ts[i];
@@ -4257,7 +3580,6 @@ extern "C" ib_status ib_adjoint_batch(const ib_table* const* tables, const ib_sh
         TRY(S.alloc(&Kh, L.total, true));
         TRY(S.alloc(&mu1, L.total, true));
         TRY(S.alloc(&mu2, L.total, true));
-        TRY(S.alloc(&grad[i], L.total, true));
         TRY(S.alloc(&segbuf, (seg + 2) * L.total, true));
         k_leap_coef<float><<<grid1(L.N, 256), 256, 0, s>>>(L, (const float*)shots[i].vel_dev, t->mask_pad[0],
                                                            dt / t->grid.h, Kh);
@@ -4265,52 +3587,34 @@ extern "C" ib_status ib_adjoint_batch(const ib_table* const* tables, const ib_sh
         ib_count_launch("setup");
         Geom<float> g;
         TRY(setup_points<float>(t, &shots[i], dt * dt / pow(t->grid.h, 2), S, g));
-        const TileBins* fb = nullptr;
-        const TileBins* tb = nullptr;
-        TRY(ib_table_bins(t, 0, false, TX2, 1, TZ2, &fb, s));
-        TRY(ib_table_bins(t, 0, true, TX2, 1, TZ2, &tb, s));
-        RowView<float> inj;
-        TRY(build_injection<float>(L, g.rec, S, inj, keep));
         StepArgs<float>& fa = fargs[i];
         memset(&fa, 0, sizeof fa);
         fa.L = L;
         float c1u[4];
         stencil_weights<float>(t->opts.space_order, fa.w2, c1u);
         fa.Kh = Kh;
-        fa.op = tview<float>(fb);
+        fa.rows = row_list<float>(t->ops[0]);
+        TRY(mark_rows<float>(fa.rows, Kh, s));
         fa.src = g.src;
         fa.wavelet = (const float*)shots[i].wavelet_dev;
         fa.rec.n = 0;
         fa.rec_step = -1;
         fa.nt = nt;
         set_damping<float>(&shots[i], dt, fa.dw, fa.da);
+        TRY(damp_field<float>(L, fa.dw, fa.da, false, S, &fa.damp));
         fa.buf0 = segbuf;
-        fa.ntx = (L.nx + TX2 - 1) / TX2;
-        fa.ntiles = fa.ntx * ((L.nz + TZ2 - 1) / TZ2);
+        fa.ntx = shape_ntx(kShapes[fshape], L);
+        fa.nrb = row_blocks(fa.rows.n, kShapes[fshape].rz);
         AdjArgs<float>& aa = aargs[i].a;
-        memset(&aa, 0, sizeof aa);
-        aa.L = L;
-        for (int k = 0; k < 5; ++k) aa.w2[k] = fa.w2[k];
-        aa.Kh = Kh;
-        aa.mask = t->mask_pad[0];
-        aa.two_dt_over_h = (float)(2.0 * dt / t->grid.h);
-        aa.opT = tview<float>(tb);
-        aa.opT.ntx = fa.ntx;
-        aa.inj = inj;
-        aa.inj.ntx = fa.ntx;
-        aa.res = (const float*)residuals[i];
-        aa.nt = nt;
-        aa.grad = grad[i];
-        aa.src = g.src;
-        aa.wavelet = (const float*)shots[i].wavelet_dev;
-        aa.gw = nullptr;
-        set_damping<float>(&shots[i], dt, aa.dw, aa.da);
+        TRY(adj_setup<float>(t, &shots[i], dt, nt, g.rec, g.src, (const float*)residuals[i], S, aa));
+        aa.ntx = adj_ntx(ashape, L);
+        aa.nrb = row_blocks(aa.nt_rows + aa.n_inj, ashape ? 0 : 1);
         aargs[i].mu1 = mu1;
         aargs[i].mu2 = mu2;
         aargs[i].seg = segbuf;
         rst[i] = {(const float*)ckpts[i], nullptr, segbuf, L.total};
-        tile0[i + 1] = tile0[i] + fa.ntiles;
-        stile0[i + 1] = stile0[i] + fa.ntx * (((L.nz + TZ2 - 1) / TZ2 + STRIP_NSUB - 1) / STRIP_NSUB);
+        tile0[i + 1] = tile0[i] + aa.nrb + adj_blocks(ashape, L);
+        stile0[i + 1] = stile0[i] + fa.nrb + shape_blocks(kShapes[fshape], L);
         maxtot = std::max(maxtot, L.total);
     }
     const int64_t nblk = tile0[nshot], nsblk = stile0[nshot];
@@ -4355,12 +3659,7 @@ extern "C" ib_status ib_adjoint_batch(const ib_table* const* tables, const ib_sh
         const int64_t c = (int64_t)k * seg;
         if (c >= nt) continue;
         const int64_t e = std::min<int64_t>(c + seg, nt);
-        switch (H) {
-            case 1: launch_adj_batch_h<1>(d_f, d_a, d_r, d_t0, d_so, nblk, d_st0, d_sso, nsblk, cgrid, nt, c, e, k, cs); break;
-            case 2: launch_adj_batch_h<2>(d_f, d_a, d_r, d_t0, d_so, nblk, d_st0, d_sso, nsblk, cgrid, nt, c, e, k, cs); break;
-            case 3: launch_adj_batch_h<3>(d_f, d_a, d_r, d_t0, d_so, nblk, d_st0, d_sso, nsblk, cgrid, nt, c, e, k, cs); break;
-            default: launch_adj_batch_h<4>(d_f, d_a, d_r, d_t0, d_so, nblk, d_st0, d_sso, nsblk, cgrid, nt, c, e, k, cs); break;
-        }
+        launch_adj_batch(H, fshape, ashape, d_f, d_a, d_r, d_t0, d_so, nblk, d_st0, d_sso, nsblk, cgrid, nt, c, e, k, cs);
         nadj += e - c;
     }
     cudaError_t ce = cudaStreamEndCapture(cs, &graph);
@@ -4381,7 +3680,8 @@ extern "C" ib_status ib_adjoint_batch(const ib_table* const* tables, const ib_sh
     }
     for (int i = 0; i < nshot; ++i) {
         const Layout& L = ts[i]->L;
-        k_unpad<float><<<grid1(L.N, 256), 256, 0, cs>>>(L, grad[i], (float*)grads[i]);
+        k_unpad_grad<float><<<grid1(L.N, 256), 256, 0, cs>>>(L, aargs[i].a.grad, aargs[i].a.Kh,
+                                                             (float)(2.0 * dt / ts[i]->grid.h), (float*)grads[i]);
         ib_count_launch("setup");
         TRY(check_finite<float>(L.N, (const float*)grads[i], (const float*)nullptr, (const float*)nullptr, cs));
     }
@@ -4393,7 +3693,6 @@ extern "C" ib_status ib_adjoint_batch(const ib_table* const* tables, const ib_sh
     cudaGraphDestroy(graph);
     cudaEventDestroy(ready);
     cudaStreamDestroy(cs);
-    for (auto& b : keep) ib_free_bins(b);
     return IB_OK;
 }
 
@@ -4428,6 +3727,10 @@ extern "C" ib_status ib_sync_status(void* stream) {
         const int zero = 0;
         IB_CUDA(cudaMemcpyToSymbolAsync(g_dev_status, &zero, sizeof(int), 0, cudaMemcpyHostToDevice, s));
         IB_CUDA(cudaStreamSynchronize(s));
+        if (word & STATUS_TIMEOUT) {
+            ib_set_error("a bounded wait between the steps of a 2D run timed out");
+            return IB_ERR_TIMEOUT;
+        }
         ib_set_error("non-finite values (NaN/Inf) in the final wavefield or gradient of a run on this device: "
                      "the scheme is unstable for that model and time step");
         return IB_ERR_UNSTABLE;
@@ -4500,23 +3803,7 @@ extern "C" ib_status ib_stability(const ib_table* tc, const ib_shot* shot, int32
 // ---------------------------------------------------------------------------
 #define IB_NOALLOC_SCRATCH_BYTES (64ll << 20)
 
-static __device__ __align__(256) unsigned char g_noalloc_scratch[IB_NOALLOC_SCRATCH_BYTES];
-
-// one warp per IB row: out[q] += Kh[q] * sum_j w_j p[q + col_j]
-__global__ void k_ib_rows_add(int64_t nrows, const int64_t* __restrict__ row_pad, const int64_t* __restrict__ row_ptr,
-                              const int64_t* __restrict__ col_pad, const float* __restrict__ w,
-                              const float* __restrict__ p, const float* __restrict__ Kh, float* out) {
-    const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    for (int64_t r = warp; r < nrows; r += ((int64_t)gridDim.x * blockDim.x) >> 5) {
-        const int64_t q = row_pad[r];
-        float s = 0.f;
-        for (int64_t j = row_ptr[r] + lane; j < row_ptr[r + 1]; j += 32) s += w[j] * p[q + col_pad[j]];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (lane == 0) out[q] += Kh[q] * s;
-    }
-}
+static __device__ __align__(256) unsigned char g_noalloc_scratch[IB_NOALLOC_SCRATCH_BYTES + 256];   // + the run's barrier word
 
 static std::mutex g_noalloc_mu;
 static void* g_noalloc_ptr[64] = {nullptr};
@@ -4591,6 +3878,8 @@ extern "C" ib_status ib_forward_noalloc(const ib_table* tc, const ib_shot* sh, d
     float* sw = (float*)carve(4 * 8 * (int64_t)std::max(sh->nsrc, 1));
     int64_t* ri = (int64_t*)carve(8 * 8 * (int64_t)std::max(sh->nrec, 1));
     float* rw = (float*)carve(4 * 8 * (int64_t)std::max(sh->nrec, 1));
+    unsigned* bar = (unsigned*)(base + IB_NOALLOC_SCRATCH_BYTES);
+    IB_CUDA(cudaMemsetAsync(bar, 0, 256, s));
     // every call starts from zero wavefields and a zero padding ring
     IB_CUDA(cudaMemsetAsync(p0, 0, sizeof(float) * L.total, s));
     IB_CUDA(cudaMemsetAsync(p1, 0, sizeof(float) * L.total, s));
@@ -4620,23 +3909,23 @@ extern "C" ib_status ib_forward_noalloc(const ib_table* tc, const ib_shot* sh, d
     a.rec = {sh->nrec, ri, rw};
     a.traces = (float*)sh->traces_dev;
     a.nt = nt;
-    const IbOp& op = t->ops[0];
-    dim3 grid2((unsigned)((L.nx + TX2 - 1) / TX2), (unsigned)((L.nz + TZ2 - 1) / TZ2));
+    a.rows = row_list<float>(t->ops[0]);
+    TRY(mark_rows<float>(a.rows, Kh, s));
+    const int shape = leap_shape(L.nx * L.nz);
     float* cur = p0;
     float* prev = p1;
-    for (int n = 0; n < nt; ++n) {
+    const RunPlan plan = run_plan<float>(L, H);
+    if (plan.blocks) {
+        TRY(launch_run<float>(a, plan, H, cur, prev, 0, 0, nt, bar, s));
+        if (nt & 1) std::swap(cur, prev);
+    }
+    for (int n = plan.blocks ? nt : 0; n < nt; ++n) {
         a.p = cur;
         a.pm = prev;
         a.out = prev;
         a.step = n;
         a.rec_step = n - 1;
-        if (H == 1) k_leap2d<float, 1, TX2, TZ2><<<grid2, 256, 0, s>>>(a);
-        else if (H == 2) k_leap2d<float, 2, TX2, TZ2><<<grid2, 256, 0, s>>>(a);
-        else if (H == 3) k_leap2d<float, 3, TX2, TZ2><<<grid2, 256, 0, s>>>(a);
-        else k_leap2d<float, 4, TX2, TZ2><<<grid2, 256, 0, s>>>(a);
-        if (op.nrows)
-            k_ib_rows_add<<<grid1(op.nrows * 32, 256), 256, 0, s>>>(op.nrows, op.row_pad, op.row_ptr, op.col_pad,
-                                                                     op.w32, cur, Kh, prev);
+        launch_leap2d(a, shape, H, s);
         IB_CHECK_LAUNCH("ib_forward_noalloc step");
         std::swap(cur, prev);
     }
