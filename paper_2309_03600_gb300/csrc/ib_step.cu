@@ -2221,6 +2221,27 @@ static void launch_tb2(const TbArgs& a, int H, int R, dim3 grid, cudaStream_t s)
     });
 }
 
+// Planes per block of the FP32 3D step on 64 x 8 column tiles.  A block costs its planes and
+// about 10 more (the 2H planes read before the first, the ring's start, the tail); three run on
+// an SM, so the launch takes ceil(blocks / (3 x 152)) such times.  The even count that minimises
+// it: 64 at 512^2 x 384 (32 planes 328 us, 64 planes 324), 10 at 131 x 97 x 110, where 32
+// planes left two thirds of the block slots empty and the others marching (51 us; 4 planes 25,
+// 10 planes 24, 16 planes 31).
+static int z_planes(const Layout& L) {
+    const int64_t tiles = ((L.nx + 63) / 64) * ((L.ny + 7) / 8);
+    int best = 32;
+    int64_t cost = INT64_MAX;
+    for (int zc = 4; zc <= 96; zc += 2) {
+        const int64_t chunks = (L.nz + zc - 1) / zc;
+        const int64_t c = (tiles * chunks + 455) / 456 * (zc + 10);
+        if (c < cost) {
+            cost = c;
+            best = zc;
+        }
+    }
+    return best;
+}
+
 template <typename T>
 static ib_status forward_2nd(ib_table* t, const ib_shot* sh, double dt, int nt, void* ckpt, int n_ckpt,
                              cudaStream_t s, const Probe* probe = nullptr) {
@@ -2286,7 +2307,7 @@ static ib_status forward_2nd(ib_table* t, const ib_shot* sh, double dt, int nt, 
         }
     }
     // planes per 3D block (IB_ZCHUNK overrides it for tuning)
-    int zchunk = 32;
+    int zchunk = d == 3 && sizeof(T) == 4 && tma_enabled() ? z_planes(L) : 32;
     if (const char* e = getenv("IB_ZCHUNK")) zchunk = std::max(1, atoi(e));
     dim3 grid3((unsigned)((L.nx + 31) / 32), (unsigned)((L.ny + 7) / 8), (unsigned)((L.nz + zchunk - 1) / zchunk));
     const int64_t nty3 = (L.ny + 7) / 8;
