@@ -1766,8 +1766,8 @@ static ib_status pack_pool(ib_table* t, const FitKind& fk, const int64_t* rows, 
         op.nnz = nnz;
         TRY(dalloc(&op.col_code, nnz));
         TRY(dalloc(&op.col_pad, nnz));
-        TRY(dalloc(&op.w64, nnz));
-        TRY(dalloc(&op.w32, nnz));
+        TRY(dalloc(&op.w64, nnz + 1));   // read in pairs: the last pair may end past nnz
+        TRY(dalloc(&op.w32, nnz + 1));
         TRY(dalloc(&op.row_lin, nrows));
         TRY(dalloc(&op.row_pad, nrows));
         TRY(dalloc(&op.row_info, 4 * nrows));
@@ -2978,7 +2978,7 @@ __global__ void k_code16(int64_t nnz, const int32_t* col_code, uint16_t* out) {
 ib_status ib_table_code16(ib_table* t, int op, const uint16_t** out, cudaStream_t s) {
     IbOp& o = t->ops[op];
     if (!o.code16 && o.nnz > 0) {
-        TRY(dalloc(&o.code16, o.nnz));
+        TRY(dalloc(&o.code16, o.nnz + 1));   // read in pairs
         k_code16<<<grid_for(o.nnz, 256), 256, 0, s>>>(o.nnz, o.col_code, o.code16);
         IB_CHECK_LAUNCH("k_code16");
         ib_count_launch("setup");

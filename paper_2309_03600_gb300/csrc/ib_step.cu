@@ -2860,13 +2860,12 @@ static ib_status forward_stag(ib_table* t, const ib_shot* sh, double dt, int nt,
 
 // ---------------------------------------------------------------------------
 // 3D staggered pressure-velocity (1st-order section: the paper's signs and the
-// backward-staggered base stencil; 3D first-order example), one thread per node:
+// backward-staggered base stencil; 3D first-order example):
 //   v_a[j] (at j + e_a/2) += b_a[j] (sum_k c_k (p[j + k e_a] - p[j - (k-1) e_a]) + G_a corrections)
 //   p[j] += kp[j] (sum_a sum_k c_k (v_a[j + (k-1) e_a] - v_a[j - k e_a]) + D corrections) + src
 // with b_a = dt / (rho h) (mean of 1/rho at the two nodes) and kp = dt rho c^2 / h.
-// The corrections of the modified rows follow each update in a pass over the
-// rows of each operator (k_ib_rows, 8 lanes per row): the updated field is not
-// read by its own update, so the pass sees the same values the fused sum would.
+// The updated field is not read by its own update, so the modified rows are updated beside
+// the others in the same launch.
 // ---------------------------------------------------------------------------
 template <typename T>
 __global__ void k_stag_coef3(Layout L, const T* vel, const T* rho, const uint8_t* mp, const uint8_t* mv0,
@@ -2887,125 +2886,275 @@ __global__ void k_stag_coef3(Layout L, const T* vel, const T* rho, const uint8_t
     }
 }
 
+// Lane gl of 8's share of sum_j w_j f[q + off_j] over the entries [j0, j1) of a 3D row: pairs
+// of adjacent entries (their codes as one 4-byte and their weights as one vector load; a pair
+// that straddles the row's ends has the foreign weight dropped), U pairs in flight.  The
+// 16-bit footprint code is decoded mostly in 32-bit arithmetic against a base moved by the code's
+// offset of 16 nodes per axis, so an entry costs about 10 instructions where 64-bit decoding took over 20.
+template <typename T>
+struct PairOf;
+template <> struct PairOf<float> { typedef float2 type; };
+template <> struct PairOf<double> { typedef double2 type; };
+template <typename T, int U>
+__device__ __forceinline__ T row_gather3(const uint16_t* __restrict__ code, const T* __restrict__ w, int64_t j0, int64_t j1,
+                                         const T* __restrict__ f, int64_t q, int px, int plane, int gl) {
+    typedef typename PairOf<T>::type V;
+    const T* base = f + (q - 16 * ((int64_t)plane + px + 1));
+    const int64_t centre = 16 * ((int64_t)plane + px + 1);
+    T v = 0;
+    for (int64_t j = (j0 & ~(int64_t)1) + 2 * gl; j < j1; j += 16 * U) {
+        T w0[U], w1[U], p0[U], p1[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int64_t e = j + 16 * u;
+            int64_t o0 = centre, o1 = centre;
+            w0[u] = w1[u] = (T)0;
+            if (e < j1) {
+                const uint32_t c = *reinterpret_cast<const uint32_t*>(code + e);
+                const V ww = *reinterpret_cast<const V*>(w + e);
+                if (e >= j0) {
+                    w0[u] = ww.x;
+                    o0 = (int64_t)(int)((c >> 10) & 63) * plane + ((int)(c & 31) + (int)((c >> 5) & 31) * px);
+                }
+                if (e + 1 < j1) {
+                    w1[u] = ww.y;
+                    o1 = (int64_t)(int)(c >> 26) * plane + ((int)((c >> 16) & 31) + (int)((c >> 21) & 31) * px);
+                }
+            }
+            p0[u] = base[o0];
+            p1[u] = base[o1];
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            v += w0[u] * p0[u];
+            v += w1[u] * p1[u];
+        }
+    }
+    return v;
+}
+template <typename T>
+__device__ __forceinline__ T sum8(T v) {
+    v += __shfl_xor_sync(0xffffffffu, v, 4, 8);
+    v += __shfl_xor_sync(0xffffffffu, v, 2, 8);
+    v += __shfl_xor_sync(0xffffffffu, v, 1, 8);
+    return v;
+}
+
+// rows of one or several operators on the same row nodes
+template <typename T>
+struct Rows3D {
+    int64_t n;
+    const int64_t* pad;
+    const int64_t* ptr[3];
+    const uint16_t* code[3];
+    const T* w[3];
+};
+
 template <typename T, int H>
 struct Stag3Args {
     Layout L;
     T c[4];              // c[k - 1]: weight of the pair at offsets +(k - 1/2), -(k - 1/2)
     T* p;
     T* v[3];
-    const T* kp;
+    const T* kp;         // sign bit of kp and b: a node of the modified rows
     const T* b[3];
+    Rows3D<T> g[3];      // gradient rows of v_a (columns p: operator 0 of each)
+    Rows3D<T> d;         // divergence rows (columns v_0, v_1, v_2)
+    int nrb[4];          // row blocks: v_0, v_1, v_2; p
+    int nbx, nby;        // column blocks along x and y
+    PointSet<T> src;     // weights include dt / h^3
+    const T* wavelet;
+    int step;
+    PointSet<T> rec;     // receivers, sampled from p before the v update
+    T* traces;
+    int nt;
+    int rec_step;
 };
+
+// Both kernels: column blocks of 256 threads own VX x-adjacent nodes per thread (16-byte
+// vectors) in a 32 VX x 8 x 1 box; row blocks update the nodes of the modified rows whole,
+// which the column blocks leave out (sign bit of their coefficient).  Two
+// launches per step: with one thread per node, a pass per operator over its rows, and
+// separate source and receiver launches a step had ten, and 64-bit divisions for every node.
+// 160 x 144 x 122, order 4, FP32: 172 -> 111 us a step (v 33, p 79; a whole warp per divergence
+// row: p 104).  The p rows, 3 gathers of about 60 entries each, bound it by instruction issue.
+static const int S3_ROWS = 32;   // rows per row block, 8 lanes each
+
+template <typename T>
+__device__ __forceinline__ bool marked3(T k) {
+    return sizeof(T) == 8 ? __double2hiint((double)k) < 0 : __float_as_int((float)k) < 0;
+}
+template <typename T, int VX>
+__device__ __forceinline__ void load3(T (&d)[VX], const T* p) {
+    typedef typename std::conditional<sizeof(T) == 4, float4, double2>::type V;
+    static_assert(sizeof(V) == sizeof(T) * VX, "16-byte vectors");
+    *reinterpret_cast<V*>(&d[0]) = *reinterpret_cast<const V*>(p);
+}
+template <typename T, int VX>
+__device__ __forceinline__ void store3(T* p, const T (&d)[VX], const T (&k)[VX], int64_t x, int64_t nx) {
+    typedef typename std::conditional<sizeof(T) == 4, float4, double2>::type V;
+    bool all = x + VX <= nx;
+#pragma unroll
+    for (int j = 0; j < VX; ++j) all = all && !marked3(k[j]);
+    if (all) {
+        *reinterpret_cast<V*>(p) = *reinterpret_cast<const V*>(&d[0]);
+    } else {
+#pragma unroll
+        for (int j = 0; j < VX; ++j)
+            if (x + j < nx && !marked3(k[j])) p[j] = d[j];
+    }
+}
 
 // v_a += b_a (forward-staggered d/dx_a p) at every interior v_a node
 template <typename T, int H>
-__global__ void __launch_bounds__(256) k_stag_v3d(Stag3Args<T, H> a) {
+__global__ void __launch_bounds__(256) k_stag_v3d(const __grid_constant__ Stag3Args<T, H> a) {
+    constexpr int VX = 16 / (int)sizeof(T), HV = (H + VX - 1) / VX, HX = HV * VX;
     const Layout& L = a.L;
+    int64_t blk = blockIdx.x;
+    record_receivers(a.rec, (const T*)a.p, a.traces, a.nt, a.rec_step, blk * 256 + threadIdx.x, (int64_t)gridDim.x * 256);
     const int64_t st[3] = {1, L.px, L.plane};
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < L.N; i += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t x = i % L.nx, r = i / L.nx, y = r % L.ny, z = r / L.ny;
-        const int64_t q = L.idx(x, y, z);
 #pragma unroll
-        for (int ax = 0; ax < 3; ++ax) {
-            const T bq = a.b[ax][q];
-            if (bq == (T)0) continue;
-            T s = 0;
-#pragma unroll
-            for (int k = 1; k <= H; ++k) s += a.c[k - 1] * (a.p[q + k * st[ax]] - a.p[q - (k - 1) * st[ax]]);
-            a.v[ax][q] += bq * s;
-        }
-    }
-}
-
-// p += kp (backward-staggered divergence of v) at every interior p node
-template <typename T, int H>
-__global__ void __launch_bounds__(256) k_stag_p3d(Stag3Args<T, H> a) {
-    const Layout& L = a.L;
-    const int64_t st[3] = {1, L.px, L.plane};
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < L.N; i += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t x = i % L.nx, r = i / L.nx, y = r % L.ny, z = r / L.ny;
-        const int64_t q = L.idx(x, y, z);
-        const T kq = a.kp[q];
-        if (kq == (T)0) continue;
-        T s = 0;
-#pragma unroll
-        for (int ax = 0; ax < 3; ++ax)
+    for (int ax = 0; ax < 3; ++ax) {
+        if (blk < a.nrb[ax]) {
+            const Rows3D<T>& R = a.g[ax];
+            const int gl = threadIdx.x & 7;
+            const int64_t r = blk * S3_ROWS + (threadIdx.x >> 3);
+            const bool act = r < R.n;
+            const int64_t q = act ? R.pad[r] : L.base;
+            const T bq = gl == 0 ? a.b[ax][q] : (T)0, vq = gl == 0 ? a.v[ax][q] : (T)0;
+            T s = row_gather3<T, 4>(R.code[0], R.w[0], act ? R.ptr[0][r] : 0, act ? R.ptr[0][r + 1] : 0, a.p, q, (int)L.px,
+                                    (int)L.plane, gl);
 #pragma unroll
             for (int k = 1; k <= H; ++k)
-                s += a.c[k - 1] * (a.v[ax][q + (k - 1) * st[ax]] - a.v[ax][q - k * st[ax]]);
-        a.p[q] += kq * s;
+                if (gl == k) s += a.c[k - 1] * (a.p[q + k * st[ax]] - a.p[q - (k - 1) * st[ax]]);
+            s = sum8(s);
+            if (act && gl == 0) a.v[ax][q] = vq + (bq < (T)0 ? -bq : bq) * s;
+            return;
+        }
+        blk -= a.nrb[ax];
     }
-}
-
-// out[q] += coef[q] sum_j w_j f[q + col_j] over the rows of one operator, 8 lanes per
-// row (rows are distinct nodes within an operator; the sum is added by a reduction
-// that returns nothing)
-template <typename T>
-__global__ void __launch_bounds__(256) k_ib_rows(int64_t nrows, const int64_t* __restrict__ row_pad,
-                                                 const int64_t* __restrict__ row_ptr,
-                                                 const int64_t* __restrict__ col_pad, const T* __restrict__ w,
-                                                 const T* __restrict__ f, const T* __restrict__ coef, T* out) {
-    const int lane = threadIdx.x & 31, gl = lane & 7;
-    const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nwarp = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t rb = warp * 4; rb < nrows; rb += nwarp * 4) {
-        const int64_t r = rb + (lane >> 3);
-        const bool act = r < nrows;
-        const int64_t q = act ? row_pad[r] : 0;
-        const int64_t j1 = act ? row_ptr[r + 1] : 0;
-        T v = 0;
-        for (int64_t j = (act ? row_ptr[r] : 0) + gl; j < j1; j += 8) v += w[j] * f[q + col_pad[j]];
-        v += __shfl_xor_sync(0xffffffffu, v, 4, 8);
-        v += __shfl_xor_sync(0xffffffffu, v, 2, 8);
-        v += __shfl_xor_sync(0xffffffffu, v, 1, 8);
-        if (act && gl == 0) atomicAdd(&out[q], coef[q] * v);
+    const int lane = threadIdx.x & 31, wy = threadIdx.x >> 5;
+    const int bx = (int)(blk % a.nbx), by = (int)(blk / a.nbx % a.nby);
+    const int64_t z = blk / a.nbx / a.nby, x = ((int64_t)bx * 32 + lane) * VX, y = by * 8 + wy;
+    if (x >= L.nx || y >= L.ny) return;
+    const int64_t q = L.idx(x, y, z);
+    T w[VX + 2 * HX], y2[2 * H][VX], z2[2 * H][VX], vv[3][VX], bb[3][VX];
+#pragma unroll
+    for (int m = 0; m < 2 * HV + 1; ++m) load3<T, VX>(*reinterpret_cast<T(*)[VX]>(&w[m * VX]), a.p + q + (m - HV) * VX);
+#pragma unroll
+    for (int k = 0; k < 2 * H; ++k) {   // offsets 1 - H .. H
+        if (k == H - 1) continue;
+        load3<T, VX>(y2[k], a.p + q + (k + 1 - H) * L.px);
+        load3<T, VX>(z2[k], a.p + q + (k + 1 - H) * L.plane);
     }
+#pragma unroll
+    for (int ax = 0; ax < 3; ++ax) {
+        load3<T, VX>(vv[ax], a.v[ax] + q);
+        load3<T, VX>(bb[ax], a.b[ax] + q);
+    }
+#pragma unroll
+    for (int j = 0; j < VX; ++j) {
+        const T c = w[HX + j];
+        T sx = 0, sy = 0, sz = 0;
+#pragma unroll
+        for (int k = 1; k <= H; ++k) {
+            sx += a.c[k - 1] * (w[HX + j + k] - w[HX + j - k + 1]);
+            sy += a.c[k - 1] * (y2[H - 1 + k][j] - (k == 1 ? c : y2[H - k][j]));
+            sz += a.c[k - 1] * (z2[H - 1 + k][j] - (k == 1 ? c : z2[H - k][j]));
+        }
+        vv[0][j] += bb[0][j] * sx;
+        vv[1][j] += bb[1][j] * sy;
+        vv[2][j] += bb[2][j] * sz;
+    }
+#pragma unroll
+    for (int ax = 0; ax < 3; ++ax) store3<T, VX>(a.v[ax] + q, vv[ax], bb[ax], x, L.nx);
 }
 
-// sources: p[corner] += w * wavelet[n] (weights include dt / h^d)
-template <typename T>
-__global__ void k_add_sources(PointSet<T> src, const T* wavelet, int n, T* p) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < 8 * src.n && src.w[i] != (T)0) atomicAdd(&p[src.idx[i]], src.w[i] * wavelet[n]);
-}
-
+// p += kp (backward-staggered divergence of v) + sources at every interior p node
 template <typename T, int H>
-static ib_status stag3_steps(ib_table* t, const ib_shot* sh, int nt, Stag3Args<T, H>& a, const Geom<T>& g,
-                             cudaStream_t s) {
+__global__ void __launch_bounds__(256) k_stag_p3d(const __grid_constant__ Stag3Args<T, H> a) {
+    constexpr int VX = 16 / (int)sizeof(T), HV = (H + VX - 1) / VX, HX = HV * VX;
     const Layout& L = a.L;
-    const int gb = grid1(L.N, 256);
-    for (int n = 0; n < nt; ++n) {
-        PROF_LAUNCH(kname<T>("stag_v3d_f32", "stag_v3d_f64"), s, { k_stag_v3d<T, H><<<gb, 256, 0, s>>>(a); });
+    int64_t blk = blockIdx.x;
+    const int64_t st[3] = {1, L.px, L.plane};
+    if (blk < a.nrb[3]) {
+        const int gl = threadIdx.x & 7;
+        const int64_t r = blk * S3_ROWS + (threadIdx.x >> 3);
+        const bool act = r < a.d.n;
+        const int64_t q = act ? a.d.pad[r] : L.base;
+        const T kq = gl == 0 ? a.kp[q] : (T)0, pq = gl == 0 ? a.p[q] : (T)0;
+        T s = 0, sv = 0;
+#pragma unroll
         for (int ax = 0; ax < 3; ++ax) {
-            const IbOp& op = t->ops[ax];
-            if (!op.nrows) continue;
-            const T* w = sizeof(T) == 8 ? (const T*)op.w64 : (const T*)op.w32;
-            PROF_LAUNCH(kname<T>("ib_rows3_f32", "ib_rows3_f64"), s, {
-                k_ib_rows<T><<<grid1(op.nrows * 8, 256), 256, 0, s>>>(op.nrows, op.row_pad, op.row_ptr, op.col_pad,
-                                                                       w, a.p, a.b[ax], a.v[ax]);
-            });
+            s += row_gather3<T, 4>(a.d.code[ax], a.d.w[ax], act ? a.d.ptr[ax][r] : 0, act ? a.d.ptr[ax][r + 1] : 0, a.v[ax],
+                                   q, (int)L.px, (int)L.plane, gl);
+#pragma unroll
+            for (int k = 1; k <= H; ++k)
+                if (gl == ((ax * H + k) & 7)) s += a.c[k - 1] * (a.v[ax][q + (k - 1) * st[ax]] - a.v[ax][q - k * st[ax]]);
         }
-        PROF_LAUNCH(kname<T>("stag_p3d_f32", "stag_p3d_f64"), s, { k_stag_p3d<T, H><<<gb, 256, 0, s>>>(a); });
-        for (int ax = 0; ax < 3; ++ax) {
-            const IbOp& op = t->ops[3 + ax];
-            if (!op.nrows) continue;
-            const T* w = sizeof(T) == 8 ? (const T*)op.w64 : (const T*)op.w32;
-            PROF_LAUNCH(kname<T>("ib_rows3_f32", "ib_rows3_f64"), s, {
-                k_ib_rows<T><<<grid1(op.nrows * 8, 256), 256, 0, s>>>(op.nrows, op.row_pad, op.row_ptr, op.col_pad,
-                                                                       w, a.v[ax], a.kp, a.p);
-            });
-        }
-        if (g.src.n) {
-            k_add_sources<T><<<1, 256, 0, s>>>(g.src, (const T*)sh->wavelet_dev, n, a.p);
-            ib_count_launch("setup");
-        }
-        if (g.rec.n) {
-            k_receivers<T><<<grid1(g.rec.n, 256), 256, 0, s>>>(g.rec, a.p, (T*)sh->traces_dev, nt, n);
-            ib_count_launch("setup");
-        }
-        IB_CHECK_LAUNCH("3D staggered step");
+        for (int i = gl; i < 8 * a.src.n; i += 8)
+            if (a.src.idx[i] == q) sv += a.src.w[i];
+        s = sum8(s);
+        sv = sum8(sv);
+        if (act && gl == 0) a.p[q] = pq + (kq < (T)0 ? -kq : kq) * s + (a.src.n ? sv * a.wavelet[a.step] : (T)0);
+        return;
     }
-    return IB_OK;
+    blk -= a.nrb[3];
+    const int lane = threadIdx.x & 31, wy = threadIdx.x >> 5;
+    const int bx = (int)(blk % a.nbx), by = (int)(blk / a.nbx % a.nby);
+    const int64_t z = blk / a.nbx / a.nby, x = ((int64_t)bx * 32 + lane) * VX, y = by * 8 + wy;
+    const bool in = x < L.nx && y < L.ny;
+    const int64_t q = L.idx(x, y, z);
+    T w[VX + 2 * HX], y2[2 * H][VX], z2[2 * H][VX], pp[VX], kk[VX];
+    if (in) {
+#pragma unroll
+        for (int m = 0; m < 2 * HV + 1; ++m) load3<T, VX>(*reinterpret_cast<T(*)[VX]>(&w[m * VX]), a.v[0] + q + (m - HV) * VX);
+#pragma unroll
+        for (int k = 0; k < 2 * H; ++k) {   // offsets -H .. H - 1
+            load3<T, VX>(y2[k], a.v[1] + q + (k - H) * L.px);
+            load3<T, VX>(z2[k], a.v[2] + q + (k - H) * L.plane);
+        }
+        load3<T, VX>(pp, a.p + q);
+        load3<T, VX>(kk, a.kp + q);
+    }
+    // does a source corner fall in this block's box? (block-uniform)
+    int here = 0;
+    if (a.src.n) {
+        for (int i = threadIdx.x; i < 8 * a.src.n; i += 256) {
+            if (a.src.w[i] == (T)0) continue;
+            const int64_t rel = a.src.idx[i] - L.base, sz = rel / L.plane, r2 = rel - sz * L.plane, sy = r2 / L.px,
+                          sx = r2 - sy * L.px;
+            here |= sz == z && sy / 8 == by && sx / (32 * VX) == bx;
+        }
+        here = __syncthreads_or(here);
+    }
+    if (!in) return;
+#pragma unroll
+    for (int j = 0; j < VX; ++j) {
+        T s = 0;
+#pragma unroll
+        for (int k = 1; k <= H; ++k) s += a.c[k - 1] * (w[HX + j + k - 1] - w[HX + j - k]);
+#pragma unroll
+        for (int k = 1; k <= H; ++k) s += a.c[k - 1] * (y2[H + k - 1][j] - y2[H - k][j]);
+#pragma unroll
+        for (int k = 1; k <= H; ++k) s += a.c[k - 1] * (z2[H + k - 1][j] - z2[H - k][j]);
+        pp[j] += kk[j] * s;
+        if (here) {
+            T sv = 0;
+            for (int i = 0; i < 8 * a.src.n; ++i)
+                if (a.src.idx[i] == q + j) sv += a.src.w[i];
+            pp[j] += sv * a.wavelet[a.step];
+        }
+    }
+    store3<T, VX>(a.p + q, pp, kk, x, L.nx);
+}
+
+template <typename T>
+__global__ void k_mark_rows3(int64_t n, const int64_t* __restrict__ pad, T* k) {
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        const T v = k[pad[i]];
+        if (!marked3(v)) k[pad[i]] = -v;
+    }
 }
 
 template <typename T>
@@ -3036,8 +3185,9 @@ static ib_status forward_stag3(ib_table* t, const ib_shot* sh, double dt, int nt
     TRY(setup_points<T>(t, sh, dt / pow(t->grid.h, 3), S, g));
     T w2u[5], c1[4];
     stencil_weights<T>(M, w2u, c1);
+    T* coef[4] = {b0, b1, b2, kp};
     auto run = [&](auto hc) -> ib_status {
-        constexpr int HH = decltype(hc)::value;
+        constexpr int HH = decltype(hc)::value, VX = 16 / (int)sizeof(T);
         Stag3Args<T, HH> a;
         memset(&a, 0, sizeof a);
         a.L = L;
@@ -3050,7 +3200,45 @@ static ib_status forward_stag3(ib_table* t, const ib_shot* sh, double dt, int nt
         a.b[0] = b0;
         a.b[1] = b1;
         a.b[2] = b2;
-        return stag3_steps<T, HH>(t, sh, nt, a, g, s);
+        // operators 0-2: gradients; 3-5: the divergence's parts, on one set of rows
+        for (int o = 0; o < 6; ++o) {
+            const IbOp& op = t->ops[o];
+            Rows3D<T>& R = o < 3 ? a.g[o] : a.d;
+            const int i = o < 3 ? 0 : o - 3;
+            R.n = op.nrows;
+            R.pad = op.row_pad;
+            R.ptr[i] = op.row_ptr;
+            R.w[i] = sizeof(T) == 8 ? (const T*)op.w64 : (const T*)op.w32;
+            TRY(ib_table_code16(t, o, &R.code[i], s));
+            if (o < 4 && op.nrows) {
+                k_mark_rows3<T><<<grid1(op.nrows, 256), 256, 0, s>>>(op.nrows, op.row_pad, coef[o]);
+                IB_CHECK_LAUNCH("k_mark_rows3");
+                ib_count_launch("setup");
+            }
+        }
+        for (int o = 0; o < 4; ++o) a.nrb[o] = (int)((t->ops[o].nrows + S3_ROWS - 1) / S3_ROWS);
+        a.nbx = (int)((L.nx + 32 * VX - 1) / (32 * VX));
+        a.nby = (int)((L.ny + 7) / 8);
+        a.src = g.src;
+        a.wavelet = (const T*)sh->wavelet_dev;
+        a.rec = g.rec;
+        a.traces = (T*)sh->traces_dev;
+        a.nt = nt;
+        const int64_t cols = (int64_t)a.nbx * a.nby * L.nz;
+        const unsigned gv = (unsigned)(cols + a.nrb[0] + a.nrb[1] + a.nrb[2]), gp = (unsigned)(cols + a.nrb[3]);
+        for (int n = 0; n < nt; ++n) {
+            a.step = n;
+            a.rec_step = n - 1;
+            PROF_LAUNCH(kname<T>("stag_v3d_f32", "stag_v3d_f64"), s, { k_stag_v3d<T, HH><<<gv, 256, 0, s>>>(a); });
+            PROF_LAUNCH(kname<T>("stag_p3d_f32", "stag_p3d_f64"), s, { k_stag_p3d<T, HH><<<gp, 256, 0, s>>>(a); });
+            IB_CHECK_LAUNCH("3D staggered step");
+        }
+        if (g.rec.n) {
+            k_receivers<T><<<grid1(g.rec.n, 256), 256, 0, s>>>(g.rec, p, (T*)sh->traces_dev, nt, nt - 1);
+            IB_CHECK_LAUNCH("k_receivers");
+            ib_count_launch("setup");
+        }
+        return IB_OK;
     };
     if (H == 1) TRY(run(std::integral_constant<int, 1>()));
     else if (H == 2) TRY(run(std::integral_constant<int, 2>()));
