@@ -2987,11 +2987,6 @@ ib_status ib_table_code16(ib_table* t, int op, const uint16_t** out, cudaStream_
     return IB_OK;
 }
 
-ib_status ib_make_bins_ext(const Layout& L, int64_t n, const int64_t* pad, int tx, int ty, int tz, TileBins& b,
-                           cudaStream_t s) {
-    return make_bins(L, n, pad, nullptr, nullptr, nullptr, tx, ty, tz, b, s);
-}
-
 ib_status ib_table_bins(ib_table* t, int op, bool transposed, int tx, int ty, int tz, const TileBins** out,
                         cudaStream_t s) {
     IbOp& o = t->ops[op];

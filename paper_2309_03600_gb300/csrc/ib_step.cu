@@ -36,8 +36,6 @@
 
 std::vector<double> ib_central_second(int M);
 std::vector<double> ib_staggered_first(int M);
-ib_status ib_make_bins_ext(const Layout& L, int64_t n, const int64_t* pad, int tx, int ty, int tz, TileBins& b,
-                           cudaStream_t s);
 
 #define TRY(x)                          \
     do {                                \
@@ -975,322 +973,6 @@ static void launch_leap3d_tma2(const StepArgs<float>& a, const CUtensorMap& tm, 
 }
 
 // ---------------------------------------------------------------------------
-// 2D staggered pressure-velocity
-//   v_a[j] (at j + e_a/2) += bh_a[j] (sum_k c_k (p[j + k e_a] - p[j - (k-1) e_a]) + IB)
-//   p[j] += kh[j] (sum_a sum_k c_k (v_a[j + (k-1) e_a] - v_a[j - k e_a]) + IB) + src
-// with bh_a = dt / (rho h) and kh = dt rho c^2 / h
-// ---------------------------------------------------------------------------
-// Producer-side partial sums of the staggered corrections.  A correction row
-// sum_e w_e f[col_e] is split by the step tile that holds col_e: the kernel
-// that has just produced f on that tile forms partial[pid] = the sum over the
-// row's entries there (values read from shared memory), and the kernel that
-// consumes the row adds its partials (1-4 per row) while it loads its tile.
-// No kernel gathers correction columns from global memory.
-template <typename T>
-struct StagPlan {
-    // producer side (this kernel writes `out`): per tile, pid positions
-    // [qptr[t], qptr[t+1]) and entries [eptr[t], eptr[t+1])
-    const int32_t* qptr;
-    const int32_t* qpid;     // global pid of each position
-    const int32_t* eptr;
-    const int32_t* emeta;    // field << 31 | (pid position - qptr[t]) << 11 | slot (lz * TX + lx) of the column
-    const T* ew;
-    T* out;
-    int max_q;               // largest pid count of a tile
-    // consumer side (this kernel reads `in`): per tile, rows [rptr[t], rptr[t+1])
-    const int32_t* rptr;
-    const int32_t* rslot;    // target << 24 | slot of the row node
-    const int32_t* rpb;      // pid range of the row
-    const int32_t* rpe;
-    const T* in;
-    int64_t n_in;            // partial sums in `in`
-};
-
-template <typename T>
-struct StagArgs {
-    Layout L;
-    StagPlan<T> pv;          // v kernel: consumes partials of p, produces those of v
-    StagPlan<T> pp;          // p kernel: consumes partials of v, produces those of p
-    const uint8_t* src_tile; // per step tile: a source corner lies in it
-    const int* step_base;    // device step offset added to step / rec_step (graph replays)
-    T c1[4];             // staggered weights for offsets +1/2 .. +(M-1)/2
-    T* p;
-    T* vx;
-    T* vz;
-    const T* bx;
-    const T* bz;
-    const T* kp;
-    TileView<T> gx, gz, dx, dz;
-    PointSet<T> src;     // weights include dt / h^d
-    const T* wavelet;
-    int step;
-    PointSet<T> rec;
-    T* traces;
-    int nt;
-    int rec_step;
-};
-
-// consumer side: correction of row i of this tile's list = sum of its partials
-template <typename T>
-__device__ __forceinline__ T plan_row_sum(const StagPlan<T>& P, int32_t i) {
-    T c = 0;
-    for (int32_t q = P.rpb[i]; q < P.rpe[i]; ++q) c += P.in[q];
-    return c;
-}
-
-// producer side, first part: stage up to STG of this tile's entries in shared memory
-template <typename T, int STG>
-__device__ __forceinline__ int32_t plan_stage(const StagPlan<T>& P, int64_t tile, int32_t* smeta, T* sw, int tid) {
-    const int32_t e0 = P.eptr[tile], e1 = P.eptr[tile + 1];
-    const int32_t n = e1 - e0 < STG ? e1 - e0 : STG;
-    for (int32_t i = tid; i < n; i += 256) {
-        cp_async<4>(&smeta[i], P.emeta + e0 + i, true);
-        cp_async<(int)sizeof(T)>(&sw[i], P.ew + e0 + i, true);
-    }
-    return n;
-}
-
-// producer side: partial[pid] = sum of w * fnew[field][slot] over the pid's entries in this tile.
-// A tile's entries are ordered by their rank within the pid, then by pid, so
-// the lanes of a warp add into different partial sums.  The first `nst`
-// entries were staged in shared memory while the tile loaded.
-template <typename T, int SLOTS>
-__device__ __forceinline__ void plan_produce(const StagPlan<T>& P, int64_t tile, const T* fnew, T* psum,
-                                             const int32_t* smeta, const T* sw, int32_t nst, int tid) {
-    const int32_t q0 = P.qptr[tile], nq = P.qptr[tile + 1] - q0;
-    const int32_t e0 = P.eptr[tile], e1 = P.eptr[tile + 1];
-    for (int32_t k = tid; k < nq; k += 256) psum[k] = (T)0;
-    __syncthreads();
-    for (int32_t i = tid; i < nst; i += 256) {
-        const uint32_t mm = (uint32_t)smeta[i];
-        atomicAdd(&psum[(mm >> 11) & 0xfffff], sw[i] * fnew[(mm >> 31) * SLOTS + (mm & 0x7ff)]);
-    }
-    constexpr int U = 8;
-    for (int32_t base = e0 + nst + tid; base < e1; base += 256 * U) {
-        int32_t m[U];
-        T w[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int32_t e = base + u * 256;
-            m[u] = e < e1 ? P.emeta[e] : 0;
-            w[u] = e < e1 ? P.ew[e] : (T)0;
-        }
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            if (base + u * 256 >= e1) continue;
-            const uint32_t mm = (uint32_t)m[u];
-            atomicAdd(&psum[(mm >> 11) & 0xfffff], w[u] * fnew[(mm >> 31) * SLOTS + (mm & 0x7ff)]);
-        }
-    }
-    __syncthreads();
-    for (int32_t k = tid; k < nq; k += 256) P.out[P.qpid[q0 + k]] = psum[k];
-}
-
-// v^{n+1/2} = v^{n-1/2} + (dt / rho) G_mod p^n on a 64 x TZ tile (256 threads as 64 x 4,
-// TZ / 4 points per thread); the p tile and the producer entries arrive by cp.async
-template <typename T, int H, int TX, int TZ, int MAXQ, int STG>
-__global__ void __launch_bounds__(256, 4) k_stag_v2d(StagArgs<T> a) {
-    static_assert(TX == 64 && TZ % 4 == 0, "64-wide tiles, 4 thread rows");
-    constexpr int NP = TZ / 4, SL = TZ * TX;
-    __shared__ __align__(16) T tile[TZ + 2 * H][TX + 2 * H];
-    __shared__ T acc[2 * SL];                        // a_x, a_z; then the new v_x, v_z
-    __shared__ T psum[MAXQ];
-    __shared__ int32_t smeta[STG];
-    __shared__ T sw[STG];
-    const int tid = threadIdx.x, tx = tid & 63, ty = tid >> 6;
-    const int64_t blk = (int64_t)blockIdx.y * gridDim.x + blockIdx.x;
-    const int64_t x0 = (int64_t)blockIdx.x * TX, z0 = (int64_t)blockIdx.y * TZ;
-    const Layout& L = a.L;
-    const int64_t origin = L.base + z0 * L.px + x0;
-    {
-        const T* pb = a.p + origin - H * L.px - H;
-#pragma unroll
-        for (int lz = ty; lz < TZ + 2 * H; lz += 4) {
-            const bool zok = z0 + lz - H < L.nz + H;
-            const T* row = pb + lz * L.px;
-            for (int lx = tx; lx < TX + 2 * H; lx += 64) {
-                const bool ok = zok && x0 + lx - H < L.nx + H;
-                cp_async<(int)sizeof(T)>(&tile[lz][lx], ok ? row + lx : a.p, ok);
-            }
-        }
-    }
-    const int32_t nst = plan_stage<T, STG>(a.pv, blk, smeta, sw, tid);
-    cp_async_commit();
-    const int sb = a.step_base ? *a.step_base : 0;
-    record_receivers(a.rec, a.p, a.traces, a.nt, sb + a.rec_step, blk * 256 + tid, launch_threads());
-    const int32_t r0 = a.pv.rptr[blk], r1 = a.pv.rptr[blk + 1];
-    // the update's own operands and this tile's row corrections while the copies fly
-    T vx[NP], vz[NP], bx[NP], bz[NP];
-#pragma unroll
-    for (int k = 0; k < NP; ++k) {
-        const int lz = ty + 4 * k;
-        const bool in = x0 + tx < L.nx && z0 + lz < L.nz;
-        const int64_t q = origin + lz * L.px + tx;
-        vx[k] = in ? a.vx[q] : (T)0;
-        vz[k] = in ? a.vz[q] : (T)0;
-        bx[k] = in ? a.bx[q] : (T)0;
-        bz[k] = in ? a.bz[q] : (T)0;
-    }
-    T corr = 0;
-    int32_t cslot = 0;
-    if (r0 + tid < r1) {
-        corr = plan_row_sum(a.pv, r0 + tid);
-        cslot = a.pv.rslot[r0 + tid];
-    }
-    cp_async_wait_all();
-    __syncthreads();
-    T ax[NP], az[NP];
-#pragma unroll
-    for (int k = 0; k < NP; ++k) {
-        const int lz = ty + 4 * k;
-        T sx = 0, sz = 0;
-#pragma unroll
-        for (int j = 1; j <= H; ++j) {
-            sx += a.c1[j - 1] * (tile[lz + H][tx + H + j] - tile[lz + H][tx + H - j + 1]);
-            sz += a.c1[j - 1] * (tile[lz + H + j][tx + H] - tile[lz + H - j + 1][tx + H]);
-        }
-        ax[k] = sx;
-        az[k] = sz;
-    }
-    if (r1 > r0) {
-#pragma unroll
-        for (int k = 0; k < NP; ++k) {
-            acc[(ty + 4 * k) * TX + tx] = ax[k];
-            acc[SL + (ty + 4 * k) * TX + tx] = az[k];
-        }
-        __syncthreads();
-        for (int32_t i = r0 + tid; i < r1; i += 256) {
-            if (i >= r0 + 256) {
-                corr = plan_row_sum(a.pv, i);
-                cslot = a.pv.rslot[i];
-            }
-            atomicAdd(&acc[(cslot >> 24) * SL + (cslot & 0xffffff)], corr);
-        }
-        __syncthreads();
-#pragma unroll
-        for (int k = 0; k < NP; ++k) {
-            ax[k] = acc[(ty + 4 * k) * TX + tx];
-            az[k] = acc[SL + (ty + 4 * k) * TX + tx];
-        }
-    }
-    const bool produce = a.pv.out != nullptr && a.pv.eptr[blk + 1] > a.pv.eptr[blk];
-    if (produce) __syncthreads();     // acc is reused for the new values
-#pragma unroll
-    for (int k = 0; k < NP; ++k) {
-        const int lz = ty + 4 * k;
-        const T nvx = vx[k] + bx[k] * ax[k];
-        const T nvz = vz[k] + bz[k] * az[k];
-        if (produce) {
-            acc[lz * TX + tx] = nvx;
-            acc[SL + lz * TX + tx] = nvz;
-        }
-        if (x0 + tx >= L.nx || z0 + lz >= L.nz) continue;
-        const int64_t q = origin + lz * L.px + tx;
-        a.vx[q] = nvx;
-        a.vz[q] = nvz;
-    }
-    if (produce) plan_produce<T, SL>(a.pv, blk, acc, psum, smeta, sw, nst, tid);
-}
-
-// p^{n+1} = p^n + dt rho c^2 D_mod v^{n+1/2} (+ source) on a 64 x TZ tile
-template <typename T, int H, int TX, int TZ, int MAXQ, int STG>
-__global__ void __launch_bounds__(256, 4) k_stag_p2d(StagArgs<T> a) {
-    static_assert(TX == 64 && TZ % 4 == 0, "64-wide tiles, 4 thread rows");
-    constexpr int NP = TZ / 4, SL = TZ * TX;
-    __shared__ __align__(16) T tvx[TZ][TX + 2 * H];
-    __shared__ __align__(16) T tvz[TZ + 2 * H][TX];
-    __shared__ T acc[SL];
-    __shared__ T psum[MAXQ];
-    __shared__ int32_t smeta[STG];
-    __shared__ T sw[STG];
-    const int tid = threadIdx.x, tx = tid & 63, ty = tid >> 6;
-    const int64_t blk = (int64_t)blockIdx.y * gridDim.x + blockIdx.x;
-    const int64_t x0 = (int64_t)blockIdx.x * TX, z0 = (int64_t)blockIdx.y * TZ;
-    const Layout& L = a.L;
-    const int64_t origin = L.base + z0 * L.px + x0;
-    {
-        const T* vb = a.vx + origin - H;
-#pragma unroll
-        for (int lz = ty; lz < TZ; lz += 4) {
-            const bool zok = z0 + lz < L.nz + H;
-            const T* row = vb + lz * L.px;
-            for (int lx = tx; lx < TX + 2 * H; lx += 64) {
-                const bool ok = zok && x0 + lx - H < L.nx + H;
-                cp_async<(int)sizeof(T)>(&tvx[lz][lx], ok ? row + lx : a.vx, ok);
-            }
-        }
-        const T* wb = a.vz + origin - H * L.px;
-        const bool xok = x0 + tx < L.nx + H;
-#pragma unroll
-        for (int lz = ty; lz < TZ + 2 * H; lz += 4) {
-            const bool ok = xok && z0 + lz - H < L.nz + H;
-            cp_async<(int)sizeof(T)>(&tvz[lz][tx], ok ? wb + lz * L.px + tx : a.vz, ok);
-        }
-    }
-    const int32_t nst = plan_stage<T, STG>(a.pp, blk, smeta, sw, tid);
-    cp_async_commit();
-    const int32_t r0 = a.pp.rptr[blk], r1 = a.pp.rptr[blk + 1];
-    T pv[NP], kv[NP];
-#pragma unroll
-    for (int k = 0; k < NP; ++k) {
-        const int lz = ty + 4 * k;
-        const bool in = x0 + tx < L.nx && z0 + lz < L.nz;
-        const int64_t q = origin + lz * L.px + tx;
-        pv[k] = in ? a.p[q] : (T)0;
-        kv[k] = in ? a.kp[q] : (T)0;
-    }
-    T corr = 0;
-    int32_t cslot = 0;
-    if (r0 + tid < r1) {
-        corr = plan_row_sum(a.pp, r0 + tid);
-        cslot = a.pp.rslot[r0 + tid];
-    }
-    const bool has_src = a.src.n > 0 && a.src_tile[blk] != 0;
-    if (has_src || r1 > r0)
-        for (int i = tid; i < SL; i += 256) acc[i] = (T)0;
-    cp_async_wait_all();
-    __syncthreads();
-    T s[NP];
-#pragma unroll
-    for (int k = 0; k < NP; ++k) {
-        const int lz = ty + 4 * k;
-        T sum = 0;
-#pragma unroll
-        for (int j = 1; j <= H; ++j) {
-            sum += a.c1[j - 1] * (tvx[lz][tx + H + j - 1] - tvx[lz][tx + H - j]);
-            sum += a.c1[j - 1] * (tvz[lz + H + j - 1][tx] - tvz[lz + H - j][tx]);
-        }
-        s[k] = pv[k] + kv[k] * sum;
-    }
-    if (has_src || r1 > r0) {
-        // acc collects kp * corrections and the source term of this tile
-        const T wv = has_src ? a.wavelet[(a.step_base ? *a.step_base : 0) + a.step] : (T)0;
-        tile_sources<T, TX, TZ>(a.src, wv, origin, L.px, acc, tid);
-        for (int32_t i = r0 + tid; i < r1; i += 256) {
-            if (i >= r0 + 256) {
-                corr = plan_row_sum(a.pp, i);
-                cslot = a.pp.rslot[i];
-            }
-            const int sl = cslot & 0xffffff;
-            atomicAdd(&acc[sl], a.kp[origin + (sl / TX) * L.px + (sl % TX)] * corr);
-        }
-        __syncthreads();
-#pragma unroll
-        for (int k = 0; k < NP; ++k) s[k] += acc[(ty + 4 * k) * TX + tx];
-    }
-    const bool produce = a.pp.out != nullptr && a.pp.eptr[blk + 1] > a.pp.eptr[blk];
-    if (produce) __syncthreads();
-#pragma unroll
-    for (int k = 0; k < NP; ++k) {
-        const int lz = ty + 4 * k;
-        if (produce) acc[lz * TX + tx] = s[k];
-        if (x0 + tx >= L.nx || z0 + lz >= L.nz) continue;
-        a.p[origin + lz * L.px + tx] = s[k];
-    }
-    if (produce) plan_produce<T, SL>(a.pp, blk, acc, psum, smeta, sw, nst, tid);
-}
-
-// ---------------------------------------------------------------------------
 // setup kernels (coefficients formed in FP64, rounded once)
 // ---------------------------------------------------------------------------
 template <typename T>
@@ -1479,21 +1161,13 @@ struct Probe {
     double* logs;       // [nslot]
 };
 
-// Renormalise the state (a, b, c) by its norm; `extra` (n_extra values, not part
-// of the norm) holds quantities linear in the state that the next step reads --
-// the staggered form's producer-side partial sums -- and is scaled alike.
+// renormalise the state (a, b, c) by its norm
 template <typename T>
-static ib_status probe_rescale(const Probe* pr, int slot, int64_t n, T* a, T* b, T* c, cudaStream_t s,
-                               T* extra = nullptr, int64_t n_extra = 0) {
+static ib_status probe_rescale(const Probe* pr, int slot, int64_t n, T* a, T* b, T* c, cudaStream_t s) {
     k_sumsq<T><<<grid1(n, 256), 256, 0, s>>>(n, a, b, c, pr->sums + slot);
     k_rescale<T><<<grid1(n, 256), 256, 0, s>>>(n, a, b, c, pr->sums + slot, pr->logs + slot);
     ib_count_launch("setup");
     ib_count_launch("setup");
-    if (extra && n_extra > 0) {
-        k_rescale<T><<<grid1(n_extra, 256), 256, 0, s>>>(n_extra, extra, (T*)nullptr, (T*)nullptr,
-                                                          pr->sums + slot, pr->logs + slot);
-        ib_count_launch("setup");
-    }
     IB_CHECK_LAUNCH("stability probe");
     return IB_OK;
 }
@@ -2486,378 +2160,6 @@ static ib_status forward_2nd(ib_table* t, const ib_shot* sh, double dt, int nt, 
     return IB_OK;
 }
 
-// Staggered step tiles: 64 x 32 (FP32) or 64 x 16 (FP64) nodes; at most
-// STAG_MAXQ partial sums produced per tile.
-static const int STAG_TX = 64, STAG_MAXQ = 1024;
-static_assert(STAG_TX * 32 <= 2048 && STAG_MAXQ <= (1 << 20), "packed producer entries: 11-bit slot, 20-bit position");
-template <typename T> struct StagTile { static const int TZ = 16, STG = 2048; };
-template <> struct StagTile<double> { static const int TZ = 16, STG = 512; };
-
-struct PlanOp {
-    int op;       // consumer operator
-    int target;   // accumulator of the consumer kernel (0: a_x / p, 1: a_z)
-    int field;    // producer field of its columns (0: v_x / p, 1: v_z)
-};
-
-// Split the rows of the consumer operators by producer tile (see StagPlan):
-// fills the consumer side of `cons` and the producer side of `prod`.
-template <typename T>
-static ib_status build_stag_plan(ib_table* t, const std::vector<PlanOp>& ops, int TZ, Scratch& S,
-                                 StagPlan<T>& cons, StagPlan<T>& prod, cudaStream_t s) {
-    const Layout& L = t->L;
-    const int64_t ntx = (L.nx + STAG_TX - 1) / STAG_TX, ntz = (L.nz + TZ - 1) / TZ, ntiles = ntx * ntz;
-    struct Ent {
-        int32_t row, ptile, slot, field;
-        double w;
-    };
-    struct Row {
-        int32_t ctile, cslot;   // consumer tile and target << 24 | slot
-    };
-    std::vector<Ent> ent;
-    std::vector<Row> rows;
-    {
-        int64_t nnz = 0, nr = 0;
-        for (const PlanOp& po : ops) {
-            nnz += t->ops[po.op].nnz;
-            nr += t->ops[po.op].nrows;
-        }
-        ent.reserve(nnz);
-        rows.reserve(nr);
-    }
-    for (const PlanOp& po : ops) {
-        const IbOp& op = t->ops[po.op];
-        const int64_t nr = op.nrows, nz = op.nnz;
-        std::vector<int64_t> lin(nr), rp(nr + 1);
-        std::vector<int32_t> code(nz);
-        std::vector<double> w(nz);
-        if (nr) {
-            IB_CUDA(cudaMemcpy(lin.data(), op.row_lin, 8 * nr, cudaMemcpyDeviceToHost));
-            IB_CUDA(cudaMemcpy(rp.data(), op.row_ptr, 8 * (nr + 1), cudaMemcpyDeviceToHost));
-        }
-        if (nz) {
-            IB_CUDA(cudaMemcpy(code.data(), op.col_code, 4 * nz, cudaMemcpyDeviceToHost));
-            IB_CUDA(cudaMemcpy(w.data(), op.w64, 8 * nz, cudaMemcpyDeviceToHost));
-        }
-        for (int64_t r = 0; r < nr; ++r) {
-            const int64_t x = lin[r] % L.nx, z = lin[r] / L.nx;
-            const int32_t key = (int32_t)rows.size();
-            rows.push_back({(int32_t)((z / TZ) * ntx + x / STAG_TX),
-                            (int32_t)(po.target << 24 | ((z % TZ) * STAG_TX + x % STAG_TX))});
-            for (int64_t e = rp[r]; e < rp[r + 1]; ++e) {
-                int dx, dy, dz;
-                unpack_off(code[e], dx, dy, dz);
-                const int64_t cx = x + dx, cz = z + dy;
-                if (cx < 0 || cx >= L.nx || cz < 0 || cz >= L.nz) {
-                    ib_set_error("correction column outside the grid");
-                    return IB_ERR_STATE;
-                }
-                ent.push_back({key, (int32_t)((cz / TZ) * ntx + cx / STAG_TX),
-                               (int32_t)((cz % TZ) * STAG_TX + cx % STAG_TX), po.field, w[e]});
-            }
-        }
-    }
-    // partial ids: one per (row, producer tile), numbered row by row.  Entries
-    // arrive grouped by row; regroup each row's entries by producer tile (a row
-    // spans a few tiles), keeping their order within a tile.
-    const int64_t nrow = (int64_t)rows.size(), nent = (int64_t)ent.size();
-    {
-        std::vector<Ent> tmp;
-        std::vector<int32_t> tiles;
-        for (int64_t i = 0; i < nent;) {
-            int64_t j = i;
-            tiles.clear();
-            for (; j < nent && ent[j].row == ent[i].row; ++j)
-                if (std::find(tiles.begin(), tiles.end(), ent[j].ptile) == tiles.end()) tiles.push_back(ent[j].ptile);
-            if (tiles.size() > 1) {
-                std::sort(tiles.begin(), tiles.end());
-                tmp.clear();
-                for (int32_t tl : tiles)
-                    for (int64_t k = i; k < j; ++k)
-                        if (ent[k].ptile == tl) tmp.push_back(ent[k]);
-                std::copy(tmp.begin(), tmp.end(), ent.begin() + i);
-            }
-            i = j;
-        }
-    }
-    std::vector<int32_t> pid(nent), rank(nent), rpb(nrow, 0), rpe(nrow, 0);
-    int32_t npid = 0;
-    for (int64_t i = 0; i < nent; ++i) {
-        const bool new_row = i == 0 || ent[i].row != ent[i - 1].row;
-        if (new_row || ent[i].ptile != ent[i - 1].ptile) {
-            if (new_row) rpb[ent[i].row] = npid;
-            ++npid;
-            rank[i] = 0;
-        } else {
-            rank[i] = rank[i - 1] + 1;
-        }
-        pid[i] = npid - 1;
-        rpe[ent[i].row] = npid;
-    }
-    // producer side: entries grouped by tile (counting sort keeps the pid order)
-    std::vector<int32_t> eptr(ntiles + 1, 0), qptr(ntiles + 1, 0), emeta(nent), qpid;
-    std::vector<T> ew(nent);
-    std::vector<int64_t> order(nent), tmp_order;
-    for (int64_t i = 0; i < nent; ++i) eptr[ent[i].ptile + 1]++;
-    for (int64_t tl = 0; tl < ntiles; ++tl) eptr[tl + 1] += eptr[tl];
-    {
-        std::vector<int32_t> fill(eptr.begin(), eptr.end() - 1);
-        for (int64_t i = 0; i < nent; ++i) order[fill[ent[i].ptile]++] = i;
-    }
-    std::vector<int32_t> pos(nent), rcount;
-    int max_q = 0;
-    for (int64_t tl = 0; tl < ntiles; ++tl) {
-        const int64_t i0 = eptr[tl], i1 = eptr[tl + 1];
-        qptr[tl] = (int32_t)qpid.size();
-        const int64_t q0 = (int64_t)qpid.size();
-        int32_t maxr = 0;
-        for (int64_t i = i0; i < i1; ++i) {
-            if ((int64_t)qpid.size() == q0 || qpid.back() != pid[order[i]]) qpid.push_back(pid[order[i]]);
-            pos[order[i]] = (int32_t)((int64_t)qpid.size() - 1 - q0);
-            maxr = std::max(maxr, rank[order[i]]);
-        }
-        max_q = std::max(max_q, (int)((int64_t)qpid.size() - q0));
-        // within the tile: by rank, then pid (a stable counting sort by rank of the
-        // pid-ordered entries), so adjacent lanes add into different partial sums
-        rcount.assign(maxr + 2, 0);
-        for (int64_t i = i0; i < i1; ++i) rcount[rank[order[i]] + 1]++;
-        for (int32_t r = 0; r <= maxr; ++r) rcount[r + 1] += rcount[r];
-        tmp_order.resize(i1 - i0);
-        for (int64_t i = i0; i < i1; ++i) tmp_order[rcount[rank[order[i]]]++] = order[i];
-        for (int64_t k = i0; k < i1; ++k) {
-            const int64_t e = tmp_order[k - i0];
-            emeta[k] = (int32_t)((uint32_t)ent[e].field << 31 | (uint32_t)pos[e] << 11 | (uint32_t)ent[e].slot);
-            ew[k] = (T)ent[e].w;
-        }
-    }
-    qptr[ntiles] = (int32_t)qpid.size();
-    if (max_q > STAG_MAXQ) {
-        ib_set_error("a staggered step tile holds more correction partial sums than the kernel's buffer");
-        return IB_ERR_STATE;
-    }
-    // consumer side: rows grouped by tile (counting sort)
-    std::vector<int32_t> rptr(ntiles + 1, 0), rslot(nrow), rb(nrow), re(nrow);
-    for (int64_t r = 0; r < nrow; ++r) rptr[rows[r].ctile + 1]++;
-    for (int64_t tl = 0; tl < ntiles; ++tl) rptr[tl + 1] += rptr[tl];
-    {
-        std::vector<int32_t> fill(rptr.begin(), rptr.end() - 1);
-        for (int64_t r = 0; r < nrow; ++r) {
-            const int32_t i = fill[rows[r].ctile]++;
-            rslot[i] = rows[r].cslot;
-            rb[i] = rpb[r];
-            re[i] = rpe[r];
-        }
-    }
-    auto up = [&](auto** dst, const auto& v) -> ib_status {
-        using E = typename std::decay<decltype(v[0])>::type;
-        E* d;
-        TRY(S.alloc(&d, (int64_t)std::max<size_t>(v.size(), 1)));
-        if (!v.empty()) IB_CUDA(cudaMemcpyAsync(d, v.data(), sizeof(E) * v.size(), cudaMemcpyHostToDevice, s));
-        *dst = d;
-        return IB_OK;
-    };
-    int32_t *d_eptr, *d_qptr, *d_qpid, *d_emeta, *d_rptr, *d_rslot, *d_rb, *d_re;
-    T* d_ew;
-    TRY(up(&d_eptr, eptr));
-    TRY(up(&d_qptr, qptr));
-    TRY(up(&d_qpid, qpid));
-    TRY(up(&d_emeta, emeta));
-    TRY(up(&d_ew, ew));
-    TRY(up(&d_rptr, rptr));
-    TRY(up(&d_rslot, rslot));
-    TRY(up(&d_rb, rb));
-    TRY(up(&d_re, re));
-    T* partial;
-    TRY(S.alloc(&partial, std::max<int64_t>(npid, 1), true));
-    IB_CUDA(cudaStreamSynchronize(s));   // host vectors go out of scope
-    prod.qptr = d_qptr;
-    prod.qpid = d_qpid;
-    prod.eptr = d_eptr;
-    prod.emeta = d_emeta;
-    prod.ew = d_ew;
-    prod.out = partial;
-    prod.max_q = max_q;
-    cons.rptr = d_rptr;
-    cons.rslot = d_rslot;
-    cons.rpb = d_rb;
-    cons.rpe = d_re;
-    cons.in = partial;
-    cons.n_in = npid;
-    return IB_OK;
-}
-
-__global__ void k_add_step(int* base, int k) {
-    if (threadIdx.x == 0 && blockIdx.x == 0) *base += k;
-}
-
-// time steps per captured graph of the staggered loop (the graph is replayed nt / STAG_GRAPH_STEPS times)
-static const int STAG_GRAPH_STEPS = 50;
-static_assert(STAG_GRAPH_STEPS == STAB_BLOCK, "the stability probe renormalises between graph replays");
-
-template <typename T>
-static ib_status forward_stag(ib_table* t, const ib_shot* sh, double dt, int nt, cudaStream_t s,
-                              const Probe* probe = nullptr) {
-    const Layout& L = t->L;
-    const int d = t->grid.ndim;
-    if (shot_damped(sh)) {
-        ib_set_error("the absorbing layer is implemented for the second-order form");
-        return IB_ERR_STATE;
-    }
-    if (d != 2) {
-        ib_set_error("the staggered form is implemented in 2D");
-        return IB_ERR_STATE;
-    }
-    const int M = t->opts.space_order;
-    const int H = M / 2;
-    Scratch S(s);
-    T *p, *vx, *vz, *kp, *bx, *bz;
-    TRY(S.alloc(&p, L.total, true));
-    TRY(S.alloc(&vx, L.total, true));
-    TRY(S.alloc(&vz, L.total, true));
-    TRY(S.alloc(&kp, L.total, true));
-    TRY(S.alloc(&bx, L.total, true));
-    TRY(S.alloc(&bz, L.total, true));
-    k_stag_coef<T><<<grid1(L.N, 256), 256, 0, s>>>(L, (const T*)sh->vel_dev, (const T*)sh->rho_dev, t->mask_pad[0],
-                                                   t->mask_pad[1], t->mask_pad[2], dt, 1.0 / t->grid.h, kp, bx, bz);
-    IB_CHECK_LAUNCH("k_stag_coef");
-    ib_count_launch("setup");
-    if (probe) {   // random p, v_x, v_z on their interior nodes, normalised together
-        k_rand_fill<T><<<grid1(L.total, 256), 256, 0, s>>>(L.total, kp, probe->seed, p, (T*)nullptr);
-        k_rand_fill<T><<<grid1(L.total, 256), 256, 0, s>>>(L.total, bx, probe->seed + 1, vx, (T*)nullptr);
-        k_rand_fill<T><<<grid1(L.total, 256), 256, 0, s>>>(L.total, bz, probe->seed + 2, vz, (T*)nullptr);
-        IB_CHECK_LAUNCH("k_rand_fill");
-        TRY(probe_rescale<T>(probe, 0, L.total, p, vx, vz, s));
-    }
-    Geom<T> g;
-    TRY(setup_points<T>(t, sh, dt / pow(t->grid.h, d), S, g));
-    StagArgs<T> a;
-    memset(&a, 0, sizeof a);
-    a.L = L;
-    {
-        T w2u[5];
-        stencil_weights<T>(M, w2u, a.c1);
-    }
-    a.p = p;
-    a.vx = vx;
-    a.vz = vz;
-    a.bx = bx;
-    a.bz = bz;
-    a.kp = kp;
-    constexpr int TZ = StagTile<T>::TZ, STG = StagTile<T>::STG;
-    // p rows read partials of v (formed by the v kernel); v rows read partials of p
-    TRY(build_stag_plan<T>(t, {{2, 0, 0}, {3, 0, 1}}, TZ, S, a.pp, a.pv, s));
-    TRY(build_stag_plan<T>(t, {{0, 0, 0}, {1, 1, 0}}, TZ, S, a.pv, a.pp, s));
-    const int64_t ntx = (L.nx + STAG_TX - 1) / STAG_TX, ntz = (L.nz + TZ - 1) / TZ;
-    {
-        std::vector<uint8_t> flag(ntx * ntz, 0);
-        std::vector<int64_t> hidx(8 * (size_t)g.src.n);
-        if (g.src.n) IB_CUDA(cudaMemcpy(hidx.data(), g.src.idx, 8 * hidx.size(), cudaMemcpyDeviceToHost));
-        for (int64_t q : hidx) {
-            const int64_t rel = q - L.base, z = rel / L.px, x = rel - z * L.px;
-            if (x >= 0 && x < L.nx && z >= 0 && z < L.nz) flag[(z / TZ) * ntx + x / STAG_TX] = 1;
-        }
-        uint8_t* d;
-        TRY(S.alloc(&d, (int64_t)flag.size()));
-        IB_CUDA(cudaMemcpyAsync(d, flag.data(), flag.size(), cudaMemcpyHostToDevice, s));
-        IB_CUDA(cudaStreamSynchronize(s));
-        a.src_tile = d;
-    }
-    a.src = g.src;
-    a.wavelet = (const T*)sh->wavelet_dev;
-    a.rec = g.rec;
-    a.traces = (T*)sh->traces_dev;
-    a.nt = nt;
-    dim3 grid2((unsigned)ntx, (unsigned)ntz);
-    auto launch_step = [&](cudaStream_t st, bool prof) -> ib_status {
-        auto v = [&]() {
-            if (H == 1) k_stag_v2d<T, 1, STAG_TX, TZ, STAG_MAXQ, STG><<<grid2, 256, 0, st>>>(a);
-            else if (H == 2) k_stag_v2d<T, 2, STAG_TX, TZ, STAG_MAXQ, STG><<<grid2, 256, 0, st>>>(a);
-            else if (H == 3) k_stag_v2d<T, 3, STAG_TX, TZ, STAG_MAXQ, STG><<<grid2, 256, 0, st>>>(a);
-            else k_stag_v2d<T, 4, STAG_TX, TZ, STAG_MAXQ, STG><<<grid2, 256, 0, st>>>(a);
-        };
-        auto pk = [&]() {
-            if (H == 1) k_stag_p2d<T, 1, STAG_TX, TZ, STAG_MAXQ, STG><<<grid2, 256, 0, st>>>(a);
-            else if (H == 2) k_stag_p2d<T, 2, STAG_TX, TZ, STAG_MAXQ, STG><<<grid2, 256, 0, st>>>(a);
-            else if (H == 3) k_stag_p2d<T, 3, STAG_TX, TZ, STAG_MAXQ, STG><<<grid2, 256, 0, st>>>(a);
-            else k_stag_p2d<T, 4, STAG_TX, TZ, STAG_MAXQ, STG><<<grid2, 256, 0, st>>>(a);
-        };
-        if (prof) {
-            PROF_LAUNCH(kname<T>("stag_v2d_f32", "stag_v2d_f64"), st, { v(); });
-            PROF_LAUNCH(kname<T>("stag_p2d_f32", "stag_p2d_f64"), st, { pk(); });
-        } else {
-            v();
-            pk();
-            ib_count_launch(kname<T>("stag_v2d_f32", "stag_v2d_f64"));
-            ib_count_launch(kname<T>("stag_p2d_f32", "stag_p2d_f64"));
-        }
-        IB_CHECK_LAUNCH("staggered step");
-        return IB_OK;
-    };
-    int* d_base;
-    TRY(S.alloc(&d_base, 1, true));
-    a.step_base = d_base;
-    const int K = STAG_GRAPH_STEPS;
-    const int nrep = (nt >= 2 * K && !getenv("IB_NO_GRAPH")) ? nt / K : 0;
-    cudaStream_t cs = s;
-    cudaEvent_t ready = nullptr;
-    if (nrep) {
-        // K steps (and the step-offset bump) as one graph, replayed nrep times on a side stream
-        IB_CUDA(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
-        IB_CUDA(cudaEventCreateWithFlags(&ready, cudaEventDisableTiming));
-        IB_CUDA(cudaEventRecord(ready, s));
-        IB_CUDA(cudaStreamWaitEvent(cs, ready, 0));
-        cudaGraph_t graph = nullptr;
-        cudaGraphExec_t exec = nullptr;
-        IB_CUDA(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
-        ib_status st = IB_OK;
-        for (int k = 0; k < K && st == IB_OK; ++k) {
-            a.step = k;
-            a.rec_step = k - 1;
-            st = launch_step(cs, false);
-        }
-        k_add_step<<<1, 32, 0, cs>>>(d_base, K);
-        cudaError_t ce = cudaStreamEndCapture(cs, &graph);
-        if (st != IB_OK) return st;
-        if (ce != cudaSuccess) return ib_cuda_fail(ce, "graph capture", __FILE__, __LINE__);
-        IB_CUDA(cudaGraphInstantiate(&exec, graph, 0));
-        for (int r = 0; r < nrep; ++r) {
-            ProfToken tk = ib_prof_begin(kname<T>("stag_graph50_f32", "stag_graph50_f64"), cs);
-            IB_CUDA(cudaGraphLaunch(exec, cs));
-            ib_prof_end(tk, cs);
-            if (probe)
-                TRY(probe_rescale<T>(probe, r + 1, L.total, p, vx, vz, cs, const_cast<T*>(a.pv.in), a.pv.n_in));
-            for (int k = 0; k < K; ++k) {
-                ib_count_launch(kname<T>("stag_v2d_f32", "stag_v2d_f64"));
-                ib_count_launch(kname<T>("stag_p2d_f32", "stag_p2d_f64"));
-            }
-        }
-        IB_CUDA(cudaStreamSynchronize(cs));
-        cudaGraphExecDestroy(exec);
-        cudaGraphDestroy(graph);
-    }
-    for (int k = 0; k < nt - nrep * K; ++k) {     // the remaining steps, offset by the graphs' bumps
-        a.step = k;
-        a.rec_step = k - 1;
-        TRY(launch_step(cs, true));
-        if (probe && (nrep * K + k + 1) % STAB_BLOCK == 0)
-            TRY(probe_rescale<T>(probe, (nrep * K + k + 1) / STAB_BLOCK, L.total, p, vx, vz, cs,
-                                 const_cast<T*>(a.pv.in), a.pv.n_in));
-    }
-    if (g.rec.n) {
-        k_receivers<T><<<grid1(g.rec.n, 256), 256, 0, cs>>>(g.rec, p, (T*)sh->traces_dev, nt, nt - 1);
-        IB_CHECK_LAUNCH("k_receivers");
-        ib_count_launch("setup");
-    }
-    if (!probe) TRY(check_finite<T>(L.total, p, vx, vz, cs));
-    if (nrep) {
-        IB_CUDA(cudaEventRecord(ready, cs));
-        IB_CUDA(cudaStreamWaitEvent(s, ready, 0));
-        IB_CUDA(cudaStreamSynchronize(cs));
-        cudaEventDestroy(ready);
-        cudaStreamDestroy(cs);
-    }
-    return IB_OK;
-}
-
 // ---------------------------------------------------------------------------
 // 3D staggered pressure-velocity (1st-order section: the paper's signs and the
 // backward-staggered base stencil; 3D first-order example):
@@ -3246,6 +2548,366 @@ static ib_status forward_stag3(ib_table* t, const ib_shot* sh, double dt, int nt
     else TRY(run(std::integral_constant<int, 4>()));
     TRY(check_finite<T>(L.total, p, v0, v1, s));
     TRY(check_finite<T>(L.total, v2, (const T*)nullptr, (const T*)nullptr, s));
+    return IB_OK;
+}
+
+// ---------------------------------------------------------------------------
+// 2D staggered pressure-velocity
+//   v_a[j] (at j + e_a/2) += bh_a[j] (sum_k c_k (p[j + k e_a] - p[j - (k-1) e_a]) + IB)
+//   p[j] += kh[j] (sum_a sum_k c_k (v_a[j + (k-1) e_a] - v_a[j - k e_a]) + IB) + src
+// with bh_a = dt / (rho h) and kh = dt rho c^2 / h.  Column and row blocks as in 3D: a thread
+// owns 16 bytes of adjacent nodes of one row, the modified rows are updated whole by 8 lanes
+// each.  The state of a 1001 x 1001 shot stays in the L2 and a kernel is a few microseconds
+// of latency; correction sums formed by the producing tiles in shared memory, which this
+// replaces, took 22 us per step and 7 ms of host plans per shot; 50 steps are now 683 us (749
+// with 16 lanes per divergence row).
+// ---------------------------------------------------------------------------
+template <typename T>
+struct Rows2D {
+    int64_t n;
+    const int64_t* pad;
+    const int64_t* ptr[2];
+    const int32_t* code[2];
+    const T* w[2];
+};
+template <typename T>
+struct Stag2Args {
+    Layout L;
+    T c[4];              // c[k - 1]: weight of the pair at offsets +(k - 1/2), -(k - 1/2)
+    T* p;
+    T* v[2];
+    const T* kp;         // sign bit of kp and b: a node of the modified rows
+    const T* b[2];
+    Rows2D<T> g[2];      // gradient rows of v_x, v_z
+    Rows2D<T> d;         // divergence rows (columns v_x, v_z)
+    int nrb[3];          // row blocks: v_x, v_z; p
+    int nbx;             // column blocks along x
+    PointSet<T> src;     // weights include dt / h^2
+    const T* wavelet;
+    const int* step_base; // device step offset added to step / rec_step (graph replays)
+    int step;
+    PointSet<T> rec;     // receivers, sampled from p before the v update
+    T* traces;
+    int nt;
+    int rec_step;
+};
+
+// lane gl of 8's share of sum_j w_j f[q + off_j] over the entries [j0, j1) of a 2D row
+template <typename T>
+__device__ __forceinline__ T row_gather2(const int32_t* __restrict__ code, const T* __restrict__ w, int64_t j0, int64_t j1,
+                                         const T* f, int64_t q, int64_t px, int gl) {
+    T v = 0;
+    for (int64_t e = j0 + gl; e < j1; e += 8) {
+        int dx, dz, dy;
+        unpack_off(code[e], dx, dz, dy);   // 2D codes: (x, z, 0)
+        v += w[e] * f[q + dz * px + dx];
+    }
+    return v;
+}
+
+// v^{n+1/2} = v^{n-1/2} + (dt / rho) G_mod p^n
+template <typename T, int H>
+__global__ void __launch_bounds__(256) k_stag_v2d(const __grid_constant__ Stag2Args<T> a) {
+    constexpr int VX = 16 / (int)sizeof(T), HV = (H + VX - 1) / VX, HX = HV * VX;
+    const Layout& L = a.L;
+    int64_t blk = blockIdx.x;
+    const int rs = a.rec_step + (a.step_base ? *a.step_base : 0);
+    record_receivers(a.rec, (const T*)a.p, a.traces, a.nt, rs, blk * 256 + threadIdx.x, (int64_t)gridDim.x * 256);
+#pragma unroll
+    for (int ax = 0; ax < 2; ++ax) {
+        if (blk < a.nrb[ax]) {
+            const Rows2D<T>& R = a.g[ax];
+            const int gl = threadIdx.x & 7;
+            const int64_t r = blk * S3_ROWS + (threadIdx.x >> 3), st = ax ? L.px : 1;
+            const bool act = r < R.n;
+            const int64_t q = act ? R.pad[r] : L.base;
+            const T bq = gl == 0 ? a.b[ax][q] : (T)0, vq = gl == 0 ? a.v[ax][q] : (T)0;
+            T s = 0;
+            if (act) s = row_gather2(R.code[0], R.w[0], R.ptr[0][r], R.ptr[0][r + 1], (const T*)a.p, q, L.px, gl);
+#pragma unroll
+            for (int k = 1; k <= H; ++k)
+                if (gl == k) s += a.c[k - 1] * (a.p[q + k * st] - a.p[q - (k - 1) * st]);
+            s = sum8(s);
+            if (act && gl == 0) a.v[ax][q] = vq + (bq < (T)0 ? -bq : bq) * s;
+            return;
+        }
+        blk -= a.nrb[ax];
+    }
+    const int lane = threadIdx.x & 31, wz = threadIdx.x >> 5;
+    const int64_t x = ((blk % a.nbx) * 32 + lane) * VX, z = blk / a.nbx * 8 + wz;
+    if (x >= L.nx || z >= L.nz) return;
+    const int64_t q = L.base + z * L.px + x;
+    T w[VX + 2 * HX], z2[2 * H][VX], vv[2][VX], bb[2][VX];
+#pragma unroll
+    for (int m = 0; m < 2 * HV + 1; ++m) load3<T, VX>(*reinterpret_cast<T(*)[VX]>(&w[m * VX]), a.p + q + (m - HV) * VX);
+#pragma unroll
+    for (int k = 0; k < 2 * H; ++k)   // offsets 1 - H .. H
+        if (k != H - 1) load3<T, VX>(z2[k], a.p + q + (k + 1 - H) * L.px);
+#pragma unroll
+    for (int ax = 0; ax < 2; ++ax) {
+        load3<T, VX>(vv[ax], a.v[ax] + q);
+        load3<T, VX>(bb[ax], a.b[ax] + q);
+    }
+#pragma unroll
+    for (int j = 0; j < VX; ++j) {
+        T sx = 0, sz = 0;
+#pragma unroll
+        for (int k = 1; k <= H; ++k) {
+            sx += a.c[k - 1] * (w[HX + j + k] - w[HX + j - k + 1]);
+            sz += a.c[k - 1] * (z2[H - 1 + k][j] - (k == 1 ? w[HX + j] : z2[H - k][j]));
+        }
+        vv[0][j] += bb[0][j] * sx;
+        vv[1][j] += bb[1][j] * sz;
+    }
+#pragma unroll
+    for (int ax = 0; ax < 2; ++ax) store3<T, VX>(a.v[ax] + q, vv[ax], bb[ax], x, L.nx);
+}
+
+// p^{n+1} = p^n + dt rho c^2 D_mod v^{n+1/2} (+ source)
+template <typename T, int H>
+__global__ void __launch_bounds__(256) k_stag_p2d(const __grid_constant__ Stag2Args<T> a) {
+    constexpr int VX = 16 / (int)sizeof(T), HV = (H + VX - 1) / VX, HX = HV * VX;
+    const Layout& L = a.L;
+    int64_t blk = blockIdx.x;
+    const int n = a.step + (a.step_base ? *a.step_base : 0);
+    if (blk < a.nrb[2]) {
+        const int gl = threadIdx.x & 7;
+        const int64_t r = blk * S3_ROWS + (threadIdx.x >> 3);
+        const bool act = r < a.d.n;
+        const int64_t q = act ? a.d.pad[r] : L.base;
+        const T kq = gl == 0 ? a.kp[q] : (T)0, pq = gl == 0 ? a.p[q] : (T)0;
+        T s = 0, sv = 0;
+#pragma unroll
+        for (int ax = 0; ax < 2; ++ax) {
+            const int64_t st = ax ? L.px : 1;
+            if (act)
+                s += row_gather2(a.d.code[ax], a.d.w[ax], a.d.ptr[ax][r], a.d.ptr[ax][r + 1], (const T*)a.v[ax], q, L.px, gl);
+#pragma unroll
+            for (int k = 1; k <= H; ++k)
+                if (gl == ax * H + k - 1) s += a.c[k - 1] * (a.v[ax][q + (k - 1) * st] - a.v[ax][q - k * st]);
+        }
+        for (int i = gl; i < 8 * a.src.n; i += 8)
+            if (a.src.idx[i] == q) sv += a.src.w[i];
+        s = sum8(s);
+        sv = sum8(sv);
+        if (act && gl == 0) a.p[q] = pq + (kq < (T)0 ? -kq : kq) * s + (a.src.n ? sv * a.wavelet[n] : (T)0);
+        return;
+    }
+    blk -= a.nrb[2];
+    const int lane = threadIdx.x & 31, wz = threadIdx.x >> 5;
+    const int64_t bx = blk % a.nbx, bz = blk / a.nbx, x = (bx * 32 + lane) * VX, z = bz * 8 + wz;
+    const bool in = x < L.nx && z < L.nz;
+    const int64_t q = L.base + z * L.px + x;
+    T w[VX + 2 * HX], z2[2 * H][VX], pp[VX], kk[VX];
+    if (in) {
+#pragma unroll
+        for (int m = 0; m < 2 * HV + 1; ++m) load3<T, VX>(*reinterpret_cast<T(*)[VX]>(&w[m * VX]), a.v[0] + q + (m - HV) * VX);
+#pragma unroll
+        for (int k = 0; k < 2 * H; ++k) load3<T, VX>(z2[k], a.v[1] + q + (k - H) * L.px);   // offsets -H .. H - 1
+        load3<T, VX>(pp, a.p + q);
+        load3<T, VX>(kk, a.kp + q);
+    }
+    // does a source corner fall in this block's box? (block-uniform)
+    int here = 0;
+    if (a.src.n) {
+        for (int i = threadIdx.x; i < 8 * a.src.n; i += 256) {
+            if (a.src.w[i] == (T)0) continue;
+            const int64_t rel = a.src.idx[i] - L.base, sz = rel / L.px, sx = rel - sz * L.px;
+            here |= sz / 8 == bz && sx / (32 * VX) == bx;
+        }
+        here = __syncthreads_or(here);
+    }
+    if (!in) return;
+#pragma unroll
+    for (int j = 0; j < VX; ++j) {
+        T s = 0;
+#pragma unroll
+        for (int k = 1; k <= H; ++k) {
+            s += a.c[k - 1] * (w[HX + j + k - 1] - w[HX + j - k]);
+            s += a.c[k - 1] * (z2[H + k - 1][j] - z2[H - k][j]);
+        }
+        pp[j] += kk[j] * s;
+        if (here) {
+            T sv = 0;
+            for (int i = 0; i < 8 * a.src.n; ++i)
+                if (a.src.idx[i] == q + j) sv += a.src.w[i];
+            pp[j] += sv * a.wavelet[n];
+        }
+    }
+    store3<T, VX>(a.p + q, pp, kk, x, L.nx);
+}
+
+__global__ void k_add_step(int* base, int k) {
+    if (threadIdx.x == 0 && blockIdx.x == 0) *base += k;
+}
+
+// time steps per captured graph of the staggered loop (the graph is replayed nt / STAG_GRAPH_STEPS times)
+static const int STAG_GRAPH_STEPS = 50;
+static_assert(STAG_GRAPH_STEPS == STAB_BLOCK, "the stability probe renormalises between graph replays");
+
+template <typename T>
+static ib_status forward_stag(ib_table* t, const ib_shot* sh, double dt, int nt, cudaStream_t s,
+                              const Probe* probe = nullptr) {
+    const Layout& L = t->L;
+    const int d = t->grid.ndim;
+    if (shot_damped(sh)) {
+        ib_set_error("the absorbing layer is implemented for the second-order form");
+        return IB_ERR_STATE;
+    }
+    if (d != 2) {
+        ib_set_error("the staggered form is implemented in 2D");
+        return IB_ERR_STATE;
+    }
+    const int M = t->opts.space_order;
+    const int H = M / 2;
+    Scratch S(s);
+    T *p, *vx, *vz, *kp, *bx, *bz;
+    TRY(S.alloc(&p, L.total, true));
+    TRY(S.alloc(&vx, L.total, true));
+    TRY(S.alloc(&vz, L.total, true));
+    TRY(S.alloc(&kp, L.total, true));
+    TRY(S.alloc(&bx, L.total, true));
+    TRY(S.alloc(&bz, L.total, true));
+    k_stag_coef<T><<<grid1(L.N, 256), 256, 0, s>>>(L, (const T*)sh->vel_dev, (const T*)sh->rho_dev, t->mask_pad[0],
+                                                   t->mask_pad[1], t->mask_pad[2], dt, 1.0 / t->grid.h, kp, bx, bz);
+    IB_CHECK_LAUNCH("k_stag_coef");
+    ib_count_launch("setup");
+    if (probe) {   // random p, v_x, v_z on their interior nodes, normalised together
+        k_rand_fill<T><<<grid1(L.total, 256), 256, 0, s>>>(L.total, kp, probe->seed, p, (T*)nullptr);
+        k_rand_fill<T><<<grid1(L.total, 256), 256, 0, s>>>(L.total, bx, probe->seed + 1, vx, (T*)nullptr);
+        k_rand_fill<T><<<grid1(L.total, 256), 256, 0, s>>>(L.total, bz, probe->seed + 2, vz, (T*)nullptr);
+        IB_CHECK_LAUNCH("k_rand_fill");
+        TRY(probe_rescale<T>(probe, 0, L.total, p, vx, vz, s));
+    }
+    Geom<T> g;
+    TRY(setup_points<T>(t, sh, dt / pow(t->grid.h, d), S, g));
+    Stag2Args<T> a;
+    memset(&a, 0, sizeof a);
+    a.L = L;
+    {
+        T w2u[5];
+        stencil_weights<T>(M, w2u, a.c);
+    }
+    a.p = p;
+    a.v[0] = vx;
+    a.v[1] = vz;
+    a.b[0] = bx;
+    a.b[1] = bz;
+    a.kp = kp;
+    // operators 0, 1: gradients; 2, 3: the divergence's parts, on one set of rows
+    T* coef[3] = {bx, bz, kp};
+    for (int o = 0; o < 4; ++o) {
+        const IbOp& op = t->ops[o];
+        Rows2D<T>& R = o < 2 ? a.g[o] : a.d;
+        const int i = o < 2 ? 0 : o - 2;
+        R.n = op.nrows;
+        R.pad = op.row_pad;
+        R.ptr[i] = op.row_ptr;
+        R.code[i] = op.col_code;
+        R.w[i] = sizeof(T) == 8 ? (const T*)op.w64 : (const T*)op.w32;
+        if (o < 3 && op.nrows) {
+            k_mark_rows3<T><<<grid1(op.nrows, 256), 256, 0, s>>>(op.nrows, op.row_pad, coef[o]);
+            IB_CHECK_LAUNCH("k_mark_rows3");
+            ib_count_launch("setup");
+        }
+        if (o < 3) a.nrb[o] = (int)((op.nrows + S3_ROWS - 1) / S3_ROWS);
+    }
+    constexpr int VX = 16 / (int)sizeof(T);
+    a.nbx = (int)((L.nx + 32 * VX - 1) / (32 * VX));
+    a.src = g.src;
+    a.wavelet = (const T*)sh->wavelet_dev;
+    a.rec = g.rec;
+    a.traces = (T*)sh->traces_dev;
+    a.nt = nt;
+    const int64_t cols = (int64_t)a.nbx * ((L.nz + 7) / 8);
+    const unsigned gv = (unsigned)(cols + a.nrb[0] + a.nrb[1]), gp = (unsigned)(cols + a.nrb[2]);
+    auto launch_step = [&](cudaStream_t st, bool prof) -> ib_status {
+        auto v = [&]() {
+            if (H == 1) k_stag_v2d<T, 1><<<gv, 256, 0, st>>>(a);
+            else if (H == 2) k_stag_v2d<T, 2><<<gv, 256, 0, st>>>(a);
+            else if (H == 3) k_stag_v2d<T, 3><<<gv, 256, 0, st>>>(a);
+            else k_stag_v2d<T, 4><<<gv, 256, 0, st>>>(a);
+        };
+        auto pk = [&]() {
+            if (H == 1) k_stag_p2d<T, 1><<<gp, 256, 0, st>>>(a);
+            else if (H == 2) k_stag_p2d<T, 2><<<gp, 256, 0, st>>>(a);
+            else if (H == 3) k_stag_p2d<T, 3><<<gp, 256, 0, st>>>(a);
+            else k_stag_p2d<T, 4><<<gp, 256, 0, st>>>(a);
+        };
+        if (prof) {
+            PROF_LAUNCH(kname<T>("stag_v2d_f32", "stag_v2d_f64"), st, { v(); });
+            PROF_LAUNCH(kname<T>("stag_p2d_f32", "stag_p2d_f64"), st, { pk(); });
+        } else {
+            v();
+            pk();
+            ib_count_launch(kname<T>("stag_v2d_f32", "stag_v2d_f64"));
+            ib_count_launch(kname<T>("stag_p2d_f32", "stag_p2d_f64"));
+        }
+        IB_CHECK_LAUNCH("staggered step");
+        return IB_OK;
+    };
+    int* d_base;
+    TRY(S.alloc(&d_base, 1, true));
+    a.step_base = d_base;
+    const int K = STAG_GRAPH_STEPS;
+    const int nrep = (nt >= 2 * K && !getenv("IB_NO_GRAPH")) ? nt / K : 0;
+    cudaStream_t cs = s;
+    cudaEvent_t ready = nullptr;
+    if (nrep) {
+        // K steps (and the step-offset bump) as one graph, replayed nrep times on a side stream
+        IB_CUDA(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
+        IB_CUDA(cudaEventCreateWithFlags(&ready, cudaEventDisableTiming));
+        IB_CUDA(cudaEventRecord(ready, s));
+        IB_CUDA(cudaStreamWaitEvent(cs, ready, 0));
+        cudaGraph_t graph = nullptr;
+        cudaGraphExec_t exec = nullptr;
+        IB_CUDA(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
+        ib_status st = IB_OK;
+        for (int k = 0; k < K && st == IB_OK; ++k) {
+            a.step = k;
+            a.rec_step = k - 1;
+            st = launch_step(cs, false);
+        }
+        k_add_step<<<1, 32, 0, cs>>>(d_base, K);
+        cudaError_t ce = cudaStreamEndCapture(cs, &graph);
+        if (st != IB_OK) return st;
+        if (ce != cudaSuccess) return ib_cuda_fail(ce, "graph capture", __FILE__, __LINE__);
+        IB_CUDA(cudaGraphInstantiate(&exec, graph, 0));
+        for (int r = 0; r < nrep; ++r) {
+            ProfToken tk = ib_prof_begin(kname<T>("stag_graph50_f32", "stag_graph50_f64"), cs);
+            IB_CUDA(cudaGraphLaunch(exec, cs));
+            ib_prof_end(tk, cs);
+            if (probe)
+                TRY(probe_rescale<T>(probe, r + 1, L.total, p, vx, vz, cs));
+            for (int k = 0; k < K; ++k) {
+                ib_count_launch(kname<T>("stag_v2d_f32", "stag_v2d_f64"));
+                ib_count_launch(kname<T>("stag_p2d_f32", "stag_p2d_f64"));
+            }
+        }
+        IB_CUDA(cudaStreamSynchronize(cs));
+        cudaGraphExecDestroy(exec);
+        cudaGraphDestroy(graph);
+    }
+    for (int k = 0; k < nt - nrep * K; ++k) {     // the remaining steps, offset by the graphs' bumps
+        a.step = k;
+        a.rec_step = k - 1;
+        TRY(launch_step(cs, true));
+        if (probe && (nrep * K + k + 1) % STAB_BLOCK == 0)
+            TRY(probe_rescale<T>(probe, (nrep * K + k + 1) / STAB_BLOCK, L.total, p, vx, vz, cs));
+    }
+    if (g.rec.n) {
+        k_receivers<T><<<grid1(g.rec.n, 256), 256, 0, cs>>>(g.rec, p, (T*)sh->traces_dev, nt, nt - 1);
+        IB_CHECK_LAUNCH("k_receivers");
+        ib_count_launch("setup");
+    }
+    if (!probe) TRY(check_finite<T>(L.total, p, vx, vz, cs));
+    if (nrep) {
+        IB_CUDA(cudaEventRecord(ready, cs));
+        IB_CUDA(cudaStreamWaitEvent(s, ready, 0));
+        IB_CUDA(cudaStreamSynchronize(cs));
+        cudaEventDestroy(ready);
+        cudaStreamDestroy(cs);
+    }
     return IB_OK;
 }
 

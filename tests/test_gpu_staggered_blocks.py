@@ -35,3 +35,18 @@ def test_staggered3d_blocks(nx, ny, nz, M):
                  np.full(sdf.shape, 1000.0))
     assert np.abs(a[:, -1]).max() > 0
     assert rel_l2(b, a) < TOL32
+
+
+@pytest.mark.parametrize("nx,nz,M", [(127, 65, 8), (129, 64, 8), (133, 71, 2), (260, 73, 6)])
+def test_staggered2d_blocks(nx, nz, M):
+    h, nt = 5.0, 60
+    sdf = inputs.flat_surface_sdf((nx, nz), h, 10.3 * h)
+    dt = 0.4 * h / 1500.0
+    # off the grid, over the corner of a block of 128 x 8 (FP32) or 64 x 8 (FP64) nodes
+    src = np.array([[min(127.5, nx - 9.5) * h, 31.5 * h]])
+    rec = np.array([[x * h, z * h] for x in range(3, nx - 3, 4) for z in (12, nz - 6)])
+    t = ib.ib_build_stencils(cuda(sdf), h, "free", "staggered", M)
+    a, b = _both(t, np.full(sdf.shape, 1500.0), inputs.ricker(100.0, dt, nt, t0=0.0), src, rec, dt, nt,
+                 np.full(sdf.shape, 1000.0))
+    assert np.abs(a[:, -1]).max() > 0
+    assert rel_l2(b, a) < TOL32
