@@ -487,7 +487,13 @@ def run_single(args, workload, steps, warmup, world, rank, local, dev, dist, wit
     value = job_value(world, upd_per_step, ms)
     launches = sum(d["launches"] for d in prof.values())
     peak, peak_kind = peaks()
-    roof = roofline_of(prof, kernel_bytes(w, stats, eb), peak, peak_kind)
+    kb = kernel_bytes(w, stats, eb)
+    if w["form"] != "staggered" and len(w["shape"]) == 2:
+        # small grids: all the steps of a shot in one launch
+        for e in ("f32", "f64"):
+            if "leap2d_" + e in kb:
+                kb["leap2d_run_" + e] = w["nt"] * kb["leap2d_" + e]
+    roof = roofline_of(prof, kb, peak, peak_kind)
     roof_step = step_roofline(prof, w, stats, peak, peak_kind) if len(w["shape"]) == 3 else None
     # ---- end to end through the C ABI with host buffers
     e2e = None
