@@ -8,13 +8,12 @@
 // the boundary ("Reconciliation with the Interior Numerical Discretization"),
 // zero Dirichlet outer edges (Examples section).
 //
-// Every step kernel owns a tile of outputs.  The bulk stencil reads a
-// shared-memory copy of the tile and its halo.  The immersed-boundary
-// corrections of the tile's rows are stored flattened per tile (output slot,
-// source offset, weight) and are added by all threads of the block with
-// shared-memory atomics -- a balanced, coalesced gather whatever the number of
-// IB rows in the tile.  The update, source injection and masking follow, and
-// the tile is written once.
+// 2D and staggered steps: column blocks for the bulk and row blocks that update the
+// immersed-boundary rows whole, in one launch (ib_leap2d.cuh, and below).  3D
+// second order: tiles marched along z, in FP32 through a TMA ring with the
+// corrections in a pass of their own, in FP64 with the tile's corrections stored
+// flattened (output slot, source offset, weight) and added by all threads of the
+// block with shared-memory atomics.
 //
 // Arithmetic: coefficients (dt^2 c^2 / h^2, dt rho c^2 / h, dt / (rho h)) are
 // formed in FP64 and rounded once; the leapfrog update is evaluated as
