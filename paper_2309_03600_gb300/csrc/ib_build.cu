@@ -1764,9 +1764,9 @@ static ib_status pack_pool(ib_table* t, const FitKind& fk, const int64_t* rows, 
         int64_t nnz = 0;
         IB_CUDA(cudaMemcpy(&nnz, op.row_ptr + nrows, sizeof(int64_t), cudaMemcpyDeviceToHost));
         op.nnz = nnz;
-        TRY(dalloc(&op.col_code, nnz));
+        TRY(dalloc(&op.col_code, nnz + 1));   // read in pairs: the last pair may end past nnz
         TRY(dalloc(&op.col_pad, nnz));
-        TRY(dalloc(&op.w64, nnz + 1));   // read in pairs: the last pair may end past nnz
+        TRY(dalloc(&op.w64, nnz + 1));
         TRY(dalloc(&op.w32, nnz + 1));
         TRY(dalloc(&op.row_lin, nrows));
         TRY(dalloc(&op.row_pad, nrows));

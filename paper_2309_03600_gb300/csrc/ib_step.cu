@@ -2188,38 +2188,38 @@ __global__ void k_stag_coef3(Layout L, const T* vel, const T* rho, const uint8_t
 }
 
 // Lane gl of 8's share of sum_j w_j f[q + off_j] over the entries [j0, j1) of a 3D row: pairs
-// of adjacent entries (their codes as one 4-byte and their weights as one vector load; a pair
-// that straddles the row's ends has the foreign weight dropped), U pairs in flight.  The
-// 16-bit footprint code is decoded mostly in 32-bit arithmetic against a base moved by the code's
-// offset of 16 nodes per axis, so an entry costs about 10 instructions where 64-bit decoding took over 20.
+// of adjacent entries (their codes and weights as one vector load each; a pair that straddles
+// the row's ends has the foreign weight dropped), U pairs in flight.
 template <typename T>
 struct PairOf;
 template <> struct PairOf<float> { typedef float2 type; };
 template <> struct PairOf<double> { typedef double2 type; };
 template <typename T, int U>
-__device__ __forceinline__ T row_gather3(const uint16_t* __restrict__ code, const T* __restrict__ w, int64_t j0, int64_t j1,
+__device__ __forceinline__ T row_gather3(const int32_t* __restrict__ code, const T* __restrict__ w, int64_t j0, int64_t j1,
                                          const T* __restrict__ f, int64_t q, int px, int plane, int gl) {
     typedef typename PairOf<T>::type V;
-    const T* base = f + (q - 16 * ((int64_t)plane + px + 1));
-    const int64_t centre = 16 * ((int64_t)plane + px + 1);
+    const T* base = f + q;
+    auto off = [&](int c) {   // unpack_off's bytes
+        return (int64_t)(int)(int8_t)(c >> 16) * plane + ((int)(int8_t)c + (int)(int8_t)(c >> 8) * px);
+    };
     T v = 0;
     for (int64_t j = (j0 & ~(int64_t)1) + 2 * gl; j < j1; j += 16 * U) {
         T w0[U], w1[U], p0[U], p1[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             const int64_t e = j + 16 * u;
-            int64_t o0 = centre, o1 = centre;
+            int64_t o0 = 0, o1 = 0;
             w0[u] = w1[u] = (T)0;
             if (e < j1) {
-                const uint32_t c = *reinterpret_cast<const uint32_t*>(code + e);
+                const int2 c = *reinterpret_cast<const int2*>(code + e);
                 const V ww = *reinterpret_cast<const V*>(w + e);
                 if (e >= j0) {
                     w0[u] = ww.x;
-                    o0 = (int64_t)(int)((c >> 10) & 63) * plane + ((int)(c & 31) + (int)((c >> 5) & 31) * px);
+                    o0 = off(c.x);
                 }
                 if (e + 1 < j1) {
                     w1[u] = ww.y;
-                    o1 = (int64_t)(int)(c >> 26) * plane + ((int)((c >> 16) & 31) + (int)((c >> 21) & 31) * px);
+                    o1 = off(c.y);
                 }
             }
             p0[u] = base[o0];
@@ -2247,7 +2247,7 @@ struct Rows3D {
     int64_t n;
     const int64_t* pad;
     const int64_t* ptr[3];
-    const uint16_t* code[3];
+    const int32_t* code[3];
     const T* w[3];
 };
 
@@ -2510,7 +2510,7 @@ static ib_status forward_stag3(ib_table* t, const ib_shot* sh, double dt, int nt
             R.pad = op.row_pad;
             R.ptr[i] = op.row_ptr;
             R.w[i] = sizeof(T) == 8 ? (const T*)op.w64 : (const T*)op.w32;
-            TRY(ib_table_code16(t, o, &R.code[i], s));
+            R.code[i] = op.col_code;
             if (o < 4 && op.nrows) {
                 k_mark_rows3<T><<<grid1(op.nrows, 256), 256, 0, s>>>(op.nrows, op.row_pad, coef[o]);
                 IB_CHECK_LAUNCH("k_mark_rows3");
