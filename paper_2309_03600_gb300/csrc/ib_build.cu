@@ -2491,6 +2491,41 @@ extern "C" void ib_table_free(ib_table* t) {
     delete t;
 }
 
+// 16-bit footprint codes of a 3D Laplacian's entries in row order, for the FP32 step's
+// correction pass.  Part of the construction: a table's first runs may come from several
+// streams, none of which may find half-filled codes.  A support that reaches beyond what a code
+// can name (16 nodes to one side of an axis, 15 to the other) leaves the table without them,
+// and its runs take the step that reads 32-bit offsets.
+__global__ void k_code16(int64_t nnz, const int32_t* col_code, uint16_t* out, int* wide) {
+    for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < nnz; j += (int64_t)gridDim.x * blockDim.x) {
+        int dx, dy, dz;
+        unpack_off(col_code[j], dx, dy, dz);
+        if (max(max(dx, dy), dz) > 15 || min(min(dx, dy), dz) < -16) *wide = 1;
+        out[j] = pack_code16(dx, dy, dz);
+    }
+}
+static ib_status build_code16(ib_table* t, cudaStream_t s, DevBuf& tmp) {
+    IbOp& o = t->ops[0];
+    if (o.nnz == 0) return IB_OK;
+    int* wide;
+    int hwide = 0;
+    TRY(tmp.alloc(&wide, 1));
+    TRY(dalloc(&o.code16, o.nnz));
+    IB_CUDA(cudaMemsetAsync(wide, 0, sizeof(int), s));
+    k_code16<<<grid_for(o.nnz, 256), 256, 0, s>>>(o.nnz, o.col_code, o.code16, wide);
+    IB_CHECK_LAUNCH("k_code16");
+    ib_count_launch("setup");
+    IB_CUDA(cudaMemcpyAsync(&hwide, wide, sizeof(int), cudaMemcpyDeviceToHost, s));
+    IB_CUDA(cudaStreamSynchronize(s));
+    if (hwide) {
+        cudaFree(o.code16);
+        o.code16 = nullptr;
+    } else {
+        t->table_bytes += 2 * o.nnz;
+    }
+    return IB_OK;
+}
+
 static ib_status build_impl(const ib_grid* grid, const double* sdf, ib_bc bc, ib_form form, const ib_opts* opts_in,
                             ib_mlp* mlp, double accept_tol, ib_table** out, cudaStream_t s) {
     double t0 = ib_wall_seconds();
@@ -2637,6 +2672,7 @@ static ib_status build_impl(const ib_grid* grid, const double* sdf, ib_bc bc, ib
             st = run_fit1d(t, g, fk, M, w2, s, tmp);
         else
             st = run_fit(t, g, fk, bp_index, bp_xb, bp_n, bplist, nbp, 0, s, tmp);
+        if (st == IB_OK && d == 3) st = build_code16(t, s, tmp);
         if (st != IB_OK) return fail(st);
     } else {
         std::vector<double> c1 = ib_staggered_first(M);
@@ -2963,27 +2999,6 @@ static ib_status make_bins(const Layout& L, int64_t n, const int64_t* pad, const
         IB_CUDA(cudaMemsetAsync(b.ent_ptr, 0, sizeof(int32_t) * (b.ntiles + 1), s));
     }
     IB_CUDA(cudaStreamSynchronize(s));
-    return IB_OK;
-}
-
-__global__ void k_code16(int64_t nnz, const int32_t* col_code, uint16_t* out) {
-    for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < nnz; j += (int64_t)gridDim.x * blockDim.x) {
-        int dx, dy, dz;
-        unpack_off(col_code[j], dx, dy, dz);
-        out[j] = pack_code16(dx, dy, dz);
-    }
-}
-
-// 16-bit footprint codes of an operator's entries in row order (kept with the table)
-ib_status ib_table_code16(ib_table* t, int op, const uint16_t** out, cudaStream_t s) {
-    IbOp& o = t->ops[op];
-    if (!o.code16 && o.nnz > 0) {
-        TRY(dalloc(&o.code16, o.nnz + 1));   // read in pairs
-        k_code16<<<grid_for(o.nnz, 256), 256, 0, s>>>(o.nnz, o.col_code, o.code16);
-        IB_CHECK_LAUNCH("k_code16");
-        ib_count_launch("setup");
-    }
-    *out = o.code16;
     return IB_OK;
 }
 

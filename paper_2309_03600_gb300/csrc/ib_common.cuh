@@ -124,7 +124,7 @@ struct IbOp {
     double* w64 = nullptr;
     float* w32 = nullptr;
     int32_t* row_info = nullptr;  // [nrows][4]
-    uint16_t* code16 = nullptr;   // [nnz] pack_code16 footprint codes (built on first use)
+    uint16_t* code16 = nullptr;   // [nnz] pack_code16 footprint codes (3D Laplacian, where they fit)
     std::vector<TileBins> bins;
     // transposed operator (adjoint): rows keyed by column node
     bool have_t = false;
@@ -170,7 +170,6 @@ ib_status ib_compact(const uint8_t* flags, int64_t n, int64_t** out, int64_t* co
 ib_status ib_table_bins(ib_table* t, int op, bool transposed, int tx, int ty, int tz,
                         const TileBins** out, cudaStream_t s);
 ib_status ib_table_transpose(ib_table* t, int op, cudaStream_t s);
-ib_status ib_table_code16(ib_table* t, int op, const uint16_t** out, cudaStream_t s);
 
 double ib_wall_seconds();
 

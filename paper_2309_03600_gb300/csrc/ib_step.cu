@@ -1979,8 +1979,10 @@ static ib_status forward_2nd(ib_table* t, const ib_shot* sh, double dt, int nt, 
             TRY(S.alloc(&tb_o2, L.total, true));
         }
     }
+    // FP32 3D: TMA, where the table's entries have 16-bit codes
+    const bool use_tma = d == 3 && sizeof(T) == 4 && tma_enabled() && (t->ops[0].nnz == 0 || t->ops[0].code16);
     // planes per 3D block (IB_ZCHUNK overrides it for tuning)
-    int zchunk = d == 3 && sizeof(T) == 4 && tma_enabled() ? z_planes(L) : 32;
+    int zchunk = use_tma ? z_planes(L) : 32;
     if (const char* e = getenv("IB_ZCHUNK")) zchunk = std::max(1, atoi(e));
     dim3 grid3((unsigned)((L.nx + 31) / 32), (unsigned)((L.ny + 7) / 8), (unsigned)((L.nz + zchunk - 1) / zchunk));
     const int64_t nty3 = (L.ny + 7) / 8;
@@ -1991,7 +1993,6 @@ static ib_status forward_2nd(ib_table* t, const ib_shot* sh, double dt, int nt, 
     memset(&rows3, 0, sizeof rows3);
     const uint16_t* code16 = nullptr;
     int* err = nullptr;
-    const bool use_tma = d == 3 && sizeof(T) == 4 && tma_enabled();
     // x-pair kernel (64 x 8 tiles; IB_TMA3_PAIRS=0 selects the 32 x 8 kernel)
     bool pairs = false;
     // correction pass: entries in flight per lane, 4 (IB_ADD3_U=8 selects 8: at
@@ -2017,8 +2018,8 @@ static ib_status forward_2nd(ib_table* t, const ib_shot* sh, double dt, int nt, 
                 rows3.code = bins->ent_code;
                 rows3.w = bins->ent_w32;
             }
-        } else if (t->ops[0].nrows > 0) {
-            TRY(ib_table_code16(t, 0, &code16, s));
+        } else {
+            code16 = t->ops[0].code16;
         }
     }
     int n0 = 0;

@@ -4,7 +4,7 @@ import numpy as np
 import pytest
 import torch
 
-from oracle import operators, propagate, stencils
+from oracle import operators, propagate, sim, stencils
 from paper_2309_03600_gb300 import inputs
 from gpu_util import cuda, gpu_rows, rel_l2, small_hills
 
@@ -49,7 +49,7 @@ def test_first_staggered_run_in_a_capture():
     assert float(ref.abs().max()) > 0 and torch.equal(out, ref)
 
 
-@pytest.mark.parametrize("form", ["staggered"])
+@pytest.mark.parametrize("form", ["staggered", "second"])
 def test_first_runs_on_two_streams(form):
     """The first two shots on a table, enqueued one after the other on two streams."""
     t, args, rho = _hills(form)
@@ -96,5 +96,22 @@ def test_wide_supports_staggered():
     assert np.abs(ref[:, -1]).max() > 0
     for prec, tol in ((torch.float64, TOL64), (torch.float32, TOL32)):
         tr = ib.ib_forward(t, cuda(1800.0 * one, prec), cuda(wv, prec), cuda(src), cuda(rec), dt, 40, rho=cuda(1000.0 * one, prec))
+        assert rel_l2(tr.double().cpu().numpy(), ref) < tol, prec
+    ib.ib_sync_status()
+
+
+def test_wide_supports_second_order():
+    t, rows, sdf, h, M, dt, src, rec, wv = _wide("second")
+    s = object.__new__(sim.Leapfrog)
+    geom = stencils.Geometry(sdf, h, M)
+    s.L, _ = operators.laplacian_matrix(geom, "free", stencils.Opts(M), ib_rows=rows[0])
+    vel = np.full(sdf.shape, 1800.0)
+    s.K = propagate.leapfrog_coefficient(vel, dt, geom.mask)
+    s.S = propagate.multilinear_matrix(src, h, sdf.shape, geom.mask).toarray().sum(0) * dt * dt / h ** 3
+    s.R, s.a = propagate.multilinear_matrix(rec, h, sdf.shape, geom.mask), None
+    ref = s.forward(wv, 40)
+    assert np.abs(ref[:, -1]).max() > 0
+    for prec, tol in ((torch.float64, TOL64), (torch.float32, TOL32)):
+        tr = ib.ib_forward(t, cuda(vel, prec), cuda(wv, prec), cuda(src), cuda(rec), dt, 40)
         assert rel_l2(tr.double().cpu().numpy(), ref) < tol, prec
     ib.ib_sync_status()
