@@ -1788,14 +1788,28 @@ static ib_status pack_pool(ib_table* t, const FitKind& fk, const int64_t* rows, 
     return IB_OK;
 }
 
-template <class T>
-static ib_status upload(DevBuf& tmp, const std::vector<T>& v, const T** out) {
-    T* d;
-    TRY(tmp.alloc(&d, (int64_t)v.size()));
-    if (!v.empty()) IB_CUDA(cudaMemcpy(d, v.data(), sizeof(T) * v.size(), cudaMemcpyHostToDevice));
-    *out = d;
-    return IB_OK;
-}
+// The host tables of a construction, laid out in one buffer and sent in one copy on the stream of
+// the kernels that read them (copies of their own on the legacy stream were not ordered before
+// a non-blocking stream's kernels, and some 30 allocations, copies and frees per operator took
+// longer than the fits of a small 2D table).
+struct HostTables {
+    std::vector<unsigned char> bytes;
+    std::vector<std::pair<const void**, size_t>> slots;   // pointers to set, and their tables' offsets
+    template <class T>
+    void add(const std::vector<T>& v, const T** out) {
+        bytes.resize((bytes.size() + 15) & ~(size_t)15);
+        slots.push_back({reinterpret_cast<const void**>(out), bytes.size()});
+        const unsigned char* p = reinterpret_cast<const unsigned char*>(v.data());
+        bytes.insert(bytes.end(), p, p + sizeof(T) * v.size());
+    }
+    ib_status send(DevBuf& tmp, cudaStream_t s) {
+        unsigned char* d;
+        TRY(tmp.alloc(&d, (int64_t)bytes.size()));
+        IB_CUDA(cudaMemcpyAsync(d, bytes.data(), bytes.size(), cudaMemcpyHostToDevice, s));
+        for (auto& e : slots) *e.first = d + e.second;
+        return IB_OK;
+    }
+};
 
 // Tables of k_fit_rows for the orders of P (same indices, balls and stencil).  *ok stays
 // false where a fit does not suit it: a basis order above 4 (its moments would outgrow the
@@ -1804,7 +1818,7 @@ static ib_status upload(DevBuf& tmp, const std::vector<T>& v, const T** out) {
 static ib_status row_fit_tables(ib_table* t, const Geo& g, const FitKind& fk, const FitParams& P,
                                 const std::vector<int>& orders, const std::vector<int8_t>* off,
                                 const std::vector<int32_t>* ball_q, const int64_t* bp_owner, int64_t nbp, RowFit& R,
-                                cudaStream_t s, DevBuf& tmp, bool* ok) {
+                                HostTables& host, cudaStream_t s, DevBuf& tmp, bool* ok) {
     const int d = g.ndim;
     *ok = false;
     memset(&R, 0, sizeof R);
@@ -1877,10 +1891,10 @@ static ib_status row_fit_tables(ib_table* t, const Geo& g, const FitKind& fk, co
             phiT.insert(phiT.end(), pT.begin(), pT.end());
             if (f + 1 < fk.nf && P.nball[f + 1] != nc) return IB_OK;   // one candidate count per field
         }
-        TRY(upload(tmp, mom, &o.mom));
-        TRY(upload(tmp, full, &o.full));
-        TRY(upload(tmp, phi, &o.phi));
-        TRY(upload(tmp, phiT, &o.phiT));
+        host.add(mom, &o.mom);
+        host.add(full, &o.full);
+        host.add(phi, &o.phi);
+        host.add(phiT, &o.phiT);
         // boundary-condition rows
         const HostTemplate ht = bc_template(fk.vector_bc, t->bc, d, Mp);
         o.nbc = (int)ht.rows.size();
@@ -1921,10 +1935,10 @@ static ib_status row_fit_tables(ib_table* t, const Geo& g, const FitKind& fk, co
             ++o.nrow;
         }
         if (o.nrow > 8 || o.nconst > 2) return IB_OK;
-        TRY(upload(tmp, pptr, &o.prog_ptr));
-        TRY(upload(tmp, prog, &o.prog));
-        TRY(upload(tmp, pc, &o.prog_c));
-        TRY(upload(tmp, crow, &o.crow));
+        host.add(pptr, &o.prog_ptr);
+        host.add(prog, &o.prog);
+        host.add(pc, &o.prog_c);
+        host.add(crow, &o.crow);
         R.bc_doubles = std::max(R.bc_doubles, (T + (o.nrow - (o.ident >= 0 ? 1 : 0)) * n) * RF_PITCH);
         // element list of the upper triangle
         std::vector<uint16_t> pair;
@@ -1943,10 +1957,10 @@ static ib_status row_fit_tables(ib_table* t, const Geo& g, const FitKind& fk, co
                 for (int c = 0; c < o.nconst; ++c) q += crow[(size_t)c * n + i] * crow[(size_t)c * n + j];
                 pconst.push_back(q);
             }
-        TRY(upload(tmp, pair, &o.pair));
-        TRY(upload(tmp, pgam, &o.pgam));
-        TRY(upload(tmp, pcoef, &o.pcoef));
-        TRY(upload(tmp, pconst, &o.pconst));
+        host.add(pair, &o.pair);
+        host.add(pgam, &o.pgam);
+        host.add(pcoef, &o.pcoef);
+        host.add(pconst, &o.pconst);
         // exterior stencil points
         std::vector<double> uE((size_t)P.rule.nE * n, 0.0);
         for (int e = 0; e < P.rule.nE; ++e) {
@@ -1962,7 +1976,7 @@ static ib_status row_fit_tables(ib_table* t, const Geo& g, const FitKind& fk, co
                 uE[(size_t)e * n + fi * T + k] = v;
             }
         }
-        TRY(upload(tmp, uE, &o.uE));
+        host.add(uE, &o.uE);
         std::vector<uint32_t> mono(T, 0);
         for (int k = 1; k < T; ++k) {
             int a = 2;
@@ -1972,7 +1986,7 @@ static ib_status row_fit_tables(ib_table* t, const Geo& g, const FitKind& fk, co
             mono[k] = (uint32_t)kid[b] | (uint32_t)a << 8 | (uint32_t)K[k][a] << 16 |
                       (uint32_t)(K[k][0] + K[k][1] + K[k][2]) << 24;
         }
-        TRY(upload(tmp, mono, &o.mono));
+        host.add(mono, &o.mono);
         for (int gi = 0; gi <= P.ngrow; ++gi) {
             const double r = o.r0 + 0.5 * gi;
             for (int a = 0; a < d; ++a) {
@@ -2036,6 +2050,7 @@ static ib_status run_fit(ib_table* t, const Geo& g, const FitKind& fk, const int
     int basis = t->opts.basis_order;
     std::vector<int> orders;
     for (int o = basis; o >= t->opts.min_order && (int)orders.size() < FIT_MAX_ORDERS; o -= 2) orders.push_back(o);
+    HostTables host;
     FitParams P;
     memset(&P, 0, sizeof P);
     P.g = g;
@@ -2071,23 +2086,14 @@ static ib_status run_fit(ib_table* t, const Geo& g, const FitKind& fk, const int
             terms.insert(terms.end(), row.begin(), row.end());
             rs.push_back((int32_t)terms.size());
         }
-        int8_t* dK;
-        int32_t* drs;
-        DevTerm* dterms;
-        TRY(tmp.alloc(&dK, (int64_t)kk.size()));
-        TRY(tmp.alloc(&drs, (int64_t)rs.size()));
-        TRY(tmp.alloc(&dterms, (int64_t)terms.size()));
-        IB_CUDA(cudaMemcpy(dK, kk.data(), kk.size(), cudaMemcpyHostToDevice));
-        IB_CUDA(cudaMemcpy(drs, rs.data(), rs.size() * 4, cudaMemcpyHostToDevice));
-        IB_CUDA(cudaMemcpy(dterms, terms.data(), terms.size() * sizeof(DevTerm), cudaMemcpyHostToDevice));
         OrderDesc& od = P.ord[oi];
+        host.add(kk, &od.K);
+        host.add(rs, &od.row_start);
+        host.add(terms, &od.terms);
         od.order = Mp;
         od.T = (int)K.size();
         od.nbc = (int)ht.rows.size();
         od.r0 = (t->opts.radius > 0.0 && oi == 0) ? t->opts.radius : (Mp + 1) / 2.0;
-        od.K = dK;
-        od.row_start = drs;
-        od.terms = dterms;
         rmax = std::max(rmax, od.r0 + 0.5 * P.ngrow);
         ncol_max = std::max(ncol_max, fk.nf * od.T);
     }
@@ -2104,14 +2110,8 @@ static ib_status run_fit(ib_table* t, const Geo& g, const FitKind& fk, const int
         std::vector<int8_t>& off = ball_off[f];
         std::vector<int32_t>& q = ball_q[f];
         make_ball(d, frac2, rmax, off, q);
-        int8_t* doff;
-        int32_t* dq;
-        TRY(tmp.alloc(&doff, (int64_t)off.size()));
-        TRY(tmp.alloc(&dq, (int64_t)q.size()));
-        IB_CUDA(cudaMemcpy(doff, off.data(), off.size(), cudaMemcpyHostToDevice));
-        IB_CUDA(cudaMemcpy(dq, q.data(), q.size() * 4, cudaMemcpyHostToDevice));
-        P.ball_off[f] = doff;
-        P.ball_q[f] = dq;
+        host.add(off, &P.ball_off[f]);
+        host.add(q, &P.ball_q[f]);
         P.nball[f] = (int)q.size();
     }
     // learned predictions of every row (checked inside k_fit)
@@ -2162,7 +2162,8 @@ static ib_status run_fit(ib_table* t, const Geo& g, const FitKind& fk, const int
     bool by_rows = false;
     int32_t* redo = nullptr;
     unsigned long long* queue = nullptr;   // next row; then the number of rows left to k_fit
-    if (nrows) TRY(row_fit_tables(t, g, fk, P, orders, ball_off, ball_q, bp_owner, nbp, R, s, tmp, &by_rows));
+    if (nrows) TRY(row_fit_tables(t, g, fk, P, orders, ball_off, ball_q, bp_owner, nbp, R, host, s, tmp, &by_rows));
+    TRY(host.send(tmp, s));
     if (by_rows) {
         TRY(tmp.alloc(&redo, nrows));
         TRY(tmp.alloc(&queue, 2));
@@ -2612,7 +2613,7 @@ static ib_status build_impl(const ib_grid* grid, const double* sdf, ib_bc bc, ib
         ib_table_free(t);
         return e;
     };
-    if (cudaMemcpyToSymbol(c_cfirst, cf, sizeof cf) != cudaSuccess) return fail(IB_ERR_CUDA);
+    if (cudaMemcpyToSymbolAsync(c_cfirst, cf, sizeof cf, 0, cudaMemcpyHostToDevice, s) != cudaSuccess) return fail(IB_ERR_CUDA);
     DevBuf tmp;
     // ---- boundary points
     uint8_t* flags;
