@@ -2145,14 +2145,15 @@ static ib_status run_fit(ib_table* t, const Geo& g, const FitKind& fk, const int
     TRY(tmp.alloc(&start, std::max<int64_t>(nrows, 1)));
     IB_CUDA(cudaMemsetAsync(cnt, 0, sizeof(int32_t) * std::max<int64_t>(nrows, 1), s));
     // room for every row's support at the first radius (a 3D order-8 row holds 64 entries of
-    // its 81 on average; the few rows that grow take what the cut supports leave): an
-    // overflow fits every row again
+    // its 81 on average; the few rows that grow take what the cut supports leave), and for 48
+    // entries a field where that radius holds fewer and most rows grow: an overflow fits every
+    // row again
     int64_t per_row = 0;
     for (int f = 0; f < fk.nf; ++f) {
         const int qlim = (int)floor(4.0 * P.ord[0].r0 * P.ord[0].r0 + 1e-9);
         for (int32_t q : ball_q[f]) per_row += q <= qlim;
     }
-    int64_t cap = std::max<int64_t>(nrows * per_row, 1024);
+    int64_t cap = std::max<int64_t>(nrows * std::max<int64_t>(per_row, 48 * fk.nf), 1024);
     int32_t* pool_code;
     int8_t* pool_field;
     double* pool_w;
