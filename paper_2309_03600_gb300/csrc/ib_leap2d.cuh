@@ -187,7 +187,10 @@ __device__ __noinline__ void leap_finish(Finish<T> a, Points<T, VX> v, int x, in
     for (int j = 0; j < VX; ++j) {
         if (x + j >= a.nx || marked(v.kh[j])) continue;
         T u = v.u[j];
-        if (a.src.n) u = add_rn(u, mul_rn(source_at(a.src, q + j), a.wv));   // the source term rounded by itself
+        if (a.src.n) {   // the source term rounded by itself; a wavelet that is not finite stays at its nodes
+            const T sw = source_at(a.src, q + j);
+            if (sw != (T)0) u = add_rn(u, mul_rn(sw, a.wv));
+        }
         if (a.damp) u -= a.damp[q + j] * (u - v.pm[j]);
         a.out[q + j] = u;
     }
@@ -496,7 +499,7 @@ __device__ __forceinline__ void leap_row(const StepArgs<T>& a, int64_t r, int64_
         for (int u = 0; u < U; ++u) {
             if (q[u] < 0) continue;
             T x = c[u] + ((c[u] - pmv[u]) + (kh[u] < (T)0 ? -kh[u] : kh[u]) * v[u]);
-            if (a.src.n) x = add_rn(x, mul_rn(sv[u], wv));
+            if (sv[u] != (T)0) x = add_rn(x, mul_rn(sv[u], wv));
             if (a.dw) x -= a.damp[q[u]] * (x - pmv[u]);
             out[q[u]] = x;
         }
@@ -1296,7 +1299,8 @@ __global__ void __launch_bounds__(RunShape<T, H, VX, RZ>::THREADS) k_leap2d_run(
                 if (slow) {
 #pragma unroll
                     for (int j = 0; j < VX; ++j) {
-                        u[k][j] = add_rn(u[k][j], mul_rn(gs[k * VX + j], wv));
+                        const T sw = gs[k * VX + j];
+                        if (sw != (T)0) u[k][j] = add_rn(u[k][j], mul_rn(sw, wv));
                         u[k][j] -= gd[k * VX + j] * (u[k][j] - pm[k][j]);
                     }
                 }

@@ -2398,7 +2398,7 @@ __global__ void __launch_bounds__(256) k_stag_p3d(const __grid_constant__ Stag3A
             if (a.src.idx[i] == q) sv += a.src.w[i];
         s = sum8(s);
         sv = sum8(sv);
-        if (act && gl == 0) a.p[q] = pq + (kq < (T)0 ? -kq : kq) * s + (a.src.n ? sv * a.wavelet[a.step] : (T)0);
+        if (act && gl == 0) a.p[q] = pq + (kq < (T)0 ? -kq : kq) * s + (sv != (T)0 ? sv * a.wavelet[a.step] : (T)0);
         return;
     }
     blk -= a.nrb[3];
@@ -2445,7 +2445,7 @@ __global__ void __launch_bounds__(256) k_stag_p3d(const __grid_constant__ Stag3A
             T sv = 0;
             for (int i = 0; i < 8 * a.src.n; ++i)
                 if (a.src.idx[i] == q + j) sv += a.src.w[i];
-            pp[j] += sv * a.wavelet[a.step];
+            if (sv != (T)0) pp[j] += sv * a.wavelet[a.step];
         }
     }
     store3<T, VX>(a.p + q, pp, kk, x, L.nx);
@@ -2690,7 +2690,7 @@ __global__ void __launch_bounds__(256) k_stag_p2d(const __grid_constant__ Stag2A
             if (a.src.idx[i] == q) sv += a.src.w[i];
         s = sum8(s);
         sv = sum8(sv);
-        if (act && gl == 0) a.p[q] = pq + (kq < (T)0 ? -kq : kq) * s + (a.src.n ? sv * a.wavelet[n] : (T)0);
+        if (act && gl == 0) a.p[q] = pq + (kq < (T)0 ? -kq : kq) * s + (sv != (T)0 ? sv * a.wavelet[n] : (T)0);
         return;
     }
     blk -= a.nrb[2];
@@ -2731,7 +2731,7 @@ __global__ void __launch_bounds__(256) k_stag_p2d(const __grid_constant__ Stag2A
             T sv = 0;
             for (int i = 0; i < 8 * a.src.n; ++i)
                 if (a.src.idx[i] == q + j) sv += a.src.w[i];
-            pp[j] += sv * a.wavelet[n];
+            if (sv != (T)0) pp[j] += sv * a.wavelet[n];
         }
     }
     store3<T, VX>(a.p + q, pp, kk, x, L.nx);
