@@ -984,6 +984,11 @@ __global__ void k_leap_coef(Layout L, const T* vel, const uint8_t* mask, double 
     }
 }
 
+// a staggered coefficient: its NaNs are not the marks of the row nodes (marked3)
+template <typename T>
+__device__ __forceinline__ T stag_coef(double v) {
+    return v == v ? (T)v : (T)__longlong_as_double(0x7ff8000000000000ll);
+}
 template <typename T>
 __global__ void k_stag_coef(Layout L, const T* vel, const T* rho, const uint8_t* mp, const uint8_t* mvx,
                             const uint8_t* mvz, double dt, double inv_h, T* kp, T* bx, T* bz) {
@@ -992,11 +997,11 @@ __global__ void k_stag_coef(Layout L, const T* vel, const T* rho, const uint8_t*
         int64_t q = L.idx(x, 0, z);
         double r0 = rho ? (double)rho[i] : 1.0;
         double c = (double)vel[i];
-        kp[q] = mp[q] ? (T)(dt * r0 * c * c * inv_h) : (T)0;
+        kp[q] = mp[q] ? stag_coef<T>(dt * r0 * c * c * inv_h) : (T)0;
         double rx = (rho && x + 1 < L.nx) ? (double)rho[i + 1] : r0;
         double rz = (rho && z + 1 < L.nz) ? (double)rho[i + L.nx] : r0;
-        bx[q] = mvx[q] ? (T)(dt * 0.5 * (1.0 / r0 + 1.0 / rx) * inv_h) : (T)0;
-        bz[q] = mvz[q] ? (T)(dt * 0.5 * (1.0 / r0 + 1.0 / rz) * inv_h) : (T)0;
+        bx[q] = mvx[q] ? stag_coef<T>(dt * 0.5 * (1.0 / r0 + 1.0 / rx) * inv_h) : (T)0;
+        bz[q] = mvz[q] ? stag_coef<T>(dt * 0.5 * (1.0 / r0 + 1.0 / rz) * inv_h) : (T)0;
     }
 }
 
@@ -2178,13 +2183,13 @@ __global__ void k_stag_coef3(Layout L, const T* vel, const T* rho, const uint8_t
         const int64_t q = L.idx(x, y, z);
         const double r0 = rho ? (double)rho[i] : 1.0;
         const double c = (double)vel[i];
-        kp[q] = mp[q] ? (T)(dt * r0 * c * c * inv_h) : (T)0;
+        kp[q] = mp[q] ? stag_coef<T>(dt * r0 * c * c * inv_h) : (T)0;
         const double rx = (rho && x + 1 < L.nx) ? (double)rho[i + 1] : r0;
         const double ry = (rho && y + 1 < L.ny) ? (double)rho[i + L.nx] : r0;
         const double rz = (rho && z + 1 < L.nz) ? (double)rho[i + L.nx * L.ny] : r0;
-        b0[q] = mv0[q] ? (T)(dt * 0.5 * (1.0 / r0 + 1.0 / rx) * inv_h) : (T)0;
-        b1[q] = mv1[q] ? (T)(dt * 0.5 * (1.0 / r0 + 1.0 / ry) * inv_h) : (T)0;
-        b2[q] = mv2[q] ? (T)(dt * 0.5 * (1.0 / r0 + 1.0 / rz) * inv_h) : (T)0;
+        b0[q] = mv0[q] ? stag_coef<T>(dt * 0.5 * (1.0 / r0 + 1.0 / rx) * inv_h) : (T)0;
+        b1[q] = mv1[q] ? stag_coef<T>(dt * 0.5 * (1.0 / r0 + 1.0 / ry) * inv_h) : (T)0;
+        b2[q] = mv2[q] ? stag_coef<T>(dt * 0.5 * (1.0 / r0 + 1.0 / rz) * inv_h) : (T)0;
     }
 }
 
@@ -2247,6 +2252,7 @@ template <typename T>
 struct Rows3D {
     int64_t n;
     const int64_t* pad;
+    const T* k;          // the row nodes' coefficients
     const int64_t* ptr[3];
     const int32_t* code[3];
     const T* w[3];
@@ -2258,7 +2264,7 @@ struct Stag3Args {
     T c[4];              // c[k - 1]: weight of the pair at offsets +(k - 1/2), -(k - 1/2)
     T* p;
     T* v[3];
-    const T* kp;         // sign bit of kp and b: a node of the modified rows
+    const T* kp;         // in kp and b, a mark (marked3) stands at the nodes of the modified rows
     const T* b[3];
     Rows3D<T> g[3];      // gradient rows of v_a (columns p: operator 0 of each)
     Rows3D<T> d;         // divergence rows (columns v_0, v_1, v_2)
@@ -2275,17 +2281,21 @@ struct Stag3Args {
 
 // Both kernels: column blocks of 256 threads own VX x-adjacent nodes per thread (16-byte
 // vectors) in a 32 VX x 8 x 1 box; row blocks update the nodes of the modified rows whole,
-// which the column blocks leave out (sign bit of their coefficient).  Two
+// which the column blocks leave out (a mark in place of their coefficient).  Two
 // launches per step: with one thread per node, a pass per operator over its rows, and
 // separate source and receiver launches a step had ten, and 64-bit divisions for every node.
 // 160 x 144 x 122, order 4, FP32: 172 -> 111 us a step (v 33, p 79; a whole warp per divergence
 // row: p 104).  The p rows, 3 gathers of about 60 entries each, bound it by instruction issue.
 static const int S3_ROWS = 32;   // rows per row block, 8 lanes each
 
-template <typename T>
-__device__ __forceinline__ bool marked3(T k) {
-    return sizeof(T) == 8 ? __double2hiint((double)k) < 0 : __float_as_int((float)k) < 0;
-}
+// The mark of a row node in a coefficient field: a NaN of a bit pattern of its own (coefficients
+// have either sign, a negative density's are negative).
+static const uint32_t MARK3_32 = 0x7fc5a3c1u;
+static const uint64_t MARK3_64 = 0x7ffd5a3c00000000ull;
+__device__ __forceinline__ bool marked3(float k) { return __float_as_uint(k) == MARK3_32; }
+__device__ __forceinline__ bool marked3(double k) { return __double2hiint(k) == (int)(MARK3_64 >> 32); }
+__device__ __forceinline__ void set_mark3(float& k) { k = __uint_as_float(MARK3_32); }
+__device__ __forceinline__ void set_mark3(double& k) { k = __longlong_as_double((long long)MARK3_64); }
 template <typename T, int VX>
 __device__ __forceinline__ void load3(T (&d)[VX], const T* p) {
     typedef typename std::conditional<sizeof(T) == 4, float4, double2>::type V;
@@ -2323,14 +2333,14 @@ __global__ void __launch_bounds__(256) k_stag_v3d(const __grid_constant__ Stag3A
             const int64_t r = blk * S3_ROWS + (threadIdx.x >> 3);
             const bool act = r < R.n;
             const int64_t q = act ? R.pad[r] : L.base;
-            const T bq = gl == 0 ? a.b[ax][q] : (T)0, vq = gl == 0 ? a.v[ax][q] : (T)0;
+            const T bq = act && gl == 0 ? R.k[r] : (T)0, vq = gl == 0 ? a.v[ax][q] : (T)0;
             T s = row_gather3<T, 4>(R.code[0], R.w[0], act ? R.ptr[0][r] : 0, act ? R.ptr[0][r + 1] : 0, a.p, q, (int)L.px,
                                     (int)L.plane, gl);
 #pragma unroll
             for (int k = 1; k <= H; ++k)
                 if (gl == k) s += a.c[k - 1] * (a.p[q + k * st[ax]] - a.p[q - (k - 1) * st[ax]]);
             s = sum8(s);
-            if (act && gl == 0) a.v[ax][q] = vq + (bq < (T)0 ? -bq : bq) * s;
+            if (act && gl == 0) a.v[ax][q] = vq + bq * s;
             return;
         }
         blk -= a.nrb[ax];
@@ -2384,7 +2394,7 @@ __global__ void __launch_bounds__(256) k_stag_p3d(const __grid_constant__ Stag3A
         const int64_t r = blk * S3_ROWS + (threadIdx.x >> 3);
         const bool act = r < a.d.n;
         const int64_t q = act ? a.d.pad[r] : L.base;
-        const T kq = gl == 0 ? a.kp[q] : (T)0, pq = gl == 0 ? a.p[q] : (T)0;
+        const T kq = act && gl == 0 ? a.d.k[r] : (T)0, pq = gl == 0 ? a.p[q] : (T)0;
         T s = 0, sv = 0;
 #pragma unroll
         for (int ax = 0; ax < 3; ++ax) {
@@ -2398,7 +2408,7 @@ __global__ void __launch_bounds__(256) k_stag_p3d(const __grid_constant__ Stag3A
             if (a.src.idx[i] == q) sv += a.src.w[i];
         s = sum8(s);
         sv = sum8(sv);
-        if (act && gl == 0) a.p[q] = pq + (kq < (T)0 ? -kq : kq) * s + (sv != (T)0 ? sv * a.wavelet[a.step] : (T)0);
+        if (act && gl == 0) a.p[q] = pq + kq * s + (sv != (T)0 ? sv * a.wavelet[a.step] : (T)0);
         return;
     }
     blk -= a.nrb[3];
@@ -2451,12 +2461,25 @@ __global__ void __launch_bounds__(256) k_stag_p3d(const __grid_constant__ Stag3A
     store3<T, VX>(a.p + q, pp, kk, x, L.nx);
 }
 
+// the row nodes' coefficients in row order, and marks in their places
 template <typename T>
-__global__ void k_mark_rows3(int64_t n, const int64_t* __restrict__ pad, T* k) {
+__global__ void k_mark_rows3(int64_t n, const int64_t* __restrict__ pad, T* k, T* rk) {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const T v = k[pad[i]];
-        if (!marked3(v)) k[pad[i]] = -v;
+        rk[i] = k[pad[i]];
+        set_mark3(k[pad[i]]);
     }
+}
+template <typename T>
+static ib_status mark_rows3(const IbOp& op, T* k, const T** rk, Scratch& S) {
+    *rk = nullptr;
+    if (!op.nrows) return IB_OK;
+    T* r;
+    TRY(S.alloc(&r, op.nrows));
+    k_mark_rows3<T><<<grid1(op.nrows, 256), 256, 0, S.s>>>(op.nrows, op.row_pad, k, r);
+    IB_CHECK_LAUNCH("k_mark_rows3");
+    ib_count_launch("setup");
+    *rk = r;
+    return IB_OK;
 }
 
 template <typename T>
@@ -2512,11 +2535,7 @@ static ib_status forward_stag3(ib_table* t, const ib_shot* sh, double dt, int nt
             R.ptr[i] = op.row_ptr;
             R.w[i] = sizeof(T) == 8 ? (const T*)op.w64 : (const T*)op.w32;
             R.code[i] = op.col_code;
-            if (o < 4 && op.nrows) {
-                k_mark_rows3<T><<<grid1(op.nrows, 256), 256, 0, s>>>(op.nrows, op.row_pad, coef[o]);
-                IB_CHECK_LAUNCH("k_mark_rows3");
-                ib_count_launch("setup");
-            }
+            if (o < 4) TRY(mark_rows3<T>(op, coef[o], &R.k, S));
         }
         for (int o = 0; o < 4; ++o) a.nrb[o] = (int)((t->ops[o].nrows + S3_ROWS - 1) / S3_ROWS);
         a.nbx = (int)((L.nx + 32 * VX - 1) / (32 * VX));
@@ -2566,6 +2585,7 @@ template <typename T>
 struct Rows2D {
     int64_t n;
     const int64_t* pad;
+    const T* k;          // the row nodes' coefficients
     const int64_t* ptr[2];
     const int32_t* code[2];
     const T* w[2];
@@ -2576,7 +2596,7 @@ struct Stag2Args {
     T c[4];              // c[k - 1]: weight of the pair at offsets +(k - 1/2), -(k - 1/2)
     T* p;
     T* v[2];
-    const T* kp;         // sign bit of kp and b: a node of the modified rows
+    const T* kp;         // in kp and b, a mark (marked3) stands at the nodes of the modified rows
     const T* b[2];
     Rows2D<T> g[2];      // gradient rows of v_x, v_z
     Rows2D<T> d;         // divergence rows (columns v_x, v_z)
@@ -2621,14 +2641,14 @@ __global__ void __launch_bounds__(256) k_stag_v2d(const __grid_constant__ Stag2A
             const int64_t r = blk * S3_ROWS + (threadIdx.x >> 3), st = ax ? L.px : 1;
             const bool act = r < R.n;
             const int64_t q = act ? R.pad[r] : L.base;
-            const T bq = gl == 0 ? a.b[ax][q] : (T)0, vq = gl == 0 ? a.v[ax][q] : (T)0;
+            const T bq = act && gl == 0 ? R.k[r] : (T)0, vq = gl == 0 ? a.v[ax][q] : (T)0;
             T s = 0;
             if (act) s = row_gather2(R.code[0], R.w[0], R.ptr[0][r], R.ptr[0][r + 1], (const T*)a.p, q, L.px, gl);
 #pragma unroll
             for (int k = 1; k <= H; ++k)
                 if (gl == k) s += a.c[k - 1] * (a.p[q + k * st] - a.p[q - (k - 1) * st]);
             s = sum8(s);
-            if (act && gl == 0) a.v[ax][q] = vq + (bq < (T)0 ? -bq : bq) * s;
+            if (act && gl == 0) a.v[ax][q] = vq + bq * s;
             return;
         }
         blk -= a.nrb[ax];
@@ -2675,7 +2695,7 @@ __global__ void __launch_bounds__(256) k_stag_p2d(const __grid_constant__ Stag2A
         const int64_t r = blk * S3_ROWS + (threadIdx.x >> 3);
         const bool act = r < a.d.n;
         const int64_t q = act ? a.d.pad[r] : L.base;
-        const T kq = gl == 0 ? a.kp[q] : (T)0, pq = gl == 0 ? a.p[q] : (T)0;
+        const T kq = act && gl == 0 ? a.d.k[r] : (T)0, pq = gl == 0 ? a.p[q] : (T)0;
         T s = 0, sv = 0;
 #pragma unroll
         for (int ax = 0; ax < 2; ++ax) {
@@ -2690,7 +2710,7 @@ __global__ void __launch_bounds__(256) k_stag_p2d(const __grid_constant__ Stag2A
             if (a.src.idx[i] == q) sv += a.src.w[i];
         s = sum8(s);
         sv = sum8(sv);
-        if (act && gl == 0) a.p[q] = pq + (kq < (T)0 ? -kq : kq) * s + (sv != (T)0 ? sv * a.wavelet[n] : (T)0);
+        if (act && gl == 0) a.p[q] = pq + kq * s + (sv != (T)0 ? sv * a.wavelet[n] : (T)0);
         return;
     }
     blk -= a.nrb[2];
@@ -2805,11 +2825,7 @@ static ib_status forward_stag(ib_table* t, const ib_shot* sh, double dt, int nt,
         R.ptr[i] = op.row_ptr;
         R.code[i] = op.col_code;
         R.w[i] = sizeof(T) == 8 ? (const T*)op.w64 : (const T*)op.w32;
-        if (o < 3 && op.nrows) {
-            k_mark_rows3<T><<<grid1(op.nrows, 256), 256, 0, s>>>(op.nrows, op.row_pad, coef[o]);
-            IB_CHECK_LAUNCH("k_mark_rows3");
-            ib_count_launch("setup");
-        }
+        if (o < 3) TRY(mark_rows3<T>(op, coef[o], &R.k, S));
         if (o < 3) a.nrb[o] = (int)((op.nrows + S3_ROWS - 1) / S3_ROWS);
     }
     constexpr int VX = 16 / (int)sizeof(T);

@@ -1,5 +1,5 @@
 """GPU: inputs at the edge of what the time steps accept -- wavelets that are not
-finite touch the nodes they belong to and no others."""
+finite, negative densities.  Each touches the nodes it belongs to and no others."""
 import numpy as np
 import pytest
 import torch
@@ -79,3 +79,25 @@ def test_nonfinite_wavelet_stays_at_the_source_staggered(ndim, prec):
                         inputs.ricker(60.0, dt, 50, t0=0.0), float("inf"))
     assert np.abs(a[:, -1]).max() > 0
     assert np.isfinite(b).all() and np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("prec", [torch.float32, torch.float64])
+@pytest.mark.parametrize("ndim", [2, 3])
+def test_negative_density(ndim, prec):
+    """The pressure does not depend on the sign of a constant density: both coefficients change sign."""
+    h = 10.0
+    if ndim == 2:
+        sdf = inputs.flat_surface_sdf((133, 71), h, 10.3 * h)
+        src, rec = np.array([[60.5 * h, 31.5 * h]]), np.array([[x * h, 12 * h] for x in range(3, 130, 4)])
+    else:
+        sdf, zs = small_hills()
+        src = np.array([[20 * h, 17 * h, 26 * h]])
+        rec = np.array([[x * h, y * h, zs[y, x] + 2 * h] for x in range(4, 36, 5) for y in range(4, 32, 5)])
+    dt = 0.3 * h / 1800.0
+    t = ib.ib_build_stencils(cuda(sdf), h, "free", "staggered", 4)
+    wv = inputs.ricker(60.0, dt, 50, t0=0.0)
+    a, b = [ib.ib_forward(t, cuda(np.full(sdf.shape, 1800.0), prec), cuda(wv, prec), cuda(src), cuda(rec), dt, 50,
+                          rho=cuda(np.full(sdf.shape, r), prec)).double().cpu().numpy() for r in (1000.0, -1000.0)]
+    ib.ib_sync_status()
+    assert np.abs(a[:, -1]).max() > 0
+    assert np.array_equal(a, b)      # every product changes sign and nothing else
