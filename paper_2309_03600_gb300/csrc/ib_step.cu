@@ -980,7 +980,9 @@ __global__ void k_leap_coef(Layout L, const T* vel, const uint8_t* mask, double 
         int64_t x = i % L.nx, r = i / L.nx, y = r % L.ny, z = r / L.ny;
         int64_t q = L.idx(x, y, z);
         double c = (double)vel[i] * dt_over_h;
-        Kh[q] = mask[q] ? (T)(c * c) : (T)0;
+        c *= c;
+        if (!(c >= 0.0)) c = __longlong_as_double(0x7ff8000000000000ll);   // a NaN without the sign bit, the mark of a row node
+        Kh[q] = mask[q] ? (T)c : (T)0;
     }
 }
 

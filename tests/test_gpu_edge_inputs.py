@@ -1,5 +1,5 @@
-"""GPU: inputs at the edge of what the time steps accept -- wavelets that are not
-finite, negative densities.  Each touches the nodes it belongs to and no others."""
+"""GPU: inputs at the edge of what the time steps accept -- NaN velocities, wavelets that are
+not finite, negative densities.  Each touches the nodes it belongs to and no others."""
 import numpy as np
 import pytest
 import torch
@@ -17,6 +17,24 @@ def _flat(nx=161, nz=71, nt=60, M=8):
                                rec_x_cells=(4, nx - 5), rec_z_cells=13)
     w["wavelet"] = inputs.ricker(60.0, w["dt"], nt, t0=0.0)
     return w
+
+
+@pytest.mark.parametrize("prec", [torch.float32, torch.float64])
+@pytest.mark.parametrize("sign", [1.0, -1.0])
+@pytest.mark.parametrize("strip", [None, "0", "1"])
+def test_nan_velocity_is_reported(prec, sign, strip, monkeypatch):
+    """A NaN of either sign in the velocity, away from the surface, makes the run's field NaN."""
+    if strip:
+        monkeypatch.setenv("IB_STRIP", strip)
+    w = _flat()
+    t = ib.ib_build_stencils(cuda(w["sdf"]), w["h"], "free", "second", 8)
+    vel = cuda(w["vel"], prec)
+    vel[40, 30] = torch.copysign(torch.tensor(float("nan"), dtype=prec), torch.tensor(sign, dtype=prec))
+    ib.ib_forward(t, vel, cuda(w["wavelet"], prec), cuda(w["src"]), cuda(w["rec"]), w["dt"], 60)
+    with pytest.raises(ib.IbError) as e:
+        ib.ib_sync_status()
+    assert e.value.status == ib.IB_ERR_UNSTABLE
+    ib.ib_sync_status()
 
 
 def _last_sample(run, wavelet, bad):
