@@ -1476,6 +1476,8 @@ static cudaError_t launch_run_shape(RunArgs<T>& r, const RunPlan& p, cudaStream_
     r.cw = p.cw;
     r.a.ntx = (r.a.L.nx + 32 * VX - 1) / (32 * VX);
     void* args[] = {&r};
+    const char* coop = getenv("IB_COOP");   // IB_COOP=0: the answer where too few SMs are usable
+    if (coop && coop[0] == '0') return cudaErrorCooperativeLaunchTooLarge;
     return cudaLaunchCooperativeKernel((const void*)k_leap2d_run<T, H, VX, RZ>, dim3((unsigned)p.blocks), dim3(threads), args,
                                        sm, s);
 }
@@ -1487,10 +1489,12 @@ static cudaError_t launch_run_h(RunArgs<T>& r, const RunPlan& p, cudaStream_t s)
     }
     return cudaErrorInvalidValue;
 }
-// steps n0 .. n1 - 1; bar: a zeroed word of this launch
+// Steps n0 .. n1 - 1; bar: a zeroed word of this launch.  *refused: the device (or the part of
+// it that this context may use) cannot hold all blocks at once, nothing was launched, and the
+// caller takes the steps launch by launch.
 template <typename T>
 static ib_status launch_run(const StepArgs<T>& a, const RunPlan& p, int H, T* buf0, T* buf1, int64_t stride, int n0, int n1,
-                            unsigned* bar, cudaStream_t s) {
+                            unsigned* bar, bool* refused, cudaStream_t s) {
     RunArgs<T> r;
     memset(&r, 0, sizeof r);
     r.a = a;
@@ -1507,6 +1511,11 @@ static ib_status launch_run(const StepArgs<T>& a, const RunPlan& p, int H, T* bu
         else if (H == 3) e = launch_run_h<T, 3>(r, p, s);
         else e = launch_run_h<T, 4>(r, p, s);
     });
+    *refused = e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported || e == cudaErrorLaunchOutOfResources;
+    if (*refused) {
+        cudaGetLastError();
+        return IB_OK;
+    }
     if (e != cudaSuccess) return ib_cuda_fail(e, "k_leap2d_run", __FILE__, __LINE__);
     return IB_OK;
 }
@@ -2079,17 +2088,20 @@ static ib_status forward_2nd(ib_table* t, const ib_shot* sh, double dt, int nt, 
         const int64_t part = ckpt ? seg : probe ? STAB_BLOCK : nt;
         unsigned* bars;
         TRY(S.alloc(&bars, (nt + part - 1) / part, true));
-        for (; n0 < nt; n0 = (int)std::min<int64_t>(n0 + part, nt)) {
+        while (n0 < nt) {
             if (ckpt) {
                 T* slot = (T*)ckpt + (n0 / seg) * 2 * L.total;
                 IB_CUDA(cudaMemcpyAsync(slot, cur, sizeof(T) * L.total, cudaMemcpyDeviceToDevice, s));
                 IB_CUDA(cudaMemcpyAsync(slot + L.total, prev, sizeof(T) * L.total, cudaMemcpyDeviceToDevice, s));
             }
             const int n1 = (int)std::min<int64_t>(n0 + part, nt);
-            TRY(launch_run<T>(a, plan, H, cur, prev, 0, n0, n1, bars + n0 / part, s));
+            bool refused;
+            TRY(launch_run<T>(a, plan, H, cur, prev, 0, n0, n1, bars + n0 / part, &refused, s));
+            if (refused) break;   // the loop below
             if ((n1 - n0) & 1) std::swap(cur, prev);
             if (probe && n1 % STAB_BLOCK == 0)
                 TRY(probe_rescale<T>(probe, n1 / STAB_BLOCK, L.total, cur, prev, (T*)nullptr, s));
+            n0 = n1;
         }
     }
     for (int n = n0; n < nt; ++n) {
@@ -3137,8 +3149,9 @@ static ib_status adjoint_2nd(ib_table* t, const ib_shot* sh, double dt, int nt, 
         // segment slots j hold p^{c - 1 + j}
         IB_CUDA(cudaMemcpyAsync(segbuf, slot + L.total, sizeof(T) * L.total, cudaMemcpyDeviceToDevice, s));
         IB_CUDA(cudaMemcpyAsync(segbuf + L.total, slot, sizeof(T) * L.total, cudaMemcpyDeviceToDevice, s));
-        if (plan.blocks) TRY(launch_run<T>(fa, plan, H, segbuf, segbuf, L.total, (int)c, (int)e, bars + k, s));
-        else for (int64_t n = c; n < e; ++n) {
+        bool refused = !plan.blocks;
+        if (!refused) TRY(launch_run<T>(fa, plan, H, segbuf, segbuf, L.total, (int)c, (int)e, bars + k, &refused, s));
+        if (refused) for (int64_t n = c; n < e; ++n) {
             fa.p = segbuf + (n - c + 1) * L.total;
             fa.pm = segbuf + (n - c) * L.total;
             fa.out = segbuf + (n - c + 2) * L.total;
@@ -3804,11 +3817,10 @@ extern "C" ib_status ib_forward_noalloc(const ib_table* tc, const ib_shot* sh, d
     float* cur = p0;
     float* prev = p1;
     const RunPlan plan = run_plan<float>(L, H);
-    if (plan.blocks) {
-        TRY(launch_run<float>(a, plan, H, cur, prev, 0, 0, nt, bar, s));
-        if (nt & 1) std::swap(cur, prev);
-    }
-    for (int n = plan.blocks ? nt : 0; n < nt; ++n) {
+    bool refused = !plan.blocks;
+    if (!refused) TRY(launch_run<float>(a, plan, H, cur, prev, 0, 0, nt, bar, &refused, s));
+    if (!refused && (nt & 1)) std::swap(cur, prev);
+    for (int n = refused ? 0 : nt; n < nt; ++n) {
         a.p = cur;
         a.pm = prev;
         a.out = prev;
