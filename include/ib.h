@@ -213,7 +213,9 @@ typedef struct {
  *   ckpt_dev   NULL, or device buffer of ib_checkpoint_bytes(table, precision,
  *              nt, n_ckpt) bytes that receives the wavefield checkpoints the
  *              adjoint needs (second-order form only); n_ckpt >= 1.
- * Errors: IB_ERR_ARG, IB_ERR_STATE, IB_ERR_OOM, IB_ERR_CUDA.
+ * Errors: IB_ERR_ARG, IB_ERR_STATE, IB_ERR_OOM, IB_ERR_CUDA; IB_ERR_TIMEOUT
+ * (3D FP32, which waits for its result; a 2D run only enqueues, and a wait that
+ * gave up in it is reported by ib_sync_status).
  */
 ib_status ib_forward(const ib_table* table, const ib_shot* shot, int32_t precision,
                      double dt, int32_t nt, void* ckpt_dev, int32_t n_ckpt, void* stream);
@@ -230,7 +232,8 @@ int64_t ib_checkpoint_bytes(const ib_table* table, int32_t precision, int32_t nt
  *   grad_vel_dev[x]     = dJ/dc(x)  (zero at exterior nodes), overwritten;
  *   grad_wavelet_dev[n] = dJ/dw[n]  if not NULL, overwritten.
  * The shot, dt, nt, precision and n_ckpt must be those of the ib_forward call
- * that filled ckpt_dev.  The shot's traces_dev is not read.
+ * that filled ckpt_dev.  The shot's traces_dev is not read.  Synchronises the
+ * stream; IB_ERR_TIMEOUT when a bounded wait of the recomputation gave up.
  */
 ib_status ib_adjoint(const ib_table* table, const ib_shot* shot, int32_t precision,
                      double dt, int32_t nt, const void* ckpt_dev, int32_t n_ckpt,
@@ -436,10 +439,12 @@ ib_status ib_profile_get(int32_t i, char* name, int32_t name_len, int64_t* launc
 /*
  * ib_selftest_bounded_wait -- diagnostics hook (no counterpart in the paper).
  * Runs one kernel that waits on a shared-memory barrier nothing will complete,
- * with the iteration bound the TMA step kernels use.  The wait gives up, the
- * kernel reports it, and the call returns IB_ERR_TIMEOUT with the context still
- * usable -- the path a stalled copy takes in ib_forward.  IB_OK would mean the
- * bound did not work.  Synchronises the stream.
+ * with the iteration bound the TMA step kernels use, and one whose blocks wait,
+ * with a short bound, for one arrival more than there are blocks at the barrier
+ * that the 2D runs in one launch use between steps.  The waits give up, the
+ * kernels report it, and the call returns IB_ERR_TIMEOUT with the context still
+ * usable -- the paths a stalled copy and a stalled block take in ib_forward.
+ * IB_OK would mean that a bound did not work.  Synchronises the stream.
  */
 ib_status ib_selftest_bounded_wait(void* stream);
 
@@ -448,8 +453,10 @@ ib_status ib_selftest_bounded_wait(void* stream);
  * error.  Every forward and adjoint run ends with a pass over its final
  * wavefields (gradients for the adjoint) that sets a per-device status word on
  * a NaN or Inf; this call then returns IB_ERR_UNSTABLE (the scheme blew up
- * for that model and time step) and clears the word.  The word is shared by
- * all streams of the device, so the report names no particular run.
+ * for that model and time step) and clears the word.  A 2D run in one launch
+ * whose wait between steps gave up sets the word too; this call then returns
+ * IB_ERR_TIMEOUT, and the results of that run are not valid.  The word is shared
+ * by all streams of the device, so the report names no particular run.
  */
 ib_status ib_sync_status(void* stream);
 

@@ -1103,7 +1103,8 @@ __global__ void k_unpad_grad(Layout L, const T* pad, const T* Kh, T two_dt_over_
 //   FP64, 201 x 201, order 4, 500 steps: 6.2 -> 1.97 ms.  A step is the barrier (about 1.5 us),
 // the halo's latency and, in FP64, 1.3 us of a pipe that issues a warp every 16 cycles.
 //   The barrier's wait is bounded (about a second): a block that gives up sets the device's
-// status word and leaves, and so do the others.
+// status word (ib_sync_status) and the call's word (the adjoint, which waits for its result,
+// returns IB_ERR_TIMEOUT) and leaves, and so do the others.
 // ---------------------------------------------------------------------------
 template <typename T>
 struct RunArgs {
@@ -1114,6 +1115,7 @@ struct RunArgs {
     int n0, n1;
     int cw;              // column warps per block
     unsigned* bar;       // barrier count, zero at launch
+    int* err;            // this call's word, set with the device's status word; or null
 };
 static const int STATUS_UNSTABLE = 1, STATUS_TIMEOUT = 2;
 static __device__ int g_dev_status;
@@ -1124,8 +1126,9 @@ __device__ __forceinline__ T* run_field(const RunArgs<T>& r, int n) {
     return ((n - r.n0) & 1) ? r.buf1 : r.buf0;
 }
 
-// all blocks of the launch; false when the wait gave up
-__device__ __forceinline__ bool grid_barrier(unsigned* bar, unsigned target, int* dead) {
+static const uint64_t BARRIER_LIMIT_NS = 1000000000ull;
+// all blocks of the launch; false when the wait gave up (after limit_ns)
+__device__ __forceinline__ bool grid_barrier(unsigned* bar, unsigned target, uint64_t limit_ns, int* dead) {
     __syncthreads();
     if (threadIdx.x == 0) {
         // the block's stores (ordered before by the barrier) are released with the arrival, and the
@@ -1140,15 +1143,18 @@ __device__ __forceinline__ bool grid_barrier(unsigned* bar, unsigned target, int
                 ok = true;
                 break;
             }
-            if ((it & 1023) == 1023 && global_ns() - t0 > 1000000000ull) break;
+            if ((it & 1023) == 1023 && global_ns() - t0 > limit_ns) break;
         }
-        if (!ok) {
-            atomicOr(&g_dev_status, STATUS_TIMEOUT);
-            *dead = 1;
-        }
+        if (!ok) *dead = 1;
     }
     __syncthreads();
     return *dead == 0;
+}
+// Self-test: every block arrives once and waits for target arrivals.
+__global__ void k_barrier_selftest(unsigned* bar, unsigned target, uint64_t limit_ns, int* gave_up) {
+    __shared__ int dead;
+    if (threadIdx.x == 0) dead = 0;
+    if (!grid_barrier(bar, target, limit_ns, &dead) && threadIdx.x == 0) atomicAdd(gave_up, 1);
 }
 
 // the shape's largest block: registers for VX x RZ points (c, p_prev, K, halo)
@@ -1356,7 +1362,13 @@ __global__ void __launch_bounds__(RunShape<T, H, VX, RZ>::THREADS) k_leap2d_run(
         }
         if (n + 1 < r.n1) {
             target += gridDim.x;
-            if (!grid_barrier(r.bar, target, &dead)) return;
+            if (!grid_barrier(r.bar, target, BARRIER_LIMIT_NS, &dead)) {
+                if (threadIdx.x == 0) {
+                    atomicOr(&g_dev_status, STATUS_TIMEOUT);
+                    if (r.err) atomicExch(r.err, 1);
+                }
+                return;
+            }
         }
     }
 }

@@ -1489,12 +1489,12 @@ static cudaError_t launch_run_h(RunArgs<T>& r, const RunPlan& p, cudaStream_t s)
     }
     return cudaErrorInvalidValue;
 }
-// Steps n0 .. n1 - 1; bar: a zeroed word of this launch.  *refused: the device (or the part of
+// Steps n0 .. n1 - 1; bar: a zeroed word of this launch; err: a zeroed word of the call, or null.  *refused: the device (or the part of
 // it that this context may use) cannot hold all blocks at once, nothing was launched, and the
 // caller takes the steps launch by launch.
 template <typename T>
 static ib_status launch_run(const StepArgs<T>& a, const RunPlan& p, int H, T* buf0, T* buf1, int64_t stride, int n0, int n1,
-                            unsigned* bar, bool* refused, cudaStream_t s) {
+                            unsigned* bar, int* err, bool* refused, cudaStream_t s) {
     RunArgs<T> r;
     memset(&r, 0, sizeof r);
     r.a = a;
@@ -1504,6 +1504,7 @@ static ib_status launch_run(const StepArgs<T>& a, const RunPlan& p, int H, T* bu
     r.n0 = n0;
     r.n1 = n1;
     r.bar = bar;
+    r.err = err;
     cudaError_t e = cudaSuccess;
     PROF_LAUNCH(kname<T>("leap2d_run_f32", "leap2d_run_f64"), s, {
         if (H == 1) e = launch_run_h<T, 1>(r, p, s);
@@ -2096,7 +2097,7 @@ static ib_status forward_2nd(ib_table* t, const ib_shot* sh, double dt, int nt, 
             }
             const int n1 = (int)std::min<int64_t>(n0 + part, nt);
             bool refused;
-            TRY(launch_run<T>(a, plan, H, cur, prev, 0, n0, n1, bars + n0 / part, &refused, s));
+            TRY(launch_run<T>(a, plan, H, cur, prev, 0, n0, n1, bars + n0 / part, nullptr, &refused, s));
             if (refused) break;   // the loop below
             if ((n1 - n0) & 1) std::swap(cur, prev);
             if (probe && n1 % STAB_BLOCK == 0)
@@ -3138,7 +3139,7 @@ static ib_status adjoint_2nd(ib_table* t, const ib_shot* sh, double dt, int nt, 
     const unsigned agrid = (unsigned)(aa.nrb + adj_blocks(ashape, L));
     const RunPlan plan = run_plan<T>(L, H);
     unsigned* bars;
-    TRY(S.alloc(&bars, n_ckpt, true));
+    TRY(S.alloc(&bars, (int64_t)n_ckpt + 1, true));   // one per segment, then the error word
     T* mu_a = mu1;   // mu^{m+1}
     T* mu_b = mu2;   // mu^{m+2}
     for (int k = n_ckpt - 1; k >= 0; --k) {
@@ -3150,7 +3151,7 @@ static ib_status adjoint_2nd(ib_table* t, const ib_shot* sh, double dt, int nt, 
         IB_CUDA(cudaMemcpyAsync(segbuf, slot + L.total, sizeof(T) * L.total, cudaMemcpyDeviceToDevice, s));
         IB_CUDA(cudaMemcpyAsync(segbuf + L.total, slot, sizeof(T) * L.total, cudaMemcpyDeviceToDevice, s));
         bool refused = !plan.blocks;
-        if (!refused) TRY(launch_run<T>(fa, plan, H, segbuf, segbuf, L.total, (int)c, (int)e, bars + k, &refused, s));
+        if (!refused) TRY(launch_run<T>(fa, plan, H, segbuf, segbuf, L.total, (int)c, (int)e, bars + k, (int*)(bars + n_ckpt), &refused, s));
         if (refused) for (int64_t n = c; n < e; ++n) {
             fa.p = segbuf + (n - c + 1) * L.total;
             fa.pm = segbuf + (n - c) * L.total;
@@ -3176,7 +3177,13 @@ static ib_status adjoint_2nd(ib_table* t, const ib_shot* sh, double dt, int nt, 
     IB_CHECK_LAUNCH("k_unpad");
     ib_count_launch("setup");
     TRY(check_finite<T>(L.N, grad_out, (const T*)nullptr, (const T*)nullptr, s));
+    int herr = 0;
+    IB_CUDA(cudaMemcpyAsync(&herr, bars + n_ckpt, sizeof(int), cudaMemcpyDeviceToHost, s));
     IB_CUDA(cudaStreamSynchronize(s));
+    if (herr) {
+        ib_set_error("a bounded wait between the steps of a 2D run timed out");
+        return IB_ERR_TIMEOUT;
+    }
     return IB_OK;
 }
 
@@ -3598,6 +3605,25 @@ extern "C" ib_status ib_adjoint_batch(const ib_table* const* tables, const ib_sh
     return IB_OK;
 }
 
+// the grid barrier with a target one arrival too high (every block gives up), and with the right one
+static ib_status selftest_barrier(Scratch& S, bool* ok) {
+    unsigned* w;
+    TRY(S.alloc(&w, 4, true));
+    for (int i = 0; i < 2; ++i) {
+        unsigned* bar = w + i;
+        unsigned target = i ? 4 : 5;
+        uint64_t limit = 20000000ull;
+        int* gave_up = (int*)(w + 2 + i);
+        void* args[] = {&bar, &target, &limit, &gave_up};
+        IB_CUDA(cudaLaunchCooperativeKernel((const void*)k_barrier_selftest, dim3(4), dim3(64), args, 0, S.s));
+    }
+    int h[2] = {0, 0};
+    IB_CUDA(cudaMemcpyAsync(h, w + 2, sizeof h, cudaMemcpyDeviceToHost, S.s));
+    IB_CUDA(cudaStreamSynchronize(S.s));
+    *ok = h[0] == 4 && h[1] == 0;
+    return IB_OK;
+}
+
 extern "C" ib_status ib_selftest_bounded_wait(void* stream) {
     ib_set_error("");
     cudaStream_t s = (cudaStream_t)stream;
@@ -3609,10 +3635,13 @@ extern "C" ib_status ib_selftest_bounded_wait(void* stream) {
     int h = 0;
     IB_CUDA(cudaMemcpyAsync(&h, err, sizeof(int), cudaMemcpyDeviceToHost, s));
     IB_CUDA(cudaStreamSynchronize(s));
-    if (h) {
-        ib_set_error("bounded device wait gave up (self-test: expected)");
+    bool barrier = false;
+    TRY(selftest_barrier(S, &barrier));
+    if (h && barrier) {
+        ib_set_error("bounded device waits gave up (self-test: expected): copy wait, grid barrier");
         return IB_ERR_TIMEOUT;
     }
+    ib_set_error(h ? "the grid barrier's bound did not work" : "the copy wait's bound did not work");
     return IB_OK;
 }
 
@@ -3818,7 +3847,7 @@ extern "C" ib_status ib_forward_noalloc(const ib_table* tc, const ib_shot* sh, d
     float* prev = p1;
     const RunPlan plan = run_plan<float>(L, H);
     bool refused = !plan.blocks;
-    if (!refused) TRY(launch_run<float>(a, plan, H, cur, prev, 0, 0, nt, bar, &refused, s));
+    if (!refused) TRY(launch_run<float>(a, plan, H, cur, prev, 0, 0, nt, bar, nullptr, &refused, s));
     if (!refused && (nt & 1)) std::swap(cur, prev);
     for (int n = refused ? 0 : nt; n < nt; ++n) {
         a.p = cur;

@@ -55,3 +55,16 @@ def test_refused_launch(prec, monkeypatch):
     assert p["leap2d_" + name]["launches"] == (440 if prec == torch.float32 else 380)
     for a, b in zip(got, ref):
         assert np.abs(b).max() > 0 and rel_l2(a, b) < tol
+
+
+def test_barrier_gives_up():
+    """The grid barrier with a target that is never reached: its blocks leave after the bound, the
+    host reads it, no run is reported as timed out, and the next run is right."""
+    w = _shot(129, 61, 8)
+    t = ib.ib_build_stencils(cuda(w["sdf"]), w["h"], "free", "second", 8)
+    args = (cuda(w["vel"]), cuda(w["wavelet"]), cuda(w["src"]), cuda(w["rec"]), w["dt"], 60)
+    ref = ib.ib_forward(t, *args)
+    assert ib.ib_selftest_bounded_wait() == ib.IB_ERR_TIMEOUT
+    assert "grid barrier" in ib.ib_last_error()
+    assert ib.ib_sync_status() == ib.IB_OK
+    assert torch.equal(ib.ib_forward(t, *args), ref)
