@@ -270,7 +270,8 @@ ib_status ib_forward_batch_ckpt(const ib_table* const* tables, const ib_shot* sh
  * ib_adjoint_batch -- ib_adjoint (same transpose, same checkpoint segments)
  * for many shots at once: every recompute step and every adjoint step is one
  * launch over the blocks of all shots, and the whole backward pass is one
- * captured graph.  Per shot i: checkpoints ckpts[i] from ib_forward_batch_ckpt
+ * captured graph (IB_BATCH_SHAPE fixes the recompute steps' blocks, as in
+ * ib_forward_batch).  Per shot i: checkpoints ckpts[i] from ib_forward_batch_ckpt
  * or ib_forward with the same dt, nt and n_ckpt; residuals[i] [nrec][nt];
  * grads[i] [N] receives dJ/dc (overwritten).  Host arrays of nshot device
  * pointers; FP32, 2D second-order tables sharing the space order; no wavelet

@@ -1467,6 +1467,11 @@ static RunPlan run_plan(const Layout& L, int H) {
     }
     return none;
 }
+// the plan of a forward or of a recomputation (IB_STRIP asks for launch by launch)
+template <typename T>
+static RunPlan run_plan_unless_forced(const Layout& L, int H) {
+    return strip_switch() < 0 ? run_plan<T>(L, H) : RunPlan{0, 0, 0, 0};
+}
 template <typename T, int H, int VX, int RZ>
 static cudaError_t launch_run_shape(RunArgs<T>& r, const RunPlan& p, cudaStream_t s) {
     const int threads = 32 * (p.cw + RUN_RW);
@@ -2082,8 +2087,7 @@ static ib_status forward_2nd(ib_table* t, const ib_shot* sh, double dt, int nt, 
     }
     // (the two-step kernel reads the coefficients unmarked)
     if (d == 2) TRY(mark_rows<T>(a.rows, Kh, s));
-    const char* forced = getenv("IB_STRIP");
-    const RunPlan plan = d == 2 && !(forced && *forced) && !tb_enabled() ? run_plan<T>(L, H) : RunPlan{0, 0, 0, 0};
+    const RunPlan plan = d == 2 && !tb_enabled() ? run_plan_unless_forced<T>(L, H) : RunPlan{0, 0, 0, 0};
     if (plan.blocks) {
         // up to the next checkpoint (or renormalisation of the probe) in one launch
         const int64_t part = ckpt ? seg : probe ? STAB_BLOCK : nt;
@@ -3137,7 +3141,7 @@ static ib_status adjoint_2nd(ib_table* t, const ib_shot* sh, double dt, int nt, 
     aa.ntx = adj_ntx(ashape, L);
     aa.nrb = row_blocks(aa.nt_rows + aa.n_inj, ashape ? 0 : 1);
     const unsigned agrid = (unsigned)(aa.nrb + adj_blocks(ashape, L));
-    const RunPlan plan = run_plan<T>(L, H);
+    const RunPlan plan = run_plan_unless_forced<T>(L, H);
     unsigned* bars;
     TRY(S.alloc(&bars, (int64_t)n_ckpt + 1, true));   // one per segment, then the error word
     T* mu_a = mu1;   // mu^{m+1}
@@ -3223,6 +3227,17 @@ static void launch_batch(int si, int H, const StepArgs<float>* args, const int64
         k_leap2d_batch<h.value, vx.value, rz.value>
             <<<(unsigned)nblk, LEAP_THREADS, sm, s>>>(args, tile0, shot_of, step, seg, kShapes[si].zc);
     });
+}
+
+// the shape by the batch's size; IB_BATCH_SHAPE=<index into kShapes> fixes it instead
+static ib_status batch_shape(int64_t points, int* si) {
+    *si = leap_shape(points);
+    const char* forced = getenv("IB_BATCH_SHAPE");
+    if (!forced || !*forced) return IB_OK;
+    *si = atoi(forced);
+    if (*si >= 0 && *si < kNumShapes) return IB_OK;
+    ib_set_error("IB_BATCH_SHAPE must name a shape index in [0, 10)");
+    return IB_ERR_ARG;
 }
 
 struct BatchSetup {
@@ -3327,16 +3342,8 @@ static ib_status forward_batch_impl(const ib_table* const* tables, const ib_shot
         TRY(setup_points<float>(ts[i], &shots[i], dt * dt / pow(ts[i]->grid.h, 2), S, geo[i]));
         total += L.N;
     }
-    // the shape by the batch's size; IB_BATCH_SHAPE=<index into kShapes> fixes it instead
-    int best = leap_shape(total);
-    const char* forced = getenv("IB_BATCH_SHAPE");
-    if (forced && *forced) {
-        best = atoi(forced);
-        if (best < 0 || best >= kNumShapes) {
-            ib_set_error("IB_BATCH_SHAPE must name a shape index in [0, 10)");
-            return IB_ERR_ARG;
-        }
-    }
+    int best;
+    TRY(batch_shape(total, &best));
     BatchSetup B;
     TRY(batch_prepare(ts.data(), shots, nshot, best, dt, nt, b0, b1, Kh, geo, S, B));
     // checkpoint copies (ib_forward's layout: slot k = [p^{k seg}, p^{k seg - 1}])
@@ -3480,7 +3487,9 @@ extern "C" ib_status ib_adjoint_batch(const ib_table* const* tables, const ib_sh
     std::vector<int64_t> tile0(nshot + 1, 0), stile0(nshot + 1, 0);
     int64_t points = 0;
     for (int i = 0; i < nshot; ++i) points += ts[i]->L.N;
-    const int fshape = leap_shape(points), ashape = adj_shape(points);
+    int fshape;
+    TRY(batch_shape(points, &fshape));
+    const int ashape = adj_shape(points);
     int64_t maxtot = 0;
     for (int i = 0; i < nshot; ++i) {
         ib_table* t = ts[i];
