@@ -68,3 +68,51 @@ def test_barrier_gives_up():
     assert "grid barrier" in ib.ib_last_error()
     assert ib.ib_sync_status() == ib.IB_OK
     assert torch.equal(ib.ib_forward(t, *args), ref)
+
+
+def _both(w, t, prec, nt, monkeypatch, **kw):
+    """The traces of the run in one launch, and of bursts launch by launch (held to the oracle elsewhere)."""
+    args = (t, cuda(w["vel"], prec), cuda(w["wavelet"], prec), cuda(w["src"]), cuda(w["rec"]), w["dt"], nt)
+    ib.ib_profile_enable(1)
+    a = ib.ib_forward(*args, **kw).double().cpu().numpy()
+    assert any(k.startswith("leap2d_run") for k in ib.ib_profile())
+    ib.ib_profile_enable(0)
+    monkeypatch.setenv("IB_STRIP", "0")
+    b = ib.ib_forward(*args, **kw).double().cpu().numpy()
+    ib.ib_sync_status()
+    assert np.abs(b[:, -1]).max() > 0
+    return a, b
+
+
+@pytest.mark.parametrize("nx,nz,M,damped", [(501, 403, 2, True), (499, 402, 4, False)])
+def test_four_points_a_thread_vs_oracle(nx, nz, M, damped, monkeypatch):
+    """FP32 grids beyond one point a thread."""
+    w, damp = _shot(nx, nz, M), ((12, 80.0) if damped else None)
+    ref = sim.Leapfrog(w["sdf"], w["vel"], w["h"], M, "free", w["dt"], w["src"], w["rec"], damp=damp).forward(w["wavelet"], 60)
+    t = ib.ib_build_stencils(cuda(w["sdf"]), w["h"], "free", "second", M)
+    a, b = _both(w, t, torch.float32, 60, monkeypatch, damp=damp)
+    assert rel_l2(a, ref) < TOL32 and rel_l2(b, ref) < TOL32
+
+
+@pytest.mark.parametrize("nx,nz,M,damped", [(601, 590, 8, True), (431, 777, 6, True)])
+def test_four_points_a_thread(nx, nz, M, damped, monkeypatch):
+    w = _shot(nx, nz, M)
+    t = ib.ib_build_stencils(cuda(w["sdf"]), w["h"], "free", "second", M)
+    a, b = _both(w, t, torch.float32, 60, monkeypatch, damp=(12, 80.0) if damped else None)
+    assert rel_l2(a, b) < TOL32
+
+
+@pytest.mark.parametrize("nx,nz,M,amp,wave,prec", [(2600, 40, 8, 2.2, 23.0, torch.float32),
+                                                   (2503, 30, 8, 2.2, 23.0, torch.float32),
+                                                   (4801, 29, 4, 3.0, 15.0, torch.float64)])
+def test_more_rows_than_a_block_holds(nx, nz, M, amp, wave, prec, monkeypatch):
+    """Wide shallow grids over a rough surface: more than 64 rows for every block a GPU of 152
+    SMs can have."""
+    w = _shot(nx, nz, M)
+    w["sdf"] = inputs.sinusoid_sdf(nx, nz, w["h"], z0=9.3 * w["h"], amp=amp * w["h"], wavelength=wave * w["h"])
+    w["src"][:, 1] = 20.5 * w["h"]
+    w["rec"][:, 1] = 14 * w["h"]
+    t = ib.ib_build_stencils(cuda(w["sdf"]), w["h"], "free", "second", M)
+    assert t.stats()["rows"][0] > 64 * 152
+    a, b = _both(w, t, prec, 40, monkeypatch)
+    assert rel_l2(a, b) < (TOL64 if prec == torch.float64 else TOL32)
