@@ -1666,6 +1666,13 @@ static ib_status excl_scan(const int64_t* in, int64_t* out, int64_t n, cudaStrea
     return IB_OK;
 }
 
+int ib_sm_count() {
+    int dev = 0, n = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        n = 1;
+    return n;
+}
+
 static int grid_for(int64_t n, int bs) {
     int64_t g = (n + bs - 1) / bs;
     if (g < 1) g = 1;
@@ -2024,7 +2031,7 @@ static ib_status launch_fit_rows(const FitParams& P, RowFit& R, cudaStream_t s) 
     IB_CUDA(cudaFuncSetAttribute(k_fit_rows<NMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
     int per_sm = 1;
     IB_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_fit_rows<NMAX>, 32, shm));
-    const int64_t blocks = std::min<int64_t>(P.nrows, (int64_t)152 * std::max(per_sm, 1));
+    const int64_t blocks = std::min<int64_t>(P.nrows, (int64_t)ib_sm_count() * std::max(per_sm, 1));
     k_fit_rows<NMAX><<<(unsigned)blocks, 32, shm, s>>>(P, R);
     IB_CHECK_LAUNCH("k_fit_rows");
     ib_count_launch("setup");
@@ -2480,7 +2487,6 @@ static void free_op(IbOp& op) {
     for (void* p : ps)
         if (p) cudaFree(p);
     for (auto& b : op.bins) ib_free_bins(b);
-    for (auto& b : op.t_bins) ib_free_bins(b);
     op = IbOp();
 }
 
@@ -3004,24 +3010,17 @@ static ib_status make_bins(const Layout& L, int64_t n, const int64_t* pad, const
     return IB_OK;
 }
 
-ib_status ib_table_bins(ib_table* t, int op, bool transposed, int tx, int ty, int tz, const TileBins** out,
-                        cudaStream_t s) {
+ib_status ib_table_bins(ib_table* t, int op, int tx, int ty, int tz, const TileBins** out, cudaStream_t s) {
     IbOp& o = t->ops[op];
-    std::vector<TileBins>& v = transposed ? o.t_bins : o.bins;
-    for (auto& b : v)
+    for (auto& b : o.bins)
         if (b.tx == tx && b.ty == ty && b.tz == tz) {
             *out = &b;
             return IB_OK;
         }
     TileBins b;
-    if (transposed) {
-        TRY(ib_table_transpose(t, op, s));
-        TRY(make_bins(t->L, o.t_nrows, o.t_row_pad, o.t_ptr, o.t_src_off, o.t_w64, tx, ty, tz, b, s));
-    } else {
-        TRY(make_bins(t->L, o.nrows, o.row_pad, o.row_ptr, o.col_pad, o.w64, tx, ty, tz, b, s, o.col_code));
-    }
-    v.push_back(b);
-    *out = &v.back();
+    TRY(make_bins(t->L, o.nrows, o.row_pad, o.row_ptr, o.col_pad, o.w64, tx, ty, tz, b, s, o.col_code));
+    o.bins.push_back(b);
+    *out = &o.bins.back();
     return IB_OK;
 }
 

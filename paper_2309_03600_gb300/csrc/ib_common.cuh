@@ -134,7 +134,6 @@ struct IbOp {
     int64_t* t_src_off = nullptr;  // padded offset from the column node to the row node
     double* t_w64 = nullptr;
     float* t_w32 = nullptr;
-    std::vector<TileBins> t_bins;
 };
 
 struct ib_table {
@@ -167,11 +166,11 @@ ib_status ib_mlp_predict_nodes(ib_mlp* m, const ib_grid* grid, const double* sdf
 ib_status ib_compact(const uint8_t* flags, int64_t n, int64_t** out, int64_t* count, cudaStream_t s);
 
 // implemented in ib_build.cu
-ib_status ib_table_bins(ib_table* t, int op, bool transposed, int tx, int ty, int tz,
-                        const TileBins** out, cudaStream_t s);
+ib_status ib_table_bins(ib_table* t, int op, int tx, int ty, int tz, const TileBins** out, cudaStream_t s);
 ib_status ib_table_transpose(ib_table* t, int op, cudaStream_t s);
 
 double ib_wall_seconds();
+int ib_sm_count();   // SMs of the current device
 
 // launch counting / sampled timing (ib_prof.cu)
 struct ProfToken {

@@ -1918,17 +1918,17 @@ static void launch_tb2(const TbArgs& a, int H, int R, dim3 grid, cudaStream_t s)
 
 // Planes per block of the FP32 3D step on 64 x 8 column tiles.  A block costs its planes and
 // about 10 more (the 2H planes read before the first, the ring's start, the tail); three run on
-// an SM, so the launch takes ceil(blocks / (3 x 152)) such times.  The even count that minimises
+// an SM, so the launch takes ceil(blocks / (3 SMs)) such times.  The even count that minimises
 // it: 64 at 512^2 x 384 (32 planes 328 us, 64 planes 324), 10 at 131 x 97 x 110, where 32
 // planes left two thirds of the block slots empty and the others marching (51 us; 4 planes 25,
 // 10 planes 24, 16 planes 31).
 static int z_planes(const Layout& L) {
-    const int64_t tiles = ((L.nx + 63) / 64) * ((L.ny + 7) / 8);
+    const int64_t tiles = ((L.nx + 63) / 64) * ((L.ny + 7) / 8), slots = 3 * (int64_t)ib_sm_count();
     int best = 32;
     int64_t cost = INT64_MAX;
     for (int zc = 4; zc <= 96; zc += 2) {
         const int64_t chunks = (L.nz + zc - 1) / zc;
-        const int64_t c = (tiles * chunks + 455) / 456 * (zc + 10);
+        const int64_t c = (tiles * chunks + slots - 1) / slots * (zc + 10);
         if (c < cost) {
             cost = c;
             best = zc;
@@ -1960,7 +1960,7 @@ static ib_status forward_2nd(ib_table* t, const ib_shot* sh, double dt, int nt, 
     Geom<T> g;
     TRY(setup_points<T>(t, sh, dt * dt / pow(t->grid.h, d), S, g));
     const TileBins* bins = nullptr;
-    if (d == 3) TRY(ib_table_bins(t, 0, false, 32, 8, 1, &bins, s));
+    if (d == 3) TRY(ib_table_bins(t, 0, 32, 8, 1, &bins, s));
     StepArgs<T> a;
     memset(&a, 0, sizeof a);
     a.L = L;
