@@ -1157,6 +1157,23 @@ struct Scratch {
     }
 };
 
+// Zeroed fields: parts of one allocation that was sized for all of them, or (at = null)
+// allocations of their own.
+struct Fields {
+    Scratch& S;
+    unsigned char* at = nullptr;
+    explicit Fields(Scratch& s) : S(s) {}
+    static int64_t bytes(int64_t n, size_t es) { return (n * (int64_t)es + 255) & ~(int64_t)255; }
+    ib_status reserve(int64_t b) { return S.alloc(&at, b, true); }
+    template <class T>
+    ib_status alloc(T** p, int64_t n) {
+        if (!at) return S.alloc(p, n, true);
+        *p = reinterpret_cast<T*>(at);
+        at += bytes(n, sizeof(T));
+        return IB_OK;
+    }
+};
+
 // power-iteration probe of ib_stability: random start, renormalisation every
 // STAB_BLOCK steps into slot k of the device arrays sums / logs
 static const int STAB_BLOCK = 50;
@@ -1429,12 +1446,12 @@ static void launch_leap2d(StepArgs<double>& a, int, int H, cudaStream_t s) {
 }
 // the absorbing layer's factor at every node (null without a layer)
 template <typename T>
-static ib_status damp_field(const Layout& L, int dw, T da, bool adjoint, Scratch& S, const T** out) {
+static ib_status damp_field(const Layout& L, int dw, T da, bool adjoint, Fields& F, const T** out) {
     *out = nullptr;
     if (!dw) return IB_OK;
     T* f;
-    TRY(S.alloc(&f, L.total, true));
-    k_damp_field<T><<<grid1(L.N, 256), 256, 0, S.s>>>(L, dw, da, adjoint, f);
+    TRY(F.alloc(&f, L.total));
+    k_damp_field<T><<<grid1(L.N, 256), 256, 0, F.S.s>>>(L, dw, da, adjoint, f);
     IB_CHECK_LAUNCH("k_damp_field");
     ib_count_launch("setup");
     *out = f;
@@ -1981,7 +1998,10 @@ static ib_status forward_2nd(ib_table* t, const ib_shot* sh, double dt, int nt, 
     T* cur = p0;   // p^n
     T* prev = p1;  // p^{n-1}
     const int shape = d == 2 ? leap_shape_shot(L) : 0;
-    if (d == 2) TRY(damp_field<T>(L, a.dw, a.da, false, S, &a.damp));
+    if (d == 2) {
+        Fields F(S);
+        TRY(damp_field<T>(L, a.dw, a.da, false, F, &a.damp));
+    }
     // two steps per launch (FP32 2D; not with checkpoints or the stability probe)
     int tbR = 0;
     TileBins tbb;
@@ -3024,7 +3044,8 @@ static ib_status build_injection(const PointSet<T>& rec, Scratch& S, AdjArgs<T>&
 // and of the receiver injection, their lists and the map between them.
 template <typename T>
 static ib_status adj_setup(ib_table* t, const ib_shot* sh, double dt, int nt, const PointSet<T>& rec,
-                           const PointSet<T>& src, const T* res, Scratch& S, AdjArgs<T>& a) {
+                           const PointSet<T>& src, const T* res, Fields& F, AdjArgs<T>& a) {
+    Scratch& S = F.S;
     const Layout& L = t->L;
     IbOp& op = t->ops[0];
     TRY(ib_table_transpose(t, 0, S.s));
@@ -3034,9 +3055,9 @@ static ib_status adj_setup(ib_table* t, const ib_shot* sh, double dt, int nt, co
     stencil_weights<T>(t->opts.space_order, a.w2, c1u);
     T* Kh;
     int32_t* map;
-    TRY(S.alloc(&Kh, L.total, true));
-    TRY(S.alloc(&map, L.total, true));
-    TRY(S.alloc(&a.grad, L.total, true));
+    TRY(F.alloc(&Kh, L.total));
+    TRY(F.alloc(&map, L.total));
+    TRY(F.alloc(&a.grad, L.total));
     k_leap_coef<T><<<grid1(L.N, 256), 256, 0, S.s>>>(L, (const T*)sh->vel_dev, t->mask_pad[0], dt / t->grid.h, Kh);
     IB_CHECK_LAUNCH("k_leap_coef");
     ib_count_launch("setup");
@@ -3057,7 +3078,7 @@ static ib_status adj_setup(ib_table* t, const ib_shot* sh, double dt, int nt, co
     a.src = src;
     a.wavelet = (const T*)sh->wavelet_dev;
     set_damping<T>(sh, dt, a.dw, a.da);
-    return damp_field<T>(L, a.dw, a.da, true, S, &a.damp);
+    return damp_field<T>(L, a.dw, a.da, true, F, &a.damp);
 }
 
 static const int kAdjRows = 32;   // rows a warp of the adjoint marches
@@ -3114,7 +3135,8 @@ static ib_status adjoint_2nd(ib_table* t, const ib_shot* sh, double dt, int nt, 
     Geom<T> g;
     TRY(setup_points<T>(t, sh, dt * dt / pow(t->grid.h, d), S, g));
     AdjArgs<T> aa;
-    TRY(adj_setup<T>(t, sh, dt, nt, g.rec, g.src, res, S, aa));
+    Fields F(S);
+    TRY(adj_setup<T>(t, sh, dt, nt, g.rec, g.src, res, F, aa));
     const int64_t seg = ckpt_seg(nt, n_ckpt);
     T* segbuf;
     TRY(S.alloc(&segbuf, (seg + 2) * L.total, true));
@@ -3135,7 +3157,7 @@ static ib_status adjoint_2nd(ib_table* t, const ib_shot* sh, double dt, int nt, 
     fa.rec_step = -1;
     fa.nt = nt;
     set_damping<T>(sh, dt, fa.dw, fa.da);
-    TRY(damp_field<T>(L, fa.dw, fa.da, false, S, &fa.damp));
+    TRY(damp_field<T>(L, fa.dw, fa.da, false, F, &fa.damp));
     aa.gw = gw;
     const int fshape = leap_shape_shot(L), ashape = sizeof(T) == 8 ? 0 : adj_shape(L.nx * L.nz);
     aa.ntx = adj_ntx(ashape, L);
@@ -3251,8 +3273,9 @@ struct BatchSetup {
 
 static ib_status batch_prepare(ib_table* const* ts, const ib_shot* shots, int nshot, int si, double dt, int nt,
                                const std::vector<float*>& buf0, const std::vector<float*>& buf1,
-                               const std::vector<float*>& Kh, const std::vector<Geom<float>>& geo, Scratch& S,
+                               const std::vector<float*>& Kh, const std::vector<Geom<float>>& geo, Fields& F,
                                BatchSetup& B) {
+    Scratch& S = F.S;
     B.args.assign(nshot, StepArgs<float>());
     B.tile0.assign(nshot + 1, 0);
     for (int i = 0; i < nshot; ++i) {
@@ -3273,7 +3296,7 @@ static ib_status batch_prepare(ib_table* const* ts, const ib_shot* shots, int ns
         a.buf0 = buf0[i];
         a.buf1 = buf1[i];
         set_damping<float>(&shots[i], dt, a.dw, a.da);
-        TRY(damp_field<float>(L, a.dw, a.da, false, S, &a.damp));
+        TRY(damp_field<float>(L, a.dw, a.da, false, F, &a.damp));
         a.ntx = shape_ntx(kShapes[si], L);
         a.nrb = row_blocks(a.rows.n, kShapes[si].rz);
         B.tile0[i + 1] = B.tile0[i] + a.nrb + shape_blocks(kShapes[si], L);
@@ -3329,11 +3352,17 @@ static ib_status forward_batch_impl(const ib_table* const* tables, const ib_shot
     std::vector<float*> b0(nshot), b1(nshot), Kh(nshot);
     std::vector<Geom<float>> geo(nshot);
     int64_t total = 0;
+    // all shots' fields in one allocation, zeroed at once (48 damped shots of 400-1200 squared, 6
+    // steps, set-up included: 9.7 ms with four allocations a shot, 8.7 with one for all)
+    Fields F(S);
+    int64_t need = 0;
+    for (int i = 0; i < nshot; ++i) need += (shot_damped(&shots[i]) ? 4 : 3) * Fields::bytes(ts[i]->L.total, 4);
+    TRY(F.reserve(need));
     for (int i = 0; i < nshot; ++i) {
         const Layout& L = ts[i]->L;
-        TRY(S.alloc(&b0[i], L.total, true));
-        TRY(S.alloc(&b1[i], L.total, true));
-        TRY(S.alloc(&Kh[i], L.total, true));
+        TRY(F.alloc(&b0[i], L.total));
+        TRY(F.alloc(&b1[i], L.total));
+        TRY(F.alloc(&Kh[i], L.total));
         k_leap_coef<float><<<grid1(L.N, 256), 256, 0, s>>>(L, (const float*)shots[i].vel_dev, ts[i]->mask_pad[0],
                                                            dt / ts[i]->grid.h, Kh[i]);
         IB_CHECK_LAUNCH("k_leap_coef");
@@ -3345,7 +3374,7 @@ static ib_status forward_batch_impl(const ib_table* const* tables, const ib_shot
     int best;
     TRY(batch_shape(total, &best));
     BatchSetup B;
-    TRY(batch_prepare(ts.data(), shots, nshot, best, dt, nt, b0, b1, Kh, geo, S, B));
+    TRY(batch_prepare(ts.data(), shots, nshot, best, dt, nt, b0, b1, Kh, geo, F, B));
     // checkpoint copies (ib_forward's layout: slot k = [p^{k seg}, p^{k seg - 1}])
     ShotCopy<float>* d_items = nullptr;
     int64_t seg = 0, maxtot = 0;
@@ -3491,14 +3520,22 @@ extern "C" ib_status ib_adjoint_batch(const ib_table* const* tables, const ib_sh
     TRY(batch_shape(points, &fshape));
     const int ashape = adj_shape(points);
     int64_t maxtot = 0;
+    // all shots' fields in one allocation: coefficients, multipliers, gradient and node map, the
+    // absorbing layer's two fields, and the segment
+    Fields F(S);
+    int64_t need = 0;
+    for (int i = 0; i < nshot; ++i)
+        need += (shot_damped(&shots[i]) ? 8 : 6) * Fields::bytes(ts[i]->L.total, 4) +
+                Fields::bytes((seg + 2) * ts[i]->L.total, 4);
+    TRY(F.reserve(need));
     for (int i = 0; i < nshot; ++i) {
         ib_table* t = ts[i];
         const Layout& L = t->L;
         float *Kh, *mu1, *mu2, *segbuf;
-        TRY(S.alloc(&Kh, L.total, true));
-        TRY(S.alloc(&mu1, L.total, true));
-        TRY(S.alloc(&mu2, L.total, true));
-        TRY(S.alloc(&segbuf, (seg + 2) * L.total, true));
+        TRY(F.alloc(&Kh, L.total));
+        TRY(F.alloc(&mu1, L.total));
+        TRY(F.alloc(&mu2, L.total));
+        TRY(F.alloc(&segbuf, (seg + 2) * L.total));
         k_leap_coef<float><<<grid1(L.N, 256), 256, 0, s>>>(L, (const float*)shots[i].vel_dev, t->mask_pad[0],
                                                            dt / t->grid.h, Kh);
         IB_CHECK_LAUNCH("k_leap_coef");
@@ -3519,12 +3556,12 @@ extern "C" ib_status ib_adjoint_batch(const ib_table* const* tables, const ib_sh
         fa.rec_step = -1;
         fa.nt = nt;
         set_damping<float>(&shots[i], dt, fa.dw, fa.da);
-        TRY(damp_field<float>(L, fa.dw, fa.da, false, S, &fa.damp));
+        TRY(damp_field<float>(L, fa.dw, fa.da, false, F, &fa.damp));
         fa.buf0 = segbuf;
         fa.ntx = shape_ntx(kShapes[fshape], L);
         fa.nrb = row_blocks(fa.rows.n, kShapes[fshape].rz);
         AdjArgs<float>& aa = aargs[i].a;
-        TRY(adj_setup<float>(t, &shots[i], dt, nt, g.rec, g.src, (const float*)residuals[i], S, aa));
+        TRY(adj_setup<float>(t, &shots[i], dt, nt, g.rec, g.src, (const float*)residuals[i], F, aa));
         aa.ntx = adj_ntx(ashape, L);
         aa.nrb = row_blocks(aa.nt_rows + aa.n_inj, ashape ? 0 : 1);
         aargs[i].mu1 = mu1;
