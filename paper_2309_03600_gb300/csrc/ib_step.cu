@@ -974,22 +974,35 @@ static void launch_leap3d_tma2(const StepArgs<float>& a, const CUtensorMap& tm, 
 // ---------------------------------------------------------------------------
 // setup kernels (coefficients formed in FP64, rounded once)
 // ---------------------------------------------------------------------------
+// a square without the sign bit that a NaN may carry (the mark of a row node); integer operations,
+// since the conversions keep the FP64 pipe busy as it is
+__device__ __forceinline__ float no_sign(float k) { return __uint_as_float(__float_as_uint(k) & 0x7fffffffu); }
+__device__ __forceinline__ double no_sign(double k) {
+    return __hiloint2double(__double2hiint(k) & 0x7fffffff, __double2loint(k));
+}
 template <typename T>
 __global__ void k_leap_coef(Layout L, const T* vel, const uint8_t* mask, double dt_over_h, T* Kh) {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < L.N; i += (int64_t)gridDim.x * blockDim.x) {
         int64_t x = i % L.nx, r = i / L.nx, y = r % L.ny, z = r / L.ny;
         int64_t q = L.idx(x, y, z);
         double c = (double)vel[i] * dt_over_h;
-        c *= c;
-        if (!(c >= 0.0)) c = __longlong_as_double(0x7ff8000000000000ll);   // a NaN without the sign bit, the mark of a row node
-        Kh[q] = mask[q] ? (T)c : (T)0;
+        Kh[q] = mask[q] ? no_sign((T)(c * c)) : (T)0;
     }
 }
 
-// a staggered coefficient: its NaNs are not the marks of the row nodes (marked3)
+// The mark of a row node in a staggered coefficient field: a NaN of a bit pattern of its own
+// (coefficients have either sign, a negative density's are negative).
+static const uint32_t MARK3_32 = 0x7fc5a3c1u;
+static const uint64_t MARK3_64 = 0x7ffd5a3c00000000ull;
+__device__ __forceinline__ bool marked3(float k) { return __float_as_uint(k) == MARK3_32; }
+__device__ __forceinline__ bool marked3(double k) { return __double2hiint(k) == (int)(MARK3_64 >> 32); }
+__device__ __forceinline__ void set_mark3(float& k) { k = __uint_as_float(MARK3_32); }
+__device__ __forceinline__ void set_mark3(double& k) { k = __longlong_as_double((long long)MARK3_64); }
+// a coefficient, whose own NaN is not that one (a conversion to FP32 gives the canonical NaN)
 template <typename T>
 __device__ __forceinline__ T stag_coef(double v) {
-    return v == v ? (T)v : (T)__longlong_as_double(0x7ff8000000000000ll);
+    if (sizeof(T) == 8 && marked3(v)) v = __longlong_as_double(0x7ff8000000000000ll);
+    return (T)v;
 }
 template <typename T>
 __global__ void k_stag_coef(Layout L, const T* vel, const T* rho, const uint8_t* mp, const uint8_t* mvx,
@@ -2327,14 +2340,6 @@ struct Stag3Args {
 // row: p 104).  The p rows, 3 gathers of about 60 entries each, bound it by instruction issue.
 static const int S3_ROWS = 32;   // rows per row block, 8 lanes each
 
-// The mark of a row node in a coefficient field: a NaN of a bit pattern of its own (coefficients
-// have either sign, a negative density's are negative).
-static const uint32_t MARK3_32 = 0x7fc5a3c1u;
-static const uint64_t MARK3_64 = 0x7ffd5a3c00000000ull;
-__device__ __forceinline__ bool marked3(float k) { return __float_as_uint(k) == MARK3_32; }
-__device__ __forceinline__ bool marked3(double k) { return __double2hiint(k) == (int)(MARK3_64 >> 32); }
-__device__ __forceinline__ void set_mark3(float& k) { k = __uint_as_float(MARK3_32); }
-__device__ __forceinline__ void set_mark3(double& k) { k = __longlong_as_double((long long)MARK3_64); }
 template <typename T, int VX>
 __device__ __forceinline__ void load3(T (&d)[VX], const T* p) {
     typedef typename std::conditional<sizeof(T) == 4, float4, double2>::type V;
