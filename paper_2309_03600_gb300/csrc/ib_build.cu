@@ -1771,8 +1771,8 @@ static ib_status pack_pool(ib_table* t, const FitKind& fk, const int64_t* rows, 
         int64_t nnz = 0;
         IB_CUDA(cudaMemcpy(&nnz, op.row_ptr + nrows, sizeof(int64_t), cudaMemcpyDeviceToHost));
         op.nnz = nnz;
-        TRY(dalloc(&op.col_code, nnz + 1));   // read in pairs: the last pair may end past nnz
-        TRY(dalloc(&op.col_pad, nnz));
+        TRY(dalloc(&op.col_code, nnz));
+        TRY(dalloc(&op.col_pad, nnz + 1));   // read in pairs: the last pair may end past nnz
         TRY(dalloc(&op.w64, nnz + 1));
         TRY(dalloc(&op.w32, nnz + 1));
         TRY(dalloc(&op.row_lin, nrows));
@@ -2499,11 +2499,11 @@ extern "C" void ib_table_free(ib_table* t) {
     delete t;
 }
 
-// 16-bit footprint codes of a 3D Laplacian's entries in row order, for the FP32 step's
-// correction pass.  Part of the construction: a table's first runs may come from several
-// streams, none of which may find half-filled codes.  A support that reaches beyond what a code
-// can name (16 nodes to one side of an axis, 15 to the other) leaves the table without them,
-// and its runs take the step that reads 32-bit offsets.
+// 16-bit footprint codes of the entries of a 3D table in row order, for the FP32 step's correction
+// pass and the rows of the staggered steps.  Part of the construction: a table's first runs may
+// come from several streams or be captured, and none may find half-filled codes.  An operator with a
+// support that reaches beyond what a code can name (16 nodes to one side of an axis, 15 to the
+// other) has none, and its runs take longer offsets.
 __global__ void k_code16(int64_t nnz, const int32_t* col_code, uint16_t* out, int* wide) {
     for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < nnz; j += (int64_t)gridDim.x * blockDim.x) {
         int dx, dy, dz;
@@ -2513,23 +2513,28 @@ __global__ void k_code16(int64_t nnz, const int32_t* col_code, uint16_t* out, in
     }
 }
 static ib_status build_code16(ib_table* t, cudaStream_t s, DevBuf& tmp) {
-    IbOp& o = t->ops[0];
-    if (o.nnz == 0) return IB_OK;
     int* wide;
-    int hwide = 0;
-    TRY(tmp.alloc(&wide, 1));
-    TRY(dalloc(&o.code16, o.nnz));
-    IB_CUDA(cudaMemsetAsync(wide, 0, sizeof(int), s));
-    k_code16<<<grid_for(o.nnz, 256), 256, 0, s>>>(o.nnz, o.col_code, o.code16, wide);
-    IB_CHECK_LAUNCH("k_code16");
-    ib_count_launch("setup");
-    IB_CUDA(cudaMemcpyAsync(&hwide, wide, sizeof(int), cudaMemcpyDeviceToHost, s));
+    int hwide[IB_MAX_OPS] = {0};
+    TRY(tmp.alloc(&wide, IB_MAX_OPS));
+    IB_CUDA(cudaMemsetAsync(wide, 0, sizeof hwide, s));
+    for (int i = 0; i < t->nops; ++i) {
+        IbOp& o = t->ops[i];
+        if (o.nnz == 0) continue;
+        TRY(dalloc(&o.code16, o.nnz + 1));   // read in pairs
+        k_code16<<<grid_for(o.nnz, 256), 256, 0, s>>>(o.nnz, o.col_code, o.code16, wide + i);
+        IB_CHECK_LAUNCH("k_code16");
+        ib_count_launch("setup");
+    }
+    IB_CUDA(cudaMemcpyAsync(hwide, wide, sizeof hwide, cudaMemcpyDeviceToHost, s));
     IB_CUDA(cudaStreamSynchronize(s));
-    if (hwide) {
-        cudaFree(o.code16);
-        o.code16 = nullptr;
-    } else {
-        t->table_bytes += 2 * o.nnz;
+    for (int i = 0; i < t->nops; ++i) {
+        IbOp& o = t->ops[i];
+        if (hwide[i]) {
+            cudaFree(o.code16);
+            o.code16 = nullptr;
+        } else if (o.nnz) {
+            t->table_bytes += 2 * o.nnz;
+        }
     }
     return IB_OK;
 }
@@ -2680,7 +2685,6 @@ static ib_status build_impl(const ib_grid* grid, const double* sdf, ib_bc bc, ib
             st = run_fit1d(t, g, fk, M, w2, s, tmp);
         else
             st = run_fit(t, g, fk, bp_index, bp_xb, bp_n, bplist, nbp, 0, s, tmp);
-        if (st == IB_OK && d == 3) st = build_code16(t, s, tmp);
         if (st != IB_OK) return fail(st);
     } else {
         std::vector<double> c1 = ib_staggered_first(M);
@@ -2729,6 +2733,7 @@ static ib_status build_impl(const ib_grid* grid, const double* sdf, ib_bc bc, ib
         fk.vector_bc = true;
         if ((st = run_fit(t, g, fk, bp_index, bp_xb, bp_n, bplist, nbp, d, s, tmp)) != IB_OK) return fail(st);
     }
+    if (d == 3 && (st = build_code16(t, s, tmp)) != IB_OK) return fail(st);
     if (cudaStreamSynchronize(s) != cudaSuccess) return fail(IB_ERR_CUDA);
     t->setup_seconds = ib_wall_seconds() - t0;
     *out = t;

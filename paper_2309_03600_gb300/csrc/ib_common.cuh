@@ -124,7 +124,7 @@ struct IbOp {
     double* w64 = nullptr;
     float* w32 = nullptr;
     int32_t* row_info = nullptr;  // [nrows][4]
-    uint16_t* code16 = nullptr;   // [nnz] pack_code16 footprint codes (3D Laplacian, where they fit)
+    uint16_t* code16 = nullptr;   // [nnz] pack_code16 footprint codes (3D, where they fit)
     std::vector<TileBins> bins;
     // transposed operator (adjoint): rows keyed by column node
     bool have_t = false;

@@ -2246,38 +2246,53 @@ __global__ void k_stag_coef3(Layout L, const T* vel, const T* rho, const uint8_t
 }
 
 // Lane gl of 8's share of sum_j w_j f[q + off_j] over the entries [j0, j1) of a 3D row: pairs
-// of adjacent entries (their codes and weights as one vector load each; a pair that straddles
-// the row's ends has the foreign weight dropped), U pairs in flight.
+// of adjacent entries (their columns and weights as one vector load each; a pair that straddles
+// the row's ends has the foreign weight dropped), U pairs in flight.  Columns are 16-bit footprint
+// codes, decoded mostly in 32-bit arithmetic against a base moved by the code's offset of 16 nodes
+// per axis, or, for a table that has none, padded offsets of 64 bits.  32-bit offsets, which need no
+// decoding but two more bytes an entry, took 5 % longer.  In FP64 the rounds past the end of the warp's
+// longest row are left out whole: an operation takes the pipe of an SM for 16 cycles whatever its
+// lanes do.
 template <typename T>
 struct PairOf;
 template <> struct PairOf<float> { typedef float2 type; };
 template <> struct PairOf<double> { typedef double2 type; };
-template <typename T, int U>
-__device__ __forceinline__ T row_gather3(const int32_t* __restrict__ code, const T* __restrict__ w, int64_t j0, int64_t j1,
+template <typename T, typename O, int U>
+__device__ __forceinline__ T row_gather3(const O* __restrict__ col, const T* __restrict__ w, int64_t j0, int64_t j1,
                                          const T* __restrict__ f, int64_t q, int px, int plane, int gl) {
-    typedef typename PairOf<T>::type V;
-    const T* base = f + q;
-    auto off = [&](int c) {   // unpack_off's bytes
-        return (int64_t)(int)(int8_t)(c >> 16) * plane + ((int)(int8_t)c + (int)(int8_t)(c >> 8) * px);
-    };
+    constexpr bool CODES = sizeof(O) == 2;
+    const int64_t centre = CODES ? 16 * ((int64_t)plane + px + 1) : 0;
+    const T* base = f + (q - centre);
+    const int64_t js = j0 & ~(int64_t)1;
+    const int most = sizeof(T) == 8 ? __reduce_max_sync(0xffffffffu, (int)(j1 - js)) : (int)(j1 - js);
     T v = 0;
-    for (int64_t j = (j0 & ~(int64_t)1) + 2 * gl; j < j1; j += 16 * U) {
+    for (int k = sizeof(T) == 8 ? 0 : 2 * gl; k < most; k += 16 * U) {
         T w0[U], w1[U], p0[U], p1[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            const int64_t e = j + 16 * u;
-            int64_t o0 = 0, o1 = 0;
+            if (sizeof(T) == 8 && k + 16 * u >= most) continue;   // warp-uniform
+            const int64_t e = js + k + 16 * u + (sizeof(T) == 8 ? 2 * gl : 0);
+            int64_t o0 = centre, o1 = centre;
             w0[u] = w1[u] = (T)0;
             if (e < j1) {
-                const int2 c = *reinterpret_cast<const int2*>(code + e);
-                const V ww = *reinterpret_cast<const V*>(w + e);
+                const typename PairOf<T>::type ww = *reinterpret_cast<const typename PairOf<T>::type*>(w + e);
+                int64_t c0, c1;
+                if constexpr (CODES) {
+                    const uint32_t c = *reinterpret_cast<const uint32_t*>(col + e);
+                    c0 = (int64_t)(int)((c >> 10) & 63) * plane + ((int)(c & 31) + (int)((c >> 5) & 31) * px);
+                    c1 = (int64_t)(int)(c >> 26) * plane + ((int)((c >> 16) & 31) + (int)((c >> 21) & 31) * px);
+                } else {
+                    const longlong2 c = *reinterpret_cast<const longlong2*>(col + e);
+                    c0 = c.x;
+                    c1 = c.y;
+                }
                 if (e >= j0) {
                     w0[u] = ww.x;
-                    o0 = off(c.x);
+                    o0 = c0;
                 }
                 if (e + 1 < j1) {
                     w1[u] = ww.y;
-                    o1 = off(c.y);
+                    o1 = c1;
                 }
             }
             p0[u] = base[o0];
@@ -2285,11 +2300,20 @@ __device__ __forceinline__ T row_gather3(const int32_t* __restrict__ code, const
         }
 #pragma unroll
         for (int u = 0; u < U; ++u) {
+            if (sizeof(T) == 8 && k + 16 * u >= most) continue;
             v += w0[u] * p0[u];
             v += w1[u] * p1[u];
         }
     }
     return v;
+}
+// c[k - 1] for a k that differs between lanes, without indexing the arguments
+template <int H, typename T>
+__device__ __forceinline__ T coef_at(const T* c, int k) {
+    T r = c[0];
+#pragma unroll
+    for (int j = 2; j <= H; ++j) r = j == k ? c[j - 1] : r;
+    return r;
 }
 template <typename T>
 __device__ __forceinline__ T sum8(T v) {
@@ -2306,7 +2330,7 @@ struct Rows3D {
     const int64_t* pad;
     const T* k;          // the row nodes' coefficients
     const int64_t* ptr[3];
-    const int32_t* code[3];
+    const void* col[3];  // the entries' columns: 16-bit codes or 64-bit offsets
     const T* w[3];
 };
 
@@ -2336,10 +2360,21 @@ struct Stag3Args {
 // which the column blocks leave out (a mark in place of their coefficient).  Two
 // launches per step: with one thread per node, a pass per operator over its rows, and
 // separate source and receiver launches a step had ten, and 64-bit divisions for every node.
-// 160 x 144 x 122, order 4, FP32: 172 -> 111 us a step (v 33, p 79; a whole warp per divergence
+// 160 x 144 x 122, order 4, FP32: 172 -> 108 us a step (v 31, p 74; a whole warp per divergence
 // row: p 104).  The p rows, 3 gathers of about 60 entries each, bound it by instruction issue.
+//   From 24 000 divergence rows on, orders 6 and 8 launch the two kinds of blocks one after the
+// other: in one kernel with columns of 100-127 registers a thread the rows' gathers have 16 warps on
+// an SM, alone 40 (FP32).  30 steps of order 8, ms, in one launch | apart | with ten launches:
+//   180 x 170 x 140   FP32 11.4 |  8.0 | 10.0    FP64 26.2 | 21.0 | 20.9
+//    60 x  60 x  80   FP32  1.6 |  1.8 |  2.6    FP64  2.7 |  3.4 |  5.1
+// In FP64 its pipe bounds the step, so vectors of nodes above the surface and idle rounds of the
+// gathers are left out.
 static const int S3_ROWS = 32;   // rows per row block, 8 lanes each
+static const int64_t S3_SPLIT_ROWS = 24000;   // divergence rows from which orders 6 and 8 take launches of their own
 
+// is any of a thread's coefficients not zero (integer operations)
+__device__ __forceinline__ bool nonzero(float k) { return (__float_as_uint(k) << 1) != 0u; }
+__device__ __forceinline__ bool nonzero(double k) { return ((__double2hiint(k) << 1) | __double2loint(k)) != 0; }
 template <typename T, int VX>
 __device__ __forceinline__ void load3(T (&d)[VX], const T* p) {
     typedef typename std::conditional<sizeof(T) == 4, float4, double2>::type V;
@@ -2361,16 +2396,21 @@ __device__ __forceinline__ void store3(T* p, const T (&d)[VX], const T (&k)[VX],
     }
 }
 
+// PART of a launch: row blocks and column blocks (S3_BOTH), or only the ones or the others; O: the
+// type of the entries' columns
+enum { S3_BOTH = 0, S3_ROWS_ONLY = 1, S3_COLUMNS = 2 };
+
 // v_a += b_a (forward-staggered d/dx_a p) at every interior v_a node
-template <typename T, int H>
+template <typename T, int H, int PART, typename O>
 __global__ void __launch_bounds__(256) k_stag_v3d(const __grid_constant__ Stag3Args<T, H> a) {
     constexpr int VX = 16 / (int)sizeof(T), HV = (H + VX - 1) / VX, HX = HV * VX;
     const Layout& L = a.L;
     int64_t blk = blockIdx.x;
-    record_receivers(a.rec, (const T*)a.p, a.traces, a.nt, a.rec_step, blk * 256 + threadIdx.x, (int64_t)gridDim.x * 256);
+    if (PART != S3_ROWS_ONLY)
+        record_receivers(a.rec, (const T*)a.p, a.traces, a.nt, a.rec_step, blk * 256 + threadIdx.x, (int64_t)gridDim.x * 256);
     const int64_t st[3] = {1, L.px, L.plane};
 #pragma unroll
-    for (int ax = 0; ax < 3; ++ax) {
+    for (int ax = 0; ax < 3 && PART != S3_COLUMNS; ++ax) {
         if (blk < a.nrb[ax]) {
             const Rows3D<T>& R = a.g[ax];
             const int gl = threadIdx.x & 7;
@@ -2378,17 +2418,21 @@ __global__ void __launch_bounds__(256) k_stag_v3d(const __grid_constant__ Stag3A
             const bool act = r < R.n;
             const int64_t q = act ? R.pad[r] : L.base;
             const T bq = act && gl == 0 ? R.k[r] : (T)0, vq = gl == 0 ? a.v[ax][q] : (T)0;
-            T s = row_gather3<T, 4>(R.code[0], R.w[0], act ? R.ptr[0][r] : 0, act ? R.ptr[0][r + 1] : 0, a.p, q, (int)L.px,
-                                    (int)L.plane, gl);
-#pragma unroll
-            for (int k = 1; k <= H; ++k)
-                if (gl == k) s += a.c[k - 1] * (a.p[q + k * st[ax]] - a.p[q - (k - 1) * st[ax]]);
+            T s = row_gather3<T, O, 4>((const O*)R.col[0], R.w[0], act ? R.ptr[0][r] : 0, act ? R.ptr[0][r + 1] : 0, a.p, q,
+                                       (int)L.px, (int)L.plane, gl);
+            T up = 0, dn = 0;   // lane k takes the stencil's pair k
+            if (gl >= 1 && gl <= H) {
+                up = a.p[q + gl * st[ax]];
+                dn = a.p[q - (gl - 1) * st[ax]];
+            }
+            s += coef_at<H>(a.c, gl) * (up - dn);
             s = sum8(s);
             if (act && gl == 0) a.v[ax][q] = vq + bq * s;
             return;
         }
         blk -= a.nrb[ax];
     }
+    if (PART == S3_ROWS_ONLY) return;
     const int lane = threadIdx.x & 31, wy = threadIdx.x >> 5;
     const int bx = (int)(blk % a.nbx), by = (int)(blk / a.nbx % a.nby);
     const int64_t z = blk / a.nbx / a.nby, x = ((int64_t)bx * 32 + lane) * VX, y = by * 8 + wy;
@@ -2407,6 +2451,14 @@ __global__ void __launch_bounds__(256) k_stag_v3d(const __grid_constant__ Stag3A
     for (int ax = 0; ax < 3; ++ax) {
         load3<T, VX>(vv[ax], a.v[ax] + q);
         load3<T, VX>(bb[ax], a.b[ax] + q);
+    }
+    if (sizeof(T) == 8) {   // the FP64 pipe bounds the step: leave out the nodes above the surface
+        bool any = false;
+#pragma unroll
+        for (int ax = 0; ax < 3; ++ax)
+#pragma unroll
+            for (int j = 0; j < VX; ++j) any = any || nonzero(bb[ax][j]);
+        if (!any) return;
     }
 #pragma unroll
     for (int j = 0; j < VX; ++j) {
@@ -2427,13 +2479,12 @@ __global__ void __launch_bounds__(256) k_stag_v3d(const __grid_constant__ Stag3A
 }
 
 // p += kp (backward-staggered divergence of v) + sources at every interior p node
-template <typename T, int H>
+template <typename T, int H, int PART, typename O>
 __global__ void __launch_bounds__(256) k_stag_p3d(const __grid_constant__ Stag3Args<T, H> a) {
     constexpr int VX = 16 / (int)sizeof(T), HV = (H + VX - 1) / VX, HX = HV * VX;
     const Layout& L = a.L;
     int64_t blk = blockIdx.x;
-    const int64_t st[3] = {1, L.px, L.plane};
-    if (blk < a.nrb[3]) {
+    if (PART == S3_ROWS_ONLY || (PART == S3_BOTH && blk < a.nrb[3])) {
         const int gl = threadIdx.x & 7;
         const int64_t r = blk * S3_ROWS + (threadIdx.x >> 3);
         const bool act = r < a.d.n;
@@ -2441,12 +2492,20 @@ __global__ void __launch_bounds__(256) k_stag_p3d(const __grid_constant__ Stag3A
         const T kq = act && gl == 0 ? a.d.k[r] : (T)0, pq = gl == 0 ? a.p[q] : (T)0;
         T s = 0, sv = 0;
 #pragma unroll
-        for (int ax = 0; ax < 3; ++ax) {
-            s += row_gather3<T, 4>(a.d.code[ax], a.d.w[ax], act ? a.d.ptr[ax][r] : 0, act ? a.d.ptr[ax][r + 1] : 0, a.v[ax],
-                                   q, (int)L.px, (int)L.plane, gl);
+        for (int ax = 0; ax < 3; ++ax)
+            s += row_gather3<T, O, 4>((const O*)a.d.col[ax], a.d.w[ax], act ? a.d.ptr[ax][r] : 0, act ? a.d.ptr[ax][r + 1] : 0,
+                                      a.v[ax], q, (int)L.px, (int)L.plane, gl);
 #pragma unroll
-            for (int k = 1; k <= H; ++k)
-                if (gl == ((ax * H + k) & 7)) s += a.c[k - 1] * (a.v[ax][q + (k - 1) * st[ax]] - a.v[ax][q - k * st[ax]]);
+        for (int i0 = 0; i0 < 3 * H; i0 += 8) {   // the 3 H pairs of the stencil, one a lane
+            const int i = i0 + gl, ax = i / H, k = i - ax * H + 1;
+            T up = 0, dn = 0;
+            if (i < 3 * H) {
+                const T* f = (ax == 0 ? a.v[0] : ax == 1 ? a.v[1] : a.v[2]) + q;
+                const int64_t d = ax == 0 ? 1 : ax == 1 ? L.px : L.plane;
+                up = f[(k - 1) * d];
+                dn = f[-k * d];
+            }
+            s += coef_at<H>(a.c, k) * (up - dn);
         }
         for (int i = gl; i < 8 * a.src.n; i += 8)
             if (a.src.idx[i] == q) sv += a.src.w[i];
@@ -2455,7 +2514,7 @@ __global__ void __launch_bounds__(256) k_stag_p3d(const __grid_constant__ Stag3A
         if (act && gl == 0) a.p[q] = pq + kq * s + (sv != (T)0 ? sv * a.wavelet[a.step] : (T)0);
         return;
     }
-    blk -= a.nrb[3];
+    if (PART == S3_BOTH) blk -= a.nrb[3];
     const int lane = threadIdx.x & 31, wy = threadIdx.x >> 5;
     const int bx = (int)(blk % a.nbx), by = (int)(blk / a.nbx % a.nby);
     const int64_t z = blk / a.nbx / a.nby, x = ((int64_t)bx * 32 + lane) * VX, y = by * 8 + wy;
@@ -2485,6 +2544,12 @@ __global__ void __launch_bounds__(256) k_stag_p3d(const __grid_constant__ Stag3A
         here = __syncthreads_or(here);
     }
     if (!in) return;
+    if (sizeof(T) == 8) {
+        bool any = false;
+#pragma unroll
+        for (int j = 0; j < VX; ++j) any = any || nonzero(kk[j]);
+        if (!any) return;
+    }
 #pragma unroll
     for (int j = 0; j < VX; ++j) {
         T s = 0;
@@ -2569,6 +2634,10 @@ static ib_status forward_stag3(ib_table* t, const ib_shot* sh, double dt, int nt
         a.b[0] = b0;
         a.b[1] = b1;
         a.b[2] = b2;
+        // IB_ROW_OFF64=1: 64-bit offsets, as where some operator's columns have no codes
+        const char* e64 = getenv("IB_ROW_OFF64");
+        bool wide = e64 && e64[0] == '1';
+        for (int o = 0; o < 6; ++o) wide = wide || (t->ops[o].nnz && !t->ops[o].code16);
         // operators 0-2: gradients; 3-5: the divergence's parts, on one set of rows
         for (int o = 0; o < 6; ++o) {
             const IbOp& op = t->ops[o];
@@ -2578,7 +2647,7 @@ static ib_status forward_stag3(ib_table* t, const ib_shot* sh, double dt, int nt
             R.pad = op.row_pad;
             R.ptr[i] = op.row_ptr;
             R.w[i] = sizeof(T) == 8 ? (const T*)op.w64 : (const T*)op.w32;
-            R.code[i] = op.col_code;
+            R.col[i] = wide ? (const void*)op.col_pad : (const void*)op.code16;
             if (o < 4) TRY(mark_rows3<T>(op, coef[o], &R.k, S));
         }
         for (int o = 0; o < 4; ++o) a.nrb[o] = (int)((t->ops[o].nrows + S3_ROWS - 1) / S3_ROWS);
@@ -2590,12 +2659,29 @@ static ib_status forward_stag3(ib_table* t, const ib_shot* sh, double dt, int nt
         a.traces = (T*)sh->traces_dev;
         a.nt = nt;
         const int64_t cols = (int64_t)a.nbx * a.nby * L.nz;
-        const unsigned gv = (unsigned)(cols + a.nrb[0] + a.nrb[1] + a.nrb[2]), gp = (unsigned)(cols + a.nrb[3]);
+        const unsigned rv = (unsigned)(a.nrb[0] + a.nrb[1] + a.nrb[2]), rp = (unsigned)a.nrb[3];
+        const bool split = wide || (HH > 2 && a.d.n >= S3_SPLIT_ROWS);
         for (int n = 0; n < nt; ++n) {
             a.step = n;
             a.rec_step = n - 1;
-            PROF_LAUNCH(kname<T>("stag_v3d_f32", "stag_v3d_f64"), s, { k_stag_v3d<T, HH><<<gv, 256, 0, s>>>(a); });
-            PROF_LAUNCH(kname<T>("stag_p3d_f32", "stag_p3d_f64"), s, { k_stag_p3d<T, HH><<<gp, 256, 0, s>>>(a); });
+            PROF_LAUNCH(kname<T>("stag_v3d_f32", "stag_v3d_f64"), s, {
+                if (!split) {
+                    k_stag_v3d<T, HH, S3_BOTH, uint16_t><<<(unsigned)cols + rv, 256, 0, s>>>(a);
+                } else {
+                    if (rv && wide) k_stag_v3d<T, HH, S3_ROWS_ONLY, int64_t><<<rv, 256, 0, s>>>(a);
+                    else if (rv) k_stag_v3d<T, HH, S3_ROWS_ONLY, uint16_t><<<rv, 256, 0, s>>>(a);
+                    k_stag_v3d<T, HH, S3_COLUMNS, uint16_t><<<(unsigned)cols, 256, 0, s>>>(a);
+                }
+            });
+            PROF_LAUNCH(kname<T>("stag_p3d_f32", "stag_p3d_f64"), s, {
+                if (!split) {
+                    k_stag_p3d<T, HH, S3_BOTH, uint16_t><<<(unsigned)cols + rp, 256, 0, s>>>(a);
+                } else {
+                    if (rp && wide) k_stag_p3d<T, HH, S3_ROWS_ONLY, int64_t><<<rp, 256, 0, s>>>(a);
+                    else if (rp) k_stag_p3d<T, HH, S3_ROWS_ONLY, uint16_t><<<rp, 256, 0, s>>>(a);
+                    k_stag_p3d<T, HH, S3_COLUMNS, uint16_t><<<(unsigned)cols, 256, 0, s>>>(a);
+                }
+            });
             IB_CHECK_LAUNCH("3D staggered step");
         }
         if (g.rec.n) {

@@ -1,5 +1,6 @@
-"""GPU: the entry codes that the 3D steps read -- there from a table's first use, in whatever
-stream or capture that falls, and for supports wider than a 16-bit code can name."""
+"""GPU: the entry codes and offsets that the 3D steps read -- there from a table's first use, in
+whatever stream or capture that falls, for supports wider than a 16-bit code can name, and in 64
+bits."""
 import numpy as np
 import pytest
 import torch
@@ -114,4 +115,26 @@ def test_wide_supports_second_order():
     for prec, tol in ((torch.float64, TOL64), (torch.float32, TOL32)):
         tr = ib.ib_forward(t, cuda(vel, prec), cuda(wv, prec), cuda(src), cuda(rec), dt, 40)
         assert rel_l2(tr.double().cpu().numpy(), ref) < tol, prec
+    ib.ib_sync_status()
+
+
+@pytest.mark.parametrize("n,M", [((30, 28, 26), 2), ((30, 28, 26), 6), ((70, 25, 30), 8), ((88, 84, 30), 8)])
+def test_staggered_rows_in_launches_of_their_own(n, M, monkeypatch):
+    """Rows with 64-bit offsets, in launches of their own, against the default: in one launch with
+    the columns on the small grids, in launches of their own from 24 000 divergence rows on."""
+    sdf, zs = small_hills(nx=n[0], ny=n[1], nz=n[2])
+    h, nt = 10.0, 40
+    dt = 0.3 * h / 1800.0
+    src = np.array([[(n[0] // 2 + 0.5) * h, n[1] // 2 * h, (n[2] - 7) * h]])
+    rec = np.array([[x * h, y * h, zs[y, x] + 2 * h] for x in range(3, n[0] - 3, 4) for y in range(3, n[1] - 3, 4)])
+    t = ib.ib_build_stencils(cuda(sdf), h, "free", "staggered", M, allow_rank_failure=True)
+    assert (t.stats()["rows"][3] >= 24000) == (n[1] == 84)
+    for prec, tol in ((torch.float64, TOL64), (torch.float32, TOL32)):
+        args = (t, cuda(np.full(sdf.shape, 1800.0), prec), cuda(inputs.ricker(60.0, dt, nt, t0=0.0), prec), cuda(src), cuda(rec), dt, nt)
+        rho = cuda(np.full(sdf.shape, 1000.0), prec)
+        monkeypatch.delenv("IB_ROW_OFF64", raising=False)
+        a = ib.ib_forward(*args, rho=rho).double().cpu().numpy()
+        monkeypatch.setenv("IB_ROW_OFF64", "1")
+        b = ib.ib_forward(*args, rho=rho).double().cpu().numpy()
+        assert np.abs(a[:, -1]).max() > 0 and rel_l2(b, a) < tol, prec
     ib.ib_sync_status()
