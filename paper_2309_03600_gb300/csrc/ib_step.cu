@@ -1948,17 +1948,28 @@ static void launch_tb2(const TbArgs& a, int H, int R, dim3 grid, cudaStream_t s)
 
 // Planes per block of the FP32 3D step on 64 x 8 column tiles.  A block costs its planes and
 // about 10 more (the 2H planes read before the first, the ring's start, the tail); three run on
-// an SM, so the launch takes ceil(blocks / (3 SMs)) such times.  The even count that minimises
-// it: 64 at 512^2 x 384 (32 planes 328 us, 64 planes 324), 10 at 131 x 97 x 110, where 32
-// planes left two thirds of the block slots empty and the others marching (51 us; 4 planes 25,
-// 10 planes 24, 16 planes 31).
-static int z_planes(const Layout& L) {
+// an SM, so the launch takes ceil(blocks / (3 SMs)) such times, and half a one for the blocks
+// that hold a source and take longer.  The even count that minimises it: 48 at 512^2 x 384 (us per
+// step with its corrections: 32 planes 465, 48 planes 457, 64 planes 461), 10 at 131 x 97 x 110,
+// where 32 planes left two thirds of the block slots empty and the others marching (51 us; 4
+// planes 25, 10 planes 24, 16 planes 31); 30 at 500 x 73 x 300, whose 400 blocks of 60 planes
+// waited for the two sources' blocks (86 us; 32 planes 80).
+//   With the absorbing layer the blocks that reach it take about twice as long (a division a
+// point), so the slots free up at different times instead of in rounds: blocks / (3 SMs) times
+// the planes and 3.5 more (the fixed part is mostly hidden behind the other blocks of the SM), and
+// half a block's whole time as the tail.  us per step with its corrections, order 8, layer of 20
+// nodes, by this rule | by the rule without a layer | at 32 planes:
+//   200 x 180 x 160   94 | 107 |  96      401 x 478 x 182  334 | 400 | 339
+//   300 x 260 x 200  170 | 186 | 172      384 x 384 x 256  310 | 354 | 310
+//   500 x  73 x 300  124 | 142 | 132      512 x 512 x 384  650 | 664 | 644
+static int z_planes(const Layout& L, bool layer) {
     const int64_t tiles = ((L.nx + 63) / 64) * ((L.ny + 7) / 8), slots = 3 * (int64_t)ib_sm_count();
     int best = 32;
-    int64_t cost = INT64_MAX;
+    double cost = INFINITY;
     for (int zc = 4; zc <= 96; zc += 2) {
-        const int64_t chunks = (L.nz + zc - 1) / zc;
-        const int64_t c = (tiles * chunks + slots - 1) / slots * (zc + 10);
+        const int64_t blocks = tiles * ((L.nz + zc - 1) / zc);
+        const double c = layer ? (double)blocks / (double)slots * (zc + 3.5) + 0.5 * (zc + 10)
+                               : ((double)((blocks + slots - 1) / slots) + 0.5) * (zc + 10);
         if (c < cost) {
             cost = c;
             best = zc;
@@ -2037,7 +2048,7 @@ static ib_status forward_2nd(ib_table* t, const ib_shot* sh, double dt, int nt, 
     // FP32 3D: TMA, where the table's entries have 16-bit codes
     const bool use_tma = d == 3 && sizeof(T) == 4 && tma_enabled() && (t->ops[0].nnz == 0 || t->ops[0].code16);
     // planes per 3D block (IB_ZCHUNK overrides it for tuning)
-    int zchunk = use_tma ? z_planes(L) : 32;
+    int zchunk = use_tma ? z_planes(L, a.dw > 0) : 32;
     if (const char* e = getenv("IB_ZCHUNK")) zchunk = std::max(1, atoi(e));
     dim3 grid3((unsigned)((L.nx + 31) / 32), (unsigned)((L.ny + 7) / 8), (unsigned)((L.nz + zchunk - 1) / zchunk));
     const int64_t nty3 = (L.ny + 7) / 8;
