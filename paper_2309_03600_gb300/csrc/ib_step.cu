@@ -1362,7 +1362,8 @@ extern "C" int64_t ib_checkpoint_bytes(const ib_table* t, int32_t precision, int
     return (int64_t)n_ckpt * 2 * t->L.total * es;
 }
 
-// Shapes of the 2D steps: vx columns a thread; rz rows (burst) or a march of zc rows.
+// Shapes of the 2D steps: vx columns a thread; rz rows (burst) or a march of zc rows.  The rules
+// below take 0, 1, 3 and marches of 4-16 rows; the others are there for IB_BATCH_SHAPE.
 struct LeapShape {
     int vx, rz, zc;
 };
@@ -1385,25 +1386,42 @@ static int strip_switch() {
     const char* e = getenv("IB_STRIP");
     return e && *e ? e[0] != '0' : -1;
 }
-// Shape of a step over `points` grid points in one launch.  A small grid needs many threads
-// with little to do, a large one few instructions a point; the march has a floor of about 25 us
-// (its 8 dependent steps).  us per step, order 8, damped, set-up included (a launch takes the
-// host about 7):
+// Rows a warp marches, for `points` grid points in one launch: few rows make many short marches,
+// which fill the SMs and end together; a march's first step reads its 2H halo rows again, so long
+// ones move less.  The even count next to 3.2 sqrt(points / 10^6), 4 to 16; us per step, order 8:
+//   10^6 points, one shot  4.2   6.0   7.5  10.5  12.0  18.0  33.6   batch  3.0   5.5   8.3  13.3  28.9
+//   4 rows                                                                 21.5  33.4  53.7  80.7   162
+//   6 rows                16.4  20.5  26.5  36.9  41.3  57.6  98.5         22.2  32.8  52.2  74.4   147
+//   8 rows                18.3  20.8  24.4  35.0  39.0  54.1  92.5         24.0  33.2  51.4  71.9   140
+//   12 rows               22.3  22.9  26.6  33.1  37.3  51.2  88.3         27.5  36.7  53.0  73.4   136
+//   16 rows               26.9  28.8  30.5  35.0  37.4  51.9  88.0         31.8  39.9  55.7  77.3   138
+//   24 rows               35.7  37.8  38.8  43.1  44.4  53.4  88.6         42.5  48.1  63.9  83.2   142
+static int march_rows(int64_t points) {
+    const int r = 2 * (int)lrint(1.6 * sqrt(1e-6 * (double)points));
+    return std::min(std::max(r, 4), 16);
+}
+// Shape of a step over `points` grid points in one launch, for half-order H.  A small grid needs many threads
+// with little to do, a large one few instructions a point.  us per step, order 8, damped, set-up
+// included (a launch takes the host about 7):
 //   10^6 points        0.16   0.42   0.79   2.1    4.2    7.5   16.8   33.6
 //   burst 1 x 1         7.2    9.3   12.3   23.9   43.6   79.3   178    358
 //   burst 2 x 2         7.1    7.2    9.2   15.7   25.2   48.5   109    219
 //   burst 4 x 2         7.2    9.0    9.2   13.6   21.0   40.3    91    182
-//   march, 16 rows     25.5   25.6   25.4   27.0   27.8   38.1    77    147
-// Longer marches were slower at every size.  Batches cross at the same sizes: 12 shots with
-// 6.5 x 10^6 points 82 (burst 4 x 2) and 70, 48 shots with 28.9 x 10^6 points 353 and 226.
-static int leap_shape(int64_t points) {
-    if (points >= 6000000) return 4;
-    if (points >= 1200000) return 3;
-    return points >= 150000 ? 1 : 0;
+// The march, at the rows above, passes the burst of 4 x 2 the earlier the wider the stencil, whose
+// rows a burst reads again for every two it writes (us per step, burst and march; the
+// strips and tiles before them took 31 at 6.0 x 10^6 points of order 2 and 42 at 5.5 x 10^6 of order 8):
+//   order 8   2.2: 12.5, 14.3   3.0: 24.9, 21.5 (batch)   4.2: 18.4, 16.4   5.5: 43.7, 32.8 (batch)
+//   order 4   3.0: 17.4, 18.6   4.1: 23.0, 22.5   5.5: 28.8, 27.1   6.6: 39.2, 32.2 (batches)
+//   order 2   4.2: 12.1, 14.2   6.0: 14.9, 16.5   6.8: 17.9, 16.6   10.5: 32.9, 29.9
+static LeapShape leap_shape(int64_t points, int H) {
+    static const int64_t march_from[4] = {6600000, 4500000, 3600000, 3000000};
+    if (points >= march_from[H - 1]) return {4, 0, march_rows(points)};
+    return kShapes[points >= 1200000 ? 3 : points >= 150000 ? 1 : 0];
 }
-static int leap_shape_shot(const Layout& L) {
+static LeapShape leap_shape_shot(const Layout& L, int H) {
     const int f = strip_switch();
-    return f < 0 ? leap_shape(L.nx * L.nz) : f ? 4 : 1;
+    if (f < 0) return leap_shape(L.nx * L.nz, H);
+    return f ? LeapShape{4, 0, march_rows(L.nx * L.nz)} : kShapes[1];
 }
 
 template <typename T>
@@ -1423,8 +1441,7 @@ static void with_h(int H, F f) {
     else f(std::integral_constant<int, 4>(), vx, rz);
 }
 template <class F>
-static void with_shape(int si, int H, F f) {
-    const LeapShape& p = kShapes[si];
+static void with_shape(const LeapShape& p, int H, F f) {
     if (p.rz == 1) with_h<1, 1>(H, f);
     else if (p.vx == 2 && p.rz == 2) with_h<2, 2>(H, f);
     else if (p.vx == 2 && p.rz == 4) with_h<2, 4>(H, f);
@@ -1433,13 +1450,12 @@ static void with_shape(int si, int H, F f) {
 }
 
 // one step of one shot; a.nrb and a.ntx are set here
-static void launch_leap2d(StepArgs<float>& a, int si, int H, cudaStream_t s) {
-    const LeapShape& p = kShapes[si];
+static void launch_leap2d(StepArgs<float>& a, const LeapShape& p, int H, cudaStream_t s) {
     a.nrb = row_blocks(a.rows.n, p.rz);
     a.ntx = shape_ntx(p, a.L);
     const unsigned grid = (unsigned)(a.nrb + shape_blocks(p, a.L));
     PROF_LAUNCH(p.rz ? "leap2d_f32" : "leap2d_strip_f32", s, {
-        with_shape(si, H, [&](auto h, auto vx, auto rz) {
+        with_shape(p, H, [&](auto h, auto vx, auto rz) {
             constexpr size_t sm = leap_smem<h.value, rz.value>();
             if (sm > 48 * 1024)
                 cudaFuncSetAttribute(k_leap2d<float, h.value, vx.value, rz.value>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1448,7 +1464,7 @@ static void launch_leap2d(StepArgs<float>& a, int si, int H, cudaStream_t s) {
         });
     });
 }
-static void launch_leap2d(StepArgs<double>& a, int, int H, cudaStream_t s) {
+static void launch_leap2d(StepArgs<double>& a, const LeapShape&, int H, cudaStream_t s) {
     const LeapShape& p = kShapes[0];
     a.nrb = row_blocks(a.rows.n, p.rz);
     a.ntx = shape_ntx(p, a.L);
@@ -2021,7 +2037,7 @@ static ib_status forward_2nd(ib_table* t, const ib_shot* sh, double dt, int nt, 
     const int64_t seg = ckpt ? ckpt_seg(nt, n_ckpt) : 0;
     T* cur = p0;   // p^n
     T* prev = p1;  // p^{n-1}
-    const int shape = d == 2 ? leap_shape_shot(L) : 0;
+    const LeapShape shape = d == 2 ? leap_shape_shot(L, H) : kShapes[0];
     if (d == 2) {
         Fields F(S);
         TRY(damp_field<T>(L, a.dw, a.da, false, F, &a.damp));
@@ -3261,7 +3277,8 @@ static ib_status adjoint_2nd(ib_table* t, const ib_shot* sh, double dt, int nt, 
     set_damping<T>(sh, dt, fa.dw, fa.da);
     TRY(damp_field<T>(L, fa.dw, fa.da, false, F, &fa.damp));
     aa.gw = gw;
-    const int fshape = leap_shape_shot(L), ashape = sizeof(T) == 8 ? 0 : adj_shape(L.nx * L.nz);
+    const LeapShape fshape = leap_shape_shot(L, H);
+    const int ashape = sizeof(T) == 8 ? 0 : adj_shape(L.nx * L.nz);
     aa.ntx = adj_ntx(ashape, L);
     aa.nrb = row_blocks(aa.nt_rows + aa.n_inj, ashape ? 0 : 1);
     const unsigned agrid = (unsigned)(aa.nrb + adj_blocks(ashape, L));
@@ -3341,27 +3358,30 @@ extern "C" ib_status ib_adjoint(const ib_table* tc, const ib_shot* sh, int32_t p
 // batched shots: one launch per time step over the blocks of every shot, captured with all
 // nt steps into one CUDA graph
 // ---------------------------------------------------------------------------
-static void launch_batch(int si, int H, const StepArgs<float>* args, const int64_t* tile0, const int32_t* shot_of,
+static void launch_batch(const LeapShape& p, int H, const StepArgs<float>* args, const int64_t* tile0, const int32_t* shot_of,
                          int step, int seg, int64_t nblk, cudaStream_t s) {
-    with_shape(si, H, [&](auto h, auto vx, auto rz) {
+    with_shape(p, H, [&](auto h, auto vx, auto rz) {
         constexpr size_t sm = leap_smem<h.value, rz.value>();
         if (sm > 48 * 1024)
             cudaFuncSetAttribute(k_leap2d_batch<h.value, vx.value, rz.value>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)sm);
         k_leap2d_batch<h.value, vx.value, rz.value>
-            <<<(unsigned)nblk, LEAP_THREADS, sm, s>>>(args, tile0, shot_of, step, seg, kShapes[si].zc);
+            <<<(unsigned)nblk, LEAP_THREADS, sm, s>>>(args, tile0, shot_of, step, seg, p.zc);
     });
 }
 
 // the shape by the batch's size; IB_BATCH_SHAPE=<index into kShapes> fixes it instead
-static ib_status batch_shape(int64_t points, int* si) {
-    *si = leap_shape(points);
+static ib_status batch_shape(int64_t points, int H, LeapShape* p) {
+    *p = leap_shape(points, H);
     const char* forced = getenv("IB_BATCH_SHAPE");
     if (!forced || !*forced) return IB_OK;
-    *si = atoi(forced);
-    if (*si >= 0 && *si < kNumShapes) return IB_OK;
-    ib_set_error("IB_BATCH_SHAPE must name a shape index in [0, 10)");
-    return IB_ERR_ARG;
+    const int si = atoi(forced);
+    if (si < 0 || si >= kNumShapes) {
+        ib_set_error("IB_BATCH_SHAPE must name a shape index in [0, 10)");
+        return IB_ERR_ARG;
+    }
+    *p = kShapes[si];
+    return IB_OK;
 }
 
 struct BatchSetup {
@@ -3373,7 +3393,7 @@ struct BatchSetup {
     int64_t nblk = 0;
 };
 
-static ib_status batch_prepare(ib_table* const* ts, const ib_shot* shots, int nshot, int si, double dt, int nt,
+static ib_status batch_prepare(ib_table* const* ts, const ib_shot* shots, int nshot, const LeapShape& p, double dt, int nt,
                                const std::vector<float*>& buf0, const std::vector<float*>& buf1,
                                const std::vector<float*>& Kh, const std::vector<Geom<float>>& geo, Fields& F,
                                BatchSetup& B) {
@@ -3399,9 +3419,9 @@ static ib_status batch_prepare(ib_table* const* ts, const ib_shot* shots, int ns
         a.buf1 = buf1[i];
         set_damping<float>(&shots[i], dt, a.dw, a.da);
         TRY(damp_field<float>(L, a.dw, a.da, false, F, &a.damp));
-        a.ntx = shape_ntx(kShapes[si], L);
-        a.nrb = row_blocks(a.rows.n, kShapes[si].rz);
-        B.tile0[i + 1] = B.tile0[i] + a.nrb + shape_blocks(kShapes[si], L);
+        a.ntx = shape_ntx(p, L);
+        a.nrb = row_blocks(a.rows.n, p.rz);
+        B.tile0[i + 1] = B.tile0[i] + a.nrb + shape_blocks(p, L);
     }
     B.nblk = B.tile0[nshot];
     TRY(S.alloc(&B.d_args, nshot));
@@ -3473,8 +3493,8 @@ static ib_status forward_batch_impl(const ib_table* const* tables, const ib_shot
         TRY(setup_points<float>(ts[i], &shots[i], dt * dt / pow(ts[i]->grid.h, 2), S, geo[i]));
         total += L.N;
     }
-    int best;
-    TRY(batch_shape(total, &best));
+    LeapShape best;
+    TRY(batch_shape(total, H, &best));
     BatchSetup B;
     TRY(batch_prepare(ts.data(), shots, nshot, best, dt, nt, b0, b1, Kh, geo, F, B));
     // checkpoint copies (ib_forward's layout: slot k = [p^{k seg}, p^{k seg - 1}])
@@ -3559,7 +3579,7 @@ extern "C" ib_status ib_forward_batch_ckpt(const ib_table* const* tables, const 
 // backward pass (segment restore, batched recompute steps, batched adjoint steps)
 // ---------------------------------------------------------------------------
 // block maps: tile0 / shot_of of the adjoint steps, stile0 / sshot_of of the recompute steps
-static void launch_adj_batch(int H, int fshape, int ashape, const StepArgs<float>* fargs, const AdjBatch<float>* aargs,
+static void launch_adj_batch(int H, const LeapShape& fshape, int ashape, const StepArgs<float>* fargs, const AdjBatch<float>* aargs,
                              const ShotCopy<float>* rst, const int64_t* tile0, const int32_t* shot_of, int64_t nblk,
                              const int64_t* stile0, const int32_t* sshot_of, int64_t nsblk, dim3 cgrid, int nt, int64_t c,
                              int64_t e, int k, cudaStream_t s) {
@@ -3618,8 +3638,8 @@ extern "C" ib_status ib_adjoint_batch(const ib_table* const* tables, const ib_sh
     std::vector<int64_t> tile0(nshot + 1, 0), stile0(nshot + 1, 0);
     int64_t points = 0;
     for (int i = 0; i < nshot; ++i) points += ts[i]->L.N;
-    int fshape;
-    TRY(batch_shape(points, &fshape));
+    LeapShape fshape;
+    TRY(batch_shape(points, H, &fshape));
     const int ashape = adj_shape(points);
     int64_t maxtot = 0;
     // all shots' fields in one allocation: coefficients, multipliers, gradient and node map, the
@@ -3660,8 +3680,8 @@ extern "C" ib_status ib_adjoint_batch(const ib_table* const* tables, const ib_sh
         set_damping<float>(&shots[i], dt, fa.dw, fa.da);
         TRY(damp_field<float>(L, fa.dw, fa.da, false, F, &fa.damp));
         fa.buf0 = segbuf;
-        fa.ntx = shape_ntx(kShapes[fshape], L);
-        fa.nrb = row_blocks(fa.rows.n, kShapes[fshape].rz);
+        fa.ntx = shape_ntx(fshape, L);
+        fa.nrb = row_blocks(fa.rows.n, fshape.rz);
         AdjArgs<float>& aa = aargs[i].a;
         TRY(adj_setup<float>(t, &shots[i], dt, nt, g.rec, g.src, (const float*)residuals[i], F, aa));
         aa.ntx = adj_ntx(ashape, L);
@@ -3671,7 +3691,7 @@ extern "C" ib_status ib_adjoint_batch(const ib_table* const* tables, const ib_sh
         aargs[i].seg = segbuf;
         rst[i] = {(const float*)ckpts[i], nullptr, segbuf, L.total};
         tile0[i + 1] = tile0[i] + aa.nrb + adj_blocks(ashape, L);
-        stile0[i + 1] = stile0[i] + fa.nrb + shape_blocks(kShapes[fshape], L);
+        stile0[i + 1] = stile0[i] + fa.nrb + shape_blocks(fshape, L);
         maxtot = std::max(maxtot, L.total);
     }
     const int64_t nblk = tile0[nshot], nsblk = stile0[nshot];
@@ -3990,7 +4010,7 @@ extern "C" ib_status ib_forward_noalloc(const ib_table* tc, const ib_shot* sh, d
     a.nt = nt;
     a.rows = row_list<float>(t->ops[0]);
     TRY(mark_rows<float>(a.rows, Kh, s));
-    const int shape = leap_shape(L.nx * L.nz);
+    const LeapShape shape = leap_shape(L.nx * L.nz, H);
     float* cur = p0;
     float* prev = p1;
     const RunPlan plan = run_plan<float>(L, H);
