@@ -3199,35 +3199,48 @@ static ib_status adj_setup(ib_table* t, const ib_shot* sh, double dt, int nt, co
     return damp_field<T>(L, a.dw, a.da, true, F, &a.damp);
 }
 
-static const int kAdjRows = 32;   // rows a warp of the adjoint marches
-// Shape of an adjoint step over `points` grid points: 0 one point a thread, 1 a march of 128
-// columns.  Whole gradients, us per step: 2 shots (10^6 points) 86 and 144, 6 shots (3.5 x 10^6)
-// 223 and 265, 12 shots (6.5 x 10^6) 449 and 403, 24 shots (13 x 10^6) 854 and 686.
-static int adj_shape(int64_t points) {
+// Shape of an adjoint step over `points` grid points: one point a thread (zc = 0) or a march of
+// 128 columns and zc rows a warp.  A march's block holds three quarters of the warps that an SM
+// could and walks its rows one pair after the other, so few rows a warp (whose halo rows come
+// from the L2) keep the SMs full and end together: marches of 32 rows took 232 us where the
+// 64 x 8 tiles before them took about 170.  us per recompute and adjoint step of a batch, order 8
+// (order 4 has the same best rows):
+//   10^6 points          0.90   1.42   2.2    2.9    3.8    5.1    6.5    9.0   12.8   15.3
+//   one point a thread     41     58     90    126    171    234    284    380    530    627
+//   4 rows                 40     49     68     92    117    158    179    231    311    371
+//   6 rows                 42     52     71     94    116    162    180    228    308    364
+//   8 rows                 46     55     73     98    123    165    178    229    307    366
+//   12 rows                57     62     83    105    131    174    189    235    315    373
+//   32 rows               104    120    129    160    187    232    246    290    362    431
+struct AdjShape {
+    int zc;
+};
+static AdjShape adj_shape(int64_t points) {
     const int f = strip_switch();
-    return f < 0 ? points >= 5000000 : f;
+    if (f == 0 || (f < 0 && points < 1200000)) return {0};
+    return {points < 8000000 ? 6 : 8};
 }
-static int64_t adj_ntx(int si, const Layout& L) { return (L.nx + (si ? 128 : 32) - 1) / (si ? 128 : 32); }
-static int64_t adj_blocks(int si, const Layout& L) {
-    const int64_t rows = (int64_t)LEAP_WARPS * (si ? kAdjRows : 1);
-    return adj_ntx(si, L) * ((L.nz + rows - 1) / rows);
+static int64_t adj_ntx(AdjShape p, const Layout& L) { return (L.nx + (p.zc ? 128 : 32) - 1) / (p.zc ? 128 : 32); }
+static int64_t adj_blocks(AdjShape p, const Layout& L) {
+    const int64_t rows = (int64_t)LEAP_WARPS * (p.zc ? p.zc : 1);
+    return adj_ntx(p, L) * ((L.nz + rows - 1) / rows);
 }
 template <class F>
-static void with_adj_shape(int si, int H, F f) {
-    if (si == 0) with_h<1, 1>(H, f);
+static void with_adj_shape(AdjShape p, int H, F f) {
+    if (p.zc == 0) with_h<1, 1>(H, f);
     else with_h<4, 0>(H, f);
 }
 
-static void launch_adj2d(const AdjArgs<float>& a, int si, int H, unsigned grid, cudaStream_t s) {
-    with_adj_shape(si, H, [&](auto h, auto vx, auto rz) {
+static void launch_adj2d(const AdjArgs<float>& a, AdjShape p, int H, unsigned grid, cudaStream_t s) {
+    with_adj_shape(p, H, [&](auto h, auto vx, auto rz) {
         constexpr size_t sm = adj_smem<h.value, rz.value>();
         if (sm)
             cudaFuncSetAttribute(k_adj2d<float, h.value, vx.value, rz.value>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)sm);
-        k_adj2d<float, h.value, vx.value, rz.value><<<grid, LEAP_THREADS, sm, s>>>(a, kAdjRows);
+        k_adj2d<float, h.value, vx.value, rz.value><<<grid, LEAP_THREADS, sm, s>>>(a, p.zc);
     });
 }
-static void launch_adj2d(const AdjArgs<double>& a, int, int H, unsigned grid, cudaStream_t s) {
+static void launch_adj2d(const AdjArgs<double>& a, AdjShape, int H, unsigned grid, cudaStream_t s) {
     with_h<1, 1>(H, [&](auto h, auto, auto) { k_adj2d<double, h.value, 1, 1><<<grid, LEAP_THREADS, 0, s>>>(a, 0); });
 }
 
@@ -3278,9 +3291,9 @@ static ib_status adjoint_2nd(ib_table* t, const ib_shot* sh, double dt, int nt, 
     TRY(damp_field<T>(L, fa.dw, fa.da, false, F, &fa.damp));
     aa.gw = gw;
     const LeapShape fshape = leap_shape_shot(L, H);
-    const int ashape = sizeof(T) == 8 ? 0 : adj_shape(L.nx * L.nz);
+    const AdjShape ashape = sizeof(T) == 8 ? AdjShape{0} : adj_shape(L.nx * L.nz);
     aa.ntx = adj_ntx(ashape, L);
-    aa.nrb = row_blocks(aa.nt_rows + aa.n_inj, ashape ? 0 : 1);
+    aa.nrb = row_blocks(aa.nt_rows + aa.n_inj, ashape.zc ? 0 : 1);
     const unsigned agrid = (unsigned)(aa.nrb + adj_blocks(ashape, L));
     const RunPlan plan = run_plan_unless_forced<T>(L, H);
     unsigned* bars;
@@ -3579,7 +3592,7 @@ extern "C" ib_status ib_forward_batch_ckpt(const ib_table* const* tables, const 
 // backward pass (segment restore, batched recompute steps, batched adjoint steps)
 // ---------------------------------------------------------------------------
 // block maps: tile0 / shot_of of the adjoint steps, stile0 / sshot_of of the recompute steps
-static void launch_adj_batch(int H, const LeapShape& fshape, int ashape, const StepArgs<float>* fargs, const AdjBatch<float>* aargs,
+static void launch_adj_batch(int H, const LeapShape& fshape, AdjShape ashape, const StepArgs<float>* fargs, const AdjBatch<float>* aargs,
                              const ShotCopy<float>* rst, const int64_t* tile0, const int32_t* shot_of, int64_t nblk,
                              const int64_t* stile0, const int32_t* sshot_of, int64_t nsblk, dim3 cgrid, int nt, int64_t c,
                              int64_t e, int k, cudaStream_t s) {
@@ -3592,7 +3605,7 @@ static void launch_adj_batch(int H, const LeapShape& fshape, int ashape, const S
                 cudaFuncSetAttribute(k_adj2d_batch<h.value, vx.value, rz.value>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)sm);
             k_adj2d_batch<h.value, vx.value, rz.value><<<(unsigned)nblk, LEAP_THREADS, sm, s>>>(
-                aargs, tile0, shot_of, (int)m, (int)(m - c), nt, kAdjRows);
+                aargs, tile0, shot_of, (int)m, (int)(m - c), nt, ashape.zc);
         });
 }
 
@@ -3640,7 +3653,7 @@ extern "C" ib_status ib_adjoint_batch(const ib_table* const* tables, const ib_sh
     for (int i = 0; i < nshot; ++i) points += ts[i]->L.N;
     LeapShape fshape;
     TRY(batch_shape(points, H, &fshape));
-    const int ashape = adj_shape(points);
+    const AdjShape ashape = adj_shape(points);
     int64_t maxtot = 0;
     // all shots' fields in one allocation: coefficients, multipliers, gradient and node map, the
     // absorbing layer's two fields, and the segment
@@ -3685,7 +3698,7 @@ extern "C" ib_status ib_adjoint_batch(const ib_table* const* tables, const ib_sh
         AdjArgs<float>& aa = aargs[i].a;
         TRY(adj_setup<float>(t, &shots[i], dt, nt, g.rec, g.src, (const float*)residuals[i], F, aa));
         aa.ntx = adj_ntx(ashape, L);
-        aa.nrb = row_blocks(aa.nt_rows + aa.n_inj, ashape ? 0 : 1);
+        aa.nrb = row_blocks(aa.nt_rows + aa.n_inj, ashape.zc ? 0 : 1);
         aargs[i].mu1 = mu1;
         aargs[i].mu2 = mu2;
         aargs[i].seg = segbuf;
