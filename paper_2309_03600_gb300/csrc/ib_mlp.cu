@@ -682,6 +682,12 @@ extern "C" ib_status ib_mlp_create(const ib_mlp_config* cfg, ib_mlp** out) {
         ib_set_error("initialising the network failed");
         return fail(IB_ERR_CUDA);
     }
+    // the copies and memsets above went to the legacy stream, which a non-blocking stream's first
+    // use of the network is not ordered after
+    if (cudaStreamSynchronize(cudaStreamLegacy) != cudaSuccess) {
+        ib_set_error("initialising the network failed");
+        return fail(IB_ERR_CUDA);
+    }
     *out = m;
     return IB_OK;
 }

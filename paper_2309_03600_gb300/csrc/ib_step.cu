@@ -1921,6 +1921,8 @@ static ib_status tb_bins(ib_table* t, int R, TileBins* out, bool* ok) {
     ib_status st = up(&b.ent_ptr, ptr);
     if (st == IB_OK) st = up(&b.ent_loc, ecode);
     if (st == IB_OK) st = up(&b.ent_w32, ew);
+    // (legacy-stream copies, which a non-blocking stream's steps are not ordered after)
+    if (st == IB_OK && cudaStreamSynchronize(cudaStreamLegacy) != cudaSuccess) st = IB_ERR_CUDA;
     if (st != IB_OK) {
         ib_free_bins(b);
         return st;
