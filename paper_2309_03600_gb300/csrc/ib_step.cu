@@ -1305,8 +1305,8 @@ static ib_status check_shot(const ib_table* t, const ib_shot* sh, int precision,
         return IB_ERR_ARG;
     }
     if (sh->nsrc > 32) {
-        // the step kernels spread each source over its 8 interpolation corners with
-        // one thread per corner of a 256-thread block
+        // the 3D second-order and the two-step kernels spread each source over its 8
+        // interpolation corners with one thread per corner of a 256-thread block
         ib_set_error("at most 32 sources per shot");
         return IB_ERR_ARG;
     }
