@@ -17,7 +17,7 @@
 // barriers of its surface tiles.
 //
 // 48 damped shots of 400-1200 squared, order 8: 171 -> 135 us a step; 24 gradients of such
-// shots: 100.6 -> 90.1 ms; one of 613 x 487, order 4: 8.9 -> 4.5 ms.
+// shots: 99 -> 75 ms; one of 613 x 487, order 4: 8.4 -> 4.7 ms.
 #pragma once
 
 __device__ __forceinline__ uint64_t global_ns();
