@@ -2394,7 +2394,7 @@ struct Stag3Args {
 //   From 24 000 divergence rows on, orders 6 and 8 launch the two kinds of blocks one after the
 // other: in one kernel with columns of 100-127 registers a thread the rows' gathers have 16 warps on
 // an SM, alone 40 (FP32).  30 steps of order 8, ms, in one launch | apart | with ten launches:
-//   180 x 170 x 140   FP32 11.4 |  8.0 | 10.0    FP64 26.2 | 21.0 | 20.9
+//   180 x 170 x 140   FP32 11.4 |  7.8 | 10.0    FP64 26.2 | 21.0 | 20.9
 //    60 x  60 x  80   FP32  1.6 |  1.8 |  2.6    FP64  2.7 |  3.4 |  5.1
 // In FP64 its pipe bounds the step, so vectors of nodes above the surface and idle rounds of the
 // gathers are left out.
@@ -2449,12 +2449,19 @@ __global__ void __launch_bounds__(256) k_stag_v3d(const __grid_constant__ Stag3A
             const T bq = act && gl == 0 ? R.k[r] : (T)0, vq = gl == 0 ? a.v[ax][q] : (T)0;
             T s = row_gather3<T, O, 4>((const O*)R.col[0], R.w[0], act ? R.ptr[0][r] : 0, act ? R.ptr[0][r + 1] : 0, a.p, q,
                                        (int)L.px, (int)L.plane, gl);
-            T up = 0, dn = 0;   // lane k takes the stencil's pair k
-            if (gl >= 1 && gl <= H) {
-                up = a.p[q + gl * st[ax]];
-                dn = a.p[q - (gl - 1) * st[ax]];
+            // lane k takes the stencil's pair k; in FP64 all lanes in one operation
+            if constexpr (sizeof(T) == 8) {
+                T up = 0, dn = 0;
+                if (gl >= 1 && gl <= H) {
+                    up = a.p[q + gl * st[ax]];
+                    dn = a.p[q - (gl - 1) * st[ax]];
+                }
+                s += coef_at<H>(a.c, gl) * (up - dn);
+            } else {
+#pragma unroll
+                for (int k = 1; k <= H; ++k)
+                    if (gl == k) s += a.c[k - 1] * (a.p[q + k * st[ax]] - a.p[q - (k - 1) * st[ax]]);
             }
-            s += coef_at<H>(a.c, gl) * (up - dn);
             s = sum8(s);
             if (act && gl == 0) a.v[ax][q] = vq + bq * s;
             return;
@@ -2524,8 +2531,17 @@ __global__ void __launch_bounds__(256) k_stag_p3d(const __grid_constant__ Stag3A
         for (int ax = 0; ax < 3; ++ax)
             s += row_gather3<T, O, 4>((const O*)a.d.col[ax], a.d.w[ax], act ? a.d.ptr[ax][r] : 0, act ? a.d.ptr[ax][r + 1] : 0,
                                       a.v[ax], q, (int)L.px, (int)L.plane, gl);
+        if constexpr (sizeof(T) == 4) {
+            const int64_t st[3] = {1, L.px, L.plane};
 #pragma unroll
-        for (int i0 = 0; i0 < 3 * H; i0 += 8) {   // the 3 H pairs of the stencil, one a lane
+            for (int ax = 0; ax < 3; ++ax)
+#pragma unroll
+                for (int k = 1; k <= H; ++k)
+                    if (gl == ((ax * H + k) & 7))
+                        s += a.c[k - 1] * (a.v[ax][q + (k - 1) * st[ax]] - a.v[ax][q - k * st[ax]]);
+        }
+#pragma unroll
+        for (int i0 = 0; i0 < (sizeof(T) == 8 ? 3 * H : 0); i0 += 8) {   // the 3 H pairs of the stencil, one a lane
             const int i = i0 + gl, ax = i / H, k = i - ax * H + 1;
             T up = 0, dn = 0;
             if (i < 3 * H) {
